@@ -1,8 +1,13 @@
-"""ctypes binding of libmonarch_attn.so: argument marshalling only.
+"""Binding of libmonarch_attn.so: argument marshalling only.
 
 Every step of the method runs inside the library's CUDA kernels.  torch is used for device
 memory and streams.  If the shared library has not been built the binding raises; there is no
 CPU fallback.
+
+The device entry points go through the extension `_native` (csrc/py_native.cpp), which checks the
+tensors, allocates output and scratch and calls the library without the interpreter in between.  It
+declines (returns None) any call that is not as documented; the checks below then say what is wrong,
+and the ctypes functions remain for the queries and the host-buffer entry point.
 """
 from __future__ import annotations
 
@@ -30,6 +35,8 @@ _TORCH_TO_CODE = {torch.float32: MA_F32, torch.float16: MA_F16, torch.bfloat16: 
 _NAME_TO_TORCH = {"f32": torch.float32, "f16": torch.float16, "bf16": torch.bfloat16}
 
 _lib = None
+_run = None     # _native.run, once loaded
+_FWD, _EX, _PADDED, _VARLEN, _OBJECTIVE, _BSHD = range(6)      # ma::Entry of csrc/internal_api.h
 
 
 class MonarchAttnError(RuntimeError):
@@ -87,6 +94,17 @@ def load_library(path: str = LIB_PATH):
     lib.monarch_attn_status_string.restype = ctypes.c_char_p
     _lib = lib
     return lib
+
+
+def _load_native():
+    global _run
+    load_library()
+    try:
+        from . import _native
+    except ImportError as e:
+        raise MonarchAttnError(-1, f"the extension _native does not load ({e}): build it with __graft_entry__.build()")
+    _run = _native.run
+    return _run
 
 
 def status_string(code: int) -> str:
@@ -170,6 +188,11 @@ def monarch_attn_workspace_bytes(batch, heads, N, d, b, T, dtype, path=MA_PATH_A
 def monarch_attn_fwd(Q, K, V, b, T, Y=None, stream=None):
     """Y = MonarchAttention(Q, K, V) with block size b, T steps, scale 1/sqrt(d).
     Q, K, V: CUDA tensors (batch, heads, N, d)."""
+    out = (_run or _load_native())(_FWD, Q, K, V, b, T, None, None, 0, None, Y, stream)
+    if out is not None:
+        if out.__class__ is int:
+            _check(out)
+        return out
     lib = load_library()
     if not Q.is_cuda:
         raise MonarchAttnError(-2, "monarch_attn_fwd needs CUDA tensors; there is no CPU path")
@@ -186,6 +209,11 @@ def monarch_attn_fwd_ex(Q, K, V, b, T, softmax_scale=None, path=MA_PATH_AUTO, wo
                         Y=None, stream=None):
     """As monarch_attn_fwd with explicit scale, path and (optionally) caller-owned workspace
     (a uint8 CUDA tensor).  Returns Y."""
+    out = (_run or _load_native())(_EX, Q, K, V, b, T, None, softmax_scale, path, workspace, Y, stream)
+    if out is not None:
+        if out.__class__ is int:
+            _check(out)
+        return out
     lib = load_library()
     if not Q.is_cuda:
         raise MonarchAttnError(-2, "monarch_attn_fwd_ex needs CUDA tensors; there is no CPU path")
@@ -206,6 +234,11 @@ def monarch_attn_fwd_objective(Q, K, V, b, T, softmax_scale=None, path=MA_PATH_A
                                Y=None, stream=None):
     """Forward pass plus the objective value: returns (Y, row_lse) with row_lse a float32 CUDA
     tensor [batch, heads, N]; row_lse.sum(-1) is f(M^(T)) of Eq. 6 per head."""
+    out = (_run or _load_native())(_OBJECTIVE, Q, K, V, b, T, None, softmax_scale, path, workspace, Y, stream)
+    if out is not None:
+        if out.__class__ is int:
+            _check(out)
+        return out
     lib = load_library()
     if not Q.is_cuda:
         raise MonarchAttnError(-2, "monarch_attn_fwd_objective needs CUDA tensors; there is no CPU path")
@@ -228,6 +261,11 @@ def monarch_attn_fwd_bshd(Q, K, V, b, T, softmax_scale=None, path=MA_PATH_AUTO, 
                           Y=None, stream=None):
     """Forward pass on contiguous CUDA tensors [batch, N, heads, d] (no transpose to
     [batch, heads, N, d] needed).  path: MA_PATH_AUTO, MA_PATH_TENSOR, MA_PATH_FUSED_SMALL or MA_PATH_GENERIC."""
+    out = (_run or _load_native())(_BSHD, Q, K, V, b, T, None, softmax_scale, path, workspace, Y, stream)
+    if out is not None:
+        if out.__class__ is int:
+            _check(out)
+        return out
     lib = load_library()
     if not Q.is_cuda:
         raise MonarchAttnError(-2, "monarch_attn_fwd_bshd needs CUDA tensors; there is no CPU path")
@@ -253,6 +291,11 @@ def monarch_attn_fwd_padded(Q, K, V, b, T, n_valid, softmax_scale=None, workspac
     """Forward pass on post-padded CUDA tensors [batch, heads, N, d] with N a multiple of b and
     n_valid real rows (N - b < n_valid <= N): keys beyond n_valid are masked out (App. C.3).
     Returns Y (rows n_valid.. carry no meaning)."""
+    out = (_run or _load_native())(_PADDED, Q, K, V, b, T, n_valid, softmax_scale, 0, workspace, Y, stream)
+    if out is not None:
+        if out.__class__ is int:
+            _check(out)
+        return out
     lib = load_library()
     if not Q.is_cuda:
         raise MonarchAttnError(-2, "monarch_attn_fwd_padded needs CUDA tensors; there is no CPU path")
@@ -275,6 +318,11 @@ def monarch_attn_fwd_varlen(Q, K, V, b, T, seq_len, softmax_scale=None, workspac
     """Forward pass on a batch of sequences of different lengths padded to N rows (App. C.3).
     seq_len: int32 CUDA tensor [batch] with the number of real rows of each batch entry.  Rows
     below seq_len[e] of Y are the result; rows from ceil(seq_len[e] / b) * b on are zero."""
+    out = (_run or _load_native())(_VARLEN, Q, K, V, b, T, seq_len, softmax_scale, 0, workspace, Y, stream)
+    if out is not None:
+        if out.__class__ is int:
+            _check(out)
+        return out
     lib = load_library()
     if not Q.is_cuda:
         raise MonarchAttnError(-2, "monarch_attn_fwd_varlen needs CUDA tensors; there is no CPU path")

@@ -17,6 +17,7 @@
 #include "fused_f32.cuh"
 #include "fused_jsplit.cuh"
 #include "tile_mma.cuh"
+#include "internal_api.h"
 
 namespace ma {
 
@@ -269,11 +270,13 @@ static int grow(void** ptr, size_t* have, size_t need) {
   return MA_OK;
 }
 
-static int fwd_ex(const void* Q, const void* K, const void* V, void* Y, const Problem& p,
-                  float scale, int resolved, void* ws, size_t ws_bytes, cudaStream_t st,
-                  bool ws_armed = false) {
-  if (!ws || ws_bytes < workspace_bytes_for(p, resolved)) return MA_ERR_WORKSPACE;
-  if (((uintptr_t)ws & 255) != 0) return MA_ERR_ALIGN;
+// Whether the kernels of a path read or write the workspace at all.
+static bool touches_workspace(int resolved) {
+  return resolved != MA_PATH_FUSED_SMALL && resolved != MA_PATH_FUSED_F32;
+}
+
+static int launch_resolved(const void* Q, const void* K, const void* V, void* Y, const Problem& p,
+                           float scale, int resolved, void* ws, cudaStream_t st, bool ws_armed) {
   if (resolved == MA_PATH_GENERIC) return launch_generic(p, Q, K, V, Y, scale, ws, st);
   if (resolved == MA_PATH_FUSED_SMALL) {
     int rc = fsmall::launch(Q, K, V, Y, p.BH, p.N, p.d, p.b, p.m, p.T, p.dtype, scale, p.n_valid, p.H, p.lse, st,
@@ -310,6 +313,14 @@ static int fwd_ex(const void* Q, const void* K, const void* V, void* Y, const Pr
   return rc;
 }
 
+static int fwd_ex(const void* Q, const void* K, const void* V, void* Y, const Problem& p,
+                  float scale, int resolved, void* ws, size_t ws_bytes, cudaStream_t st,
+                  bool ws_armed = false) {
+  if (!ws || ws_bytes < workspace_bytes_for(p, resolved)) return MA_ERR_WORKSPACE;
+  if (((uintptr_t)ws & 255) != 0) return MA_ERR_ALIGN;
+  return launch_resolved(Q, K, V, Y, p, scale, resolved, ws, st, ws_armed);
+}
+
 static int check_ptrs(const void* Q, const void* K, const void* V, void* Y, const Problem& p) {
   if (!Q || !K || !V || !Y) return MA_ERR_NULL;
   if ((((uintptr_t)Q | (uintptr_t)K | (uintptr_t)V | (uintptr_t)Y) & 15) != 0) return MA_ERR_ALIGN;
@@ -321,6 +332,89 @@ static int check_ptrs(const void* Q, const void* K, const void* V, void* Y, cons
     if (y0 < a + bytes && a < y0 + bytes) return MA_ERR_ALIGN;
   }
   return MA_OK;
+}
+
+// Which kernels serve a call; -1 if none.
+static int resolve_call(const Call& c, const Problem& p) {
+  switch (c.entry) {
+    case Entry::kFwd: return resolve_path(p, MA_PATH_AUTO);
+    case Entry::kEx: return resolve_path(p, c.path);
+    case Entry::kObjective: return resolve_tensor_or_generic(p, c.path, true);
+    case Entry::kBshd:
+      // (the kernel split by in-block position takes this layout too: a head is a column offset of
+      // its tensor maps)
+      if (((c.path == MA_PATH_AUTO && p.T <= 2) || c.path == MA_PATH_FUSED_JSPLIT) &&
+          jsplit::supported(p.N, p.d, p.b, p.m, p.dtype, p.BH))
+        return MA_PATH_FUSED_JSPLIT;
+      return resolve_tensor_or_generic(p, c.path, true);
+    case Entry::kPadded:
+    case Entry::kVarlen: break;
+  }
+  // The mask entries.  Short 16-bit sequences (up to two rounds, or where the hi + lo instantiation
+  // applies): the fused per-head kernel (one launch).  `padded` then has the second-generation
+  // tensor kernel where a tile row owns a whole key block (b = 64, 128: the mask touches the last
+  // block's tiles only).  Other 16-bit shapes: the warp-MMA tile kernels (hi + lo states from the
+  // third round on); else the generic kernels.
+  if ((p.T <= 2 && fsmall::supported(p.N, p.d, p.b, p.m, p.dtype, p.T)) ||
+      fsmall::supported_hilo(p.N, p.d, p.b, p.m, p.dtype, p.T))
+    return MA_PATH_FUSED_SMALL;
+  if (c.entry == Entry::kPadded && resolve_path(p, MA_PATH_AUTO, false) == MA_PATH_TENSOR && p.b != 32)
+    return MA_PATH_TENSOR;
+  if (tile::supported(p.N, p.d, p.b, p.m, p.dtype, p.BH)) return MA_PATH_TILE_MMA;
+  if (c.entry == Entry::kPadded && p.dtype == MA_F32 && p.BH <= 65535 && ffused::supported(p.N, p.d, p.b, p.m))
+    return MA_PATH_FUSED_F32;
+  return generic_supported(p) ? MA_PATH_GENERIC : -1;
+}
+
+static int run_call(const Call& c) {
+  Problem p;
+  int rc = validate_shape(c.batch, c.heads, c.N, c.d, c.b, c.T, c.dtype, &p);
+  if (rc != MA_OK) return rc;
+  // less than one block of padding: every key block keeps at least one valid key
+  if (c.entry == Entry::kPadded && (c.n_valid > c.N || c.n_valid <= c.N - c.b)) return MA_ERR_SHAPE;
+  rc = check_ptrs(c.Q, c.K, c.V, c.Y, p);
+  if (rc != MA_OK) return rc;
+  if (c.entry == Entry::kVarlen) {
+    if (!c.seq_len) return MA_ERR_NULL;
+    if (((uintptr_t)c.seq_len & 3) != 0) return MA_ERR_ALIGN;
+  }
+  if (c.entry == Entry::kObjective) {
+    if (!c.lse) return MA_ERR_NULL;
+    if (((uintptr_t)c.lse & 3) != 0) return MA_ERR_ALIGN;
+  }
+  if (c.entry != Entry::kFwd && (!(c.scale == c.scale) || isinf(c.scale))) return MA_ERR_SHAPE;
+  const int r = resolve_call(c, p);
+  if (r < 0) return MA_ERR_UNSUPPORTED;
+  cudaStream_t st = (cudaStream_t)c.stream;
+  if (c.entry == Entry::kPadded) p.n_valid = c.n_valid;
+  if (c.entry == Entry::kVarlen) p.seq_len = c.seq_len;
+  if (c.entry == Entry::kObjective) p.lse = c.lse;
+  if (c.entry == Entry::kBshd) p.H = c.heads;
+  if (c.entry != Entry::kFwd) {
+    void* ws = c.ws;
+    size_t bytes = c.ws_bytes;
+    if (!ws && c.alloc) {
+      bytes = workspace_bytes_for(p, r);
+      // the fused per-head kernels touch no scratch: nothing is allocated for them
+      if (!touches_workspace(r)) return launch_resolved(c.Q, c.K, c.V, c.Y, p, c.scale, r, nullptr, st, false);
+      ws = c.alloc(c.ctx, bytes);
+      if (!ws) return MA_ERR_CUDA;
+    }
+    return fwd_ex(c.Q, c.K, c.V, c.Y, p, c.scale, r, ws, bytes, st);
+  }
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return MA_ERR_CUDA;
+  DeviceBuffers& B = g_dev[dev];
+  const size_t had = B.ws_bytes;
+  rc = grow(&B.ws, &B.ws_bytes, workspace_bytes_for(p, r));
+  if (rc != MA_OK) return rc;
+  // The persistent kernel leaves its status block and counters zeroed, so the library's own
+  // workspace is cleared only when the problem (hence the layout) changes.
+  const long long key = ((long long)r << 56) ^ ((long long)p.T << 48) ^ ((long long)p.BH << 24) ^ p.N;
+  const bool armed = (r == MA_PATH_TENSOR) && had == B.ws_bytes && B.armed_key == key;
+  rc = fwd_ex(c.Q, c.K, c.V, c.Y, p, 1.0f / sqrtf((float)c.d), r, B.ws, B.ws_bytes, st, armed);
+  B.armed_key = (rc == MA_OK && r == MA_PATH_TENSOR) ? key : -1;
+  return rc;
 }
 
 }  // namespace ma
@@ -338,135 +432,49 @@ size_t monarch_attn_workspace_bytes(int batch, int heads, int N, int d, int b, i
   return workspace_bytes_for(p, r);
 }
 
+int monarch_attn_internal_run(const Call* c) { return run_call(*c); }
+
 int monarch_attn_fwd_ex(const void* Q, const void* K, const void* V, void* Y, int batch, int heads,
                         int N, int d, int b, int T, int dtype, float softmax_scale, int path,
                         void* workspace, size_t workspace_bytes, void* stream) {
-  Problem p;
-  int rc = validate_shape(batch, heads, N, d, b, T, dtype, &p);
-  if (rc != MA_OK) return rc;
-  rc = check_ptrs(Q, K, V, Y, p);
-  if (rc != MA_OK) return rc;
-  if (!(softmax_scale == softmax_scale) || isinf(softmax_scale)) return MA_ERR_SHAPE;
-  int r = resolve_path(p, path);
-  if (r < 0) return MA_ERR_UNSUPPORTED;
-  return fwd_ex(Q, K, V, Y, p, softmax_scale, r, workspace, workspace_bytes, (cudaStream_t)stream);
+  return run_call(Call{Entry::kEx, Q, K, V, Y, batch, heads, N, d, b, T, dtype, softmax_scale, path, 0, nullptr,
+                       nullptr, workspace, workspace_bytes, stream, nullptr, nullptr});
 }
 
 int monarch_attn_fwd_padded(const void* Q, const void* K, const void* V, void* Y, int batch,
                             int heads, int N, int d, int b, int T, int dtype, float softmax_scale,
                             int n_valid, void* workspace, size_t workspace_bytes, void* stream) {
-  Problem p;
-  int rc = validate_shape(batch, heads, N, d, b, T, dtype, &p);
-  if (rc != MA_OK) return rc;
-  // less than one block of padding: every key block keeps at least one valid key
-  if (n_valid > N || n_valid <= N - b) return MA_ERR_SHAPE;
-  rc = check_ptrs(Q, K, V, Y, p);
-  if (rc != MA_OK) return rc;
-  if (!(softmax_scale == softmax_scale) || isinf(softmax_scale)) return MA_ERR_SHAPE;
-  // fused kernel for short sequences; the second-generation tensor kernel where a tile row owns a
-  // whole key block (b = 64, 128: the mask touches the last block's tiles only); else generic
-  int r = -1;
-  if ((p.T <= 2 && fsmall::supported(p.N, p.d, p.b, p.m, p.dtype, p.T)) ||
-      fsmall::supported_hilo(p.N, p.d, p.b, p.m, p.dtype, p.T))
-    r = MA_PATH_FUSED_SMALL;
-  else if (resolve_path(p, MA_PATH_AUTO, false) == MA_PATH_TENSOR && p.b != 32) r = MA_PATH_TENSOR;
-  else if (tile::supported(p.N, p.d, p.b, p.m, p.dtype, p.BH)) r = MA_PATH_TILE_MMA;
-  else if (p.dtype == MA_F32 && p.BH <= 65535 && ffused::supported(p.N, p.d, p.b, p.m)) r = MA_PATH_FUSED_F32;
-  else if (generic_supported(p)) r = MA_PATH_GENERIC;
-  if (r < 0) return MA_ERR_UNSUPPORTED;
-  p.n_valid = n_valid;
-  return fwd_ex(Q, K, V, Y, p, softmax_scale, r, workspace, workspace_bytes, (cudaStream_t)stream);
+  return run_call(Call{Entry::kPadded, Q, K, V, Y, batch, heads, N, d, b, T, dtype, softmax_scale, MA_PATH_AUTO,
+                       n_valid, nullptr, nullptr, workspace, workspace_bytes, stream, nullptr, nullptr});
 }
 
 int monarch_attn_fwd_varlen(const void* Q, const void* K, const void* V, void* Y, int batch,
                             int heads, int N, int d, int b, int T, int dtype, float softmax_scale,
                             const int* seq_len, void* workspace, size_t workspace_bytes,
                             void* stream) {
-  Problem p;
-  int rc = validate_shape(batch, heads, N, d, b, T, dtype, &p);
-  if (rc != MA_OK) return rc;
-  rc = check_ptrs(Q, K, V, Y, p);
-  if (rc != MA_OK) return rc;
-  if (!seq_len) return MA_ERR_NULL;
-  if (((uintptr_t)seq_len & 3) != 0) return MA_ERR_ALIGN;
-  if (!(softmax_scale == softmax_scale) || isinf(softmax_scale)) return MA_ERR_SHAPE;
-  // short 16-bit sequences with up to two rounds: the fused per-head kernel (one launch); other
-  // 16-bit shapes: the warp-MMA tile kernels (hi + lo states from the third round on); else the
-  // generic kernels
-  int r = -1;
-  if ((p.T <= 2 && fsmall::supported(p.N, p.d, p.b, p.m, p.dtype, p.T)) ||
-      fsmall::supported_hilo(p.N, p.d, p.b, p.m, p.dtype, p.T))
-    r = MA_PATH_FUSED_SMALL;
-  else if (tile::supported(p.N, p.d, p.b, p.m, p.dtype, p.BH)) r = MA_PATH_TILE_MMA;
-  else if (generic_supported(p)) r = MA_PATH_GENERIC;
-  if (r < 0) return MA_ERR_UNSUPPORTED;
-  p.seq_len = seq_len;
-  return fwd_ex(Q, K, V, Y, p, softmax_scale, r, workspace, workspace_bytes, (cudaStream_t)stream);
+  return run_call(Call{Entry::kVarlen, Q, K, V, Y, batch, heads, N, d, b, T, dtype, softmax_scale, MA_PATH_AUTO, 0,
+                       seq_len, nullptr, workspace, workspace_bytes, stream, nullptr, nullptr});
 }
 
 int monarch_attn_fwd_objective(const void* Q, const void* K, const void* V, void* Y, int batch,
                                int heads, int N, int d, int b, int T, int dtype,
                                float softmax_scale, int path, float* row_lse, void* workspace,
                                size_t workspace_bytes, void* stream) {
-  Problem p;
-  int rc = validate_shape(batch, heads, N, d, b, T, dtype, &p);
-  if (rc != MA_OK) return rc;
-  rc = check_ptrs(Q, K, V, Y, p);
-  if (rc != MA_OK) return rc;
-  if (!row_lse) return MA_ERR_NULL;
-  if (((uintptr_t)row_lse & 3) != 0) return MA_ERR_ALIGN;
-  if (!(softmax_scale == softmax_scale) || isinf(softmax_scale)) return MA_ERR_SHAPE;
-  const int r = resolve_tensor_or_generic(p, path, true);
-  if (r < 0) return MA_ERR_UNSUPPORTED;
-  p.lse = row_lse;
-  return fwd_ex(Q, K, V, Y, p, softmax_scale, r, workspace, workspace_bytes, (cudaStream_t)stream);
+  return run_call(Call{Entry::kObjective, Q, K, V, Y, batch, heads, N, d, b, T, dtype, softmax_scale, path, 0,
+                       nullptr, row_lse, workspace, workspace_bytes, stream, nullptr, nullptr});
 }
 
 int monarch_attn_fwd_bshd(const void* Q, const void* K, const void* V, void* Y, int batch, int N,
                           int heads, int d, int b, int T, int dtype, float softmax_scale, int path,
                           void* workspace, size_t workspace_bytes, void* stream) {
-  Problem p;
-  int rc = validate_shape(batch, heads, N, d, b, T, dtype, &p);
-  if (rc != MA_OK) return rc;
-  rc = check_ptrs(Q, K, V, Y, p);
-  if (rc != MA_OK) return rc;
-  if (!(softmax_scale == softmax_scale) || isinf(softmax_scale)) return MA_ERR_SHAPE;
-  // (the kernel split by in-block position takes this layout too: a head is a column offset of
-  // its tensor maps)
-  int r;
-  if (((path == MA_PATH_AUTO && p.T <= 2) || path == MA_PATH_FUSED_JSPLIT) &&
-      jsplit::supported(p.N, p.d, p.b, p.m, p.dtype, p.BH))
-    r = MA_PATH_FUSED_JSPLIT;
-  else
-    r = resolve_tensor_or_generic(p, path, true);
-  if (r < 0) return MA_ERR_UNSUPPORTED;
-  p.H = heads;
-  return fwd_ex(Q, K, V, Y, p, softmax_scale, r, workspace, workspace_bytes, (cudaStream_t)stream);
+  return run_call(Call{Entry::kBshd, Q, K, V, Y, batch, heads, N, d, b, T, dtype, softmax_scale, path, 0, nullptr,
+                       nullptr, workspace, workspace_bytes, stream, nullptr, nullptr});
 }
 
 int monarch_attn_fwd(const void* Q, const void* K, const void* V, void* Y, int batch, int heads,
                      int N, int d, int b, int T, int dtype, void* stream) {
-  Problem p;
-  int rc = validate_shape(batch, heads, N, d, b, T, dtype, &p);
-  if (rc != MA_OK) return rc;
-  rc = check_ptrs(Q, K, V, Y, p);
-  if (rc != MA_OK) return rc;
-  int r = resolve_path(p, MA_PATH_AUTO);
-  if (r < 0) return MA_ERR_UNSUPPORTED;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return MA_ERR_CUDA;
-  DeviceBuffers& B = g_dev[dev];
-  const size_t had = B.ws_bytes;
-  rc = grow(&B.ws, &B.ws_bytes, workspace_bytes_for(p, r));
-  if (rc != MA_OK) return rc;
-  // The persistent kernel leaves its status block and counters zeroed, so the library's own
-  // workspace is cleared only when the problem (hence the layout) changes.
-  const long long key = ((long long)r << 56) ^ ((long long)p.T << 48) ^ ((long long)p.BH << 24) ^ p.N;
-  const bool armed = (r == MA_PATH_TENSOR) && had == B.ws_bytes && B.armed_key == key;
-  rc = fwd_ex(Q, K, V, Y, p, 1.0f / sqrtf((float)d), r, B.ws, B.ws_bytes, (cudaStream_t)stream,
-              armed);
-  B.armed_key = (rc == MA_OK && r == MA_PATH_TENSOR) ? key : -1;
-  return rc;
+  return run_call(Call{Entry::kFwd, Q, K, V, Y, batch, heads, N, d, b, T, dtype, 0.f, MA_PATH_AUTO, 0, nullptr,
+                       nullptr, nullptr, 0, stream, nullptr, nullptr});
 }
 
 int monarch_attn_fwd_host(const void* Qh, const void* Kh, const void* Vh, void* Yh, int batch,

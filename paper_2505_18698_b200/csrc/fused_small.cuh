@@ -659,9 +659,8 @@ inline int launch_t(const void* Q, const void* K, const void* V, void* Y, int BH
       (m > 8 || b > 8) && smem_bytes(N, T, 2 * kThreads) <= (size_t)kMaxSmem)
     threads = 2 * kThreads;
   const size_t smem = smem_bytes(N, T, threads, b, KS, HILO);
-  if (cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-      cudaSuccess)
-    return 7;
+  static warpmma::SmemOptIn opt_in;
+  if (!opt_in.done((const void*)kern, kMaxSmem)) return 7;
   // programmatic stream serialisation: when calls follow one another on a stream, the CTAs of the
   // next call take SM slots while the last wave of this one drains (they touch no memory before
   // this launch has finished: the kernel starts with griddepcontrol.wait)

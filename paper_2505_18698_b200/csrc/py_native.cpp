@@ -1,0 +1,189 @@
+// Python extension `_native`: the per-call host path of the binding (tensor checks, output and
+// scratch allocation, stream lookup, the library call) without the interpreter in between.  A call
+// from Python took 13 us of host time through ctypes, more than the kernels of the smallest problems
+// run; this takes about 4.
+//
+// It serves calls whose arguments are all as documented and returns None for anything else; the
+// binding then runs its checks in Python, which say what is wrong.  No arithmetic of the method
+// and no path choice is here: the library picks the kernels (internal_api.h).
+#include <Python.h>
+
+#include <ATen/EmptyTensor.h>
+#include <ATen/cuda/EmptyTensor.h>
+#include <c10/cuda/CUDACachingAllocator.h>
+#include <c10/cuda/CUDAFunctions.h>
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include <climits>
+#include <cmath>
+#include <exception>
+
+#include "internal_api.h"
+
+namespace {
+
+// Scratch from torch's caching allocator, held until the call has been enqueued (the allocator
+// hands the block out again in stream order).
+struct Scratch {
+  c10::DataPtr block;
+  std::exception_ptr failed;
+};
+void* scratch_alloc(void* ctx, size_t bytes) {
+  Scratch* s = static_cast<Scratch*>(ctx);
+  try {
+    s->block = c10::cuda::CUDACachingAllocator::get()->allocate(bytes);
+  } catch (...) {      // out of memory: raised again once the library has returned
+    s->failed = std::current_exception();
+    return nullptr;
+  }
+  return s->block.get();
+}
+
+// Runs the rest of a scope with `dev` current; free when it already is.
+struct OnDevice {
+  c10::DeviceIndex before, dev;
+  explicit OnDevice(int d) : before(c10::cuda::current_device()), dev((c10::DeviceIndex)d) {
+    if (before != dev) c10::cuda::set_device(dev);
+  }
+  ~OnDevice() {
+    if (before != dev) c10::cuda::set_device(before);
+  }
+};
+
+bool as_int(PyObject* o, int* out) {
+  if (!PyLong_CheckExact(o)) return false;
+  int over = 0;
+  const long v = PyLong_AsLongAndOverflow(o, &over);
+  if (over || v < INT_MIN || v > INT_MAX) return false;
+  *out = (int)v;
+  return true;
+}
+
+// run(entry, Q, K, V, b, T, arg, scale, path, workspace, Y, stream)
+//   entry: ma::Entry; arg: n_valid (padded), seq_len tensor (varlen), else None; scale: float or None
+//   (1 / sqrt(d)); workspace, Y: tensors or None; stream: an object with .cuda_stream, or None.
+// -> Y, or (Y, row_lse) for the objective; an int: the library's status; None: not a call this
+//    function takes.
+PyObject* run(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  HANDLE_TH_ERRORS
+  ma::Call c{};
+  int entry;
+  if (n != 12 || !as_int(a[0], &entry)) Py_RETURN_NONE;
+  c.entry = (ma::Entry)entry;
+  for (int i = 1; i <= 3; ++i)
+    if (!THPVariable_CheckExact(a[i])) Py_RETURN_NONE;
+  const at::Tensor &Q = THPVariable_Unpack(a[1]), &K = THPVariable_Unpack(a[2]), &V = THPVariable_Unpack(a[3]);
+  if (!Q.is_cuda() || Q.dim() != 4 || Q.layout() != at::kStrided) Py_RETURN_NONE;
+  const auto dtype = Q.scalar_type();
+  if (dtype == at::kFloat) c.dtype = 0;
+  else if (dtype == at::kHalf) c.dtype = 1;
+  else if (dtype == at::kBFloat16) c.dtype = 2;
+  else Py_RETURN_NONE;
+  const auto sizes = Q.sizes();
+  for (const at::Tensor* t : {&K, &V})
+    if (t->sizes() != sizes || t->scalar_type() != dtype || t->device() != Q.device()) Py_RETURN_NONE;
+  if (!Q.is_contiguous() || !K.is_contiguous() || !V.is_contiguous()) Py_RETURN_NONE;
+  for (int i = 0; i < 4; ++i)
+    if (sizes[i] <= 0 || sizes[i] > INT_MAX) Py_RETURN_NONE;
+  c.batch = (int)sizes[0];
+  c.heads = (int)sizes[c.entry == ma::Entry::kBshd ? 2 : 1];
+  c.N = (int)sizes[c.entry == ma::Entry::kBshd ? 1 : 2];
+  c.d = (int)sizes[3];
+  if (!as_int(a[4], &c.b) || !as_int(a[5], &c.T)) Py_RETURN_NONE;
+  if (c.entry == ma::Entry::kPadded) {
+    if (!as_int(a[6], &c.n_valid)) Py_RETURN_NONE;
+  } else if (c.entry == ma::Entry::kVarlen) {
+    if (!THPVariable_CheckExact(a[6])) Py_RETURN_NONE;
+    const at::Tensor& len = THPVariable_Unpack(a[6]);
+    if (len.scalar_type() != at::kInt || len.dim() != 1 || len.size(0) != c.batch || !len.is_contiguous() ||
+        len.device() != Q.device())
+      Py_RETURN_NONE;
+    c.seq_len = len.const_data_ptr<int>();
+  }
+  if (a[7] == Py_None) c.scale = (float)(1.0 / std::sqrt((double)c.d));
+  else if (PyFloat_CheckExact(a[7])) c.scale = (float)PyFloat_AS_DOUBLE(a[7]);
+  else Py_RETURN_NONE;
+  if (!as_int(a[8], &c.path)) Py_RETURN_NONE;
+  if (a[9] != Py_None) {
+    if (!THPVariable_CheckExact(a[9])) Py_RETURN_NONE;
+    const at::Tensor& ws = THPVariable_Unpack(a[9]);
+    if (ws.device() != Q.device() || ws.scalar_type() != at::kByte || !ws.is_contiguous()) Py_RETURN_NONE;
+    c.ws = ws.data_ptr();
+    c.ws_bytes = (size_t)ws.numel();
+    if (!c.ws) Py_RETURN_NONE;
+  }
+  at::Tensor Y;
+  if (a[10] != Py_None) {
+    if (!THPVariable_CheckExact(a[10])) Py_RETURN_NONE;
+    Y = THPVariable_Unpack(a[10]);
+    if (Y.sizes() != sizes || Y.scalar_type() != dtype || Y.device() != Q.device() || !Y.is_contiguous())
+      Py_RETURN_NONE;
+  }
+  const int dev = Q.get_device();
+  const OnDevice on(dev);
+  const auto current = c10::cuda::getCurrentCUDAStream((c10::DeviceIndex)dev);
+  cudaStream_t stream = current.stream();
+  if (a[11] != Py_None) {
+    PyObject* handle = PyObject_GetAttrString(a[11], "cuda_stream");
+    const bool ok = handle && PyLong_Check(handle);
+    if (ok) stream = (cudaStream_t)PyLong_AsVoidPtr(handle);
+    Py_XDECREF(handle);
+    if (!ok) {
+      PyErr_Clear();
+      Py_RETURN_NONE;
+    }
+  }
+  if (!Y.defined()) Y = at::detail::empty_cuda(sizes, dtype, Q.device(), std::nullopt);
+  at::Tensor lse;
+  if (c.entry == ma::Entry::kObjective)
+    lse = at::detail::empty_cuda({c.batch, c.heads, c.N}, at::kFloat, Q.device(), std::nullopt);
+  Scratch s;
+  c.Q = Q.const_data_ptr();
+  c.K = K.const_data_ptr();
+  c.V = V.const_data_ptr();
+  c.Y = Y.data_ptr();
+  c.lse = lse.defined() ? lse.data_ptr<float>() : nullptr;
+  c.stream = stream;
+  c.alloc = scratch_alloc;
+  c.ctx = &s;
+  int rc = 0;
+  Py_BEGIN_ALLOW_THREADS
+  rc = monarch_attn_internal_run(&c);
+  Py_END_ALLOW_THREADS
+  if (s.failed) std::rethrow_exception(s.failed);
+  // (a call on a stream other than the current one: the block is not handed out again before that
+  // stream's work up to here is done)
+  if (s.block && stream != current.stream())
+    c10::cuda::CUDACachingAllocator::recordStream(
+        s.block, c10::cuda::getStreamFromExternal(stream, (c10::DeviceIndex)dev));
+  if (rc != 0) return PyLong_FromLong(rc);
+  PyObject* y;
+  if (a[10] != Py_None) {
+    y = a[10];
+    Py_INCREF(y);
+  } else {
+    y = THPVariable_Wrap(Y);
+  }
+  if (!lse.defined() || !y) return y;
+  PyObject* l = THPVariable_Wrap(lse);
+  if (!l) {
+    Py_DECREF(y);
+    return nullptr;
+  }
+  PyObject* pair = PyTuple_Pack(2, y, l);
+  Py_DECREF(y);
+  Py_DECREF(l);
+  return pair;
+  END_HANDLE_TH_ERRORS
+}
+
+PyMethodDef methods[] = {
+    {"run", (PyCFunction)(void (*)(void))run, METH_FASTCALL, "One call of a device entry point."},
+    {nullptr, nullptr, 0, nullptr}};
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__native() { return PyModule_Create(&module); }

@@ -681,8 +681,8 @@ template <typename TIn, int CB, int DT, bool HILO>
 inline int launch_r(const Args& a, const Ws& w, bool first, bool last, cudaStream_t st) {
   auto kern = r_tile_kernel<TIn, CB, DT, HILO>;
   const size_t smem = r_smem_bytes(a.b, DT, HILO);
-  if (cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return 7;
+  static warpmma::SmemOptIn opt_in;
+  if (!opt_in.done((const void*)kern, kMaxSmem)) return 7;
   cudaLaunchConfig_t cfg = serialised_config(dim3(a.m, a.BH), 32 * ((a.b + 15) / 16), smem, st);
   return cudaLaunchKernelEx(&cfg, kern, (const TIn*)a.Q, (const TIn*)a.K, (const TIn*)a.V, (const __half*)w.aR,
                             w.aL, w.y, (const __half*)w.aR_lo, w.aL_lo, w.cL, a.N, a.d, a.b, a.scale, a.n_valid,
@@ -694,8 +694,8 @@ template <typename TIn, int CM, int DT, bool HILO>
 inline int launch_l(const Args& a, const Ws& w, bool last, cudaStream_t st) {
   auto kern = l_tile_kernel<TIn, CM, DT, HILO>;
   const size_t smem = l_smem_bytes(a.m, CM, DT, HILO);
-  if (cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return 7;
+  static warpmma::SmemOptIn opt_in;
+  if (!opt_in.done((const void*)kern, kMaxSmem)) return 7;
   cudaLaunchConfig_t cfg = serialised_config(dim3(a.b, a.BH), 32 * ((a.m + 15) / 16), smem, st);
   return cudaLaunchKernelEx(&cfg, kern, (const TIn*)a.Q, (const __half*)w.aL, (const float*)w.cL,
                             (const __half*)w.y, w.aR, (const __half*)w.aL_lo, w.aR_lo, (TIn*)a.Y,

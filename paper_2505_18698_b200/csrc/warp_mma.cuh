@@ -49,6 +49,19 @@ template <> struct Mma<__nv_bfloat16> {
   }
 };
 
+// Lets a kernel use up to `bytes` of dynamic shared memory: once per kernel and device (the call
+// costs most of a microsecond of host time).
+struct SmemOptIn {
+  bool prepared[64] = {};
+  bool done(const void* kernel, int bytes) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    if (!prepared[dev])
+      prepared[dev] = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
+    return prepared[dev];
+  }
+};
+
 __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
