@@ -17,6 +17,7 @@
 #include "fused_f32.cuh"
 #include "fused_jsplit.cuh"
 #include "tile_mma.cuh"
+#include "tile_tc.cuh"
 #include "internal_api.h"
 
 namespace ma {
@@ -224,7 +225,7 @@ static size_t workspace_bytes_for(const Problem& p, int resolved) {
   if (resolved == MA_PATH_GENERIC) return generic_layout(p, nullptr).bytes;
   if (resolved == MA_PATH_FUSED_SMALL || resolved == MA_PATH_FUSED_F32 || resolved == MA_PATH_FUSED_JSPLIT)
     return kStatusBytes;   // no states leave the chip
-  if (resolved == MA_PATH_TILE_MMA) return tile::workspace_bytes(p.BH, p.N, p.d, p.T);
+  if (resolved == MA_PATH_TILE_MMA) return tile::workspace_bytes(p.BH, p.N, p.d, p.b, p.T);
   if (resolved == MA_PATH_TENSOR_BASIC) return tensor::workspace_bytes(p.BH, p.N, p.d, p.b, p.T);
   if (resolved == MA_PATH_TENSOR || resolved == MA_PATH_TENSOR_TMEM)
     return tp::workspace_bytes(p.BH, p.N, p.T, tp::uses_hilo(p.dtype, p.b));
@@ -275,6 +276,18 @@ static bool touches_workspace(int resolved) {
   return resolved != MA_PATH_FUSED_SMALL && resolved != MA_PATH_FUSED_F32;
 }
 
+// MA_PATH_TILE_MMA has two sets of kernels: tcgen05 tiles (tile_tc.cuh: f16 states, up to two rounds,
+// d <= 64) and warp-MMA tiles (tile_mma.cuh: hi + lo states for three or more rounds, wider heads,
+// negative scales).  Where both apply the tcgen05 tiles pay for their set-up and longer chain once
+// there are tiles enough to keep several in flight on every SM: measured over N = 960 .. 10240 and 8
+// to 64 heads they are 1.0-1.9 x as fast from 448 tiles of 128 rows on (two rounds of blocks of
+// more than 32: from 160 on), and 0.65-0.97 x below.
+static bool tiles_on_tensor_cores(const Problem& p, float scale) {
+  if (p.T > 2 || !(scale >= 0.f) || !ttc::supported(p.N, p.d, p.b, p.m, p.dtype, p.BH)) return false;
+  const long long tiles = (long long)p.BH * p.N / 128;
+  return tiles >= (p.T == 2 && p.b > 32 ? 160 : 448);
+}
+
 static int launch_resolved(const void* Q, const void* K, const void* V, void* Y, const Problem& p,
                            float scale, int resolved, void* ws, cudaStream_t st, bool ws_armed) {
   if (resolved == MA_PATH_GENERIC) return launch_generic(p, Q, K, V, Y, scale, ws, st);
@@ -292,6 +305,13 @@ static int launch_resolved(const void* Q, const void* K, const void* V, void* Y,
   if (resolved == MA_PATH_FUSED_JSPLIT) {
     int rc = jsplit::launch(Q, K, V, Y, p.BH, p.T, p.dtype, scale, (int*)ws, st, p.H);
     if (rc == MA_OK) g_last_launches = 1;
+    return rc;
+  }
+  if (resolved == MA_PATH_TILE_MMA && tiles_on_tensor_cores(p, scale)) {
+    const tile::Ws w = tile::ws_layout(ws, p.BH, p.N, p.d, p.b, false);
+    const int rc = ttc::launch({Q, K, V, Y, p.BH, p.N, p.d, p.b, p.m, p.T, p.dtype, p.H, p.heads, p.n_valid, scale, p.lse, p.seq_len},
+                               {w.aL, w.aR, w.y, w.cL, (int*)ws}, st);
+    if (rc == MA_OK) g_last_launches = 2 * p.T;
     return rc;
   }
   if (resolved == MA_PATH_TILE_MMA) {

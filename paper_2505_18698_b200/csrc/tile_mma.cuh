@@ -629,7 +629,7 @@ struct Ws {
   float* cL;
   size_t bytes;
 };
-inline Ws ws_layout(void* base, int BH, int N, int d, bool hilo) {
+inline Ws ws_layout(void* base, int BH, int N, int d, int b, bool hilo) {
   auto up = [](size_t x) { return (x + 255) / 256 * 256; };
   Ws w;
   char* c = (char*)base;
@@ -638,7 +638,7 @@ inline Ws ws_layout(void* base, int BH, int N, int d, bool hilo) {
   w.aL = (__half*)(c + off); off += big;
   w.aR = (__half*)(c + off); off += big;
   w.y = (__half*)(c + off); off += big;
-  w.cL = (float*)(c + off); off += up((size_t)BH * N * 4);
+  w.cL = (float*)(c + off); off += up((size_t)BH * b * ((N / b + 3) / 4 * 4) * 4);   // rows of m floats, 16-byte aligned
   w.aL_lo = w.aR_lo = nullptr;
   if (hilo) {
     w.aL_lo = (__half*)(c + off); off += big;
@@ -647,7 +647,7 @@ inline Ws ws_layout(void* base, int BH, int N, int d, bool hilo) {
   w.bytes = off;
   return w;
 }
-inline size_t workspace_bytes(int BH, int N, int d, int T) { return ws_layout(nullptr, BH, N, d, uses_hilo(T)).bytes; }
+inline size_t workspace_bytes(int BH, int N, int d, int b, int T) { return ws_layout(nullptr, BH, N, d, b, uses_hilo(T)).bytes; }
 
 // Launch configuration with programmatic stream serialisation (see grid_dependency_sync).
 inline cudaLaunchConfig_t serialised_config(dim3 grid, int threads, size_t smem, cudaStream_t st) {
@@ -707,7 +707,7 @@ inline int launch_l(const Args& a, const Ws& w, bool last, cudaStream_t st) {
 
 template <typename TIn, int DT, bool HILO>
 inline int launch_td(const Args& a, void* ws, cudaStream_t st, int* launches) {
-  const Ws w = ws_layout(ws, a.BH, a.N, a.d, HILO);
+  const Ws w = ws_layout(ws, a.BH, a.N, a.d, a.b, HILO);
   int n = 0;
   for (int t = 1; t <= a.T; ++t) {
     const bool first = t == 1, last = t == a.T;

@@ -1,0 +1,1029 @@
+// Tensor-core tiles of both half-steps for sm_100a (tcgen05 + TMA), one launch per half-step: 16-bit
+// inputs, d <= 64 (a multiple of 8), any b, m <= 128, key padding mask and per-sequence lengths (App.
+// C.3), either layout, row log-sum-exp output.  MA_PATH_TILE_MMA takes these kernels for up to two
+// rounds where there are tiles enough to fill the GPU (the rule is in api.cu).
+//
+// What bounds a tile.  Its chain load -> score MMA -> softmax -> apply MMA -> epilogue -> store is 4-5
+// us long, most of it latency, while its pipe time is half a microsecond (128 x 128 exponentials at
+// 16 per clock and SM).  So as many chains as possible have to be in flight with as few hand-overs as
+// possible: two CTAs share an SM, each with two compute groups of four warps (thread = score row,
+// one tile per group: softmax and epilogue) over one ring of six 16 KB operand slots, and four service
+// threads (producer, MMA issuer, one store thread per group) that serve only that CTA.
+//
+// One tile shape for everything: 128 score rows = 128 / B blocks of B rows (B = b or m rounded up
+// to 32, 64 or 128; rows past the block are zero-filled by TMA), one M = N = 128 score MMA, of which a
+// row owns the B columns of its own block (at B = 64 the wasted half costs no time: M = 64 MMAs run
+// at half rate).  The weights go back to tensor memory over the scores, zeros outside the window,
+// and are the A operand of the apply MMA; only the non-final L half-step, whose contraction runs
+// over the rows of the weights, passes them through shared memory.
+//   TMEM columns of a group: scores 0-127; weights (16-bit pairs) 0-63; apply accumulator 64-127; in
+//   the non-final L half-step sixteen copies of c_R in 0-15.
+//   Slots of a tile: the first operand (alpha_R or Q(.,j)), the second (K or alpha_L).  A third operand
+//   (V, y) lands over the first once the score MMA has read it, under the softmax; the weights of the
+//   non-final L half-step go over alpha_L (at B = 128 their second half takes a slot of its own); rows
+//   are staged for their store over an operand that is dead by then.
+//
+// Arithmetic and states are f16 (bf16 inputs are converted in shared memory: the rounding of alpha_L
+// is the dominant error of a 16-bit pipeline and f16 has three more bits).  alpha_R is stored divided
+// by c_R, and the columns of the non-final L weights are rescaled by powers of two before they are
+// rounded (the quotient is invariant), so that a column of small weights keeps its bits however small
+// c_R is; c_R sums the weights as rounded.
+//
+// Measured (B200, us per call, against the warp-MMA tiles that served these shapes): 8 heads of N =
+// 7600 in blocks of 128, d = 48, two rounds 43.9 / 61.9; 32 heads of N = 8192 as 128 blocks of 64, one
+// round (bf16) 64 / 95, two rounds (f16) 119 / 214; 64 heads of 60 blocks of 64, two rounds 102 / 150.
+#pragma once
+#include <type_traits>
+
+#include "tensor_path.cuh"
+
+namespace ma {
+namespace ttc {
+
+using namespace ma::tensor;
+
+constexpr int kThreads = 384;                // two compute groups of four warps, four service warps
+constexpr int kCtasPerSm = 2;
+constexpr int kSlot = kTileBytes;            // 16 KB
+constexpr int kSlots = 6;
+constexpr int kOffOnes = kSlots * kSlot;     // 2 KB of ones
+constexpr int kOffVec = kOffOnes + 2048;     // c_L of a tile's rows: three tiles of 128 floats
+constexpr int kOffCol = kOffVec + 3 * 512;   // per group: column maxima, then scales, of the non-final L weights
+constexpr int kOffScale = kOffCol + 2 * 512;
+constexpr int kOffBar = kOffScale + 2 * 512;
+constexpr int kSmem = kOffBar + 384 + 1024;  // + alignment slack
+static_assert(kCtasPerSm * (kSmem + 1024) <= 228 * 1024, "two CTAs per SM");
+
+struct Params {
+  // Loads and stores of one tile, all with 64-column rows and 128 rows in 128-byte swizzle.
+  // R: dims (d, b, m, heads, batch), box (64, B, 128 / B, 1, 1): blocks of rows (k, .)
+  // L: dims (d, m, b, heads, batch), box (64, B, 128 / B, 1, 1): blocks of rows (., j)
+  CUtensorMap rQ, rK, rV, rAR, rAL, rY;      // R half-step: loads Q, K, V, alpha_R; stores alpha_L, y
+  CUtensorMap lQ, lAL, lY, lAR, lOut;        // L half-step: loads Q, alpha_L, y; stores alpha_R, Y
+  float* cL;               // [BH][b][mp]: -c_L log2 e, the addend of the next L half-step's logits
+  uint8_t *aL, *aR, *y;    // state arrays, for L2 discards once a tile has been consumed (d = 64)
+  float* lse;              // optional [BH][N]
+  const int* seq_len;      // optional [BH / heads]
+  int* status;             // set by a wait that ran out
+  int N, b, m, mp, BH, H, heads, n_valid;
+  int first, last;         // this launch's half-step: of the first round, of the last round
+  int tiles, per_head;     // tiles of this launch, tiles of a head
+  int discard;
+  long long wait_cycles;
+  float scale;
+};
+
+struct __align__(16) Shared {
+  uint64_t load[3], empty[kSlots];                     // by tile, by slot
+  uint64_t mma1[2], weights[2], first[2], mma2[2];     // by group from here on
+  uint64_t third[2], prep[2], oread[2], o_free[2], staged[2], out_free[2], cols[2];
+  uint32_t tmem;
+  volatile int abort_flag;
+  int4 tile[3], out[2];      // {head or -1, first block or position, slot, keys that count}, {head or -1, first .., slot, is y}
+};
+static_assert(sizeof(Shared) <= 384, "barrier block");
+
+// ------------------------------------------------------------------------------------ PTX helpers
+__device__ __forceinline__ void load_5d(void* dst, const CUtensorMap* tm, uint64_t* bar, int r, int blk, int h0, int h1) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], [%2];" ::"r"(
+          smem_u32(dst)),
+      "l"((uint64_t)tm), "r"(smem_u32(bar)), "r"(0), "r"(r), "r"(blk), "r"(h0), "r"(h1)
+      : "memory");
+}
+__device__ __forceinline__ void store_5d(const CUtensorMap* tm, const void* src, int blk, int h0, int h1) {
+  asm volatile("cp.async.bulk.tensor.5d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5, %6}], [%1];" ::"l"((uint64_t)tm),
+               "r"(smem_u32(src)), "r"(0), "r"(0), "r"(blk), "r"(h0), "r"(h1)
+               : "memory");
+}
+__device__ __forceinline__ void bulk_1d(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
+               "l"(src), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
+}
+template <int N>
+__device__ __forceinline__ void st_cols(uint32_t taddr, const uint32_t* r);
+template <>
+__device__ __forceinline__ void st_cols<8>(uint32_t taddr, const uint32_t* r) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr), "r"(r[0]),
+               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
+}
+template <>
+__device__ __forceinline__ void st_cols<16>(uint32_t taddr, const uint32_t* r) {
+  tmem_st16(taddr, reinterpret_cast<const float*>(r));
+}
+template <>
+__device__ __forceinline__ void st_cols<32>(uint32_t taddr, const uint32_t* r) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
+      "%12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, "
+      "%30, %31, %32};" ::"r"(taddr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+      "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
+      "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
+      "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+      : "memory");
+}
+__device__ __forceinline__ float ld_col(uint32_t taddr) {
+  uint32_t r;
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr) : "memory");
+  return __uint_as_float(r);
+}
+template <bool ACC>
+__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(b_desc), "r"(idesc), "n"(ACC ? 1 : 0)
+      : "memory");
+}
+
+// Bounded wait: after a timeout (status word and abort flag set) every wait of the CTA returns at
+// once, the tile ends with garbage and the CTA leaves at the tile's last barrier.
+__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Shared* sh, const Params& P, int where) {
+  const uint32_t addr = smem_u32(bar);
+  uint32_t done = 0;
+  long long t0 = 0;
+  for (int n = 0;; ++n) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(addr), "r"(parity)
+        : "memory");
+    if (done) return true;
+    if (sh->abort_flag) return false;
+    if (n == 0) {
+      t0 = clock64();
+    } else if (clock64() - t0 > P.wait_cycles) {
+      report_timeout(P.status, where);
+      sh->abort_flag = 1;
+      return false;
+    }
+  }
+}
+
+__device__ __forceinline__ void arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ bool test_bar(uint64_t* bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(done)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+
+// ------------------------------------------------------------------------------------ kernel
+// MODE 0: R tiles, 1: L tiles of blocks (rows of blocks) padded to B.  FULL: nothing is padded or masked.
+template <typename TIn, int B, bool FULL, int MODE>
+struct Kernel {
+  typedef __half TA;                    // arithmetic and states
+  static constexpr bool kConvert = !std::is_same<TIn, TA>::value;
+  static constexpr bool R = MODE == 0;
+  static constexpr int kBlocks = 128 / B;
+  static constexpr int FT = Fmt<TA>::code;
+  static constexpr uint32_t kIdScore = instr_desc(128, 128, FT, 0, 0), kIdApply = instr_desc(128, 64, FT, 0, 1);
+
+  // Slots of a tile: two, and a third for the weights of a non-final L tile of 128 columns.
+  static __device__ __forceinline__ int slots(const Params& P) { return B == 128 && !R && !P.last ? 3 : 2; }
+  static __device__ __forceinline__ int wrap(int s) { return s >= kSlots ? s - kSlots : s; }
+  static __device__ __forceinline__ bool prepares(const Params& P) { return kConvert || (!FULL && P.seq_len != nullptr); }
+
+  // ================================================================ producer (one thread)
+  // Requests the first two operands of the CTA's tiles.
+  static __device__ __forceinline__ void produce(const Params& P, uint8_t* smem, Shared* sh) {
+    int q = 0, i3 = 0, ends = 0;
+    uint32_t par_e = (1u << kSlots) - 1;      // per slot: parity of its next "empty"
+    const int ns = slots(P);
+    for (int g = blockIdx.x;; g += gridDim.x) {
+      const bool end = g >= P.tiles;
+      const int h = end ? -1 : g / P.per_head, idx0 = end ? 0 : (g - h * P.per_head) * kBlocks;
+      int n_valid = P.n_valid;
+      if (!FULL && !end && P.seq_len != nullptr) {
+        n_valid = min(max(P.seq_len[h / P.heads], 1), P.N);
+        if (R && idx0 * P.b >= n_valid) continue;      // key blocks that are absent from a shorter sequence
+      }
+      for (int s = 0; s < ns; ++s) {
+        const int e = wrap(q + s);
+        if (!wait_bar(&sh->empty[e], (par_e >> e) & 1, sh, P, 11)) return;
+        par_e ^= 1u << e;
+      }
+      uint64_t* bar = &sh->load[i3];
+      sh->tile[i3] = make_int4(h, idx0, q, n_valid);
+      if (end) {                              // once for each group
+        arrive(bar);
+        if (++ends == 2) return;
+      } else {
+        const int h0 = P.H ? h % P.H : h, h1 = P.H ? h / P.H : 0;
+        uint8_t *s0 = smem + q * kSlot, *s1 = smem + wrap(q + 1) * kSlot;
+        if (R) {
+          mbar_expect_tx(bar, 2 * kSlot);
+          if (P.first) load_5d(s0, &P.rQ, bar, 0, idx0, h0, h1);
+          else load_5d(s0, &P.rAR, bar, 0, idx0, h, 0);
+          load_5d(s1, &P.rK, bar, 0, idx0, h0, h1);
+        } else {
+          float* sC = reinterpret_cast<float*>(smem + kOffVec) + i3 * 128;
+          const int nj = min(kBlocks, P.b - idx0);
+          mbar_expect_tx(bar, 2 * kSlot + nj * P.mp * 4);
+          load_5d(s0, &P.lQ, bar, 0, idx0, h0, h1);
+          load_5d(s1, &P.lAL, bar, 0, idx0, h, 0);
+          const float* c = P.cL + ((size_t)h * P.b + idx0) * P.mp;
+          for (int jj = 0; jj < nj; ++jj) bulk_1d(sC + jj * B, c + (size_t)jj * P.mp, P.mp * 4, bar);
+        }
+      }
+      q = wrap(q + ns);
+      i3 = i3 == 2 ? 0 : i3 + 1;
+    }
+  }
+
+  // ================================================================ issuer (one thread): all MMAs
+  // Polls: what is ready first, the scores of the next tile or the apply MMA of an earlier one, is
+  // issued first.
+  static __device__ __forceinline__ void issue(const Params& P, uint8_t* smem, Shared* sh, uint32_t tmem) {
+    const bool prep = prepares(P), last = P.last != 0;
+    auto apply = [&](uint32_t d, const uint8_t* x, uint64_t* done) {     // weights (TMEM) times the rows of a slot
+      const uint64_t dX = smem_desc(smem_u32(x), 16, 1024);
+      umma_ts<false>(d + 64, d, dX, kIdApply);
+#pragma unroll
+      for (int ks = 1; ks < 8; ++ks) umma_ts<true>(d + 64, d + 8 * ks, dX + 128 * ks, kIdApply);
+      umma_commit(done);
+    };
+    int n1 = 0, n2 = 0, i1 = 0, i2 = 0;       // tiles and load barriers of the two MMAs
+    uint32_t par1 = 0, par_t = 0, par_r = 0;                 // (bit w: group w)
+    bool second = false, end = false, idle = false;
+    long long t0 = 0;
+    while (!end || n2 < n1) {
+      bool did = false;
+      const int w1 = n1 & 1, w2 = n2 & 1;
+      const uint32_t d1 = tmem + 128 * w1, d2 = tmem + 128 * w2;
+      if (n2 < n1) {
+        if (!second && test_bar(&sh->weights[w2], (n2 >> 1) & 1)) {
+          if (R || !last || prep || test_bar(&sh->third[w2], (par_t >> w2) & 1)) {
+            const int q2 = sh->tile[i2].z;
+            uint8_t *s0 = smem + q2 * kSlot, *s1 = smem + wrap(q2 + 1) * kSlot;
+            tc_fence_after();
+            if (R) {
+              apply(d2, s1, last ? &sh->first[w2] : &sh->mma2[w2]);
+              second = last;
+            } else if (last) {
+              par_t ^= 1u << w2;
+              apply(d2, s0, &sh->mma2[w2]);
+              umma_commit(&sh->empty[q2]);
+            } else {
+              const uint64_t dQ = smem_desc(smem_u32(s0), 16, 1024), dO = smem_desc(smem_u32(smem + kOffOnes), 16, 1024);
+              if constexpr (B == 128) {
+                const int e1 = wrap(q2 + 1), e2 = wrap(q2 + 2);
+                const uint32_t lo = smem_u32(smem) + min(e1, e2) * kSlot, hi = smem_u32(smem) + max(e1, e2) * kSlot;
+                const uint64_t dP = smem_desc(lo, hi - lo, 1024);
+                constexpr uint32_t id = instr_desc(128, 64, FT, 1, 1), id1 = instr_desc(128, 16, FT, 1, 0);
+                umma_c<false>(d2 + 64, dP, dQ, id);
+                umma_c<false>(d2, dP, dO, id1);
+#pragma unroll
+                for (int ks = 1; ks < 8; ++ks) {
+                  umma_c<true>(d2 + 64, dP + 128 * ks, dQ + 128 * ks, id);
+                  umma_c<true>(d2, dP + 128 * ks, dO, id1);
+                }
+                umma_commit(&sh->empty[e2]);
+              } else {
+                // two groups of 64 rows; their accumulators take the lower and upper 16 lanes of
+                // every warp's part of tensor memory
+                const uint64_t dP = smem_desc(smem_u32(s1), 16, 1024);
+                constexpr uint32_t id = instr_desc(64, 64, FT, 1, 1), id1 = instr_desc(64, 16, FT, 1, 0);
+#pragma unroll
+                for (int g = 0; g < 2; ++g) {
+                  const uint32_t d = d2 + ((uint32_t)(16 * g) << 16);
+#pragma unroll
+                  for (int ks = 0; ks < 4; ++ks) {
+                    const uint64_t off = 512 * g + 128 * ks;
+                    if (ks == 0) {
+                      umma_c<false>(d + 64, dP + off, dQ + off, id);
+                      umma_c<false>(d, dP + off, dO, id1);
+                    } else {
+                      umma_c<true>(d + 64, dP + off, dQ + off, id);
+                      umma_c<true>(d, dP + off, dO, id1);
+                    }
+                  }
+                }
+              }
+              umma_commit(&sh->mma2[w2]);
+              umma_commit(&sh->empty[wrap(q2 + 1)]);
+            }
+            if (!second) {
+              i2 = i2 == 2 ? 0 : i2 + 1;
+              ++n2;
+            }
+            did = true;
+          }
+        } else if (second && test_bar(&sh->oread[w2], (par_r >> w2) & 1) &&
+                   (prep || test_bar(&sh->third[w2], (par_t >> w2) & 1))) {
+          par_r ^= 1u << w2;              // alpha_L is out: y = R V through the same columns
+          par_t ^= 1u << w2;
+          tc_fence_after();
+          apply(d2, smem + sh->tile[i2].z * kSlot, &sh->mma2[w2]);
+          second = false;
+          i2 = i2 == 2 ? 0 : i2 + 1;
+          ++n2;
+          did = true;
+        }
+      }
+      if (!end && n1 < n2 + 2 && test_bar(&sh->load[i1], par1) && (n1 < 2 || test_bar(&sh->o_free[w1], ((n1 >> 1) & 1) ^ 1))) {
+        const int4 t = sh->tile[i1];
+        if (t.x < 0) {
+          end = true;
+        } else if (!prep || test_bar(&sh->prep[w1], (n1 >> 1) & 1)) {
+          const int q1 = t.z;
+          tc_fence_after();
+          const uint64_t da = smem_desc(smem_u32(smem + q1 * kSlot), 16, 1024);
+          const uint64_t db = smem_desc(smem_u32(smem + wrap(q1 + 1) * kSlot), 16, 1024);
+          umma_c<false>(d1, da, db, kIdScore);
+          umma_c<true>(d1, da + 2, db + 2, kIdScore);
+          umma_c<true>(d1, da + 4, db + 4, kIdScore);
+          umma_c<true>(d1, da + 6, db + 6, kIdScore);
+          umma_commit(&sh->mma1[w1]);
+          if (R && !last) umma_commit(&sh->empty[q1]);
+          if (++i1 == 3) {
+            i1 = 0;
+            par1 ^= 1;
+          }
+          ++n1;
+          did = true;
+        }
+      }
+      if (did) {
+        idle = false;
+      } else if (!idle) {
+        idle = true;
+        t0 = clock64();
+      } else if (sh->abort_flag) {
+        return;
+      } else if (clock64() - t0 > P.wait_cycles) {
+        report_timeout(P.status, 20);
+        sh->abort_flag = 1;
+        return;
+      }
+    }
+  }
+
+  // ================================================================ store thread of group w
+  // Stores what the group has staged; sh->out[w] says what and where.
+  static __device__ __forceinline__ void store(const Params& P, uint8_t* smem, Shared* sh, int w) {
+    for (uint32_t par = 0;; par ^= 1) {
+      if (!wait_bar(&sh->staged[w], par, sh, P, 40)) break;
+      const int4 o = sh->out[w];          // head, first block or position, slot, y?
+      arrive(&sh->out_free[w]);
+      if (o.x < 0) break;
+      const uint8_t* s = smem + o.z * kSlot;
+      if (R) store_5d(o.w ? &P.rY : &P.rAL, s, o.y, o.x, 0);
+      else if (!P.last) store_5d(&P.lAR, s, o.y, o.x, 0);
+      else store_5d(&P.lOut, s, o.y, P.H ? o.x % P.H : o.x, P.H ? o.x / P.H : 0);
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+      asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+      arrive(&sh->empty[o.z]);
+    }
+    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+  }
+
+  // ================================================================ compute warps (thread = score row)
+  // bf16 -> f16 in a slot, rows of absent blocks zeroed.
+  static __device__ __forceinline__ void prepare(const Params& P, uint8_t* tile, bool convert, int idx0, int mv, int row) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int ch = q * 128 + row, r = ch >> 3;
+      uint4* p = reinterpret_cast<uint4*>(tile + ch * 16);
+      const bool absent = !FULL && P.seq_len != nullptr && (R ? idx0 + r / B >= mv : r % B >= mv);
+      if (absent) {
+        *p = make_uint4(0u, 0u, 0u, 0u);
+      } else if (kConvert && convert) {
+        uint4 v = *p;
+        uint32_t* w = reinterpret_cast<uint32_t*>(&v);
+#pragma unroll
+        for (int e = 0; e < 4; ++e)     // a bf16 is the upper half of an fp32; saturates at +-65504
+          asm("cvt.rn.satfinite.f16x2.f32 %0, %1, %2;"
+              : "=r"(w[e])
+              : "f"(__uint_as_float(w[e] & 0xffff0000u)), "f"(__uint_as_float(w[e] << 16)));
+        *p = v;
+      }
+    }
+    fence_proxy_async();
+  }
+  // Zero weights beside the B columns of a row's own block, in tensor memory.
+  static __device__ __forceinline__ void zeros_beside(uint32_t t_row, int r_blk) {
+    if constexpr (B < 128) {
+      uint32_t z[B / 2];
+#pragma unroll
+      for (int i = 0; i < B / 2; ++i) z[i] = 0u;
+#pragma unroll
+      for (int q = 1; q < 128 / B; ++q) st_cols<B / 2>(t_row + (B / 2) * ((r_blk + q) % (128 / B)), z);
+    }
+  }
+  // CH scores of an R row: p = exp2(f s - f mx), sums of p and p s, packed weights.
+  template <int CH>
+  static __device__ __forceinline__ void r_weights(const float* s, int col0, int lim, float f, float off, float2* a2,
+                                                   float2* z2, uint32_t* u) {
+    if (FULL || lim >= col0 + CH) {
+      const float2 f2 = make_float2(f, f), off2 = make_float2(off, off);
+#pragma unroll
+      for (int i = 0; i < CH / 2; ++i) {
+        const float2 x = make_float2(s[2 * i], s[2 * i + 1]);
+        const float2 z = ffma2(x, f2, off2);
+        const float2 p = make_float2(fast_exp2(z.x), fast_exp2(z.y));
+        z2[i & 1] = ffma2(p, x, z2[i & 1]);
+        a2[i & 1] = fadd2(a2[i & 1], p);
+        u[i] = pack2<TA>(p.x, p.y);
+      }
+    } else {       // keys past the block or past n_valid: weight 0
+#pragma unroll
+      for (int i = 0; i < CH / 2; ++i) {
+        const bool v0 = col0 + 2 * i < lim, v1 = col0 + 2 * i + 1 < lim;
+        const float p0 = v0 ? fast_exp2(fmaf(s[2 * i], f, off)) : 0.f, p1 = v1 ? fast_exp2(fmaf(s[2 * i + 1], f, off)) : 0.f;
+        z2[i & 1].x = fmaf(p0, v0 ? s[2 * i] : 0.f, z2[i & 1].x);
+        z2[i & 1].y = fmaf(p1, v1 ? s[2 * i + 1] : 0.f, z2[i & 1].y);
+        a2[i & 1] = fadd2(a2[i & 1], make_float2(p0, p1));
+        u[i] = pack2<TA>(p0, p1);
+      }
+    }
+  }
+  template <int CH>
+  static __device__ __forceinline__ void mask(float* s, int col0, int lim) {
+    if (!FULL && lim < col0 + CH) {
+#pragma unroll
+      for (int i = 0; i < CH; ++i)
+        if (col0 + i >= lim) s[i] = -INFINITY;
+    }
+  }
+  template <int CH>
+  static __device__ __forceinline__ void fold_max(const float* s, float* m4) {
+#pragma unroll
+    for (int i = 0; i < CH / 2; ++i) m4[i & 3] = max3(m4[i & 3], s[2 * i], s[2 * i + 1]);
+  }
+
+  // R: softmax over the keys of the row's block (Eq. 7; alpha_R arrives divided by c_R), weights to
+  // tensor memory, -c_L log2 e (Eq. 10) to global.  Returns 1 / sum.
+  static __device__ __forceinline__ float r_softmax(const Params& P, int h, int k, int n_valid, uint32_t t_row, int r_blk, int r_pos) {
+    const float f = P.scale * kLog2e;
+    const uint32_t tS = t_row + B * r_blk;
+    const int lim = FULL ? B : max(1, min(P.b, n_valid - k * P.b));      // keys of this block that count
+    float2 a2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, z2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+    float mx;
+    if constexpr (B >= 64) {
+      // two passes over the scores (a row does not fit the registers that four CTAs leave a thread), the
+      // next chunk's load in flight
+      {
+        float x[32];
+#pragma unroll
+        for (int cc = 0; cc < B / 32; ++cc) {
+          tmem_ld32(tS + 32 * cc, x);
+          tmem_ld_wait();
+          mask<32>(x, 32 * cc, lim);
+          fold_max<32>(x, m4);
+        }
+      }
+      float c16[2][16];
+      tmem_ld16(tS, c16[0]);
+      mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+#pragma unroll
+      for (int cc = 0; cc < B / 16; ++cc) {
+        tmem_ld_wait();
+        if (cc < B / 16 - 1) tmem_ld16(tS + 16 * (cc + 1), c16[(cc + 1) & 1]);
+        uint32_t u[8];
+        r_weights<16>(c16[cc & 1], 16 * cc, lim, f, -mx * f, a2, z2, u);
+        st_cols<8>(t_row + (B / 2) * r_blk + 8 * cc, u);       // over columns of the scores already read
+      }
+    } else {
+      float x[B];
+#pragma unroll
+      for (int cc = 0; cc < B / 32; ++cc) tmem_ld32(tS + 32 * cc, x + 32 * cc);
+      tmem_ld_wait();
+      mask<B>(x, 0, lim);
+      fold_max<B>(x, m4);
+      mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+#pragma unroll
+      for (int cc = 0; cc < B / 32; ++cc) {
+        uint32_t u[16];
+        r_weights<32>(x + 32 * cc, 32 * cc, lim, f, -mx * f, a2, z2, u);
+        st_cols<16>(t_row + (B / 2) * r_blk + 16 * cc, u);
+      }
+    }
+    zeros_beside(t_row, r_blk);
+    const float sum = (a2[0].x + a2[0].y) + (a2[1].x + a2[1].y);
+    const float sz = (z2[0].x + z2[0].y) + (z2[1].x + z2[1].y);
+    const float inv_s = 1.f / sum;
+    if (FULL || (r_pos < P.b && k < P.m))
+      P.cL[((size_t)h * P.b + r_pos) * P.mp + k] = fast_log2(sum) - f * (sz * inv_s - mx);
+    tmem_st_wait();
+    return inv_s;
+  }
+
+  // CH scores of an L row to logits z = f s - c_L (Eq. 8), in place.
+  template <int CH>
+  static __device__ __forceinline__ void l_logits(float* s, const float* c, float f) {
+    const float4* c4 = reinterpret_cast<const float4*>(c);
+    const float2 f2 = make_float2(f, f);
+#pragma unroll
+    for (int i = 0; i < CH / 4; ++i) {
+      const float4 k4 = c4[i];
+      const float2 za = ffma2(make_float2(s[4 * i], s[4 * i + 1]), f2, make_float2(k4.x, k4.y));
+      const float2 zb = ffma2(make_float2(s[4 * i + 2], s[4 * i + 3]), f2, make_float2(k4.z, k4.w));
+      s[4 * i] = za.x; s[4 * i + 1] = za.y; s[4 * i + 2] = zb.x; s[4 * i + 3] = zb.y;
+    }
+  }
+  // CH logits to weights exp2(z - mx), in place.
+  template <int CH>
+  static __device__ __forceinline__ void l_weights(float* z, float mx, float2* a2) {
+    const float2 nmx2 = make_float2(-mx, -mx);
+#pragma unroll
+    for (int i = 0; i < CH / 2; ++i) {
+      const float2 d = fadd2(make_float2(z[2 * i], z[2 * i + 1]), nmx2);
+      const float2 p = make_float2(fast_exp2(d.x), fast_exp2(d.y));
+      a2[i & 1] = fadd2(a2[i & 1], p);
+      z[2 * i] = p.x;
+      z[2 * i + 1] = p.y;
+    }
+  }
+  template <int CH>
+  static __device__ __forceinline__ void pack_cols(const float* v, uint32_t* u) {
+#pragma unroll
+    for (int i = 0; i < CH / 2; ++i) u[i] = pack2<TA>(v[2 * i], v[2 * i + 1]);
+  }
+  // 16 weights of a row, times `on` and the column scales, to the shared-memory operand: `base` is the
+  // row's 128 bytes in the 64-column chunk, col its first column there (128-byte swizzle).
+  static __device__ __forceinline__ void emit16(const float* v, uint8_t* base, int col, float on, const float* scale, int row) {
+    const float2 on2 = make_float2(on, on);
+    const float4* g4 = reinterpret_cast<const float4*>(scale);
+    uint32_t u[8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float2 a = fmul2(make_float2(v[4 * i], v[4 * i + 1]), on2), b = fmul2(make_float2(v[4 * i + 2], v[4 * i + 3]), on2);
+      const float4 g = g4[i];
+      a = fmul2(a, make_float2(g.x, g.y));
+      b = fmul2(b, make_float2(g.z, g.w));
+      u[2 * i] = pack2<TA>(a.x, a.y);
+      u[2 * i + 1] = pack2<TA>(b.x, b.y);
+    }
+    const int c0 = col >> 3;
+    *reinterpret_cast<uint4*>(base + ((c0 ^ (row & 7)) << 4)) = make_uint4(u[0], u[1], u[2], u[3]);
+    *reinterpret_cast<uint4*>(base + (((c0 + 1) ^ (row & 7)) << 4)) = make_uint4(u[4], u[5], u[6], u[7]);
+  }
+  // Maxima of 32 columns over the warp's rows, to the shared maxima.
+  static __device__ __forceinline__ void fold_columns(const float* v, float on, unsigned* sMax, int lane) {
+    unsigned keep = 0u;
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+      const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(v[i] * on));
+      if (lane == i) keep = w;
+    }
+    atomicMax(sMax + lane, keep);
+  }
+
+
+  static __device__ __forceinline__ void compute(const Params& P, uint8_t* smem, Shared* sh, uint32_t tmem, int w) {
+    const int row = threadIdx.x & 127, warp = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
+    const uint32_t t_row = tmem + 128 * w + ((uint32_t)(warp * 32) << 16);     // this warp's TMEM lanes
+    const bool prep = prepares(P), last = P.last != 0;
+    int i3 = w;
+    // Parities: load (round of three tiles), one phase per tile of the group, and the barriers that
+    // only some tiles use.
+    uint32_t par_l = 0, par = 0, par_t = 0, par_1 = 0, par_c = 0, par_o = 1;
+#define MA_WAIT(BAR, PAR, WHERE) \
+  if (!__all_sync(0xffffffffu, wait_bar(&(BAR), PAR, sh, P, WHERE))) return
+    // Staged rows (or the end) to the store thread, once it has taken the word of the one before.
+    auto hand_over = [&](int h, int idx0, int slot, int is_y) {
+      const bool ok = wait_bar(&sh->out_free[w], par_o, sh, P, 38);
+      par_o ^= 1;
+      if (row == 0) sh->out[w] = make_int4(h, idx0, slot, is_y);
+      arrive(&sh->staged[w]);
+      return ok;
+    };
+    for (;; par ^= 1) {
+      MA_WAIT(sh->load[i3], par_l, 30);
+      const int4 t = sh->tile[i3];               // head, first block or position, slot, keys that count
+      if (t.x < 0) {
+        hand_over(-1, 0, 0, 0);
+        return;
+      }
+      const float* sC = reinterpret_cast<const float*>(smem + kOffVec) + i3 * 128;
+      if (i3 == 0) {
+        i3 = 2;
+      } else {
+        i3 -= 1;
+        par_l ^= 1;
+      }
+      const int h = t.x, idx0 = t.y, e0 = t.z, e1 = wrap(e0 + 1);
+      uint8_t *s0 = smem + e0 * kSlot, *s1 = smem + e1 * kSlot;
+      const int r_blk = row / B, r_pos = row % B;   // block of the tile, row in it
+      const int mv = FULL ? P.m : (t.w + P.b - 1) / P.b;                            // blocks that are present
+      if (prep) {
+        prepare(P, s0, !R || P.first, idx0, mv, row);      // Q, but not alpha_R
+        prepare(P, s1, R, idx0, mv, row);                   // K, but not alpha_L
+        arrive(&sh->prep[w]);
+      }
+      MA_WAIT(sh->mma1[w], par, 31);
+      tc_fence_after();
+      if (last && warp == 0 && elect_one()) {    // the third operand, over the first: the score MMA has read it
+        mbar_expect_tx(&sh->third[w], kSlot);
+        if (R) load_5d(s0, &P.rV, &sh->third[w], 0, idx0, P.H ? h % P.H : h, P.H ? h / P.H : 0);
+        else load_5d(s0, &P.lY, &sh->third[w], 0, idx0, h, 0);
+      }
+      __syncwarp();
+      if (FULL && P.discard) {     // the state rows the score MMA consumed are read exactly once: drop them from L2
+        if (!R) discard_line(P.aL + ((size_t)(h * P.b + idx0) * P.m + row) * 128);
+        else if (!P.first) discard_line(P.aR + ((size_t)(h * P.m + idx0) * P.b + row) * 128);
+      }
+      float mul;                                 // of the accumulator rows in the epilogue
+      if constexpr (R) {
+        mul = r_softmax(P, h, idx0 + r_blk, t.w, t_row, r_blk, r_pos);
+      } else {
+        // ============================================================ L: softmax over the blocks
+        const float f = P.scale * kLog2e;
+        const uint32_t tS = t_row + B * r_blk;
+        const float* cv = sC + B * r_blk;
+        const int lim = FULL ? B : mv;
+        float2 a2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+        float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+        float mx;
+        {
+          // logits back over the scores, then weights (final: 16-bit, as the MMA's operand)
+          float x[2][16];
+          tmem_ld16(tS, x[0]);
+#pragma unroll
+          for (int cc = 0; cc < B / 16; ++cc) {
+            float* cur = x[cc & 1];
+            tmem_ld_wait();
+            if (cc < B / 16 - 1) tmem_ld16(tS + 16 * (cc + 1), x[(cc + 1) & 1]);
+            l_logits<16>(cur, cv + 16 * cc, f);
+            mask<16>(cur, 16 * cc, lim);
+            fold_max<16>(cur, m4);
+            tmem_st16(tS + 16 * cc, cur);
+          }
+          mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+          tmem_st_wait();
+          tmem_ld16(tS, x[0]);
+#pragma unroll
+          for (int cc = 0; cc < B / 16; ++cc) {
+            float* cur = x[cc & 1];
+            tmem_ld_wait();
+            if (cc < B / 16 - 1) tmem_ld16(tS + 16 * (cc + 1), x[(cc + 1) & 1]);
+            l_weights<16>(cur, mx, a2);
+            if (last) {
+              uint32_t u[8];
+              pack_cols<16>(cur, u);
+              st_cols<8>(t_row + (B / 2) * r_blk + 8 * cc, u);
+            } else {
+              tmem_st16(tS + 16 * cc, cur);
+            }
+          }
+        }
+        if (last) zeros_beside(t_row, r_blk);
+        const float sum = (a2[0].x + a2[0].y) + (a2[1].x + a2[1].y);
+        mul = 1.f / sum;
+        tmem_st_wait();
+        if (last) {
+          // Row b l + j (l = r_pos, j = idx0 + r_blk) of the final L half-step: its log-sum-exp; summed
+          // over the rows of a head it is the value of the objective (Eq. 6) at the returned matrix.
+          if (P.lse != nullptr && r_pos < P.m && idx0 + r_blk < P.b)
+            P.lse[(size_t)h * P.N + (size_t)r_pos * P.b + idx0 + r_blk] = (mx + fast_log2(sum)) * kLn2;
+          if (!FULL && r_pos >= mv) mul = 0.f;        // rows of absent blocks
+        } else {
+          // alpha_R(k,j) = sum_l L[l,k] Q(l,j) / c_R: the contraction runs over the rows of the weights,
+          // so they are normalised before they are rounded, and go through shared memory (over
+          // alpha_L, which the score MMA has read; at B = 128 with a slot of their own for one half).
+          const float on = FULL || r_pos < mv ? mul : 0.f;     // rows past the last block: weight 0
+          float* scale = reinterpret_cast<float*>(smem + kOffScale) + 128 * w;
+          {
+            // column k times 2^-(exponent of its largest weight)
+            unsigned* sMax = reinterpret_cast<unsigned*>(smem + kOffCol) + 128 * w;
+            float x[32];
+#pragma unroll 1
+            for (int cc = 0; cc < B / 32; ++cc) {
+              tmem_ld32(tS + 32 * cc, x);
+              tmem_ld_wait();
+              fold_columns(x, on, sMax + B * r_blk + 32 * cc, lane);
+            }
+            arrive(&sh->cols[w]);
+            MA_WAIT(sh->cols[w], par_c, 34);
+            scale[row] = __uint_as_float((253u << 23) - (sMax[row] & 0x7f800000u));
+            sMax[row] = 0u;
+            arrive(&sh->cols[w]);
+            MA_WAIT(sh->cols[w], par_c ^ 1, 35);
+          }
+          float x[2][16];
+          tmem_ld16(tS, x[0]);
+          const int e2 = wrap(e1 + 1);
+          uint8_t* p_lo = smem + (B == 128 ? min(e1, e2) : e1) * kSlot + row * 128;
+          uint8_t* p_hi = smem + (B == 128 ? max(e1, e2) : e1) * kSlot + row * 128;
+          const int win = B == 32 ? 32 * (r_blk & 1) : 0;
+#pragma unroll
+          for (int cc = 0; cc < B / 16; ++cc) {
+            tmem_ld_wait();
+            if (cc < B / 16 - 1) tmem_ld16(tS + 16 * (cc + 1), x[(cc + 1) & 1]);
+            emit16(x[cc & 1], cc < 4 ? p_lo : p_hi, win + (16 * cc & 63), on, scale + B * r_blk + 16 * cc, row);
+          }
+          if constexpr (B == 32) {               // zeros beside the window
+            const int c0 = (32 - win) >> 3;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4*>(p_lo + (((c0 + c) ^ (row & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
+          }
+          fence_proxy_async();
+        }
+      }
+      if (last && prep) {
+        MA_WAIT(sh->third[w], par_t, 36);
+        par_t ^= 1;
+        prepare(P, s0, R, idx0, mv, row);                   // V, but not y
+      }
+      tc_fence_before();
+      arrive(&sh->weights[w]);
+      // ============================================================== epilogue
+      float o[32];
+      if (R && last) {                           // alpha_L, over K; then y, over V
+        MA_WAIT(sh->first[w], par_1, 32);
+        par_1 ^= 1;
+        tc_fence_after();
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          tmem_ld32(t_row + 64 + 32 * hf, o);
+          tmem_ld_wait();
+          store_row32<TA>(s1, row, 32 * hf, o, mul);
+        }
+        tc_fence_before();
+        arrive(&sh->oread[w]);
+        fence_proxy_async();
+        if (!__all_sync(0xffffffffu, hand_over(h, idx0, e1, 0))) return;
+      }
+      MA_WAIT(sh->mma2[w], par, 33);
+      tc_fence_after();
+      int out_row = row;
+      if (!R && !last) {
+        if constexpr (!R && B < 128) out_row = ((lane >> 4) << 6) + 16 * warp + (lane & 15);
+        const float cr = ld_col(t_row);
+        tmem_ld_wait();
+        mul = cr > 1e-30f ? 1.f / cr : 0.f;
+      }
+      if (FULL && P.discard && !R && last) discard_line(P.y + ((size_t)(h * P.b + idx0) * P.m + row) * 128);
+      // rows go: alpha_L over K, y over V (first slot), alpha_R over Q (first), Y over alpha_L (second)
+      const bool to_first = R ? last : !last;
+      uint8_t* dst = to_first ? s0 : s1;
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        tmem_ld32(t_row + 64 + 32 * hf, o);
+        tmem_ld_wait();
+        if (hf == 1) {                           // the next tile's scores may come
+          tc_fence_before();
+          arrive(&sh->o_free[w]);
+        }
+        if (!R && last) {
+          if (!FULL && mul == 0.f) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) o[i] = 0.f;
+          }
+          store_row32<TIn>(dst, out_row, 32 * hf, o, mul);
+        } else {
+          store_row32<TA>(dst, out_row, 32 * hf, o, mul);
+        }
+      }
+      fence_proxy_async();
+      if (!__all_sync(0xffffffffu, hand_over(h, idx0, to_first ? e0 : e1, R && last))) return;
+    }
+#undef MA_WAIT
+  }
+};
+
+template <typename TIn, int B, bool FULL, int MODE>
+__global__ void __launch_bounds__(kThreads, kCtasPerSm) monarch_tiles(const __grid_constant__ Params P) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  Shared* sh = reinterpret_cast<Shared*>(smem + kOffBar);
+  const int tid = threadIdx.x, warp = tid >> 5;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (tid == 0) {
+    for (int i = 0; i < 3; ++i) mbar_init(&sh->load[i], 1);
+    for (int i = 0; i < kSlots; ++i) mbar_init(&sh->empty[i], 1);
+    for (int w = 0; w < 2; ++w) {
+      mbar_init(&sh->mma1[w], 1);
+      mbar_init(&sh->first[w], 1);
+      mbar_init(&sh->mma2[w], 1);
+      mbar_init(&sh->third[w], 1);
+      mbar_init(&sh->out_free[w], 1);
+      mbar_init(&sh->prep[w], 128);
+      mbar_init(&sh->weights[w], 128);
+      mbar_init(&sh->oread[w], 128);
+      mbar_init(&sh->o_free[w], 128);
+      mbar_init(&sh->staged[w], 128);
+      mbar_init(&sh->cols[w], 128);
+    }
+    sh->abort_flag = 0;
+    fence_barrier_init();
+  }
+  if (tid < 128) {
+    const uint32_t one2 = pack2<__half>(1.f, 1.f);
+    *reinterpret_cast<uint4*>(smem + kOffOnes + tid * 16) = make_uint4(one2, one2, one2, one2);
+  }
+  for (int i = tid; i < 3 * 128; i += kThreads) reinterpret_cast<float*>(smem + kOffVec)[i] = 0.f;
+  if (tid < 256) reinterpret_cast<unsigned*>(smem + kOffCol)[tid] = 0u;
+  if (warp == 8) tmem_alloc(&sh->tmem, 256);
+  fence_proxy_async();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = sh->tmem;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (MODE == 0 && P.first && blockIdx.x == 0 && tid == 0) *P.status = 0;
+  using K = Kernel<TIn, B, FULL, MODE>;
+  // registers: 384 threads at the launch's 80; 128 x 48 + 256 x 96 make use of all of them
+  if (warp >= 8) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+    if (elect_one()) {
+      if (warp == 8) K::produce(P, smem, sh);
+      else if (warp == 9) K::issue(P, smem, sh, tmem);
+      else K::store(P, smem, sh, warp - 10);
+    }
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 96;");
+    K::compute(P, smem, sh, tmem, warp >> 2);
+  }
+  __syncwarp();
+  tc_fence_before();
+  __syncthreads();
+  if (sh->abort_flag) {                 // what is in flight lands before the CTA leaves
+    const long long t0 = clock64();
+    while (clock64() - t0 < 200000) __nanosleep(1000);
+    __syncthreads();
+  }
+  if (warp == 8) tmem_dealloc(tmem, 256);
+}
+
+// ------------------------------------------------------------------------------------ host side
+struct Args {
+  const void *Q, *K, *V;
+  void* Y;
+  int BH, N, d, b, m, T, dtype, H, heads, n_valid;
+  float scale;
+  float* lse;
+  const int* seq_len;
+};
+struct States {
+  void *aL, *aR, *y;       // f16, BH * N rows of d
+  float* cL;               // BH * b rows of pad4(m)
+  int* status;
+};
+inline int pad4(int m) { return (m + 3) & ~3; }
+inline bool supported(int N, int d, int b, int m, int dtype, int BH) {
+  return (dtype == 1 || dtype == 2) && d % 8 == 0 && d <= 64 && b <= 128 && m <= 128 && (long long)BH * N < (1LL << 31);
+}
+// 2T launches, one per half-step.
+int launch(const Args& a, const States& s, cudaStream_t st);
+
+#ifdef MA_TU_TILE_TC
+inline int pad_block(int x) { return x <= 32 ? 32 : (x <= 64 ? 64 : 128); }
+
+// View (d, i, k, h0, h1) with byte strides s1 .. s4; box of 128 rows: B of the second dimension,
+// 128 / B of the third.
+inline bool make_map5(CUtensorMap* tm, int dtype, const void* base, const uint64_t (&n)[5], const uint64_t (&s)[4], int B) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[5], strides[4];
+  for (int i = 0; i < 5; ++i) dims[i] = n[i];
+  for (int i = 0; i < 4; ++i) strides[i] = s[i];
+  cuuint32_t box[5] = {kD, (cuuint32_t)B, (cuuint32_t)(128 / B), 1, 1}, es[5] = {1, 1, 1, 1, 1};
+  return fn(tm, dtype == 1 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base),
+            dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+inline bool make_maps(Params* P, const Args& a, const States& s) {
+  const uint64_t d2 = (uint64_t)a.d * 2, b = a.b, m = a.m, N = a.N, BH = a.BH, H = a.H ? a.H : 1;
+  const int BR = pad_block(a.b), BL = pad_block(a.m);
+  // inputs and output: rows d2 (or heads * d2) apart
+  const uint64_t row = d2 * H, h0 = a.H ? a.H : BH, h1 = a.H ? BH / a.H : 1;
+  const uint64_t s0 = a.H ? d2 : N * d2, s1 = N * d2 * (a.H ? H : BH);
+  const uint64_t rn[5] = {(uint64_t)a.d, b, m, h0, h1}, rs[4] = {row, b * row, s0, s1};
+  const uint64_t ln[5] = {(uint64_t)a.d, m, b, h0, h1}, ls[4] = {b * row, row, s0, s1};
+  // states: alpha_L, y [BH][b][m][d]; alpha_R [BH][m][b][d] -- every load reads contiguous rows, the
+  // permutation between the half-steps is in the strides of the stores
+  const uint64_t srn[5] = {(uint64_t)a.d, b, m, BH, 1}, sln[5] = {(uint64_t)a.d, m, b, BH, 1};
+  const uint64_t l_st[4] = {m * d2, d2, N * d2, N * d2 * BH}, l_ld[4] = {d2, m * d2, N * d2, N * d2 * BH};
+  const uint64_t r_ld[4] = {d2, b * d2, N * d2, N * d2 * BH}, r_st[4] = {b * d2, d2, N * d2, N * d2 * BH};
+  return make_map5(&P->rQ, a.dtype, a.Q, rn, rs, BR) && make_map5(&P->rK, a.dtype, a.K, rn, rs, BR) &&
+         make_map5(&P->rV, a.dtype, a.V, rn, rs, BR) && make_map5(&P->rAR, 1, s.aR, srn, r_ld, BR) &&
+         make_map5(&P->rAL, 1, s.aL, srn, l_st, BR) && make_map5(&P->rY, 1, s.y, srn, l_st, BR) &&
+         make_map5(&P->lQ, a.dtype, a.Q, ln, ls, BL) && make_map5(&P->lAL, 1, s.aL, sln, l_ld, BL) &&
+         make_map5(&P->lY, 1, s.y, sln, l_ld, BL) && make_map5(&P->lAR, 1, s.aR, sln, r_st, BL) &&
+         make_map5(&P->lOut, a.dtype, a.Y, ln, ls, BL);
+}
+// Tensor maps depend only on the addresses and the shape; encoding eleven of them costs several
+// times the launch, so the maps of the last few problems are kept.
+struct MapKey {
+  const void *Q, *K, *V, *Y, *aL, *aR;
+  int BH, N, d, b, dtype, H, dev;
+  bool operator==(const MapKey& o) const {
+    return Q == o.Q && K == o.K && V == o.V && Y == o.Y && aL == o.aL && aR == o.aR && BH == o.BH && N == o.N && d == o.d &&
+           b == o.b && dtype == o.dtype && H == o.H && dev == o.dev;
+  }
+};
+struct MapCache {
+  static constexpr int kEntries = 16;
+  MapKey key[kEntries];
+  Params maps[kEntries];
+  bool used[kEntries] = {};
+  int next = 0, last = 0;
+};
+inline bool cached_maps(Params* P, const Args& a, const States& s, int dev) {
+  static thread_local MapCache c;
+  const MapKey key{a.Q, a.K, a.V, a.Y, s.aL, s.aR, a.BH, a.N, a.d, a.b, a.dtype, a.H, dev};
+  for (int i = 0; i < MapCache::kEntries; ++i) {
+    const int e = (c.last + i) % MapCache::kEntries;
+    if (c.used[e] && c.key[e] == key) {
+      c.last = e;
+      *P = c.maps[e];
+      return true;
+    }
+  }
+  if (!make_maps(P, a, s)) return false;
+  const int e = c.next;
+  c.next = (c.next + 1) % MapCache::kEntries;
+  c.key[e] = key;
+  c.maps[e] = *P;
+  c.used[e] = true;
+  c.last = e;
+  return true;
+}
+struct Device {
+  int dev = -1, sms = 0;
+};
+inline bool current_device(Device* d) {
+  static int sms[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+  if (sms[dev] == 0 && cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
+  d->dev = dev;
+  d->sms = sms[dev];
+  return d->sms > 0;
+}
+template <typename TIn, int B, bool FULL, int MODE>
+inline int launch_kernel(const Params& P, const Device& dev, cudaStream_t st) {
+  auto kern = monarch_tiles<TIn, B, FULL, MODE>;
+  static bool prepared[64] = {};
+  if (!prepared[dev.dev]) {
+    if (cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess) return 7;
+    prepared[dev.dev] = true;
+  }
+  // (the next half-step's CTAs take SM slots and set up as this one's drain; they wait for its end
+  // before they touch memory)
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(P.tiles < kCtasPerSm * dev.sms ? P.tiles : kCtasPerSm * dev.sms);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = kSmem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, P) == cudaSuccess ? 0 : 7;
+}
+template <typename TIn, int MODE>
+inline int launch_half(Params& P, const Device& dev, cudaStream_t st, bool masked) {
+  const int x = MODE == 0 ? P.b : P.m, n = MODE == 0 ? P.m : P.b, B = pad_block(x);      // n blocks of x rows
+  P.per_head = (n + 128 / B - 1) / (128 / B);
+  P.tiles = P.BH * P.per_head;
+  const bool full = !masked && x == B && n % (128 / B) == 0;
+#define MA_H(B) (full ? launch_kernel<TIn, B, true, MODE>(P, dev, st) : launch_kernel<TIn, B, false, MODE>(P, dev, st))
+  return B == 32 ? MA_H(32) : (B == 64 ? MA_H(64) : MA_H(128));
+#undef MA_H
+}
+template <typename TIn>
+inline int launch_t(const Args& a, const States& s, cudaStream_t st) {
+  Device dev;
+  Params P;
+  if (!current_device(&dev) || !cached_maps(&P, a, s, dev.dev)) return 7;
+  P.cL = s.cL;
+  P.aL = (uint8_t*)s.aL; P.aR = (uint8_t*)s.aR; P.y = (uint8_t*)s.y;
+  P.lse = a.lse; P.seq_len = a.seq_len; P.status = s.status;
+  P.N = a.N; P.b = a.b; P.m = a.m; P.mp = pad4(a.m); P.BH = a.BH; P.H = a.H; P.heads = a.heads; P.n_valid = a.n_valid;
+  P.discard = a.d == 64;       // (a row is then a line)
+  P.wait_cycles = kWaitCycles;
+  P.scale = a.scale;
+  for (int t = 0; t < a.T; ++t) {
+    P.first = t == 0;
+    P.last = t == a.T - 1;
+    const int rc = launch_half<TIn, 0>(P, dev, st, a.n_valid < a.N || a.seq_len != nullptr);
+    if (rc != 0) return rc;
+    const int rl = launch_half<TIn, 1>(P, dev, st, a.seq_len != nullptr);
+    if (rl != 0) return rl;
+  }
+  return 0;
+}
+int launch(const Args& a, const States& s, cudaStream_t st) {
+  return a.dtype == 1 ? launch_t<__half>(a, s, st) : launch_t<__nv_bfloat16>(a, s, st);
+}
+#endif  // MA_TU_TILE_TC
+
+}  // namespace ttc
+}  // namespace ma

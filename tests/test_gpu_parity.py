@@ -972,3 +972,47 @@ def test_seeded_sweep_of_shapes_through_every_entry_point(seed):
         assert err <= TOL[dtype], (what, err)
         done += 1
     assert done >= 80
+
+
+# ------------------------------------------------------------------ tcgen05 tiles of MA_PATH_TILE_MMA
+@pytest.mark.parametrize("BH,N,b,d,T,dtype,mode", [
+    (64, 31 * 33, 33, 24, 2, "f16", "fwd"),       # one row more than a 32-row block; m one less
+    (56, 1024, 32, 48, 2, "bf16", "bshd"),        # four full blocks a tile, rows narrower than the tile
+    (60, 960, 30, 64, 1, "f16", "objective"),     # ragged blocks, the last tile of a head half empty
+    (30, 65 * 63, 65, 64, 2, "f16", "padded"),    # one row more than a 64-row block
+    (12, 128 * 128, 128, 64, 2, "f16", "varlen"),  # whole tiles, most blocks of some sequences absent
+    (12, 127 * 60, 127, 56, 1, "bf16", "padded"),
+    (16, 64 * 128, 64, 64, 2, "bf16", "varlen"), (40, 2048, 64, 64, 1, "f16", "fwd"), (150, 3 * 128, 128, 8, 2, "f16", "fwd"),
+])
+def test_tensor_core_tiles_agree_with_the_generic_kernels(BH, N, b, d, T, dtype, mode):
+    """Enough tiles for the tcgen05 kernels of the tile path: every head against the fp32 kernels on the
+    same values, at the edges of the 32 / 64 / 128-row blocks and through every entry point."""
+    batch, heads = 2, BH // 2
+    Q, K, V = (torch.from_numpy(x).cuda() for x in wl.make_qkv(batch, heads, N, d, dtype, min(8, d), 1.0, seed=N + T))
+    x16 = [x.to(binding.torch_dtype(dtype)) for x in (Q, K, V)]
+    rows, lens = slice(None), None
+    if mode == "padded":
+        nv = N - b // 2
+        Y, ref = (binding.monarch_attn_fwd_padded(*x, b, T, nv) for x in (x16, (Q, K, V)))
+        rows = slice(0, nv)
+    elif mode == "varlen":
+        sl = torch.tensor([N - b // 3, N // 3], dtype=torch.int32, device="cuda")
+        lens = sl.tolist()
+        for x in x16:
+            x[1, :, -(-lens[1] // b) * b:] = float("nan")          # absent blocks: never read
+        Y, ref = (binding.monarch_attn_fwd_varlen(*x, b, T, sl) for x in (x16, (Q, K, V)))
+        assert bool((Y[1, :, -(-lens[1] // b) * b:] == 0).all())
+    elif mode == "bshd":
+        Y = binding.monarch_attn_fwd_bshd(*(x.transpose(1, 2).contiguous() for x in x16), b, T).transpose(1, 2)
+        ref = binding.monarch_attn_fwd_ex(Q, K, V, b, T, path=binding.MA_PATH_GENERIC)
+    elif mode == "objective":
+        (Y, lse), (ref, lse_ref) = (binding.monarch_attn_fwd_objective(*x, b, T, path=p)
+                                    for x, p in ((x16, binding.MA_PATH_TILE_MMA), ((Q, K, V), binding.MA_PATH_GENERIC)))
+        assert float((lse - lse_ref).abs().max()) <= 5e-2
+    else:
+        Y = binding.monarch_attn_fwd_ex(*x16, b, T, path=binding.MA_PATH_TILE_MMA)
+        ref = binding.monarch_attn_fwd_ex(Q, K, V, b, T, path=binding.MA_PATH_GENERIC)
+    for e in range(batch):
+        r = slice(0, lens[e]) if lens else rows
+        err = ((Y[e, :, r].float() - ref[e, :, r]).flatten(1).norm(dim=1) / ref[e, :, r].flatten(1).norm(dim=1)).max()
+        assert float(err) <= (2e-3 if dtype == "f16" else 5e-3), (e, float(err))
