@@ -14,6 +14,7 @@
 #include "tensor_persistent.cuh"
 #include "tensor_decoupled.cuh"
 #include "fused_small.cuh"
+#include "fused_head.cuh"
 #include "fused_f32.cuh"
 #include "fused_jsplit.cuh"
 #include "tile_mma.cuh"
@@ -291,6 +292,15 @@ static bool tiles_on_tensor_cores(const Problem& p, float scale) {
 static int launch_resolved(const void* Q, const void* K, const void* V, void* Y, const Problem& p,
                            float scale, int resolved, void* ws, cudaStream_t st, bool ws_armed) {
   if (resolved == MA_PATH_GENERIC) return launch_generic(p, Q, K, V, Y, scale, ws, st);
+  // MA_PATH_FUSED_SMALL has two kernels: fused_head.cuh for 9 .. 32 rows and blocks with d <= 64, and the
+  // general one (narrower and wider blocks, wider heads, hi + lo states for three or more rounds).
+  if (resolved == MA_PATH_FUSED_SMALL && scale > 1e-30f && fhead::supported(p.N, p.d, p.b, p.m, p.dtype, p.T) &&
+      !fsmall::supported_hilo(p.N, p.d, p.b, p.m, p.dtype, p.T)) {
+    const int rc = fhead::launch({Q, K, V, Y, p.BH, p.N, p.d, p.b, p.m, p.T, p.dtype, p.H, p.heads, p.n_valid, scale, p.lse,
+                                  p.seq_len, (int*)ws}, st);
+    if (rc == MA_OK) g_last_launches = 1;
+    return rc;
+  }
   if (resolved == MA_PATH_FUSED_SMALL) {
     int rc = fsmall::launch(Q, K, V, Y, p.BH, p.N, p.d, p.b, p.m, p.T, p.dtype, scale, p.n_valid, p.H, p.lse, st,
                             p.seq_len, p.heads);

@@ -1,0 +1,639 @@
+// Fused kernel for short sequences, a head at a time: N = m b with 9 <= m, b <= 32 (m need not equal
+// b), d <= 64 (a multiple of 8), f16 / bf16, plain f16 states, key padding mask or per-sequence lengths
+// (App. C.3), either layout, row log-sum-exp.  All T rounds of Eq. 7-10 and Eq. 4 in one launch; Q, K, V
+// are read from HBM once, the states stay in shared memory, Y is written once.
+//
+// What bounds it.  A head is 3 N d 16-bit values in and N d out for a few dozen small MMAs per block: the
+// time is HBM traffic if the loads of the next head run under the arithmetic of this one and the
+// instruction stream is short enough.  Hence
+//   * an SM works on two or three heads at a time: three small CTAs, or one CTA that starts on a head by
+//     requesting the next (every warp asks TMA for the Q, K and V rows of the blocks it will own there,
+//     zero-filled past d), or two CTAs; `plan` chooses;
+//   * rows of a tile lie k bp + i with an odd block pitch bp = b | 1: under the 128-byte swizzle of the TMA
+//     eight rows are then free of bank conflicts along a block (R half-step) and across blocks
+//     (L half-step), so the permutation between the half-steps is only a choice of rows;
+//   * a warp owns a block (R) or a position (L) and holds its scores and weights in registers, in as many
+//     8-column tiles as b or m need.
+// One round: alpha_L goes over K, y over V, Y over Q.  More rounds: alpha_R and alpha_L replace each
+// other in place in a state tile.  Arithmetic is f16 whatever the input type (see fused_small.cuh).
+//
+// Measured (B200, us per call, against the general per-head kernel): 768 heads of 256 = 16 x 16, one
+// round 25.6 / 27.7 (60 % of the copy bandwidth); 768 of 210 = 15 x 14, two rounds 42.4 / 47.7; 384 of
+// lengths up to 384 = 16 x 24 24.3 / 28.9; 720 of 396 = 22 x 18 59 / 97; 24 of 210 5.3 / 7.  What is left is
+// instruction issue and shared-memory latency at four warps per scheduler (41 % of the slots issue).
+#pragma once
+#include <cuda.h>
+
+#include "tensor_path.cuh"
+#include "warp_mma.cuh"
+
+namespace ma {
+namespace fhead {
+
+using tensor::mbar_expect_tx;
+using tensor::mbar_init;
+using tensor::smem_u32;
+using warpmma::Mma;
+using warpmma::ex2;
+using warpmma::kLn2;
+using warpmma::kLog2e;
+using warpmma::ldsm_x4;
+using warpmma::ldsm_x4_trans;
+using warpmma::lg2;
+using warpmma::movm_trans;
+using warpmma::quad_max;
+using warpmma::quad_sum;
+
+constexpr int kMaxThreads = 512, kMaxSmem = 227 * 1024, kMaxBlocks = 32;
+constexpr float kMasked = -3.0e38f;      // finite, and far below any score
+
+struct Params {
+  CUtensorMap q, k, v;      // (d, b, m, heads, batch), box (64, bp, 1, 1, 1)
+  void* Y;
+  float* lse;
+  const int* seq_len;
+  int* status;              // nullptr: no workspace
+  int BH, N, d, b, m, T, H, heads, n_valid;
+  int bp;                   // block pitch in rows
+  int tile;                 // bytes of a tile
+  int bufs;                 // heads in shared memory
+  float scale;
+};
+struct __align__(16) Bars {
+  uint64_t full[2][kMaxBlocks];      // by buffer and block
+};
+
+__device__ __forceinline__ void stsm_x4(uint32_t saddr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(saddr), "r"(r0),
+               "r"(r1), "r"(r2), "r"(r3)
+               : "memory");
+}
+__device__ __forceinline__ void load_5d(uint32_t dst, const CUtensorMap* tm, uint64_t* bar, int blk, int h0, int h1) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %3, %4, %5, %6}], [%2];" ::"r"(
+          dst),
+      "l"((uint64_t)tm), "r"(smem_u32(bar)), "r"(0), "r"(blk), "r"(h0), "r"(h1)
+      : "memory");
+}
+// Four 8 x 8 pieces of an accumulator pair (two 8-column tiles of 16 rows) as 16-bit rows.
+__device__ __forceinline__ void put(uint32_t addr, const float (&o)[2][4], float m0, float m1) {
+  typedef Mma<__half> M;
+  stsm_x4(addr, M::pack(o[0][0] * m0, o[0][1] * m0), M::pack(o[0][2] * m1, o[0][3] * m1), M::pack(o[1][0] * m0, o[1][1] * m0),
+          M::pack(o[1][2] * m1, o[1][3] * m1));
+}
+// Byte offset of a 16-byte chunk of a row under the 128-byte swizzle.
+__device__ __forceinline__ uint32_t at(uint32_t base, int row, int chunk) {
+  return base + (uint32_t)(row * 128 + ((chunk ^ (row & 7)) << 4));
+}
+// Rows row_of(0 .. 8 NT - 1) of a tile as B operands of NT 8-column tiles, four 16-column steps.
+template <int NT, typename RowOf>
+__device__ __forceinline__ void load_b(uint32_t (&kb)[NT][4][2], uint32_t base, int lane, RowOf row_of) {
+#pragma unroll
+  for (int np = 0; np < NT / 2; ++np) {
+    const uint32_t ad = at(base, row_of(16 * np + (lane & 7) + (lane >> 4) * 8), (lane >> 3) & 1);
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) {
+      uint32_t r[4];
+      ldsm_x4(r, ad ^ (ks << 5));
+      kb[2 * np][ks][0] = r[0]; kb[2 * np][ks][1] = r[1];
+      kb[2 * np + 1][ks][0] = r[2]; kb[2 * np + 1][ks][1] = r[3];
+    }
+  }
+  if (NT & 1) {
+    const uint32_t ad = at(base, row_of(8 * (NT - 1) + (lane & 7)), lane >> 3);
+#pragma unroll
+    for (int k2 = 0; k2 < 2; ++k2) {
+      uint32_t r[4];
+      ldsm_x4(r, ad ^ (k2 << 6));
+      kb[NT - 1][2 * k2][0] = r[0]; kb[NT - 1][2 * k2][1] = r[1];
+      kb[NT - 1][2 * k2 + 1][0] = r[2]; kb[NT - 1][2 * k2 + 1][1] = r[3];
+    }
+  }
+}
+// The 16 x 8 NT weights of a row tile as A fragments of (NT + 1) / 2 16-column steps.
+template <int NT>
+__device__ __forceinline__ void pack_a(uint32_t (&pa)[(NT + 1) / 2][4], const float (&s)[NT][4]) {
+  typedef Mma<__half> M;
+#pragma unroll
+  for (int kk = 0; kk < (NT + 1) / 2; ++kk) {
+    pa[kk][0] = M::pack(s[2 * kk][0], s[2 * kk][1]);
+    pa[kk][1] = M::pack(s[2 * kk][2], s[2 * kk][3]);
+    pa[kk][2] = 2 * kk + 1 < NT ? M::pack(s[(2 * kk + 1) % NT][0], s[(2 * kk + 1) % NT][1]) : 0u;
+    pa[kk][3] = 2 * kk + 1 < NT ? M::pack(s[(2 * kk + 1) % NT][2], s[(2 * kk + 1) % NT][3]) : 0u;
+  }
+}
+
+// Shared memory of a CTA: `bufs` x (Q, K, V), the state tile (more than one round), c_L ([position]
+// [nm * 8 blocks]), a dump for matrix-store rows past a block, barriers.
+inline size_t smem_bytes(int tile, int bufs, bool multi, int b, int nm) {
+  return (size_t)tile * (3 * bufs + (multi ? 1 : 0)) + (size_t)b * nm * 8 * 4 + 128 + sizeof(Bars) + 1024 + 16;
+}
+
+// NB, NM: 8-column tiles that hold b keys / m blocks.
+template <typename TIn, int NB, int NM, bool MULTI>
+__global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __grid_constant__ Params P) {
+  typedef Mma<__half> M;
+  constexpr int RB = (NB + 1) / 2, RM = (NM + 1) / 2;      // 16-row tiles
+  extern __shared__ uint8_t smem_raw[];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  const int tile = P.tile, b = P.b, bp = P.bp;
+  const uint32_t s0 = smem_u32(smem);
+  const uint32_t sS = s0 + 3 * P.bufs * tile;              // state tile (MULTI)
+  float* sCL = reinterpret_cast<float*>(smem + (3 * P.bufs + (MULTI ? 1 : 0)) * tile);
+  uint8_t* tail = reinterpret_cast<uint8_t*>(sCL + b * NM * 8);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const uint32_t dump = smem_u32(tail) + (lane & 7) * 16;
+  Bars* bars = reinterpret_cast<Bars*>(tail + 128);
+  if (tid == 0) {
+    for (int i = 0; i < P.bufs; ++i)
+      for (int k = 0; k < P.m; ++k) mbar_init(&bars->full[i][k], 1);
+    tensor::fence_barrier_init();
+  }
+  __syncthreads();
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+
+  auto valid_of = [&](int h) { return P.seq_len != nullptr ? min(max(P.seq_len[h / P.heads], 1), P.N) : P.n_valid; };
+  const int nw = blockDim.x >> 5;
+  const float fl = P.scale * kLog2e;
+  // per-lane row within 16 and 16-byte chunk: A operands, transposed B operands, matrix stores
+  const int a_row = lane & 15, a_ch = lane >> 4;
+
+  // Requests the blocks of head h that this warp owns in the R half-step (absent ones excepted).
+  auto request = [&](int h, int buf) {
+    if (lane != 0 || h >= P.BH) return;
+    const int h0 = P.H ? h % P.H : h, h1 = P.H ? h / P.H : 0;
+    const int m = P.seq_len != nullptr ? (valid_of(h) + b - 1) / b : P.m;
+    for (int k = warp; k < m; k += nw) {
+      uint64_t* bar = &bars->full[buf][k];
+      const uint32_t dst = s0 + 3 * buf * tile + k * bp * 128;
+      mbar_expect_tx(bar, 3 * bp * 128);
+      load_5d(dst, &P.q, bar, k, h0, h1);
+      load_5d(dst + tile, &P.k, bar, k, h0, h1);
+      load_5d(dst + 2 * tile, &P.v, bar, k, h0, h1);
+    }
+  };
+  request(blockIdx.x, 0);
+  int buf = 0;
+  uint32_t par = 0;                 // bit 16 buf + r: parity of the warp's r-th block in that buffer
+  for (int h = blockIdx.x; h < P.BH; h += gridDim.x) {
+    if (P.bufs == 2) request(h + gridDim.x, buf ^ 1);
+    const uint32_t sQ = s0 + 3 * buf * tile, sK = sQ + tile, sV = sK + tile;
+    const int n_valid = valid_of(h);
+    const int m = P.seq_len != nullptr ? (n_valid + b - 1) / b : P.m;
+    const size_t head_base = P.H == 0 ? (size_t)h * P.N * P.d : ((size_t)(h / P.H) * P.N * P.H + (h % P.H)) * P.d;
+    const size_t row_stride = P.H == 0 ? (size_t)P.d : (size_t)P.H * P.d;
+    for (int step = 1; step <= P.T; ++step) {
+      const bool first = !MULTI || step == 1, last = !MULTI || step == P.T;
+      // ================================================================ R half-step (Eq. 7, 9, 10)
+      for (int k = warp, r = 0; k < m; k += nw, ++r) {
+        if (first) {
+          if (!tensor::mbar_wait(&bars->full[buf][k], (par >> (16 * buf + r)) & 1) && P.status != nullptr)
+            tensor::report_timeout(P.status, 2);
+          par ^= 1u << (16 * buf + r);
+          if (!Mma<TIn>::is_f16) {      // bf16: to f16 in place, the block's three operands
+            for (int e = lane; e < b * 8; e += 32) {
+#pragma unroll
+              for (int a = 0; a < 3; ++a) {
+                uint4* p = reinterpret_cast<uint4*>(smem + (sQ - s0) + a * tile + (k * bp) * 128 + e * 16);
+                *p = warpmma::to_f16x8(*p, (const TIn*)nullptr);
+              }
+            }
+          }
+          __syncwarp();
+        }
+        const uint32_t sA = first ? sQ : sS;                 // alpha_R (= Q rows while L is the identity)
+        const uint32_t dst = MULTI ? sS : sK;                // alpha_L
+        const int r0 = k * bp;
+        const int lim = min(b, n_valid - k * b);             // keys of this block that count
+        uint32_t pa[RB][RB][4];                              // unnormalised weights: the largest is exactly 1
+        float inv[RB][2];
+        {
+          uint32_t kb[NB][4][2];
+          load_b<NB>(kb, sK, lane, [&](int i) { return r0 + min(i, b - 1); });
+#pragma unroll
+          for (int rt = 0; rt < RB; ++rt) {
+            float s[NB][4];
+#pragma unroll
+            for (int nt = 0; nt < NB; ++nt)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) s[nt][e] = 0.f;
+            const uint32_t ad = at(sA, r0 + min(16 * rt + a_row, b - 1), a_ch);
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks) {
+              uint32_t a[4];
+              ldsm_x4(a, ad ^ (ks << 5));
+#pragma unroll
+              for (int nt = 0; nt < NB; ++nt) M::run(s[nt], a, kb[nt][ks]);
+            }
+            // rows j = 16 rt + g (c0, c1) and + 8 (c2, c3); columns i = 8 nt + 2 t, + 1.  Columns past the
+            // block, in the last column tile, and padded keys of the last block: a score of weight 0.
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              if (8 * (NB - 1) + 2 * t + (e & 1) >= lim) s[NB - 1][e] = kMasked;
+            if (lim < b) {
+#pragma unroll
+              for (int nt = 0; nt < NB - 1; ++nt)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                  if (8 * nt + 2 * t + (e & 1) >= lim) s[nt][e] = kMasked;
+            }
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) {
+              float mx = kMasked;
+#pragma unroll
+              for (int nt = 0; nt < NB; ++nt) mx = fmaxf(mx, fmaxf(s[nt][2 * hh], s[nt][2 * hh + 1]));
+              mx = quad_max(mx);
+              const float off = -mx * fl;
+              float sum = 0.f, sz = 0.f;
+#pragma unroll
+              for (int nt = 0; nt < NB; ++nt)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                  const float x = s[nt][2 * hh + e];
+                  const float p = ex2(fmaf(x, fl, off));
+                  s[nt][2 * hh + e] = p;
+                  sum += p;
+                  sz = fmaf(p, x, sz);               // 0 times a finite number where masked (0 log 0 = 0)
+                }
+              sum = quad_sum(sum);
+              sz = quad_sum(sz);
+              inv[rt][hh] = 1.f / sum;
+              // -c_L log2 e = log2 sum + max - sum R z (Eq. 10), the addend of the L logits
+              const int j = 16 * rt + g + 8 * hh;
+              if (t == 0 && j < b) sCL[j * NM * 8 + k] = lg2(sum) - off - fl * (sz * inv[rt][hh]);
+            }
+            pack_a<NB>(pa[rt], s);
+          }
+        }
+        __syncwarp();
+        // second products, 16 columns at a time; a warp alone reads and writes the rows of its block
+        uint32_t kt[RB], st[RB];
+#pragma unroll
+        for (int kk = 0; kk < RB; ++kk) {
+          kt[kk] = at(0, r0 + min(16 * kk + a_row, b - 1), a_ch);
+          st[kk] = at(0, r0 + 16 * kk + a_row, a_ch);
+        }
+#pragma unroll
+        for (int np = 0; np < 4; ++np) {
+          uint32_t bk[RB][4], bv[RB][4];
+#pragma unroll
+          for (int kk = 0; kk < RB; ++kk) {
+            ldsm_x4_trans(bk[kk], sK + (kt[kk] ^ (np << 5)));
+            if (last) ldsm_x4_trans(bv[kk], sV + (kt[kk] ^ (np << 5)));
+          }
+          __syncwarp();
+#pragma unroll
+          for (int rt = 0; rt < RB; ++rt) {
+            const bool on = 16 * rt + a_row < b;
+            float o[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+            for (int kk = 0; kk < RB; ++kk) {
+              M::run(o[0], pa[rt][kk], bk[kk]);
+              M::run(o[1], pa[rt][kk], bk[kk] + 2);
+            }
+            put(on ? dst + (st[rt] ^ (np << 5)) : dump, o, inv[rt][0], inv[rt][1]);
+            if (last) {
+              float y[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+              for (int kk = 0; kk < RB; ++kk) {
+                M::run(y[0], pa[rt][kk], bv[kk]);
+                M::run(y[1], pa[rt][kk], bv[kk] + 2);
+              }
+              put(on ? sV + (st[rt] ^ (np << 5)) : dump, y, inv[rt][0], inv[rt][1]);
+            }
+          }
+        }
+      }
+      __syncthreads();
+
+      // ================================================================ L half-step (Eq. 8, 9 / Eq. 4)
+      for (int j = warp; j < b; j += nw) {
+        const uint32_t sA = MULTI ? sS : sK;                 // alpha_L
+        float c[NM][2];
+#pragma unroll
+        for (int nt = 0; nt < NM; ++nt) {
+          const float2 v = *reinterpret_cast<const float2*>(sCL + j * NM * 8 + 8 * nt + 2 * t);
+          c[nt][0] = 8 * nt + 2 * t < m ? v.x : kMasked;
+          c[nt][1] = 8 * nt + 2 * t + 1 < m ? v.y : kMasked;
+        }
+        uint32_t pa[RM][RM][4];                              // weights, rows l (final, unnormalised)
+        float inv[RM][2];
+        float w[MULTI ? RM : 1][MULTI ? NM : 1][4];          // normalised weights (non-final)
+        {
+          uint32_t kb[NM][4][2];
+          load_b<NM>(kb, sA, lane, [&](int k) { return min(k, m - 1) * bp + j; });
+#pragma unroll
+          for (int rt = 0; rt < RM; ++rt) {
+            float s[NM][4];
+#pragma unroll
+            for (int nt = 0; nt < NM; ++nt)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) s[nt][e] = 0.f;
+            const uint32_t ad = at(sQ, min(16 * rt + a_row, m - 1) * bp + j, a_ch);
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks) {
+              uint32_t a[4];
+              ldsm_x4(a, ad ^ (ks << 5));
+#pragma unroll
+              for (int nt = 0; nt < NM; ++nt) M::run(s[nt], a, kb[nt][ks]);
+            }
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) {
+              float mx = kMasked;
+#pragma unroll
+              for (int nt = 0; nt < NM; ++nt)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                  const float z = fmaf(s[nt][2 * hh + e], fl, c[nt][e]);
+                  s[nt][2 * hh + e] = z;
+                  mx = fmaxf(mx, z);
+                }
+              mx = quad_max(mx);
+              float sum = 0.f;
+#pragma unroll
+              for (int nt = 0; nt < NM; ++nt)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                  const float p = ex2(s[nt][2 * hh + e] - mx);
+                  s[nt][2 * hh + e] = p;
+                  sum += p;
+                }
+              sum = quad_sum(sum);
+              inv[rt][hh] = 1.f / sum;
+              const int l = 16 * rt + g + 8 * hh;
+              // log-sum-exp of row b l + j of the final L half-step: summed over a head's rows it is the
+              // objective (Eq. 6) at the returned matrix
+              if (last && P.lse != nullptr && t == 0 && l < m) P.lse[(size_t)h * P.N + (size_t)l * b + j] = (mx + lg2(sum)) * kLn2;
+              if (MULTI && !last) {
+                const float on = l < m ? inv[rt][hh] : 0.f;      // (rows past the last block: not in sums over rows)
+#pragma unroll
+                for (int nt = 0; nt < NM; ++nt) {
+                  s[nt][2 * hh] *= on;
+                  s[nt][2 * hh + 1] *= on;
+                }
+              }
+            }
+            if (last) {
+              pack_a<NM>(pa[rt], s);
+            } else if (MULTI) {
+#pragma unroll
+              for (int nt = 0; nt < NM; ++nt)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) w[MULTI ? rt : 0][MULTI ? nt : 0][e] = s[nt][e];
+            }
+          }
+        }
+        __syncwarp();
+        uint32_t kt[RM], st[RM];
+#pragma unroll
+        for (int kk = 0; kk < RM; ++kk) {
+          kt[kk] = at(0, min(16 * kk + a_row, m - 1) * bp + j, a_ch);
+          st[kk] = at(0, (16 * kk + a_row) * bp + j, a_ch);
+        }
+        if (last) {
+          // Y(l,j) = sum_k L[j,k,l] y(k,j), over the rows of Q the scores were formed from
+#pragma unroll
+          for (int np = 0; np < 4; ++np) {
+            uint32_t by[RM][4];
+#pragma unroll
+            for (int kk = 0; kk < RM; ++kk) ldsm_x4_trans(by[kk], sV + (kt[kk] ^ (np << 5)));
+#pragma unroll
+            for (int rt = 0; rt < RM; ++rt) {
+              float o[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+              for (int kk = 0; kk < RM; ++kk) {
+                M::run(o[0], pa[rt][kk], by[kk]);
+                M::run(o[1], pa[rt][kk], by[kk] + 2);
+              }
+              put(16 * rt + a_row < m ? sQ + (st[rt] ^ (np << 5)) : dump, o, inv[rt][0], inv[rt][1]);
+            }
+          }
+          __syncwarp();
+          const int ch = lane & 7;
+          if (ch * 8 < P.d)
+            for (int l = lane >> 3; l < P.m; l += 4) {
+              // (rows of blocks that are absent from a shorter sequence: zeros)
+              const uint4 v = l < m ? *reinterpret_cast<const uint4*>(smem + (at(sQ, l * bp + j, ch) - s0)) : make_uint4(0u, 0u, 0u, 0u);
+              TIn* gp = (TIn*)P.Y + head_base + (size_t)(l * b + j) * row_stride + ch * 8;
+              *reinterpret_cast<uint4*>(gp) = warpmma::from_f16x8(v, gp);
+            }
+        } else if constexpr (MULTI) {
+          // alpha_R(k,j) = sum_l L[j,k,l] Q(l,j) / c_R, c_R(k,j) = sum_l L[j,k,l]: the contraction runs over
+          // the rows of the weights, so the A fragments are their transpose.  Column k is multiplied by
+          // g_k = 2^-(exponent of its largest weight) first (the quotient is invariant), which keeps its
+          // significant weights in the normal f16 range however small c_R is; c_R comes out of the same
+          // MMAs against a B fragment of ones, i.e. over the weights as rounded.
+          uint32_t tp[RM][2][NM];
+#pragma unroll
+          for (int nt = 0; nt < NM; ++nt) {
+            float gk[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              float cm = 0.f;
+#pragma unroll
+              for (int rt = 0; rt < RM; ++rt) cm = fmaxf(cm, fmaxf(w[rt][nt][e], w[rt][nt][2 + e]));
+              cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, 4));
+              cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, 8));
+              cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, 16));
+              gk[e] = __uint_as_float((253u << 23) - (__float_as_uint(cm) & 0x7f800000u));
+            }
+#pragma unroll
+            for (int rt = 0; rt < RM; ++rt)
+#pragma unroll
+              for (int hh = 0; hh < 2; ++hh)
+                tp[rt][hh][nt] = movm_trans(M::pack(w[rt][nt][2 * hh] * gk[0], w[rt][nt][2 * hh + 1] * gk[1]));
+          }
+          const uint32_t ones[2] = {0x3C003C00u, 0x3C003C00u};
+#pragma unroll
+          for (int kq = 0; kq < RM; ++kq) {
+            uint32_t pk[RM][4];      // A[k][l]: rows k = 16 kq .., contraction over l = 16 ls ..
+            float cr[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int ls = 0; ls < RM; ++ls) {
+              pk[ls][0] = tp[ls][0][2 * kq];
+              pk[ls][1] = 2 * kq + 1 < NM ? tp[ls][0][(2 * kq + 1) % NM] : 0u;
+              pk[ls][2] = tp[ls][1][2 * kq];
+              pk[ls][3] = 2 * kq + 1 < NM ? tp[ls][1][(2 * kq + 1) % NM] : 0u;
+              M::run(cr, pk[ls], ones);
+            }
+            const float i0 = cr[0] > 1e-30f ? 1.f / cr[0] : 0.f, i1 = cr[2] > 1e-30f ? 1.f / cr[2] : 0.f;
+#pragma unroll
+            for (int np = 0; np < 4; ++np) {
+              float o[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+              for (int ls = 0; ls < RM; ++ls) {
+                uint32_t bq[4];      // B[l][v] = Q(l,j)[v], read transposed
+                ldsm_x4_trans(bq, sQ + (kt[ls] ^ (np << 5)));
+                M::run(o[0], pk[ls], bq);
+                M::run(o[1], pk[ls], bq + 2);
+              }
+              put(16 * kq + a_row < m ? sS + (st[kq] ^ (np << 5)) : dump, o, i0, i1);
+            }
+          }
+        }
+      }
+      if (!last) __syncthreads();
+    }
+    // The head's buffer is free (and c_L, and the state tile) when every warp is done with it.
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+    if (P.bufs == 2) buf ^= 1;
+    else request(h + gridDim.x, 0);
+  }
+}
+
+inline bool shape_ok(int d, int b, int m, int dtype) {
+  return (dtype == 1 || dtype == 2) && d % 8 == 0 && d <= 64 && b > 8 && b <= 32 && m > 8 && m <= 32;
+}
+struct Plan {
+  int bp, tile, bufs, warps, ctas;      // ctas: per SM
+  size_t smem;
+};
+inline bool plan(int b, int m, int T, int BH, int num_sms, Plan* p) {
+  const int nm = (m + 7) / 8;
+  const bool multi = T > 1;
+  // The odd pitch where it fits; without it the L half-step's rows conflict (8-way for b = 16, 24, 32,
+  // which the general kernel then serves faster: N = 576 as 24 x 24, 768 heads, 120 against 125 us).
+  for (int odd = 1; odd >= (b % 8 != 0 ? 0 : 1); --odd) {
+    p->bp = odd ? (b | 1) : b;
+    p->tile = (m * p->bp * 128 + 1023) / 1024 * 1024;
+    const size_t one = smem_bytes(p->tile, 1, multi, b, nm), two = smem_bytes(p->tile, 2, multi, b, nm);
+    if (one > (size_t)kMaxSmem) continue;
+    const int fit = (int)((size_t)(227 * 1024) / (one + 1024));      // CTAs per SM by shared memory
+    // At most one head per SM: one CTA with as many warps as a half-step has tiles.  More: the 16 warps
+    // an SM holds (128 registers) go to as many CTAs as fit, up to three, each with a head of its own
+    // (768 heads of 130 = 13 x 10, two rounds: 34.6 us with three, 39.8 with two); except that where no
+    // third fits and there are heads left for a second turn, one CTA of all 16 with the next head's
+    // loads under way is faster (768 heads of 256 = 16 x 16: 25.6 against 27.4 us).
+    p->ctas = BH <= num_sms ? 1 : (fit < 3 ? fit : 3);
+    p->bufs = 1;
+    if (p->ctas <= 2 && BH > p->ctas * num_sms && two <= (size_t)kMaxSmem) {
+      p->ctas = 1;
+      p->bufs = 2;
+    }
+    const int most = 16 / p->ctas;
+    // the fewest warps that take the fewest rounds of tiles over both half-steps
+    int best = 1 << 30;
+    for (int w = 1; w <= most; ++w) {
+      const int rounds = (m + w - 1) / w + (b + w - 1) / w;
+      if (rounds < best) {
+        best = rounds;
+        p->warps = w;
+      }
+    }
+    p->smem = p->bufs == 2 ? two : one;
+    return true;
+  }
+  return false;
+}
+inline bool supported(int N, int d, int b, int m, int dtype, int T) {
+  (void)N;
+  Plan p;
+  return shape_ok(d, b, m, dtype) && plan(b, m, T, 1, 1, &p);
+}
+struct Args {
+  const void *Q, *K, *V;
+  void* Y;
+  int BH, N, d, b, m, T, dtype, H, heads, n_valid;
+  float scale;
+  float* lse;
+  const int* seq_len;
+  int* status;
+};
+int launch(const Args& a, cudaStream_t st);
+
+#ifdef MA_TU_FUSED_HEAD
+inline bool make_map(CUtensorMap* tm, const Args& a, const void* base, int bp) {
+  tensor::EncodeTiledFn fn = tensor::encode_fn();
+  if (!fn) return false;
+  const cuuint64_t d2 = (cuuint64_t)a.d * 2, H = a.H ? a.H : 1, row = d2 * H, N = a.N, BH = a.BH;
+  cuuint64_t dims[5] = {(cuuint64_t)a.d, (cuuint64_t)a.b, (cuuint64_t)a.m, a.H ? (cuuint64_t)a.H : BH, a.H ? BH / a.H : 1};
+  cuuint64_t strides[4] = {row, a.b * row, a.H ? d2 : N * d2, N * d2 * (a.H ? H : BH)};
+  cuuint32_t box[5] = {64, (cuuint32_t)bp, 1, 1, 1}, es[5] = {1, 1, 1, 1, 1};
+  return fn(tm, a.dtype == 1 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims,
+            strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+struct MapKey {
+  const void *Q, *K, *V;
+  int BH, N, d, b, dtype, H, bp, dev;
+  bool operator==(const MapKey& o) const {
+    return Q == o.Q && K == o.K && V == o.V && BH == o.BH && N == o.N && d == o.d && b == o.b && dtype == o.dtype && H == o.H &&
+           bp == o.bp && dev == o.dev;
+  }
+};
+// The maps of the last few problems are kept (encoding three costs more host time than the launch).
+struct MapCache {
+  static constexpr int kEntries = 16;
+  MapKey key[kEntries];
+  CUtensorMap maps[kEntries][3];
+  bool used[kEntries] = {};
+  int next = 0;
+};
+inline bool get_maps(Params* P, const Args& a, const Plan& p, int dev) {
+  static thread_local MapCache c;
+  const MapKey key{a.Q, a.K, a.V, a.BH, a.N, a.d, a.b, a.dtype, a.H, p.bp, dev};
+  int e = 0;
+  while (e < MapCache::kEntries && !(c.used[e] && c.key[e] == key)) ++e;
+  if (e == MapCache::kEntries) {
+    e = c.next;
+    c.next = (c.next + 1) % MapCache::kEntries;
+    c.used[e] = false;
+    if (!make_map(&c.maps[e][0], a, a.Q, p.bp) || !make_map(&c.maps[e][1], a, a.K, p.bp) || !make_map(&c.maps[e][2], a, a.V, p.bp))
+      return false;
+    c.key[e] = key;
+    c.used[e] = true;
+  }
+  P->q = c.maps[e][0];
+  P->k = c.maps[e][1];
+  P->v = c.maps[e][2];
+  return true;
+}
+template <typename TIn, int NB, int NM, bool MULTI>
+inline int launch_k(const Params& P, const Plan& p, int num_sms, cudaStream_t st) {
+  auto kern = monarch_fused_head<TIn, NB, NM, MULTI>;
+  static warpmma::SmemOptIn opt_in;
+  if (!opt_in.done((const void*)kern, kMaxSmem)) return 7;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  const int slots = p.ctas * num_sms;
+  cfg.gridDim = dim3(P.BH < slots ? P.BH : slots);
+  cfg.blockDim = dim3(32 * p.warps);
+  cfg.dynamicSmemBytes = p.smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, P) == cudaSuccess ? 0 : 7;
+}
+template <typename TIn, bool MULTI>
+inline int launch_n(const Params& P, const Plan& p, int num_sms, cudaStream_t st) {
+  const int nb = (P.b + 7) / 8, nm = (P.m + 7) / 8;
+#define MA_FH(B)                                            \
+  (nm == 2 ? launch_k<TIn, B, 2, MULTI>(P, p, num_sms, st)  \
+           : (nm == 3 ? launch_k<TIn, B, 3, MULTI>(P, p, num_sms, st) : launch_k<TIn, B, 4, MULTI>(P, p, num_sms, st)))
+  return nb == 2 ? MA_FH(2) : (nb == 3 ? MA_FH(3) : MA_FH(4));
+#undef MA_FH
+}
+int launch(const Args& a, cudaStream_t st) {
+  static int sms[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 7;
+  if (sms[dev] == 0 && cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 7;
+  Plan p;
+  Params P;
+  if (!plan(a.b, a.m, a.T, a.BH, sms[dev], &p)) return 4;
+  if (!get_maps(&P, a, p, dev)) return 7;
+  P.Y = a.Y; P.lse = a.lse; P.seq_len = a.seq_len; P.status = a.status;
+  P.BH = a.BH; P.N = a.N; P.d = a.d; P.b = a.b; P.m = a.m; P.T = a.T; P.H = a.H; P.heads = a.heads; P.n_valid = a.n_valid;
+  P.bp = p.bp; P.tile = p.tile; P.bufs = p.bufs;
+  P.scale = a.scale;
+  if (a.dtype == 1) return a.T > 1 ? launch_n<__half, true>(P, p, sms[dev], st) : launch_n<__half, false>(P, p, sms[dev], st);
+  return a.T > 1 ? launch_n<__nv_bfloat16, true>(P, p, sms[dev], st) : launch_n<__nv_bfloat16, false>(P, p, sms[dev], st);
+}
+#endif  // MA_TU_FUSED_HEAD
+
+}  // namespace fhead
+}  // namespace ma

@@ -1016,3 +1016,38 @@ def test_tensor_core_tiles_agree_with_the_generic_kernels(BH, N, b, d, T, dtype,
         r = slice(0, lens[e]) if lens else rows
         err = ((Y[e, :, r].float() - ref[e, :, r]).flatten(1).norm(dim=1) / ref[e, :, r].flatten(1).norm(dim=1)).max()
         assert float(err) <= (2e-3 if dtype == "f16" else 5e-3), (e, float(err))
+
+
+# ------------------------------------------------------------------ per-head kernel fed by TMA
+@pytest.mark.parametrize("b,m,T,dtype,BH", [
+    (9, 9, 2, "f16", 2), (16, 16, 1, "bf16", 400), (17, 16, 2, "f16", 310), (16, 17, 1, "f16", 150),   # two, one, three
+    (10, 13, 2, "bf16", 600), (24, 18, 1, "f16", 300), (25, 15, 2, "f16", 6), (32, 13, 2, "bf16", 160),  # heads per SM
+    (12, 32, 1, "f16", 449), (32, 17, 1, "f16", 5), (18, 24, 2, "f16", 7), (30, 18, 1, "bf16", 300),
+])
+@pytest.mark.parametrize("mode", ["bshd", "padded", "varlen"])
+def test_per_head_kernel_agrees_with_the_generic_kernels(b, m, T, dtype, BH, mode):
+    """9 .. 32 blocks and rows at the edges of their 8-column and 16-row tiles, in every split of an SM
+    between heads, every head against the fp32 kernels on the same values."""
+    N, d = b * m, 64 if mode != "varlen" else 56
+    batch, heads = (BH, 1) if mode == "varlen" else (1, BH)
+    Q, K, V = (torch.from_numpy(x).cuda() for x in wl.make_qkv(batch, heads, N, d, dtype, 8, 1.0, seed=N + T))
+    x16 = [x.to(binding.torch_dtype(dtype)) for x in (Q, K, V)]
+    valid = torch.full((batch,), N)
+    if mode == "padded":
+        valid[:] = N - b + 1
+        Y, ref = (binding.monarch_attn_fwd_padded(*x, b, T, N - b + 1) for x in (x16, (Q, K, V)))
+    elif mode == "varlen":
+        valid = torch.linspace(1, N, batch).to(torch.int32)
+        Y, ref = (binding.monarch_attn_fwd_varlen(*x, b, T, valid.cuda()) for x in (x16, (Q, K, V)))
+    else:
+        Y, lse = binding.monarch_attn_fwd_objective(*x16, b, T, path=binding.MA_PATH_FUSED_SMALL)
+        ref, lse_ref = binding.monarch_attn_fwd_objective(Q, K, V, b, T, path=binding.MA_PATH_GENERIC)
+        assert float((lse - lse_ref).abs().max()) <= (5e-2 if dtype == "f16" else 1e-1)
+        Ys = binding.monarch_attn_fwd_bshd(*(x.transpose(1, 2).contiguous() for x in x16), b, T, path=binding.MA_PATH_FUSED_SMALL)
+        assert torch.equal(Ys.transpose(1, 2), Y)
+    assert binding.monarch_attn_last_launch_count() >= 1
+    for e in range(batch):
+        r = slice(0, int(valid[e]))
+        err = ((Y[e, :, r].float() - ref[e, :, r]).flatten(1).norm(dim=1) / ref[e, :, r].flatten(1).norm(dim=1)).max()
+        assert float(err) <= (3e-3 if dtype == "f16" else 6e-3), (e, float(err))
+        assert not bool(Y[e, :, -(-int(valid[e]) // b) * b:].any())
