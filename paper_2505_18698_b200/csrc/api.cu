@@ -48,6 +48,7 @@ static int validate_shape(int batch, int heads, int N, int d, int b, int T, int 
 // ------------------------------------------------------------------ generic path
 constexpr size_t kStatusBytes = 256;
 constexpr size_t kMaxSmem = 227 * 1024;
+constexpr int kSmsB200 = 148;     // (path choice needs no device: the workspace query runs without one)
 
 static bool generic_supported(const Problem& p) {
   if (p.BH > 65535) return false;   // gridDim.y
@@ -184,7 +185,7 @@ static int resolve_path(const Problem& p, int path, bool plain = true) {
     if (p.b <= 32 && fsmall::supported(p.N, p.d, p.b, p.m, p.dtype, p.T)) return MA_PATH_FUSED_SMALL;
     if (tile::supported(p.N, p.d, p.b, p.m, p.dtype, p.BH)) return MA_PATH_TILE_MMA;
     // fp32 inputs: short sequences in one launch with the states in shared memory
-    if (p.dtype == MA_F32 && p.BH <= 65535 && ffused::supported(p.N, p.d, p.b, p.m)) return MA_PATH_FUSED_F32;
+    if (p.dtype == MA_F32 && p.BH <= 65535 && ffused::chosen(p.N, p.d, p.b, p.m, p.BH, kSmsB200)) return MA_PATH_FUSED_F32;
     if (generic_supported(p)) return MA_PATH_GENERIC;
     return -1;
   }
@@ -391,7 +392,7 @@ static int resolve_call(const Call& c, const Problem& p) {
   if (c.entry == Entry::kPadded && resolve_path(p, MA_PATH_AUTO, false) == MA_PATH_TENSOR && p.b != 32)
     return MA_PATH_TENSOR;
   if (tile::supported(p.N, p.d, p.b, p.m, p.dtype, p.BH)) return MA_PATH_TILE_MMA;
-  if (c.entry == Entry::kPadded && p.dtype == MA_F32 && p.BH <= 65535 && ffused::supported(p.N, p.d, p.b, p.m))
+  if (c.entry == Entry::kPadded && p.dtype == MA_F32 && p.BH <= 65535 && ffused::chosen(p.N, p.d, p.b, p.m, p.BH, kSmsB200))
     return MA_PATH_FUSED_F32;
   return generic_supported(p) ? MA_PATH_GENERIC : -1;
 }

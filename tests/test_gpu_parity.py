@@ -1051,3 +1051,28 @@ def test_per_head_kernel_agrees_with_the_generic_kernels(b, m, T, dtype, BH, mod
         err = ((Y[e, :, r].float() - ref[e, :, r]).flatten(1).norm(dim=1) / ref[e, :, r].flatten(1).norm(dim=1)).max()
         assert float(err) <= (3e-3 if dtype == "f16" else 6e-3), (e, float(err))
         assert not bool(Y[e, :, -(-int(valid[e]) // b) * b:].any())
+
+
+# ------------------------------------------------------------------ register tiles of the fused fp32 kernel
+@pytest.mark.parametrize("N,b,d,T,batch,heads", [
+    (272, 17, 64, 2, 1, 1), (136, 8, 64, 3, 2, 1), (255, 15, 62, 2, 1, 12),    # one position, two, four per tile
+    (384, 24, 64, 3, 8, 12), (425, 25, 36, 2, 12, 12), (512, 32, 40, 1, 1, 40),   # three and four key tiles, m = 17
+    (264, 8, 64, 2, 8, 12), (198, 33, 63, 2, 1, 7), (9, 3, 3, 4, 200, 1),         # 33 blocks / 33 keys: any sizes
+    (600, 24, 64, 2, 1, 2),                                                       # a position or two beside K
+])
+def test_fused_f32_kernel_at_the_edges_of_its_tiles(N, b, d, T, batch, heads):
+    """Positions left over from a tile, keys and blocks left over from a group's columns, head sizes that are
+    no multiple of four, with the mask, against the fp64 oracle; and the same through the other layout."""
+    Q, K, V = wl.make_qkv(batch, heads, N, d, "f32", 3, 0.5, seed=N + T)
+    x = [binding.to_device(t, "f32") for t in (Q, K, V)]
+    Y = binding.monarch_attn_fwd_padded(*x, b, T, N - b // 2)
+    assert binding.monarch_attn_last_launch_count() == 1
+    few = slice(0, 2)
+    ref = mo.monarch_attention(Q[few, few], K[few, few], V[few, few], b, T, n_valid=N - b // 2)
+    rows = slice(0, N - b // 2)
+    assert rel_err(Y[few, few, rows].double().cpu().numpy(), ref[:, :, rows]) <= 1e-5
+    a = binding.monarch_attn_fwd_ex(*x, b, T, path=binding.MA_PATH_FUSED_F32)
+    c = binding.monarch_attn_fwd_bshd(*(t.transpose(1, 2).contiguous() for t in x), b, T, path=binding.MA_PATH_FUSED_F32)
+    assert torch.equal(c.transpose(1, 2), a)
+    g = binding.monarch_attn_fwd_ex(*x, b, T, path=binding.MA_PATH_GENERIC)
+    assert float((a - g).norm() / g.norm()) <= 1e-5
