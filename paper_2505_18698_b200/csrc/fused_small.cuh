@@ -47,8 +47,8 @@ using warpmma::quad_max;
 using warpmma::quad_sum;
 
 constexpr int kThreads = 256, kWarps = 8, kRowBytes = 128, kMaxSmem = 227 * 1024;
-// where stmatrix rows past the end of a block go: 16 bytes per thread
-inline size_t dump_bytes(int threads) { return (size_t)threads * 16; }
+// where stmatrix rows past the end of a block go: eight rows of 16 bytes (nothing reads them)
+constexpr size_t kDumpBytes = 128;
 
 // Four 8x8 16-bit matrices from accumulator-layout registers; lane L gives the address of row L & 7
 // of matrix L >> 3.
@@ -103,9 +103,9 @@ inline size_t tile_bytes(int N, int b, int ks) {
   return ks == 4 ? (size_t)N * kRowBytes : (size_t)m * ((size_t)b * (32 * ks + 16) + 16);
 }
 inline int ksteps_for(int d) { return d <= 64 ? 4 : (d <= 80 ? 5 : 8); }
-inline size_t smem_bytes(int N, int T, int threads = kThreads, int b = 16, int ks = 4, bool hilo = false) {
+inline size_t smem_bytes(int N, int T, int b = 16, int ks = 4, bool hilo = false) {
   // (alignment slack: the XOR-swizzled layout needs a 1024-byte aligned base, the padded one 128)
-  return (size_t)(T == 1 ? 3 : (hilo ? 5 : 4)) * tile_bytes(N, b, ks) + (((size_t)N * 4 + 15) & ~(size_t)15) + dump_bytes(threads) +
+  return (size_t)(T == 1 ? 3 : (hilo ? 5 : 4)) * tile_bytes(N, b, ks) + (((size_t)N * 4 + 15) & ~(size_t)15) + kDumpBytes +
          (ks == 4 ? 1024 : 128);
 }
 
@@ -116,7 +116,7 @@ inline size_t smem_bytes(int N, int T, int threads = kThreads, int b = 16, int k
 // three or more rounds on peaky logits need (plain 16-bit states, fed back round after round, lose
 // 1e-2 on about one head in 300 at T = 3).
 template <typename TIn, int BP, int MP, bool EXACT = false, int KS = 4, bool HILO = false>
-__global__ void __launch_bounds__((KS == 4 && !HILO && BP <= 32 && (BP == 16 || MP == 16)) ? 2 * kThreads : kThreads, 1)
+__global__ void __launch_bounds__((HILO || (KS == 4 && BP <= 32 && (BP == 16 || MP == 16))) ? 2 * kThreads : kThreads, 1)
 monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const TIn* __restrict__ V,
                     TIn* __restrict__ Y, int N, int d, int b, int m, int T_steps, float scale,
                     int n_valid, int H, float* __restrict__ lse, const int* __restrict__ seq_len,
@@ -154,10 +154,10 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
   // the rows (., j)), and V has a tile of its own from the start
   float* sCL = reinterpret_cast<float*>(smem + (T_steps == 1 ? 3 : (HILO ? 5 : 4)) * (size_t)tile);   // [k*b + j]
   const uint32_t sQ_u = (uint32_t)__cvta_generic_to_shared(sQ);
-  // stmatrix writes whole 8-row matrices: rows past a block's end land in a per-lane dump slot
+  // stmatrix writes whole 8-row matrices: rows past a block's end land in a dump slot
   const uint32_t dump_u =
       (uint32_t)__cvta_generic_to_shared(reinterpret_cast<uint8_t*>(sCL) + (((size_t)N * 4 + 15) & ~(size_t)15)) +
-      threadIdx.x * 16;   // 16-byte aligned like every stmatrix row
+      (threadIdx.x & 7) * 16;   // 16-byte aligned like every stmatrix row
   const int st_row = (threadIdx.x & 7) + ((threadIdx.x >> 3) & 1) * 8;   // row within a 16-row tile
   const int st_nt = (threadIdx.x >> 4) & 1;                              // which of a pair of 8-column tiles
   const uint32_t sK_u = sQ_u + tile, sV_u = sK_u + tile;
@@ -632,14 +632,14 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
 
 inline bool supported(int N, int d, int b, int m, int dtype, int T) {
   return (dtype == 1 || dtype == 2) && d % 8 == 0 && d <= 128 && b <= (d <= 64 ? 64 : 32) && m <= 32 &&
-         smem_bytes(N, T, kThreads, b, ksteps_for(d)) <= (size_t)kMaxSmem;
+         smem_bytes(N, T, b, ksteps_for(d)) <= (size_t)kMaxSmem;
 }
 
 // Three or more rounds with hi + lo states: blocks and block counts up to 16, d <= 80, five tiles in
 // shared memory.
 inline bool supported_hilo(int N, int d, int b, int m, int dtype, int T) {
   return (dtype == 1 || dtype == 2) && T >= 3 && d % 8 == 0 && d <= 80 && b <= 16 && m <= 16 &&
-         smem_bytes(N, T, kThreads, b, ksteps_for(d), true) <= (size_t)kMaxSmem;
+         smem_bytes(N, T, b, ksteps_for(d), true) <= (size_t)kMaxSmem;
 }
 
 int launch(const void* Q, const void* K, const void* V, void* Y, int BH, int N, int d, int b,
@@ -652,13 +652,14 @@ inline int launch_t(const void* Q, const void* K, const void* V, void* Y, int BH
                     int m, int T, float scale, int n_valid, int H, float* lse, cudaStream_t st,
                     const int* seq_len, int heads) {
   auto kern = monarch_fused_small<TIn, BP, MP, EXACT, KS, HILO>;
-  // The 16 x 16 kernel is compiled for 128 registers: two CTAs of 8 warps per SM where shared memory
-  // lets two fit, else one CTA of 16 warps (each warp then owns at most one tile per half-step).
-  int threads = kThreads;
-  if (KS == 4 && !HILO && BP <= 32 && (BP == 16 || MP == 16) && 2 * (smem_bytes(N, T) + 1024) > (size_t)228 * 1024 &&
-      (m > 8 || b > 8) && smem_bytes(N, T, 2 * kThreads) <= (size_t)kMaxSmem)
-    threads = 2 * kThreads;
-  const size_t smem = smem_bytes(N, T, threads, b, KS, HILO);
+  // Two CTAs of 8 warps per SM where shared memory lets two fit, else one CTA of 16 warps (each warp then
+  // owns at most one tile of a half-step of 16 blocks), for the instantiations compiled for 128 registers.
+  // The hi + lo states leave room for one CTA, and where two fit a grid of one CTA per SM or fewer gains
+  // from 16 warps as well (128 heads of 256 = 16 x 16, d = 72, three rounds: 17.5 against 22.6 us).
+  const size_t smem = smem_bytes(N, T, b, KS, HILO);
+  const bool wide = HILO || (KS == 4 && BP <= 32 && (BP == 16 || MP == 16));
+  const bool one = 2 * (smem + 1024) > (size_t)228 * 1024 || (HILO && BH <= 148);
+  const int threads = wide && one && (m > 8 || b > 8) ? 2 * kThreads : kThreads;
   static warpmma::SmemOptIn opt_in;
   if (!opt_in.done((const void*)kern, kMaxSmem)) return 7;
   // programmatic stream serialisation: when calls follow one another on a stream, the CTAs of the
