@@ -114,11 +114,12 @@ int monarch_attn_fwd_ex(const void* Q, const void* K, const void* V, void* Y,
 
 /* End-to-end variant: Q, K, V, Y are HOST pointers (pinned memory gives asynchronous copies).
  * Copies Q, K, V to device staging buffers owned by the library, runs monarch_attn_fwd, copies Y
- * back; does not synchronise.  The (batch, head) units are independent (Sec. 3), so the call is
- * cut into four chunks of units (measured best of 1-8 on C2 and C5): a chunk's kernels and the copy of its result run on two
- * streams owned by the library while the next chunk's inputs come in on `stream` (fork and join by
- * events, so work queued on `stream` after the call still sees Y_host complete).  Grows the staging buffers on
- * demand. */
+ * back; does not synchronise.  The (batch, head) units are independent (Sec. 3), so a call of more
+ * than a few megabytes is cut into two or three chunks of units: a chunk's kernels and the copy of its
+ * result run on two streams owned by the library while the next chunk's inputs come in on `stream`
+ * (fork and join by events, so work queued on `stream` after the call still sees Y_host complete).
+ * Where the kernels write each row of Y once (short sequences) and Y_host is pinned, they write it
+ * directly instead of a copy back.  Grows the staging buffers on demand. */
 int monarch_attn_fwd_host(const void* Q_host, const void* K_host, const void* V_host, void* Y_host,
                           int batch, int heads, int N, int d, int b, int T,
                           int dtype, void* stream);

@@ -26,7 +26,8 @@ int monarch_attn_set_trace_buffer(void* device_buffer, size_t bytes);
  *           dependency waits of the second half-step can never be satisfied.  Together they let a
  *           test watch a wait run out: the kernel ends by itself, results are garbage, and
  *           monarch_attn_device_status reports MA_ERR_TIMEOUT.  Nothing faults or hangs.
- *   knob 3: number of chunks monarch_attn_fwd_host cuts a call into (1..8, default 4). */
+ *   knob 3: number of chunks monarch_attn_fwd_host cuts a call into (1..8; 0, the default: by
+ *           the size of the tensors). */
 int monarch_attn_debug_knob(int knob, long long value);
 
 #ifdef __cplusplus

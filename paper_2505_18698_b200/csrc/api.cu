@@ -250,7 +250,7 @@ struct DeviceBuffers {
   cudaEvent_t all_back = nullptr;
 };
 constexpr int kHostChunks = 8;
-static int g_host_chunks = 4;   // chunks a host call is cut into (<= kHostChunks)
+static int g_host_chunks = 0;   // chunks a host call is cut into (<= kHostChunks); 0: by size
 static DeviceBuffers g_dev[kMaxDevices];
 
 static int grow(void** ptr, size_t* have, size_t need) {
@@ -536,7 +536,28 @@ int monarch_attn_fwd_host(const void* Qh, const void* Kh, const void* Vh, void* 
   // into chunks of units: copy in on `stream`, compute on the library's compute stream, copy back
   // on its copy-back stream, chained by events.
   const size_t unit = (size_t)p.N * p.d * esize(p.dtype);
-  const int chunks = (unit % 16 == 0 && p.BH >= g_host_chunks) ? g_host_chunks : 1;
+  // The per-head kernels write each row of Y once, in whole lines: to pinned memory they write it
+  // directly, and the copy back is gone.
+  char* direct = nullptr;
+  const int r = resolve_path(p, MA_PATH_AUTO);
+  if (r == MA_PATH_FUSED_SMALL || r == MA_PATH_FUSED_F32) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, Yh) == cudaSuccess && at.type == cudaMemoryTypeHost && at.devicePointer &&
+        ((uintptr_t)at.devicePointer & 15) == 0)
+      direct = (char*)at.devicePointer;
+    else
+      cudaGetLastError();
+  }
+  // Every copy costs 3-4 us beyond its bytes, and copies in slow down while others go back; the copies
+  // and kernels of a chunk overlap the copies of the next.  Measured with 1, 2, 3, 4 and 6 chunks (us): 0.2 MB
+  // a tensor 46, 52, 62, 75, 98; 2.4 MB 220, 227, 235, 249, 268; 9.4 MB 717, 661, 661, 664, 692; 20 MB 1521, 1388,
+  // 1345, 1346, 1354; 25 MB 1866, 1684, 1633, 1645, 1662.  The long sequences' kernels and the copy back
+  // they need weigh more: four.
+  const size_t bytes = (size_t)p.BH * unit;
+  const int want = g_host_chunks > 0 ? g_host_chunks : (!direct ? 4 : (bytes < ((size_t)4 << 20) ? 1 : (bytes < ((size_t)14 << 20) ? 2 : 3)));
+  const int chunks = (unit % 16 == 0 && p.BH >= want) ? want : 1;
+  // one chunk: everything in order on the caller's stream
+  cudaStream_t compute = chunks > 1 ? B.compute : st, back = chunks > 1 ? B.d2h : st;
   int launches = 0;
   for (int c = 0; c < chunks; ++c) {
     const int u0 = (int)((long long)p.BH * c / chunks), u1 = (int)((long long)p.BH * (c + 1) / chunks);
@@ -545,20 +566,23 @@ int monarch_attn_fwd_host(const void* Qh, const void* Kh, const void* Vh, void* 
         cudaMemcpyAsync(s + one + off, (const char*)Kh + off, len, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(s + 2 * one + off, (const char*)Vh + off, len, cudaMemcpyHostToDevice, st) != cudaSuccess)
       return MA_ERR_CUDA;
-    if (cudaEventRecord(B.chunk_in[c], st) != cudaSuccess ||
-        cudaStreamWaitEvent(B.compute, B.chunk_in[c], 0) != cudaSuccess)
+    if (chunks > 1 && (cudaEventRecord(B.chunk_in[c], st) != cudaSuccess ||
+                       cudaStreamWaitEvent(compute, B.chunk_in[c], 0) != cudaSuccess))
       return MA_ERR_CUDA;
-    rc = monarch_attn_fwd(s + off, s + one + off, s + 2 * one + off, s + 3 * one + off, 1, u1 - u0, N, d, b,
-                          T, dtype, (void*)B.compute);
+    rc = monarch_attn_fwd(s + off, s + one + off, s + 2 * one + off, direct ? direct + off : s + 3 * one + off, 1, u1 - u0, N,
+                          d, b, T, dtype, (void*)compute);
     if (rc != MA_OK) return rc;
     launches += g_last_launches;
-    if (cudaEventRecord(B.chunk_done[c], B.compute) != cudaSuccess ||
-        cudaStreamWaitEvent(B.d2h, B.chunk_done[c], 0) != cudaSuccess ||
-        cudaMemcpyAsync((char*)Yh + off, s + 3 * one + off, len, cudaMemcpyDeviceToHost, B.d2h) != cudaSuccess)
+    if (direct) continue;
+    if (chunks > 1 && (cudaEventRecord(B.chunk_done[c], compute) != cudaSuccess ||
+                       cudaStreamWaitEvent(back, B.chunk_done[c], 0) != cudaSuccess))
+      return MA_ERR_CUDA;
+    if (cudaMemcpyAsync((char*)Yh + off, s + 3 * one + off, len, cudaMemcpyDeviceToHost, back) != cudaSuccess)
       return MA_ERR_CUDA;
   }
   // the caller's stream is done when the last result is back
-  if (cudaEventRecord(B.all_back, B.d2h) != cudaSuccess || cudaStreamWaitEvent(st, B.all_back, 0) != cudaSuccess)
+  if (chunks > 1 && (cudaEventRecord(B.all_back, direct ? compute : back) != cudaSuccess ||
+                     cudaStreamWaitEvent(st, B.all_back, 0) != cudaSuccess))
     return MA_ERR_CUDA;
   g_last_launches = launches;
   return MA_OK;
@@ -627,7 +651,7 @@ int monarch_attn_debug_knob(int knob, long long value) {
   } else if (knob == 2) {
     tp::knobs().skip_first_half_step = value != 0;
   } else if (knob == 3) {
-    g_host_chunks = value < 1 ? 1 : (value > kHostChunks ? kHostChunks : (int)value);
+    g_host_chunks = value < 1 ? 0 : (value > kHostChunks ? kHostChunks : (int)value);
   } else {
     return MA_ERR_SHAPE;
   }
