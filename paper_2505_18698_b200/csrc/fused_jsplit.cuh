@@ -1,29 +1,38 @@
 // Fused kernel for N = 1024 as 32 blocks of 32 (d = 64, f16/bf16): all T rounds of Eq. 7-10 and the
-// Monarch multiply of Eq. 4 in ONE launch, the states alpha_L, alpha_R, y, c_L (Sec. 3
-// 'Implementation') never leaving shared memory.
+// Monarch multiply of Eq. 4 in ONE launch, the states alpha_L, alpha_R, y, c_L (Sec. 3 'Implementation')
+// never leaving shared memory.
 //
 // A head of this size does not fit one SM (Q, K, V and a state are 128 KB each), so it is split by
 // in-block position: within a head the whole recursion is independent across the position j (row
 // (l, j) of the Monarch matrix is L[j,:,l] (x) R[:,j,:]; R[k,j,:], c_L[j,k], alpha_L[j,k,:],
 // L[j,:,:], alpha_R[k,j,:], c_R[k,j], y[j,k,:] only ever read quantities with the same j, plus all
-// of K and V and the 32 rows (l, j) of Q).  A CTA owns 8 positions of one head: K stays resident
-// (128 KB, read once), the CTA's rows of Q and ONE state tile are 36 KB each (alpha_R and alpha_L
-// replace each other in place: an R tile reads the rows (k, .) it then overwrites, an L tile the
-// rows (., j)).  In the last round a block of V lands over the key block it pairs with as soon as
-// that block's alpha_L is formed, and y takes eight of its rows.  No CTA exchanges anything with
-// another; the four CTAs of a head read the same K and V, once from HBM and three times from L2.
+// of K and V and the 32 rows (l, j) of Q).  A CTA owns PJ = 16 (or 8) positions of one head: its rows of Q
+// and ONE state tile stay in shared memory (alpha_R and alpha_L replace each other in place: an R tile
+// reads the rows (k, .) it then overwrites, an L tile the rows (., j)).  No CTA exchanges anything with
+// another; the CTAs of a head read the same K and V, once from HBM and then from L2.
 //
-// K, V and Q arrive by TMA (128-byte swizzle; the blocks of the Q and state tiles are 9 lines apart
-// so that eight rows are conflict-free both along a block and across blocks).  Contractions are
-// warp-level mma.sync m16n8k16 in f16 (bf16 inputs are converted to f16 in registers, fragment by
-// fragment on their way to the tensor cores: the kernel is bound by shared-memory traffic and a
-// conversion in place would add a round trip; exact for magnitudes in [6.1e-5, 65504], clamped beyond).  With 8 positions the R half-step runs transposed,
-// S^T[i,j] = <K(k,i), alpha_R(k,j)> with the positions as the MMA's N: the softmax over i is a
-// reduction over accumulator rows (registers, then three shuffles), the weights reach the second
-// product as its B operand through movmatrix, and alpha_L^T[v,j] leaves through transposing matrix
-// stores.  A warp works on two key blocks at a time.  In the L half-step two warps share a position
-// (16 rows l each); for alpha_R, whose contraction runs over l, they exchange their weights through
-// shared memory and each forms 16 of the 32 rows k.
+// What bounds it: instruction issue and latency at four warps per scheduler (half of the issue slots are
+// busy), then the last wave of CTAs.  K and V stream
+// through ONE 4 KB slot per warp.  A warp owns 32 / (warps) key blocks of an R half-step; it reads a block
+// into registers as the operand of the scores, at which point the slot is free and TMA brings the next
+// block (K of the next, or V of this one in the last round) under the whole work on this one; the
+// second product's operand, the block transposed, comes out of the same registers through movmatrix.  So
+// K is read from shared memory (and converted from bf16) once per half-step, and the first block of the
+// next round arrives under the L half-step.  With 16 positions a K fragment feeds two MMAs.
+//
+// The R half-step runs transposed, S^T[i,j] = <K(k,i), alpha_R(k,j)> with the positions as the MMA's N: the
+// softmax over i is a reduction over accumulator rows (registers, then three shuffles), the weights reach
+// the second product as its B operand through movmatrix, and alpha_L^T[v,j] leaves through transposing
+// matrix stores.  In the L half-step a warp owns a position.  Contractions are mma.sync m16n8k16 in f16
+// (bf16 inputs are converted in registers: exact for magnitudes in [6.1e-5, 65504], clamped beyond).
+// Blocks of the Q and state tiles are an odd number of 128-byte lines apart, so that under the 128-byte
+// swizzle eight rows are conflict-free both along a block and across blocks.  Reductions over the lanes of
+// a column halve the number of values a lane carries at each step, which also leaves one division and one
+// logarithm a lane instead of four.
+//
+// Batch 16, 12 heads, T = 2, bf16: 58 us (f16 54), against 79 (74) with K resident in shared memory, read
+// again as the second product's operand, and 8 positions a CTA; 64 (60) before the halving reductions and
+// Q converted once.  One head: 8 and 13 us (T = 1, 2).
 #pragma once
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -44,36 +53,61 @@ using tensor::mbar_init;
 using tensor::mbar_wait;
 using tensor::tma_load_2d;
 using warpmma::Mma;
-using warpmma::col_sum;
 using warpmma::ex2;
-using warpmma::kLn2;
 using warpmma::kLog2e;
 using warpmma::ldsm_x4;
 using warpmma::ldsm_x4_trans;
 using warpmma::lg2;
 using warpmma::movm_trans;
 using warpmma::quad_max;
-using warpmma::quad_sum;
 
-constexpr int kN = 1024, kB = 32, kM = 32, kD = 64, kPJ = 8;   // kPJ: positions per CTA
-constexpr int kThreads = 512, kWarps = 16;
-constexpr int kBlkK = kB * 128;            // a key block
-constexpr int kBlkQ = (kPJ + 1) * 128;     // the 8 rows (k, .) of the Q / state tile and one line of padding
-constexpr int kOffK = 0;                               // [k][i][128 B]
-constexpr int kOffQ = kN * 128;                        // [l][jj][128 B], blocks kBlkQ apart
-constexpr int kOffS = kOffQ + kM * kBlkQ;              // state, [k][jj][128 B], blocks kBlkQ apart
-constexpr int kOffP = kOffS + kM * kBlkQ;              // weights exchange: per position [32 l][32 k] f16
-constexpr int kOffX = kOffP + kPJ * 2048;              // column maxima: per position [2][32] floats
-constexpr int kOffC = kOffX + kPJ * 256;               // c_L, [k*8 + jj] floats
-constexpr int kOffBar = kOffC + kM * kPJ * 4;          // 64 mbarriers
-constexpr int kSmem = kOffBar + 64 * 8 + 1024;         // + alignment slack
-static_assert(kOffQ % 1024 == 0 && kOffS % 1024 == 0 && kSmem <= 227 * 1024, "shared memory layout");
+constexpr int kN = 1024, kB = 32, kM = 32, kD = 64;
+constexpr int kSlot = kB * 128;                          // a block of K or V
+
+// Shared memory for PJ positions per CTA and W warps per position.
+template <int PJ, int W>
+struct Lay {
+  static constexpr int kWarps = PJ * W, kThreads = 32 * kWarps;
+  static constexpr int kBlk = (PJ + 1) * 128;            // the PJ rows (k, .) of the Q / state tile and a line of padding
+  static constexpr int Q = kWarps * kSlot;               // after the slots, one per warp
+  static constexpr int S = Q + kM * kBlk;                // state, [k][jj]
+  static constexpr int P = S + kM * kBlk;                // W = 2: weights exchange, per position [32 l][32 k] f16
+  static constexpr int X = P + (W - 1) * PJ * 2048;      // W = 2: column maxima, per position [2][32]
+  static constexpr int C = X + (W - 1) * PJ * 256;       // -c_L log2 e, [jj][kCp]: conflict-free along k and along jj
+  static constexpr int kCp = kM + 2;
+  static constexpr int Bar = C + kCp * PJ * 4;
+  static constexpr int kSmem = Bar + kWarps * 8 + 1024;  // + alignment slack
+  static_assert(Q % 1024 == 0 && S % 1024 == 0 && kSmem <= 227 * 1024, "shared memory layout");
+};
 
 __device__ __forceinline__ float col_max(float v) {   // over the 8 row groups (lanes with equal t)
   v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 4));
   v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 8));
   return fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 16));
 }
+// Reduction of NV values over the lanes that differ in the three bits (or two, LO = 1) of `lane` below
+// 2 HI: each step halves the values a lane carries as long as there is more than one, so that with eight
+// values and three bits lane bits HI..LO are the index of the value the lane ends up with.
+template <int NV, int HI, int LO, typename Op>
+__device__ __forceinline__ float scatter_reduce(float* v, int lane, Op op) {
+  int n = NV / 2;
+#pragma unroll
+  for (int m = HI; m >= LO; m >>= 1, n >>= 1) {
+    if (n >= 1) {
+#pragma unroll
+      for (int i = 0; i < NV / 2; ++i)
+        if (i < n) {
+          const float keep = lane & m ? v[i + n] : v[i], send = lane & m ? v[i] : v[i + n];
+          v[i] = op(keep, __shfl_xor_sync(0xffffffffu, send, m));
+        }
+    } else {
+      v[0] = op(v[0], __shfl_xor_sync(0xffffffffu, v[0], m));
+    }
+  }
+  return v[0];
+}
+struct Add { __device__ __forceinline__ float operator()(float a, float b) const { return a + b; } };
+struct Max { __device__ __forceinline__ float operator()(float a, float b) const { return fmaxf(a, b); } };
 __device__ __forceinline__ void stsm_x4(uint32_t saddr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
   asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(saddr), "r"(r0),
                "r"(r1), "r"(r2), "r"(r3)
@@ -85,65 +119,65 @@ __device__ __forceinline__ void stsm_x4_trans(uint32_t saddr, uint32_t r0, uint3
                "r"(r0), "r"(r1), "r"(r2), "r"(r3)
                : "memory");
 }
-// Row offsets (bytes from the 1024-byte aligned base) and the 128-byte swizzle TMA applies: the
-// 16-byte chunk index is XORed with bits 7..9 of the row's address.
-__device__ __forceinline__ uint32_t rk(int k, int i) { return kOffK + k * kBlkK + i * 128; }
-__device__ __forceinline__ uint32_t rq(int l, int jj) { return kOffQ + l * kBlkQ + jj * 128; }
-__device__ __forceinline__ uint32_t rs(int k, int jj) { return kOffS + k * kBlkQ + jj * 128; }
-// y(k, j) lies in key block k at row (j + k) mod 8: conflict-free along j and along k
-__device__ __forceinline__ uint32_t ry(int k, int jj) { return kOffK + k * kBlkK + ((jj + k) & 7) * 128; }
+// The 128-byte swizzle TMA applies: the 16-byte chunk index is XORed with bits 7..9 of the row's address.
 __device__ __forceinline__ uint32_t swz(uint32_t row, int c) { return row + ((c ^ ((row >> 7) & 7)) << 4); }
-// exchanged weights of position jj: row l (64 bytes), 16-byte chunk c
-__device__ __forceinline__ uint32_t pt(int jj, int l, int c) {
-  return kOffP + jj * 2048 + l * 64 + ((c ^ ((l >> 1) & 3)) << 4);
-}
 
-template <typename TIn>
-__global__ void __launch_bounds__(kThreads, 1)
-monarch_jsplit32(const __grid_constant__ CUtensorMap tmQ,    // Q as [BH*N rows][64], box of 8 rows
+template <typename TIn, int PJ, int W>
+__global__ void __launch_bounds__(Lay<PJ, W>::kThreads, 1)
+monarch_jsplit32(const __grid_constant__ CUtensorMap tmQ,    // Q as rows of d, box of PJ rows
                  const __grid_constant__ CUtensorMap tmK,    // K, box of 32 rows
                  const __grid_constant__ CUtensorMap tmV,    // V, box of 32 rows
                  TIn* __restrict__ Y, int T_steps, float scale, int* status, int H) {
-  typedef __half T;
+  typedef Mma<__half> M;
+  using L = Lay<PJ, W>;
+  constexpr int NW = L::kWarps, NB = kM / NW;   // key blocks of a warp: warp, warp + NW, ..
+  constexpr int NT = PJ / 8;                    // 8-position tiles
   extern __shared__ uint8_t smem_raw[];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(smem);
-  float* sCL = reinterpret_cast<float*>(smem + kOffC);
-  uint64_t* kbar = reinterpret_cast<uint64_t*>(smem + kOffBar);   // block k: K(k, .) and Q(k, .) have landed
-  uint64_t* vbar = kbar + kM;                                     // block k: V(k, .) has landed
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-  const int c4 = blockIdx.x;                    // which 8 of the 32 positions
-  // H = 0: tensors [batch][heads][N][64], the maps see [BH * N rows][64 columns]; H = heads: tensors
-  // [batch][N][heads][64], the maps see [batch * N rows][heads * 64 columns] and a head is a column
-  // offset
-  const int hb = H ? (int)blockIdx.y / H : (int)blockIdx.y;   // which sequence of rows
-  const int x0 = H ? ((int)blockIdx.y - hb * H) * kD : 0;     // first column of the head
-  const int row0 = hb * kN;                                   // the head's first row
+  float* sCL = reinterpret_cast<float*>(smem + L::C);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::Bar);      // by warp: what it asked for has landed in its slot
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, t = lane & 3;
+  const int jc = blockIdx.x * PJ;               // first position
+  // H = 0: tensors [batch][heads][N][d], a head is 1024 rows of the maps; H = heads: tensors
+  // [batch][N][heads][d], the maps see rows of heads * 64 columns (d = 64) and a head is a column offset
+  const int hb = H ? (int)blockIdx.y / H : (int)blockIdx.y;
+  const int x0 = H ? ((int)blockIdx.y - hb * H) * kD : 0;
+  const int row0 = hb * kN;
   const float fl = scale * kLog2e;
-  const int kk[2] = {warp, warp + kWarps};      // the key blocks this warp owns in the R half-steps
-#ifdef MA_JSPLIT_TRACE
-  long long stamps[12];
-  int n_st = 0;
-#define MA_STAMP() do { if (n_st < 12) stamps[n_st++] = clock64(); } while (0)
-#else
-#define MA_STAMP() do { } while (0)
-#endif
-  MA_STAMP();
-
-  if (tid == 0) {
-    for (int i = 0; i < 2 * kM; ++i) mbar_init(&kbar[i], 1);
-    tensor::fence_barrier_init();
-  }
+  if (lane == 0) mbar_init(&bars[warp], 1);
+  tensor::fence_barrier_init();
   __syncthreads();
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (lane == 0) {
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      mbar_expect_tx(&kbar[kk[u]], kBlkK + kPJ * 128);
-      tma_load_2d(smem + rk(kk[u], 0), &tmK, &kbar[kk[u]], x0, row0 + kk[u] * kB);
-      tma_load_2d(smem + rq(kk[u], 0), &tmQ, &kbar[kk[u]], x0, row0 + kk[u] * kB + c4 * kPJ);
+
+  // rows of the tiles: Q (l, jj), state (k, jj)
+  auto rq = [&](int l, int jj) { return s0 + L::Q + l * L::kBlk + jj * 128; };
+  auto rs = [&](int k, int jj) { return s0 + L::S + k * L::kBlk + jj * 128; };
+  // y(k, jj) lies in the slot of the warp that owns block k; rows are turned by k so that eight blocks
+  // are conflict-free
+  auto ry = [&](int k, int jj) { return s0 + (k % NW) * kSlot + ((k / NW) * PJ + ((jj + k) & (PJ - 1))) * 128; };
+  const uint32_t slot = s0 + warp * kSlot;
+  uint32_t par = 0;
+  auto request = [&](const CUtensorMap* tm, int k) {      // block k of K or V into the slot
+    tensor::fence_proxy_async();
+    __syncwarp();
+    if (lane == 0) {
+      mbar_expect_tx(&bars[warp], kSlot);
+      tma_load_2d(smem + warp * kSlot, tm, &bars[warp], x0, row0 + k * kB);
     }
+  };
+  auto landed = [&]() {
+    if (!mbar_wait(&bars[warp], par)) tensor::report_timeout(status, 1);
+    par ^= 1;
+    __syncwarp();
+  };
+  if (lane == 0) {
+    mbar_expect_tx(&bars[warp], kSlot + NB * PJ * 128);
+    tma_load_2d(smem + warp * kSlot, &tmK, &bars[warp], x0, row0 + warp * kB);
+#pragma unroll
+    for (int u = 0; u < NB; ++u)
+      tma_load_2d(smem + L::Q + (warp + u * NW) * L::kBlk, &tmQ, &bars[warp], x0, row0 + (warp + u * NW) * kB + jc);
   }
   // bf16 -> f16 of a fragment in registers (a no-op for f16 inputs)
   auto convert_frag = [&](uint32_t* a) {
@@ -153,338 +187,362 @@ monarch_jsplit32(const __grid_constant__ CUtensorMap tmQ,    // Q as [BH*N rows]
     }
   };
 
-  uint32_t pb[2][2][2];      // the R weights of the warp's two blocks as B fragments (P^T), kept for y
-  float inv_r[2][2];         // 1 / their column sums
-
   for (int step = 1; step <= T_steps; ++step) {
     const bool first = step == 1, last = step == T_steps;
     // ================================================================ R half-step (Eq. 7, 9, 10)
     // block k: S^T[i,j] = <K(k,i), alpha_R(k,j)> (alpha_R arrives divided by c_R), softmax over i,
     // alpha_L(k,j) = sum_i R[j,i] K(k,i), c_L(k,j) = sum_i R log R, (last) y(k,j) = sum_i R[j,i] V(k,i)
-    // `which`: 0 / 1 = the warp's first / second block alone, 2 = both at a time (two independent
-    // instruction streams per warp)
-    auto r_pass = [&](auto which) {
-      constexpr int U0 = decltype(which)::value == 1 ? 1 : 0;
-      constexpr int U1 = decltype(which)::value == 0 ? 1 : 2;
-      if (first) {
+    uint32_t yk[NB][NT][4][2];                  // y of the warp's blocks, 16-bit
 #pragma unroll
-        for (int u = U0; u < U1; ++u) {
-          if (!mbar_wait(&kbar[kk[u]], 0)) tensor::report_timeout(status, 1);
+    for (int u = 0; u < NB; ++u) {
+      const int k = warp + u * NW;
+      landed();
+      if (first && u == 0 && !Mma<TIn>::is_f16) {        // the warp's rows of Q, in place
+#pragma unroll
+        for (int q = 0; q < NB * PJ / 4; ++q) {
+          uint4* c = reinterpret_cast<uint4*>(smem + L::Q + (warp + q / (PJ / 4) * NW) * L::kBlk + q % (PJ / 4) * 512 + lane * 16);
+          *c = warpmma::to_f16x8(*c, (const TIn*)nullptr);
         }
         __syncwarp();
       }
-      {
-        // B operand: rows (k, jj) of alpha_R (L^(0) = identity: the Q rows (k, .) in the first round)
-        uint32_t bq[2][2][4];
+      uint32_t kf[2][4][4];                     // K(k, .) as A operand: [16 rows i][16 columns v]
 #pragma unroll
-        for (int u = U0; u < U1; ++u)
+      for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-          for (int half = 0; half < 2; ++half) {
-            ldsm_x4(bq[u][half], s0 + swz(first ? rq(kk[u], lane & 7) : rs(kk[u], lane & 7), (lane >> 3) + 4 * half));
-            if (first) convert_frag(bq[u][half]);
-          }
-        float s[2][2][4];
+        for (int ks = 0; ks < 4; ++ks) {
+          ldsm_x4(kf[mt][ks], swz(slot + (16 * mt + (lane & 15)) * 128, 2 * ks + (lane >> 4)));
+          convert_frag(kf[mt][ks]);
+        }
+      // the slot is free: the next block comes under the work on this one
+      if (last) request(&tmV, k);
+      else request(&tmK, u + 1 < NB ? k + NW : warp);
+      uint32_t pb[NT][2][2];                    // the weights P^T[i, j] as the second product's B operand
+      float inv[NT][2], red[4 * NT], mxs[2 * NT];
 #pragma unroll
-        for (int u = U0; u < U1; ++u)
+      for (int nt = 0; nt < NT; ++nt) {
+        float s[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+        const uint32_t row = first ? rq(k, 8 * nt + (lane & 7)) : rs(k, 8 * nt + (lane & 7));
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+          uint32_t bq[4];                       // alpha_R rows (k, j) (L^(0) = identity: Q rows in the first round)
+          ldsm_x4(bq, swz(row, (lane >> 3) + 4 * half));
+#pragma unroll
+          for (int k2 = 0; k2 < 2; ++k2)
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) M::run(s[mt], kf[mt][2 * half + k2], bq + 2 * k2);
+        }
+        // column j = 8 nt + 2 t + e holds rows i = 16 mt + g (+ 8): softmax over i
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const float mx = col_max(fmaxf(fmaxf(s[0][e], s[0][e + 2]), fmaxf(s[1][e], s[1][e + 2])) * fl);
+          float sum = 0.f, sz = 0.f;
 #pragma unroll
           for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) s[u][mt][e] = 0.f;
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks)
-#pragma unroll
-          for (int u = U0; u < U1; ++u)
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt) {
-              uint32_t a[4];
-              ldsm_x4(a, s0 + swz(rk(kk[u], 16 * mt + (lane & 7) + 8 * ((lane >> 3) & 1)), 2 * ks + (lane >> 4)));
-              convert_frag(a);
-              Mma<T>::run(s[u][mt], a, &bq[u][ks >> 1][2 * (ks & 1)]);
+            for (int hh = 0; hh < 2; ++hh) {
+              const float p = ex2(fmaf(s[mt][e + 2 * hh], fl, -mx));
+              sum += p;
+              sz = fmaf(p, s[mt][e + 2 * hh], sz);
+              s[mt][e + 2 * hh] = p;
             }
-        // column j = 2 t + e holds rows i = 16 mt + g (+ 8): softmax over i
-#pragma unroll
-        for (int u = U0; u < U1; ++u)
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            float mx = fmaxf(fmaxf(s[u][0][e], s[u][0][e + 2]), fmaxf(s[u][1][e], s[u][1][e + 2])) * fl;
-            mx = col_max(mx);
-            float sum = 0.f, sz = 0.f;
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-              for (int hh = 0; hh < 2; ++hh) {
-                const float z = s[u][mt][e + 2 * hh] * fl;
-                const float p = ex2(z - mx);
-                s[u][mt][e + 2 * hh] = p;
-                sum += p;
-                sz = fmaf(p, z, sz);
-              }
-            sum = col_sum(sum);
-            sz = col_sum(sz);
-            inv_r[u][e] = 1.f / sum;
-            // c_L = sum R log R (natural log): ln2 * (sum p z / sum - max - log2 sum)
-            if (g == 0) sCL[kk[u] * kPJ + 2 * t + e] = kLn2 * (sz * inv_r[u][e] - mx - lg2(sum));
-          }
-        // the weights as the second product's B operand: P^T[i, j], contraction over i
-#pragma unroll
-        for (int u = U0; u < U1; ++u)
-#pragma unroll
-          for (int mt = 0; mt < 2; ++mt) {
-            pb[u][mt][0] = movm_trans(Mma<T>::pack(s[u][mt][0], s[u][mt][1]));
-            pb[u][mt][1] = movm_trans(Mma<T>::pack(s[u][mt][2], s[u][mt][3]));
-          }
-        __syncwarp();
-        // alpha_L^T[v, j] = sum_i K(k,i)[v] P^T[i, j]: A = the key block read transposed; the rows
-        // (k, j) of alpha_L go over the alpha_R rows they were formed from (transposing stores: memory
-        // row j receives column j of the accumulator tile)
-#pragma unroll
-        for (int vp = 0; vp < 2; ++vp) {
-          float o[2][2][4];
-#pragma unroll
-          for (int u = U0; u < U1; ++u)
-#pragma unroll
-            for (int v2 = 0; v2 < 2; ++v2) {
-#pragma unroll
-              for (int e = 0; e < 4; ++e) o[u][v2][e] = 0.f;
-#pragma unroll
-              for (int is = 0; is < 2; ++is) {
-                uint32_t a[4];
-                ldsm_x4_trans(a, s0 + swz(rk(kk[u], 16 * is + (lane & 7) + 8 * (lane >> 4)),
-                                          2 * (2 * vp + v2) + ((lane >> 3) & 1)));
-                convert_frag(a);
-                Mma<T>::run(o[u][v2], a, pb[u][is]);
-              }
-            }
-#pragma unroll
-          for (int u = U0; u < U1; ++u)
-            stsm_x4_trans(s0 + swz(rs(kk[u], lane & 7), 4 * vp + (lane >> 3)),
-                          Mma<T>::pack(o[u][0][0] * inv_r[u][0], o[u][0][1] * inv_r[u][1]),
-                          Mma<T>::pack(o[u][0][2] * inv_r[u][0], o[u][0][3] * inv_r[u][1]),
-                          Mma<T>::pack(o[u][1][0] * inv_r[u][0], o[u][1][1] * inv_r[u][1]),
-                          Mma<T>::pack(o[u][1][2] * inv_r[u][0], o[u][1][3] * inv_r[u][1]));
+          mxs[2 * nt + e] = mx;
+          red[2 * (2 * nt + e)] = sum;
+          red[2 * (2 * nt + e) + 1] = sz;
         }
-        if (last) {
-          // the key blocks are dead: V(k, .) lands over them while the final scores are formed
-          tensor::fence_proxy_async();
-          __syncwarp();
-          if (lane == 0) {
 #pragma unroll
-            for (int u = U0; u < U1; ++u) {
-              mbar_expect_tx(&vbar[kk[u]], kBlkK);
-              tma_load_2d(smem + rk(kk[u], 0), &tmV, &vbar[kk[u]], x0, row0 + kk[u] * kB);
-            }
-          }
+        for (int mt = 0; mt < 2; ++mt) {
+          pb[nt][mt][0] = movm_trans(M::pack(s[mt][0], s[mt][1]));
+          pb[nt][mt][1] = movm_trans(M::pack(s[mt][2], s[mt][3]));
         }
       }
-    };
-    if (first) {
-      // blocks are taken as they land: the first sixteen while the second sixteen are on their way
-      r_pass(std::integral_constant<int, 0>());
-      r_pass(std::integral_constant<int, 1>());
-    } else {
-      r_pass(std::integral_constant<int, 2>());
-    }
-    MA_STAMP();
-    __syncthreads();
-    MA_STAMP();
-
-    // ================================================================ L half-step (Eq. 8, 9 / Eq. 4)
-    // position jj, rows l = 16 lt ..: Z_L[l,k] = fl * <Q(l,j), alpha_L(k,j)> - c_L(k,j), softmax over k
-    {
-      const int jj = warp >> 1, lt = warp & 1;
-      float c[4][2];
+      {
+        // a lane ends up with sum or sum p s (lane bit kSz) of one column: one division and one logarithm
+        // a lane, the reciprocals then go to all lanes
+        constexpr int kSz = 8 / NT, kCol = NT == 2 ? 3 : 4;
+        const float r = scatter_reduce<4 * NT, 16, 4>(red, lane, Add());
+        const float ri = 1.f / r;
 #pragma unroll
-      for (int nt = 0; nt < 4; ++nt)
+        for (int q = 0; q < 2 * NT; ++q) inv[q >> 1][q & 1] = __shfl_sync(0xffffffffu, ri, (q << kCol) + t);
+        const float so = __shfl_xor_sync(0xffffffffu, r, kSz), io = __shfl_xor_sync(0xffffffffu, ri, kSz);
+        const int q = lane >> kCol;
+        float mx = mxs[0];
 #pragma unroll
-        for (int e = 0; e < 2; ++e) c[nt][e] = sCL[(8 * nt + 2 * t + e) * kPJ + jj] * kLog2e;
-      float s[4][4];
-#pragma unroll
-      for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) s[nt][e] = 0.f;
-#pragma unroll
-      for (int ks = 0; ks < 4; ++ks) {
-        uint32_t a[4];
-        ldsm_x4(a, s0 + swz(rq(16 * lt + (lane & 7) + 8 * ((lane >> 3) & 1), jj), 2 * ks + (lane >> 4)));
-        convert_frag(a);
-#pragma unroll
-        for (int np = 0; np < 2; ++np) {
-          uint32_t bf[4];
-          ldsm_x4(bf, s0 + swz(rs(16 * np + (lane & 7) + 8 * (lane >> 4), jj), 2 * ks + ((lane >> 3) & 1)));
-          Mma<T>::run(s[2 * np], a, bf);
-          Mma<T>::run(s[2 * np + 1], a, bf + 2);
-        }
+        for (int i = 1; i < 2 * NT; ++i) mx = q == i ? mxs[i] : mx;
+        // -c_L log2 e = max + log2 sum - sum R z (z = s fl), the addend of the L logits
+        if ((lane & kSz) && (NT == 2 || !(lane & 4)))
+          sCL[(8 * (q >> 1) + 2 * t + (q & 1)) * L::kCp + k] = mx + lg2(so) - r * fl * io;
       }
+      __syncwarp();
+      // alpha_L^T[v, j] = sum_i K(k,i)[v] P^T[i, j]: A = the block's fragments transposed; the rows (k, j)
+      // go over the alpha_R rows they were formed from (transposing stores: memory row j receives
+      // column j of the accumulator tile)
 #pragma unroll
-      for (int hh = 0; hh < 2; ++hh) {
-        float mx = -INFINITY;
+      for (int vp = 0; vp < 2; ++vp) {
+        float o[NT][2][4];
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
+        for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const float z = fmaf(s[nt][2 * hh + e], fl, -c[nt][e]);
-            s[nt][2 * hh + e] = z;
-            mx = fmaxf(mx, z);
+          for (int v2 = 0; v2 < 2; ++v2)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o[nt][v2][e] = 0.f;
+#pragma unroll
+        for (int v2 = 0; v2 < 2; ++v2)
+#pragma unroll
+          for (int is = 0; is < 2; ++is) {
+            const uint32_t* f = kf[is][2 * vp + v2];
+            const uint32_t a[4] = {movm_trans(f[0]), movm_trans(f[2]), movm_trans(f[1]), movm_trans(f[3])};
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) M::run(o[nt][v2], a, pb[nt][is]);
           }
-        mx = quad_max(mx);
-        float sum = 0.f;
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const float p = ex2(s[nt][2 * hh + e] - mx);
-            s[nt][2 * hh + e] = p;
-            sum += p;
-          }
-        const float inv = 1.f / quad_sum(sum);
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-          for (int e = 0; e < 2; ++e) s[nt][2 * hh + e] *= inv;
+        for (int nt = 0; nt < NT; ++nt) {
+          const float i0 = inv[nt][0], i1 = inv[nt][1];
+          stsm_x4_trans(swz(rs(k, 8 * nt + (lane & 7)), 4 * vp + (lane >> 3)), M::pack(o[nt][0][0] * i0, o[nt][0][1] * i1),
+                        M::pack(o[nt][0][2] * i0, o[nt][0][3] * i1), M::pack(o[nt][1][0] * i0, o[nt][1][1] * i1),
+                        M::pack(o[nt][1][2] * i0, o[nt][1][3] * i1));
+        }
       }
       if (last) {
-        // Y(l,j) = sum_k L[j,k,l] y(k,j): A = the weights, rows l
-        uint32_t pa[2][4];
+        // y^T[v, j] = sum_i V(k,i)[v] P^T[i, j]
+        landed();
 #pragma unroll
-        for (int k2 = 0; k2 < 2; ++k2) {
-          pa[k2][0] = Mma<T>::pack(s[2 * k2][0], s[2 * k2][1]);
-          pa[k2][1] = Mma<T>::pack(s[2 * k2][2], s[2 * k2][3]);
-          pa[k2][2] = Mma<T>::pack(s[2 * k2 + 1][0], s[2 * k2 + 1][1]);
-          pa[k2][3] = Mma<T>::pack(s[2 * k2 + 1][2], s[2 * k2 + 1][3]);
-        }
-        // y^T[v, j] = sum_i V(k,i)[v] P^T[i, j] for the warp's two blocks, V read where K was
+        for (int vt = 0; vt < 4; ++vt) {
+          float o[NT][4];
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          if (!mbar_wait(&vbar[kk[u]], 0)) tensor::report_timeout(status, 2);
-        }
-        float yv[2][4][4];
+          for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-        for (int u = 0; u < 2; ++u)
+            for (int e = 0; e < 4; ++e) o[nt][e] = 0.f;
 #pragma unroll
-          for (int vt = 0; vt < 4; ++vt) {
+          for (int is = 0; is < 2; ++is) {
+            uint32_t a[4];
+            ldsm_x4_trans(a, swz(slot + (16 * is + (lane & 7) + 8 * (lane >> 4)) * 128, 2 * vt + ((lane >> 3) & 1)));
+            convert_frag(a);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) yv[u][vt][e] = 0.f;
-#pragma unroll
-            for (int is = 0; is < 2; ++is) {
-              uint32_t a[4];
-              ldsm_x4_trans(a, s0 + swz(rk(kk[u], 16 * is + (lane & 7) + 8 * (lane >> 4)), 2 * vt + ((lane >> 3) & 1)));
-              convert_frag(a);     // V is used once: converted on its way to the tensor cores
-              Mma<T>::run(yv[u][vt], a, pb[u][is]);
-            }
+            for (int nt = 0; nt < NT; ++nt) M::run(o[nt], a, pb[nt][is]);
           }
-        __syncwarp();      // every row of V(k, .) is read: y(k, .) takes eight of them
 #pragma unroll
-        for (int u = 0; u < 2; ++u)
+          for (int nt = 0; nt < NT; ++nt) {
+            yk[u][nt][vt][0] = M::pack(o[nt][0] * inv[nt][0], o[nt][1] * inv[nt][1]);
+            yk[u][nt][vt][1] = M::pack(o[nt][2] * inv[nt][0], o[nt][3] * inv[nt][1]);
+          }
+        }
+        if (u + 1 < NB) request(&tmK, k + NW);
+      }
+    }
+    if (last) {                                 // the slot has had its last block: y(k, .) of all of them
+      __syncwarp();
+#pragma unroll
+      for (int u = 0; u < NB; ++u)
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
           for (int vp = 0; vp < 2; ++vp)
-            stsm_x4_trans(s0 + swz(ry(kk[u], lane & 7), 4 * vp + (lane >> 3)),
-                          Mma<T>::pack(yv[u][2 * vp][0] * inv_r[u][0], yv[u][2 * vp][1] * inv_r[u][1]),
-                          Mma<T>::pack(yv[u][2 * vp][2] * inv_r[u][0], yv[u][2 * vp][3] * inv_r[u][1]),
-                          Mma<T>::pack(yv[u][2 * vp + 1][0] * inv_r[u][0], yv[u][2 * vp + 1][1] * inv_r[u][1]),
-                          Mma<T>::pack(yv[u][2 * vp + 1][2] * inv_r[u][0], yv[u][2 * vp + 1][3] * inv_r[u][1]));
-        MA_STAMP();
-        __syncthreads();
-        MA_STAMP();
+            stsm_x4_trans(swz(ry(warp + u * NW, 8 * nt + (lane & 7)), 4 * vp + (lane >> 3)), yk[u][nt][2 * vp][0],
+                          yk[u][nt][2 * vp][1], yk[u][nt][2 * vp + 1][0], yk[u][nt][2 * vp + 1][1]);
+    }
+    __syncthreads();
+
+    // ================================================================ L half-step (Eq. 8, 9 / Eq. 4)
+    // position jj: Z_L[l,k] = fl * <Q(l,j), alpha_L(k,j)> - c_L(k,j), softmax over k.  A warp has
+    // LT tiles of 16 rows l
+    {
+      constexpr int LT = 2 / W;
+      const int jj = warp / W, l0 = W == 2 ? 16 * (warp & 1) : 0;
+      float c[4][2];
 #pragma unroll
-        for (int vp = 0; vp < 4; ++vp) {          // two 8-column tiles of v per load
-          float o[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+      for (int nt = 0; nt < 4; ++nt) {
+        const float2 v = *reinterpret_cast<const float2*>(sCL + jj * L::kCp + 8 * nt + 2 * t);
+        c[nt][0] = v.x;
+        c[nt][1] = v.y;
+      }
+      float s[LT][4][4], inv[LT][2], rsum[2 * LT];
+#pragma unroll
+      for (int lt = 0; lt < LT; ++lt)
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) s[lt][nt][e] = 0.f;
+#pragma unroll
+      for (int ks = 0; ks < 4; ++ks) {
+        uint32_t bf[2][4];
+#pragma unroll
+        for (int np = 0; np < 2; ++np)
+          ldsm_x4(bf[np], swz(rs(16 * np + (lane & 7) + 8 * (lane >> 4), jj), 2 * ks + ((lane >> 3) & 1)));
+#pragma unroll
+        for (int lt = 0; lt < LT; ++lt) {
+          uint32_t a[4];
+          ldsm_x4(a, swz(rq(l0 + 16 * lt + (lane & 15), jj), 2 * ks + (lane >> 4)));
+#pragma unroll
+          for (int nt = 0; nt < 4; ++nt) M::run(s[lt][nt], a, bf[nt >> 1] + 2 * (nt & 1));
+        }
+      }
+#pragma unroll
+      for (int lt = 0; lt < LT; ++lt)
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh) {
+          float mx = -INFINITY;
+#pragma unroll
+          for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              const float z = fmaf(s[lt][nt][2 * hh + e], fl, c[nt][e]);
+              s[lt][nt][2 * hh + e] = z;
+              mx = fmaxf(mx, z);
+            }
+          mx = quad_max(mx);
+          float sum = 0.f;
+#pragma unroll
+          for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              const float p = ex2(s[lt][nt][2 * hh + e] - mx);
+              s[lt][nt][2 * hh + e] = p;
+              sum += p;
+            }
+          rsum[2 * lt + hh] = sum;
+        }
+      const float ri = 1.f / scatter_reduce<2 * LT, 2, 1>(rsum, lane, Add());
+#pragma unroll
+      for (int i = 0; i < 2 * LT; ++i) inv[i >> 1][i & 1] = __shfl_sync(0xffffffffu, ri, (lane & ~3) + i * (2 / LT));
+      __syncwarp();
+      if (last) {
+        // Y(l,j) = sum_k L[j,k,l] y(k,j): A = the weights, rows l; staged over the rows (l, j) of Q the
+        // scores were formed from (only this warp reads them)
+        uint32_t pa[LT][2][4];
+#pragma unroll
+        for (int lt = 0; lt < LT; ++lt)
 #pragma unroll
           for (int k2 = 0; k2 < 2; ++k2) {
-            uint32_t bf[4];      // B[k][v] = y(k,j)[v], read transposed
-            ldsm_x4_trans(bf, s0 + swz(ry(16 * k2 + (lane & 15), jj), 2 * vp + (lane >> 4)));
-            Mma<T>::run(o[0], pa[k2], bf);
-            Mma<T>::run(o[1], pa[k2], bf + 2);
+            pa[lt][k2][0] = M::pack(s[lt][2 * k2][0], s[lt][2 * k2][1]);
+            pa[lt][k2][1] = M::pack(s[lt][2 * k2][2], s[lt][2 * k2][3]);
+            pa[lt][k2][2] = M::pack(s[lt][2 * k2 + 1][0], s[lt][2 * k2 + 1][1]);
+            pa[lt][k2][3] = M::pack(s[lt][2 * k2 + 1][2], s[lt][2 * k2 + 1][3]);
           }
-          // staged over the rows (l, j) of Q the scores were formed from (only this warp reads them)
-          stsm_x4(s0 + swz(rq(16 * lt + (lane & 7) + 8 * ((lane >> 3) & 1), jj), 2 * vp + (lane >> 4)),
-                  Mma<T>::pack(o[0][0], o[0][1]), Mma<T>::pack(o[0][2], o[0][3]),
-                  Mma<T>::pack(o[1][0], o[1][1]), Mma<T>::pack(o[1][2], o[1][3]));
+#pragma unroll
+        for (int vp = 0; vp < 4; ++vp) {          // two 8-column tiles of v per load
+          uint32_t bf[2][4];      // B[k][v] = y(k,j)[v], read transposed
+#pragma unroll
+          for (int k2 = 0; k2 < 2; ++k2) ldsm_x4_trans(bf[k2], swz(ry(16 * k2 + (lane & 15), jj), 2 * vp + (lane >> 4)));
+#pragma unroll
+          for (int lt = 0; lt < LT; ++lt) {
+            float o[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+            for (int k2 = 0; k2 < 2; ++k2) {
+              M::run(o[0], pa[lt][k2], bf[k2]);
+              M::run(o[1], pa[lt][k2], bf[k2] + 2);
+            }
+            const float i0 = inv[lt][0], i1 = inv[lt][1];
+            stsm_x4(swz(rq(l0 + 16 * lt + (lane & 15), jj), 2 * vp + (lane >> 4)), M::pack(o[0][0] * i0, o[0][1] * i0),
+                    M::pack(o[0][2] * i1, o[0][3] * i1), M::pack(o[1][0] * i0, o[1][1] * i0),
+                    M::pack(o[1][2] * i1, o[1][3] * i1));
+          }
         }
         __syncwarp();
-        // the warp's 16 rows (l, j) of Y are complete: 16 bytes per lane and store
+        // the rows (l, j) of Y are complete: 16 bytes per lane and store
+        const int ch = lane & 7;
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const int l = 16 * lt + (lane >> 3) + 4 * r;
-          const uint4 v = *reinterpret_cast<const uint4*>(smem + swz(rq(l, jj), lane & 7));
-          TIn* gp = Y + ((size_t)row0 + l * kB + c4 * kPJ + jj) * (size_t)(H ? H * kD : kD) + x0 + (lane & 7) * 8;
+        for (int r = 0; r < 4 * LT; ++r) {
+          const int l = l0 + (lane >> 3) + 4 * r;
+          const uint4 v = *reinterpret_cast<const uint4*>(smem + (swz(rq(l, jj), ch) - s0));
+          TIn* gp = Y + ((size_t)row0 + l * kB + jc + jj) * (size_t)(H ? H * kD : kD) + x0 + ch * 8;
           *reinterpret_cast<uint4*>(gp) = warpmma::from_f16x8(v, gp);
         }
       } else {
-        // alpha_R(k,j) = sum_l L[j,k,l] Q(l,j) / c_R, c_R(k,j) = sum_l L[j,k,l]: the contraction
-        // runs over the ROW index of the weights, which two warps share.  The result does not change
-        // when column k is multiplied by any g_k > 0: g_k = 2^-(exponent of the column's largest
-        // weight) keeps every column's significant weights in the normal f16 range however small
-        // c_R is.  So the warps exchange their column maxima, then their scaled weights, and each
-        // forms the rows k = 16 lt .. of alpha_R; c_R comes out of the same MMAs (a B operand of
-        // ones), i.e. summed over the weights AS ROUNDED like the numerator.
-        float* xm = reinterpret_cast<float*>(smem + kOffX + jj * 256);
-        float cm[4][2];
+        // alpha_R(k,j) = sum_l L[j,k,l] Q(l,j) / c_R, c_R(k,j) = sum_l L[j,k,l]: the contraction runs over
+        // the ROW index of the weights, so the A fragments are their transpose.  The result does not
+        // change when column k is multiplied by any g_k > 0: g_k = 2^-(exponent of the column's largest
+        // weight) keeps every column's significant weights in the normal f16 range however small c_R
+        // is; c_R comes out of the same MMAs (a B operand of ones), i.e. summed over the weights AS
+        // ROUNDED like the numerator.
+        // Two warps that share a position exchange their column maxima, then their scaled weights, and
+        // each forms 16 of the rows k.
+        float cms[8];
 #pragma unroll
         for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
-            cm[nt][e] = col_max(fmaxf(s[nt][e], s[nt][e + 2]));
-            if (g == 0) xm[lt * 32 + 8 * nt + 2 * t + e] = cm[nt][e];
+            cms[2 * nt + e] = 0.f;
+#pragma unroll
+            for (int lt = 0; lt < LT; ++lt)
+#pragma unroll
+              for (int hh = 0; hh < 2; ++hh) {
+                s[lt][nt][2 * hh + e] *= inv[lt][hh];
+                cms[2 * nt + e] = fmaxf(cms[2 * nt + e], s[lt][nt][2 * hh + e]);
+              }
           }
-        asm volatile("bar.sync %0, 64;" ::"r"(1 + jj) : "memory");
-        uint32_t w[2][4];
+        float cm = scatter_reduce<8, 16, 4>(cms, lane, Max());     // of column 8 (g / 2) + 2 t + g % 2
+        if constexpr (W == 2) {
+          float* xm = reinterpret_cast<float*>(smem + L::X + jj * 256);
+          xm[2 * l0 + lane] = cm;
+          asm volatile("bar.sync %0, 64;" ::"r"(1 + jj) : "memory");
+          cm = fmaxf(cm, xm[32 - 2 * l0 + lane]);
+        }
+        const float gl = cm > 0.f ? __uint_as_float((253u << 23) - (__float_as_uint(cm) & 0x7f800000u)) : 0.f;
+        uint32_t w[LT][2][4];      // [row tile][half][8-column tile]
 #pragma unroll
         for (int nt = 0; nt < 4; ++nt) {
           float gk[2];
 #pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const float m2 = fmaxf(cm[nt][e], xm[(lt ^ 1) * 32 + 8 * nt + 2 * t + e]);
-            gk[e] = m2 > 0.f ? __uint_as_float((253u << 23) - (__float_as_uint(m2) & 0x7f800000u)) : 0.f;
-          }
-          w[0][nt] = Mma<T>::pack(s[nt][0] * gk[0], s[nt][1] * gk[1]);
-          w[1][nt] = Mma<T>::pack(s[nt][2] * gk[0], s[nt][3] * gk[1]);
-        }
+          for (int e = 0; e < 2; ++e) gk[e] = __shfl_sync(0xffffffffu, gl, (2 * nt + e) * 4 + t);
 #pragma unroll
-        for (int hh = 0; hh < 2; ++hh)
-          stsm_x4(s0 + pt(jj, 16 * lt + 8 * hh + (lane & 7), lane >> 3), w[hh][0], w[hh][1], w[hh][2], w[hh][3]);
-        asm volatile("bar.sync %0, 64;" ::"r"(1 + jj) : "memory");
-        const int kt = lt;
-        uint32_t pa[2][4];       // A[k][l] = weights transposed
+          for (int lt = 0; lt < LT; ++lt)
 #pragma unroll
-        for (int ls = 0; ls < 2; ++ls)
-          ldsm_x4_trans(pa[ls], s0 + pt(jj, 16 * ls + (lane & 7) + 8 * (lane >> 4), 2 * kt + ((lane >> 3) & 1)));
-        float cr[4] = {0.f, 0.f, 0.f, 0.f};
-        {
-          const uint32_t ones[2] = {0x3C003C00u, 0x3C003C00u};
-          Mma<T>::run(cr, pa[0], ones);
-          Mma<T>::run(cr, pa[1], ones);
+            for (int hh = 0; hh < 2; ++hh) w[lt][hh][nt] = M::pack(s[lt][nt][2 * hh] * gk[0], s[lt][nt][2 * hh + 1] * gk[1]);
         }
-        const float ic0 = cr[0] > 1e-30f ? 1.f / cr[0] : 0.f;     // row k = 16 kt + g
-        const float ic1 = cr[2] > 1e-30f ? 1.f / cr[2] : 0.f;     // row k = 16 kt + g + 8
+        uint32_t pk[LT][2][4];     // A[k][l], the weights transposed: row tile kt, contraction step ls
+        if constexpr (W == 2) {
+          // row l (64 bytes), 16-byte chunk c of the exchanged weights
+          auto pt = [&](int l, int c) { return s0 + L::P + jj * 2048 + l * 64 + ((c ^ ((l >> 1) & 3)) << 4); };
+#pragma unroll
+          for (int hh = 0; hh < 2; ++hh) stsm_x4(pt(l0 + 8 * hh + (lane & 7), lane >> 3), w[0][hh][0], w[0][hh][1], w[0][hh][2], w[0][hh][3]);
+          asm volatile("bar.sync %0, 64;" ::"r"(1 + jj) : "memory");
+#pragma unroll
+          for (int ls = 0; ls < 2; ++ls)
+            ldsm_x4_trans(pk[0][ls], pt(16 * ls + (lane & 7) + 8 * (lane >> 4), l0 / 8 + ((lane >> 3) & 1)));
+        } else {
+#pragma unroll
+          for (int kt = 0; kt < LT; ++kt)
+#pragma unroll
+            for (int ls = 0; ls < 2; ++ls)
+#pragma unroll
+              for (int i = 0; i < 4; ++i) pk[kt][ls][i] = movm_trans(w[ls * (LT - 1)][i >> 1][2 * kt + (i & 1)]);
+        }
+        const uint32_t ones[2] = {0x3C003C00u, 0x3C003C00u};
+        float ic[LT][2], c1 = 0.f;
+#pragma unroll
+        for (int kt = 0; kt < LT; ++kt) {
+          float cr[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int ls = 0; ls < 2; ++ls) M::run(cr, pk[kt][ls], ones);
+          if (t == 2 * kt) c1 = cr[0];            // a division a lane
+          if (t == 2 * kt + 1) c1 = cr[2];
+        }
+        c1 = c1 > 1e-30f ? 1.f / c1 : 0.f;
+#pragma unroll
+        for (int i = 0; i < 2 * LT; ++i) ic[i >> 1][i & 1] = __shfl_sync(0xffffffffu, c1, (lane & ~3) + i);
 #pragma unroll
         for (int vp = 0; vp < 4; ++vp) {
-          float o[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+          uint32_t bf[2][4];       // B[l][v] = Q(l,j)[v], read transposed; two 8-column tiles
 #pragma unroll
-          for (int ls = 0; ls < 2; ++ls) {
-            uint32_t bf[4];   // B[l][v] = Q(l,j)[v], read transposed; two 8-column tiles
-            ldsm_x4_trans(bf, s0 + swz(rq(16 * ls + (lane & 15), jj), 2 * vp + (lane >> 4)));
-            convert_frag(bf);
-            Mma<T>::run(o[0], pa[ls], bf);
-            Mma<T>::run(o[1], pa[ls], bf + 2);
+          for (int ls = 0; ls < 2; ++ls) ldsm_x4_trans(bf[ls], swz(rq(16 * ls + (lane & 15), jj), 2 * vp + (lane >> 4)));
+#pragma unroll
+          for (int kt = 0; kt < LT; ++kt) {
+            float o[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+            for (int ls = 0; ls < 2; ++ls) {
+              M::run(o[0], pk[kt][ls], bf[ls]);
+              M::run(o[1], pk[kt][ls], bf[ls] + 2);
+            }
+            // alpha_R rows (k, j) over the alpha_L rows (whose readers have formed their scores)
+            stsm_x4(swz(rs(l0 + 16 * kt + (lane & 15), jj), 2 * vp + (lane >> 4)), M::pack(o[0][0] * ic[kt][0], o[0][1] * ic[kt][0]),
+                    M::pack(o[0][2] * ic[kt][1], o[0][3] * ic[kt][1]), M::pack(o[1][0] * ic[kt][0], o[1][1] * ic[kt][0]),
+                    M::pack(o[1][2] * ic[kt][1], o[1][3] * ic[kt][1]));
           }
-          // alpha_R rows (k, j) over the alpha_L rows (both warps have formed their scores)
-          stsm_x4(s0 + swz(rs(16 * kt + (lane & 7) + 8 * ((lane >> 3) & 1), jj), 2 * vp + (lane >> 4)),
-                  Mma<T>::pack(o[0][0] * ic0, o[0][1] * ic0), Mma<T>::pack(o[0][2] * ic1, o[0][3] * ic1),
-                  Mma<T>::pack(o[1][0] * ic0, o[1][1] * ic0), Mma<T>::pack(o[1][2] * ic1, o[1][3] * ic1));
         }
       }
     }
-    MA_STAMP();
-    __syncthreads();
-    MA_STAMP();
+    if (!last) __syncthreads();
   }
-#ifdef MA_JSPLIT_TRACE
-  if (blockIdx.x == 0 && blockIdx.y == 0 && lane == 0) {
-    long long* out = reinterpret_cast<long long*>(Y) + 16384 + warp * 16;   // probe builds only
-    for (int i = 0; i < n_st; ++i) out[i] = stamps[i] - stamps[0];
-  }
-#endif
-#undef MA_STAMP
 }
 
 inline bool supported(int N, int d, int b, int m, int dtype, int BH) {
@@ -498,7 +556,7 @@ int launch(const void* Q, const void* K, const void* V, void* Y, int BH, int T, 
 #ifdef MA_TU_FUSED_JSPLIT
 struct Maps {
   const void *q = nullptr, *k = nullptr, *v = nullptr;
-  int BH = 0, dtype = 0, dev = -1, H = 0;
+  int BH = 0, dtype = 0, dev = -1, H = 0, pj = 0;
   CUtensorMap tmQ, tmK, tmV;
 };
 inline bool make_map(CUtensorMap* tm, int dtype, const void* base, uint64_t rows, uint32_t box_rows, int H) {
@@ -516,23 +574,19 @@ inline bool make_map(CUtensorMap* tm, int dtype, const void* base, uint64_t rows
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <typename TIn>
-inline int launch_t(const Maps& mp, void* Y, int BH, int T, float scale, int* status, cudaStream_t st,
-                    int dev, int H) {
-  auto kern = monarch_jsplit32<TIn>;
-  static bool prepared[64] = {};
-  if (!prepared[dev]) {
-    if (cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess)
-      return 7;
-    prepared[dev] = true;
-  }
+template <typename TIn, int PJ, int W>
+inline int launch_t(const Maps& mp, void* Y, int BH, int T, float scale, int* status, cudaStream_t st, int H) {
+  auto kern = monarch_jsplit32<TIn, PJ, W>;
+  using L = Lay<PJ, W>;
+  static warpmma::SmemOptIn opt_in;
+  if (!opt_in.done((const void*)kern, L::kSmem)) return 7;
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kB / kPJ, BH);     // the four CTAs of a head are neighbours: they share K and V in L2
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kSmem;
+  cfg.gridDim = dim3(kB / PJ, BH);      // the CTAs of a head are neighbours: they share K and V in L2
+  cfg.blockDim = dim3(L::kThreads);
+  cfg.dynamicSmemBytes = L::kSmem;
   cfg.stream = st;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
@@ -543,28 +597,34 @@ int launch(const void* Q, const void* K, const void* V, void* Y, int BH, int T, 
            int* status, cudaStream_t st, int H) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 7;
+  // As long as one wave holds four CTAs a head, two warps share a position: 13.5 us against 19.0 (T = 2).
+  // Beyond that a K fragment used for two tiles of positions wins: 48 heads 20.6 against 26.9 us, 80 heads
+  // (three waves against two) 38.2 against 38.6, 192 heads 58.1 against 76.1.
+  const int pj = BH * (kB / 8) <= 148 ? 8 : 16;
   // the tensor maps of the last few (Q, K, V) triples are kept: encoding three maps costs more host
   // time than the launch itself
-  static thread_local Maps cache[4];
+  static thread_local Maps cache[8];
   static thread_local int next = 0;
   const Maps* mp = nullptr;
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 8; ++i)
     if (cache[i].q == Q && cache[i].k == K && cache[i].v == V && cache[i].BH == BH && cache[i].dtype == dtype &&
-        cache[i].dev == dev && cache[i].H == H)
+        cache[i].dev == dev && cache[i].H == H && cache[i].pj == pj)
       mp = &cache[i];
   if (!mp) {
     Maps& m = cache[next];
-    next = (next + 1) % 4;
+    next = (next + 1) % 8;
     m.dev = -1;
     const uint64_t rows = (uint64_t)BH * kN;
-    if (!make_map(&m.tmQ, dtype, Q, rows, kPJ, H) || !make_map(&m.tmK, dtype, K, rows, kB, H) ||
+    if (!make_map(&m.tmQ, dtype, Q, rows, pj, H) || !make_map(&m.tmK, dtype, K, rows, kB, H) ||
         !make_map(&m.tmV, dtype, V, rows, kB, H))
       return 7;
-    m.q = Q; m.k = K; m.v = V; m.BH = BH; m.dtype = dtype; m.dev = dev; m.H = H;
+    m.q = Q; m.k = K; m.v = V; m.BH = BH; m.dtype = dtype; m.dev = dev; m.H = H; m.pj = pj;
     mp = &m;
   }
-  if (dtype == 1) return launch_t<__half>(*mp, Y, BH, T, scale, status, st, dev, H);
-  return launch_t<__nv_bfloat16>(*mp, Y, BH, T, scale, status, st, dev, H);
+  if (dtype == 1)
+    return pj == 8 ? launch_t<__half, 8, 2>(*mp, Y, BH, T, scale, status, st, H) : launch_t<__half, 16, 1>(*mp, Y, BH, T, scale, status, st, H);
+  return pj == 8 ? launch_t<__nv_bfloat16, 8, 2>(*mp, Y, BH, T, scale, status, st, H)
+                 : launch_t<__nv_bfloat16, 16, 1>(*mp, Y, BH, T, scale, status, st, H);
 }
 #endif  // MA_TU_FUSED_JSPLIT
 

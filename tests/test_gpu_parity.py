@@ -879,6 +879,22 @@ def test_position_split_kernel_matches_oracle(T, dtype, batch, heads, s):
     assert binding.monarch_attn_last_launch_count() == 1
 
 
+@pytest.mark.parametrize("BH", [37, 38, 75])      # the last one with four CTAs a head, the first with two, two waves
+@pytest.mark.parametrize("T,dtype,bshd", [(1, "bf16", False), (2, "f16", False), (3, "bf16", True)])
+def test_position_split_kernel_agrees_in_both_splits(T, dtype, bshd, BH):
+    """The two splits of a head over CTAs, every head against the fp32 kernels on the same values."""
+    Q, K, V = (torch.from_numpy(x).cuda() for x in wl.make_qkv(1, BH, 1024, 64, dtype, 16, 1.0 if T < 3 else 0.5, seed=BH + T))
+    x16 = [x.to(binding.torch_dtype(dtype)) for x in (Q, K, V)]
+    if bshd:
+        Y = binding.monarch_attn_fwd_bshd(*(x.transpose(1, 2).contiguous() for x in x16), 32, T,
+                                          path=binding.MA_PATH_FUSED_JSPLIT).transpose(1, 2)
+    else:
+        Y = binding.monarch_attn_fwd_ex(*x16, 32, T, path=binding.MA_PATH_FUSED_JSPLIT)
+    ref = binding.monarch_attn_fwd_ex(Q, K, V, 32, T, path=binding.MA_PATH_GENERIC)
+    err = ((Y.float() - ref).flatten(2).norm(dim=2) / ref.flatten(2).norm(dim=2)).max()
+    assert float(err) <= (3e-3 if dtype == "f16" else 1e-2), float(err)
+
+
 def test_position_split_kernel_is_the_default_for_its_shape_and_nothing_else():
     Q, K, V = wl.make_qkv(1, 6, 1024, 64, "bf16", 16, 1.0, seed=11)
     Qd, Kd, Vd = (binding.to_device(x, "bf16") for x in (Q, K, V))
