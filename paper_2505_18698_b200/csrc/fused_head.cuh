@@ -18,9 +18,11 @@
 // other in place in a state tile.  Arithmetic is f16 whatever the input type (see fused_small.cuh).
 //
 // Measured (B200, us per call, against the general per-head kernel): 768 heads of 256 = 16 x 16, one
-// round 25.6 / 27.7 (60 % of the copy bandwidth); 768 of 210 = 15 x 14, two rounds 42.4 / 47.7; 384 of
-// lengths up to 384 = 16 x 24 24.3 / 28.9; 720 of 396 = 22 x 18 59 / 97; 24 of 210 5.3 / 7.  What is left is
-// instruction issue and shared-memory latency at four warps per scheduler (41 % of the slots issue).
+// round 25.2 / 27.7 (61 % of the copy bandwidth); 768 of 210 = 15 x 14, two rounds 41.5 / 47.7; 384 of
+// lengths up to 384 = 16 x 24 23.4 / 28.9; 720 of 396 = 22 x 18 64 / 97; 24 of 210 5 / 7.  Row and column
+// reductions that halve the values a lane carries, with one division a lane, took 3 % (16 x 16) to 11 %
+// (10 x 24, two rounds) off.  What is left is instruction issue and shared-memory latency at four warps
+// per scheduler, and the last of six turns of heads, which few SMs take.
 #pragma once
 #include <cuda.h>
 
@@ -42,7 +44,7 @@ using warpmma::ldsm_x4_trans;
 using warpmma::lg2;
 using warpmma::movm_trans;
 using warpmma::quad_max;
-using warpmma::quad_sum;
+using warpmma::scatter_reduce;
 
 constexpr int kMaxThreads = 512, kMaxSmem = 227 * 1024, kMaxBlocks = 32;
 constexpr float kMasked = -3.0e38f;      // finite, and far below any score
@@ -207,7 +209,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
         const int r0 = k * bp;
         const int lim = min(b, n_valid - k * b);             // keys of this block that count
         uint32_t pa[RB][RB][4];                              // unnormalised weights: the largest is exactly 1
-        float inv[RB][2];
+        float inv[RB][2], off[2 * RB], red[4 * RB];          // red: sum of the weights, sum of weight times score
         {
           uint32_t kb[NB][4][2];
           load_b<NB>(kb, sK, lane, [&](int i) { return r0 + min(i, b - 1); });
@@ -244,27 +246,40 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
 #pragma unroll
               for (int nt = 0; nt < NB; ++nt) mx = fmaxf(mx, fmaxf(s[nt][2 * hh], s[nt][2 * hh + 1]));
               mx = quad_max(mx);
-              const float off = -mx * fl;
+              off[2 * rt + hh] = -mx * fl;
               float sum = 0.f, sz = 0.f;
 #pragma unroll
               for (int nt = 0; nt < NB; ++nt)
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
                   const float x = s[nt][2 * hh + e];
-                  const float p = ex2(fmaf(x, fl, off));
+                  const float p = ex2(fmaf(x, fl, off[2 * rt + hh]));
                   s[nt][2 * hh + e] = p;
                   sum += p;
                   sz = fmaf(p, x, sz);               // 0 times a finite number where masked (0 log 0 = 0)
                 }
-              sum = quad_sum(sum);
-              sz = quad_sum(sz);
-              inv[rt][hh] = 1.f / sum;
-              // -c_L log2 e = log2 sum + max - sum R z (Eq. 10), the addend of the L logits
-              const int j = 16 * rt + g + 8 * hh;
-              if (t == 0 && j < b) sCL[j * NM * 8 + k] = lg2(sum) - off - fl * (sz * inv[rt][hh]);
+              red[2 * (2 * rt + hh)] = sum;
+              red[2 * (2 * rt + hh) + 1] = sz;
             }
             pack_a<NB>(pa[rt], s);
           }
+          // a lane ends up with both sums of row q = t (two row tiles), or with one of them: one division a
+          // lane, the reciprocals then go to the row's four lanes
+          const float r = scatter_reduce<4 * RB, 2, 1>(red, lane, warpmma::Add());
+          const float ri = 1.f / r;
+          const int q = RB == 2 ? t : t >> 1, j = 16 * (q >> 1) + g + 8 * (q & 1);
+#pragma unroll
+          for (int i = 0; i < 2 * RB; ++i) inv[i >> 1][i & 1] = __shfl_sync(0xffffffffu, ri, (lane & ~3) + i * (2 / RB));
+          float so = r, sz = red[1], io = ri, mo = off[0];
+          if (RB == 1) {
+            sz = r;
+            so = __shfl_xor_sync(0xffffffffu, r, 1);
+            io = __shfl_xor_sync(0xffffffffu, ri, 1);
+          }
+#pragma unroll
+          for (int i = 1; i < 2 * RB; ++i) mo = q == i ? off[i] : mo;
+          // -c_L log2 e = log2 sum + max - sum R z (Eq. 10), the addend of the L logits
+          if ((RB == 2 || (t & 1)) && j < b) sCL[j * NM * 8 + k] = lg2(so) - mo - fl * (sz * io);
         }
         __syncwarp();
         // second products, 16 columns at a time; a warp alone reads and writes the rows of its block
@@ -318,7 +333,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
           c[nt][1] = 8 * nt + 2 * t + 1 < m ? v.y : kMasked;
         }
         uint32_t pa[RM][RM][4];                              // weights, rows l (final, unnormalised)
-        float inv[RM][2];
+        float inv[RM][2], red[2 * RM], mxs[2 * RM];
         float w[MULTI ? RM : 1][MULTI ? NM : 1][4];          // normalised weights (non-final)
         {
           uint32_t kb[NM][4][2];
@@ -359,20 +374,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
                   s[nt][2 * hh + e] = p;
                   sum += p;
                 }
-              sum = quad_sum(sum);
-              inv[rt][hh] = 1.f / sum;
-              const int l = 16 * rt + g + 8 * hh;
-              // log-sum-exp of row b l + j of the final L half-step: summed over a head's rows it is the
-              // objective (Eq. 6) at the returned matrix
-              if (last && P.lse != nullptr && t == 0 && l < m) P.lse[(size_t)h * P.N + (size_t)l * b + j] = (mx + lg2(sum)) * kLn2;
-              if (MULTI && !last) {
-                const float on = l < m ? inv[rt][hh] : 0.f;      // (rows past the last block: not in sums over rows)
-#pragma unroll
-                for (int nt = 0; nt < NM; ++nt) {
-                  s[nt][2 * hh] *= on;
-                  s[nt][2 * hh + 1] *= on;
-                }
-              }
+              red[2 * rt + hh] = sum;
+              mxs[2 * rt + hh] = mx;
             }
             if (last) {
               pack_a<NM>(pa[rt], s);
@@ -382,6 +385,19 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
 #pragma unroll
                 for (int e = 0; e < 4; ++e) w[MULTI ? rt : 0][MULTI ? nt : 0][e] = s[nt][e];
             }
+          }
+          const float r = scatter_reduce<2 * RM, 2, 1>(red, lane, warpmma::Add());     // of row q
+          const float ri = 1.f / r;
+#pragma unroll
+          for (int i = 0; i < 2 * RM; ++i) inv[i >> 1][i & 1] = __shfl_sync(0xffffffffu, ri, (lane & ~3) + i * (2 / RM));
+          // log-sum-exp of row b l + j of the final L half-step: summed over a head's rows it is the
+          // objective (Eq. 6) at the returned matrix
+          if (last && P.lse != nullptr) {
+            const int q = RM == 2 ? t : t >> 1, l = 16 * (q >> 1) + g + 8 * (q & 1);
+            float mx = mxs[0];
+#pragma unroll
+            for (int i = 1; i < 2 * RM; ++i) mx = q == i ? mxs[i] : mx;
+            if ((RM == 2 || !(t & 1)) && l < m) P.lse[(size_t)h * P.N + (size_t)l * b + j] = (mx + lg2(r)) * kLn2;
           }
         }
         __syncwarp();
@@ -424,20 +440,32 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
           // g_k = 2^-(exponent of its largest weight) first (the quotient is invariant), which keeps its
           // significant weights in the normal f16 range however small c_R is; c_R comes out of the same
           // MMAs against a B fragment of ones, i.e. over the weights as rounded.
+          constexpr int kCols = NM == 2 ? 4 : 8, kColStep = 32 / kCols;     // columns 8 (i / 2) + 2 t + i % 2 by i
+          float cms[kCols];
+#pragma unroll
+          for (int i = 0; i < kCols; ++i) cms[i] = 0.f;
+#pragma unroll
+          for (int rt = 0; rt < RM; ++rt)
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) {
+              // (rows past the last block: not in sums over rows)
+              const float on = 16 * rt + g + 8 * hh < m ? inv[rt][hh] : 0.f;
+#pragma unroll
+              for (int nt = 0; nt < NM; ++nt)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                  w[rt][nt][2 * hh + e] *= on;
+                  cms[2 * nt + e] = fmaxf(cms[2 * nt + e], w[rt][nt][2 * hh + e]);
+                }
+            }
+          const float cm = scatter_reduce<kCols, 16, 4>(cms, lane, warpmma::Max());
+          const float gl = __uint_as_float((253u << 23) - (__float_as_uint(cm) & 0x7f800000u));
           uint32_t tp[RM][2][NM];
 #pragma unroll
           for (int nt = 0; nt < NM; ++nt) {
             float gk[2];
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              float cm = 0.f;
-#pragma unroll
-              for (int rt = 0; rt < RM; ++rt) cm = fmaxf(cm, fmaxf(w[rt][nt][e], w[rt][nt][2 + e]));
-              cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, 4));
-              cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, 8));
-              cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, 16));
-              gk[e] = __uint_as_float((253u << 23) - (__float_as_uint(cm) & 0x7f800000u));
-            }
+            for (int e = 0; e < 2; ++e) gk[e] = __shfl_sync(0xffffffffu, gl, (2 * nt + e) * kColStep + t);
 #pragma unroll
             for (int rt = 0; rt < RM; ++rt)
 #pragma unroll
@@ -445,19 +473,26 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
                 tp[rt][hh][nt] = movm_trans(M::pack(w[rt][nt][2 * hh] * gk[0], w[rt][nt][2 * hh + 1] * gk[1]));
           }
           const uint32_t ones[2] = {0x3C003C00u, 0x3C003C00u};
+          uint32_t pk[RM][RM][4];    // A[k][l]: rows k = 16 kq .., contraction over l = 16 ls ..
+          float c1 = 0.f;
 #pragma unroll
           for (int kq = 0; kq < RM; ++kq) {
-            uint32_t pk[RM][4];      // A[k][l]: rows k = 16 kq .., contraction over l = 16 ls ..
             float cr[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
             for (int ls = 0; ls < RM; ++ls) {
-              pk[ls][0] = tp[ls][0][2 * kq];
-              pk[ls][1] = 2 * kq + 1 < NM ? tp[ls][0][(2 * kq + 1) % NM] : 0u;
-              pk[ls][2] = tp[ls][1][2 * kq];
-              pk[ls][3] = 2 * kq + 1 < NM ? tp[ls][1][(2 * kq + 1) % NM] : 0u;
-              M::run(cr, pk[ls], ones);
+              pk[kq][ls][0] = tp[ls][0][2 * kq];
+              pk[kq][ls][1] = 2 * kq + 1 < NM ? tp[ls][0][(2 * kq + 1) % NM] : 0u;
+              pk[kq][ls][2] = tp[ls][1][2 * kq];
+              pk[kq][ls][3] = 2 * kq + 1 < NM ? tp[ls][1][(2 * kq + 1) % NM] : 0u;
+              M::run(cr, pk[kq][ls], ones);
             }
-            const float i0 = cr[0] > 1e-30f ? 1.f / cr[0] : 0.f, i1 = cr[2] > 1e-30f ? 1.f / cr[2] : 0.f;
+            if (t == 2 * kq) c1 = cr[0];      // a division a lane
+            if (t == 2 * kq + 1) c1 = cr[2];
+          }
+          c1 = c1 > 1e-30f ? 1.f / c1 : 0.f;
+#pragma unroll
+          for (int kq = 0; kq < RM; ++kq) {
+            const float i0 = __shfl_sync(0xffffffffu, c1, (lane & ~3) + 2 * kq), i1 = __shfl_sync(0xffffffffu, c1, (lane & ~3) + 2 * kq + 1);
 #pragma unroll
             for (int np = 0; np < 4; ++np) {
               float o[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
@@ -465,8 +500,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
               for (int ls = 0; ls < RM; ++ls) {
                 uint32_t bq[4];      // B[l][v] = Q(l,j)[v], read transposed
                 ldsm_x4_trans(bq, sQ + (kt[ls] ^ (np << 5)));
-                M::run(o[0], pk[ls], bq);
-                M::run(o[1], pk[ls], bq + 2);
+                M::run(o[0], pk[kq][ls], bq);
+                M::run(o[1], pk[kq][ls], bq + 2);
               }
               put(16 * kq + a_row < m ? sS + (st[kq] ^ (np << 5)) : dump, o, i0, i1);
             }

@@ -60,6 +60,7 @@ using warpmma::ldsm_x4_trans;
 using warpmma::lg2;
 using warpmma::movm_trans;
 using warpmma::quad_max;
+using warpmma::scatter_reduce;
 
 constexpr int kN = 1024, kB = 32, kM = 32, kD = 64;
 constexpr int kSlot = kB * 128;                          // a block of K or V
@@ -85,29 +86,6 @@ __device__ __forceinline__ float col_max(float v) {   // over the 8 row groups (
   v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 8));
   return fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 16));
 }
-// Reduction of NV values over the lanes that differ in the three bits (or two, LO = 1) of `lane` below
-// 2 HI: each step halves the values a lane carries as long as there is more than one, so that with eight
-// values and three bits lane bits HI..LO are the index of the value the lane ends up with.
-template <int NV, int HI, int LO, typename Op>
-__device__ __forceinline__ float scatter_reduce(float* v, int lane, Op op) {
-  int n = NV / 2;
-#pragma unroll
-  for (int m = HI; m >= LO; m >>= 1, n >>= 1) {
-    if (n >= 1) {
-#pragma unroll
-      for (int i = 0; i < NV / 2; ++i)
-        if (i < n) {
-          const float keep = lane & m ? v[i + n] : v[i], send = lane & m ? v[i] : v[i + n];
-          v[i] = op(keep, __shfl_xor_sync(0xffffffffu, send, m));
-        }
-    } else {
-      v[0] = op(v[0], __shfl_xor_sync(0xffffffffu, v[0], m));
-    }
-  }
-  return v[0];
-}
-struct Add { __device__ __forceinline__ float operator()(float a, float b) const { return a + b; } };
-struct Max { __device__ __forceinline__ float operator()(float a, float b) const { return fmaxf(a, b); } };
 __device__ __forceinline__ void stsm_x4(uint32_t saddr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
   asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(saddr), "r"(r0),
                "r"(r1), "r"(r2), "r"(r3)
@@ -259,7 +237,7 @@ monarch_jsplit32(const __grid_constant__ CUtensorMap tmQ,    // Q as rows of d, 
         // a lane ends up with sum or sum p s (lane bit kSz) of one column: one division and one logarithm
         // a lane, the reciprocals then go to all lanes
         constexpr int kSz = 8 / NT, kCol = NT == 2 ? 3 : 4;
-        const float r = scatter_reduce<4 * NT, 16, 4>(red, lane, Add());
+        const float r = scatter_reduce<4 * NT, 16, 4>(red, lane, warpmma::Add());
         const float ri = 1.f / r;
 #pragma unroll
         for (int q = 0; q < 2 * NT; ++q) inv[q >> 1][q & 1] = __shfl_sync(0xffffffffu, ri, (q << kCol) + t);
@@ -401,7 +379,7 @@ monarch_jsplit32(const __grid_constant__ CUtensorMap tmQ,    // Q as rows of d, 
             }
           rsum[2 * lt + hh] = sum;
         }
-      const float ri = 1.f / scatter_reduce<2 * LT, 2, 1>(rsum, lane, Add());
+      const float ri = 1.f / scatter_reduce<2 * LT, 2, 1>(rsum, lane, warpmma::Add());
 #pragma unroll
       for (int i = 0; i < 2 * LT; ++i) inv[i >> 1][i & 1] = __shfl_sync(0xffffffffu, ri, (lane & ~3) + i * (2 / LT));
       __syncwarp();
@@ -470,7 +448,7 @@ monarch_jsplit32(const __grid_constant__ CUtensorMap tmQ,    // Q as rows of d, 
                 cms[2 * nt + e] = fmaxf(cms[2 * nt + e], s[lt][nt][2 * hh + e]);
               }
           }
-        float cm = scatter_reduce<8, 16, 4>(cms, lane, Max());     // of column 8 (g / 2) + 2 t + g % 2
+        float cm = scatter_reduce<8, 16, 4>(cms, lane, warpmma::Max());     // of column 8 (g / 2) + 2 t + g % 2
         if constexpr (W == 2) {
           float* xm = reinterpret_cast<float*>(smem + L::X + jj * 256);
           xm[2 * l0 + lane] = cm;

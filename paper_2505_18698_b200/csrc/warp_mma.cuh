@@ -111,6 +111,30 @@ __device__ __forceinline__ float col_sum(float v) {   // over the 8 row groups (
   return v + __shfl_xor_sync(0xffffffffu, v, 16);
 }
 
+// Reduction of NV values (a power of two) over the lanes that differ in bits HI .. LO of `lane`.  Each step
+// halves the values a lane carries as long as there is more than one: lane bits HI, HI / 2, .. are the
+// leading bits of the index of the values it ends up with, NV / (lanes) of them, or one, in v[0], ..
+template <int NV, int HI, int LO, typename Op>
+__device__ __forceinline__ float scatter_reduce(float* v, int lane, Op op) {
+  int n = NV / 2;
+#pragma unroll
+  for (int m = HI; m >= LO; m >>= 1, n >>= 1) {
+    if (n >= 1) {
+#pragma unroll
+      for (int i = 0; i < NV / 2; ++i)
+        if (i < n) {
+          const float keep = lane & m ? v[i + n] : v[i], send = lane & m ? v[i] : v[i + n];
+          v[i] = op(keep, __shfl_xor_sync(0xffffffffu, send, m));
+        }
+    } else {
+      v[0] = op(v[0], __shfl_xor_sync(0xffffffffu, v[0], m));
+    }
+  }
+  return v[0];
+}
+struct Add { __device__ __forceinline__ float operator()(float a, float b) const { return a + b; } };
+struct Max { __device__ __forceinline__ float operator()(float a, float b) const { return fmaxf(a, b); } };
+
 __device__ __forceinline__ uint4 to_f16x8(uint4 v, const __half*) { return v; }
 __device__ __forceinline__ uint4 to_f16x8(uint4 v, const __nv_bfloat16*) {
   uint32_t* w = reinterpret_cast<uint32_t*>(&v);
