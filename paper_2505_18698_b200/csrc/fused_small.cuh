@@ -34,7 +34,6 @@ namespace ma {
 namespace fsmall {
 
 using warpmma::Mma;
-using warpmma::col_sum;
 using warpmma::ex2;
 using warpmma::kLn2;
 using warpmma::kLog2e;
@@ -44,7 +43,7 @@ using warpmma::ldsm_x4_trans;
 using warpmma::lg2;
 using warpmma::movm_trans;
 using warpmma::quad_max;
-using warpmma::quad_sum;
+using warpmma::scatter_reduce;
 
 constexpr int kThreads = 256, kWarps = 8, kRowBytes = 128, kMaxSmem = 227 * 1024;
 // where stmatrix rows past the end of a block go: eight rows of 16 bytes (nothing reads them)
@@ -109,13 +108,11 @@ inline size_t smem_bytes(int N, int T, int b = 16, int ks = 4, bool hilo = false
          (ks == 4 ? 1024 : 128);
 }
 
-// BP: b rounded up to 16, 32, 48 or 64; MP: m rounded up to 16 or 32.  EXACT: b = BP, m = MP, d = 64
-// and no mask, known at compile time: every clamp, mask and bounds predicate below folds away and
-// the index products become shifts (the instruction stream, not a pipe, bounds this kernel).
+// BP: b rounded up to 16, 32, 48 or 64; MP: m rounded up to 16 or 32.
 // HILO: alpha_L, alpha_R and the weights that feed them are hi + lo pairs of f16 (two more tiles): what
 // three or more rounds on peaky logits need (plain 16-bit states, fed back round after round, lose
 // 1e-2 on about one head in 300 at T = 3).
-template <typename TIn, int BP, int MP, bool EXACT = false, int KS = 4, bool HILO = false>
+template <typename TIn, int BP, int MP, int KS = 4, bool HILO = false>
 __global__ void __launch_bounds__((HILO || (KS == 4 && BP <= 32 && (BP == 16 || MP == 16))) ? 2 * kThreads : kThreads, 1)
 monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const TIn* __restrict__ V,
                     TIn* __restrict__ Y, int N, int d, int b, int m, int T_steps, float scale,
@@ -130,15 +127,8 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
   // m = ceil(length / b) blocks and the appendix's mask in the last of them.  Rows are addressed
   // by (block, position) with the block size b only, so running the smaller problem is a matter
   // of the block count; the rows of Y past it are zeroed, the rows of Q, K, V past it never read.
-  if (EXACT) {
-    b = BP;
-    m = MP;
-    N = BP * MP;
-    d = 64;
-    n_valid = 0x7fffffff;
-  }
   const int m_alloc = m;
-  if (!EXACT && seq_len != nullptr) {
+  if (seq_len != nullptr) {
     n_valid = min(max(seq_len[blockIdx.x / heads], 1), N);
     m = (n_valid + b - 1) / b;
   }
@@ -281,16 +271,16 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
             }
           }
           // rows j = j0 + g (c0, c1) and j0 + g + 8 (c2, c3); columns i = 8 nt + 2t, +1
+          float red[4], mxs[2];      // sum of the weights and of weight times logit, by row
 #pragma unroll
           for (int hh = 0; hh < 2; ++hh) {
-            const int j = j0 + g + 8 * hh;
             float mx = -INFINITY;
 #pragma unroll
             for (int nt = 0; nt < BP / 8; ++nt)
 #pragma unroll
               for (int e = 0; e < 2; ++e) {
                 const int i = 8 * nt + 2 * t + e;
-                const bool valid = EXACT || (i < b && k * b + i < n_valid);
+                const bool valid = i < b && k * b + i < n_valid;
                 const float z = valid ? s[nt][2 * hh + e] * fl : -INFINITY;
                 s[nt][2 * hh + e] = z;
                 mx = fmaxf(mx, z);
@@ -307,11 +297,20 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
                 sum += p;
                 if (z > -INFINITY) sz = fmaf(p, z, sz);      // 0 log 0 = 0
               }
-            sum = quad_sum(sum);
-            sz = quad_sum(sz);
-            inv_s[rt][hh] = 1.f / sum;
-            // c_L = sum R log R (natural log): ln2 * (sum p z / sum - max - log2 sum)
-            if (t == 0 && j < b) sCL[k * b + j] = kLn2 * (sz * inv_s[rt][hh] - mx - lg2(sum));
+            red[2 * hh] = sum;
+            red[2 * hh + 1] = sz;
+            mxs[hh] = mx;
+          }
+          {
+            // lane t ends up with one sum (odd t: of weight times logit) of row half t / 2: one division a lane
+            const float r = scatter_reduce<4, 2, 1>(red, lane, warpmma::Add());
+            const float ri = 1.f / r;
+            inv_s[rt][0] = __shfl_sync(0xffffffffu, ri, lane & ~3);
+            inv_s[rt][1] = __shfl_sync(0xffffffffu, ri, (lane & ~3) + 2);
+            const float so = __shfl_xor_sync(0xffffffffu, r, 1), io = __shfl_xor_sync(0xffffffffu, ri, 1);
+            const int j = j0 + g + 4 * (t & 2);
+            // -c_L log2 e = max + log2 sum - sum R z, the addend of the L logits
+            if ((t & 1) && j < b) sCL[k * b + j] = (t & 2 ? mxs[1] : mxs[0]) + lg2(so) - r * io;
           }
 #pragma unroll
           for (int kk = 0; kk < BP / 16; ++kk) {
@@ -394,7 +393,7 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
         for (int nt = 0; nt < MP / 8; ++nt)
 #pragma unroll
           for (int e = 0; e < 2; ++e)
-            c[nt][e] = sCL[min(8 * nt + 2 * t + e, m - 1) * b + j] * kLog2e;
+            c[nt][e] = sCL[min(8 * nt + 2 * t + e, m - 1) * b + j];
         float pn[MP / 16][2][MP / 8][2];           // normalised weights [row tile][half][nt][e]
 #pragma unroll
         for (int rt = 0; rt < MP / 16; ++rt) {
@@ -434,7 +433,7 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
               }
             }
           }
-          float inv_s[2];
+          float inv_s[2], red[2], mxs[2];
 #pragma unroll
           for (int hh = 0; hh < 2; ++hh) {
             float mx = -INFINITY;
@@ -442,7 +441,7 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
             for (int nt = 0; nt < MP / 8; ++nt)
 #pragma unroll
               for (int e = 0; e < 2; ++e) {
-                const float z = (8 * nt + 2 * t + e < m) ? fmaf(s[nt][2 * hh + e], fl, -c[nt][e])
+                const float z = (8 * nt + 2 * t + e < m) ? fmaf(s[nt][2 * hh + e], fl, c[nt][e])
                                                          : -INFINITY;
                 s[nt][2 * hh + e] = z;
                 mx = fmaxf(mx, z);
@@ -457,12 +456,19 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
                 s[nt][2 * hh + e] = p;
                 sum += p;
               }
-            sum = quad_sum(sum);
-            inv_s[hh] = 1.f / sum;
+            red[hh] = sum;
+            mxs[hh] = mx;
+          }
+          {
+            const float r = scatter_reduce<2, 2, 1>(red, lane, warpmma::Add());      // of row half t / 2
+            const float ri = 1.f / r;
+            inv_s[0] = __shfl_sync(0xffffffffu, ri, lane & ~3);
+            inv_s[1] = __shfl_sync(0xffffffffu, ri, (lane & ~3) + 2);
             // log-sum-exp of row b l + j of the final L half-step: summed over a head's rows it is
             // the objective (Eq. 6) at the returned matrix
-            if (last && lse != nullptr && t == 0 && l0 + g + 8 * hh < m)
-              lse[(size_t)h_idx * N + (size_t)(l0 + g + 8 * hh) * b + j] = (mx + log2f(sum)) * kLn2;
+            const int l = l0 + g + 4 * (t & 2);
+            if (last && lse != nullptr && !(t & 1) && l < m)
+              lse[(size_t)h_idx * N + (size_t)l * b + j] = ((t & 2 ? mxs[1] : mxs[0]) + log2f(r)) * kLn2;
           }
           if (last) {
             // Y(l,j) = sum_k L[j,k,l] y(k,j)   (A = weights rows l, B = y rows (k,j) transposed)
@@ -530,20 +536,22 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
           // of the column's largest weight) keeps every column's significant weights in the normal
           // f16 range however small c_R is.
           uint32_t tp[MP / 16][2][MP / 8], tpl[HILO ? MP / 16 : 1][2][HILO ? MP / 8 : 1];
-          float cs[MP / 8][2];
+          constexpr int kCols = MP / 4, kColStep = 32 / kCols;      // columns k = 8 (i / 2) + 2 t + i % 2 by i
+          float cs[kCols], cms[kCols];
+#pragma unroll
+          for (int i = 0; i < kCols; ++i) {
+            cms[i] = 0.f;
+#pragma unroll
+            for (int rt = 0; rt < MP / 16; ++rt)
+              cms[i] = fmaxf(cms[i], fmaxf(pn[rt][0][i >> 1][i & 1], pn[rt][1][i >> 1][i & 1]));
+          }
+          const float cm = scatter_reduce<kCols, 16, 4>(cms, lane, warpmma::Max());
+          const float gl = cm > 0.f ? __uint_as_float((253u << 23) - (__float_as_uint(cm) & 0x7f800000u)) : 0.f;
 #pragma unroll
           for (int nt = 0; nt < MP / 8; ++nt) {
             float gk[2];
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              float cm = 0.f;
-#pragma unroll
-              for (int rt = 0; rt < MP / 16; ++rt) cm = fmaxf(cm, fmaxf(pn[rt][0][nt][e], pn[rt][1][nt][e]));
-              cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, 4));
-              cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, 8));
-              cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, 16));
-              gk[e] = cm > 0.f ? __uint_as_float((253u << 23) - (__float_as_uint(cm) & 0x7f800000u)) : 0.f;
-            }
+            for (int e = 0; e < 2; ++e) gk[e] = __shfl_sync(0xffffffffu, gl, (2 * nt + e) * kColStep + t);
             // column sums of the weights AS ROUNDED to 16 bit: numerator (the MMA below) and
             // denominator of the weighted mean must see the same weights
             float c0 = 0.f, c1 = 0.f;
@@ -564,21 +572,18 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
                 c0 += f.x;
                 c1 += f.y;
               }
-            cs[nt][0] = col_sum(c0);
-            cs[nt][1] = col_sum(c1);
+            cs[2 * nt] = c0;
+            cs[2 * nt + 1] = c1;
           }
+          const float cr = scatter_reduce<kCols, 16, 4>(cs, lane, warpmma::Add());
+          const float icl = cr > 1e-30f ? 1.f / cr : 0.f;
 #pragma unroll
           for (int kt = 0; kt < MP / 16; ++kt) {
             if (16 * kt >= m) continue;
-            // 1 / c_R of rows k = 16 kt + g and + 8: column k = 8 nt + 2 t' + e sits in lane t'
-            float ic[2];
+            float ic[2];      // 1 / c_R of rows k = 16 kt + g and + 8
 #pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-              const float v0 = __shfl_sync(0xffffffffu, cs[2 * kt + hh][0], g >> 1);
-              const float v1 = __shfl_sync(0xffffffffu, cs[2 * kt + hh][1], g >> 1);
-              const float cr = (g & 1) ? v1 : v0;
-              ic[hh] = cr > 1e-30f ? 1.f / cr : 0.f;
-            }
+            for (int hh = 0; hh < 2; ++hh)
+              ic[hh] = __shfl_sync(0xffffffffu, icl, (2 * (2 * kt + hh) + (g & 1)) * kColStep + (g >> 1));
             uint32_t pa[MP / 16][4], pal[HILO ? MP / 16 : 1][4];
 #pragma unroll
             for (int ls = 0; ls < MP / 16; ++ls) {
@@ -647,15 +652,16 @@ int launch(const void* Q, const void* K, const void* V, void* Y, int BH, int N, 
            const int* seq_len = nullptr, int heads = 1);
 
 #ifdef MA_TU_FUSED_SMALL
-template <typename TIn, int BP, int MP, bool EXACT = false, int KS = 4, bool HILO = false>
+template <typename TIn, int BP, int MP, int KS = 4, bool HILO = false>
 inline int launch_t(const void* Q, const void* K, const void* V, void* Y, int BH, int N, int d, int b,
                     int m, int T, float scale, int n_valid, int H, float* lse, cudaStream_t st,
                     const int* seq_len, int heads) {
-  auto kern = monarch_fused_small<TIn, BP, MP, EXACT, KS, HILO>;
+  auto kern = monarch_fused_small<TIn, BP, MP, KS, HILO>;
   // Two CTAs of 8 warps per SM where shared memory lets two fit, else one CTA of 16 warps (each warp then
   // owns at most one tile of a half-step of 16 blocks), for the instantiations compiled for 128 registers.
   // The hi + lo states leave room for one CTA, and where two fit a grid of one CTA per SM or fewer gains
-  // from 16 warps as well (128 heads of 256 = 16 x 16, d = 72, three rounds: 17.5 against 22.6 us).
+  // from 16 warps as well (128 heads of 256 = 16 x 16, d = 72, three rounds: 17.5 against 22.6 us; 17.1 with row and column
+  // sums spread over the lanes, one division a lane).
   const size_t smem = smem_bytes(N, T, b, KS, HILO);
   const bool wide = HILO || (KS == 4 && BP <= 32 && (BP == 16 || MP == 16));
   const bool one = 2 * (smem + 1024) > (size_t)228 * 1024 || (HILO && BH <= 148);
@@ -687,20 +693,14 @@ inline int launch_d(const void* Q, const void* K, const void* V, void* Y, int BH
                     const int* seq_len, int heads) {
 #define MA_FS_ARGS Q, K, V, Y, BH, N, d, b, m, T, scale, n_valid, H, lse, st, seq_len, heads
   if (supported_hilo(N, d, b, m, 1, T))   // three or more rounds: hi + lo states
-    return d <= 64 ? launch_t<TIn, 16, 16, false, 4, true>(MA_FS_ARGS) : launch_t<TIn, 16, 16, false, 5, true>(MA_FS_ARGS);
-  if (d == 64 && n_valid >= N && seq_len == nullptr) {   // exact fits, no mask
-    if (b == 16 && m == 16) return launch_t<TIn, 16, 16, true>(MA_FS_ARGS);
-    if (b == 32 && m == 32) return launch_t<TIn, 32, 32, true>(MA_FS_ARGS);
-    if (b == 16 && m == 32) return launch_t<TIn, 16, 32, true>(MA_FS_ARGS);
-    if (b == 32 && m == 16) return launch_t<TIn, 32, 16, true>(MA_FS_ARGS);
-  }
+    return d <= 64 ? launch_t<TIn, 16, 16, 4, true>(MA_FS_ARGS) : launch_t<TIn, 16, 16, 5, true>(MA_FS_ARGS);
   if (d > 80) {          // rows of up to 128 columns
-    if (b <= 16) return m <= 16 ? launch_t<TIn, 16, 16, false, 8>(MA_FS_ARGS) : launch_t<TIn, 16, 32, false, 8>(MA_FS_ARGS);
-    return m <= 16 ? launch_t<TIn, 32, 16, false, 8>(MA_FS_ARGS) : launch_t<TIn, 32, 32, false, 8>(MA_FS_ARGS);
+    if (b <= 16) return m <= 16 ? launch_t<TIn, 16, 16, 8>(MA_FS_ARGS) : launch_t<TIn, 16, 32, 8>(MA_FS_ARGS);
+    return m <= 16 ? launch_t<TIn, 32, 16, 8>(MA_FS_ARGS) : launch_t<TIn, 32, 32, 8>(MA_FS_ARGS);
   }
   if (d > 64) {          // rows of up to 80 columns (d = 72)
-    if (b <= 16) return m <= 16 ? launch_t<TIn, 16, 16, false, 5>(MA_FS_ARGS) : launch_t<TIn, 16, 32, false, 5>(MA_FS_ARGS);
-    return m <= 16 ? launch_t<TIn, 32, 16, false, 5>(MA_FS_ARGS) : launch_t<TIn, 32, 32, false, 5>(MA_FS_ARGS);
+    if (b <= 16) return m <= 16 ? launch_t<TIn, 16, 16, 5>(MA_FS_ARGS) : launch_t<TIn, 16, 32, 5>(MA_FS_ARGS);
+    return m <= 16 ? launch_t<TIn, 32, 16, 5>(MA_FS_ARGS) : launch_t<TIn, 32, 32, 5>(MA_FS_ARGS);
   }
   if (b > 48) return m <= 16 ? launch_t<TIn, 64, 16>(MA_FS_ARGS) : launch_t<TIn, 64, 32>(MA_FS_ARGS);
   if (b > 32) return m <= 16 ? launch_t<TIn, 48, 16>(MA_FS_ARGS) : launch_t<TIn, 48, 32>(MA_FS_ARGS);
