@@ -551,16 +551,22 @@ int monarch_attn_fwd_host(const void* Qh, const void* Kh, const void* Vh, void* 
   // Every copy costs 3-4 us beyond its bytes, and copies in slow down while others go back; the copies
   // and kernels of a chunk overlap the copies of the next.  Measured with 1, 2, 3, 4 and 6 chunks (us): 0.2 MB
   // a tensor 46, 52, 62, 75, 98; 2.4 MB 220, 227, 235, 249, 268; 9.4 MB 717, 661, 661, 664, 692; 20 MB 1521, 1388,
-  // 1345, 1346, 1354; 25 MB 1866, 1684, 1633, 1645, 1662.  The long sequences' kernels and the copy back
-  // they need weigh more: four.
+  // 1345, 1346, 1354; 25 MB 1866, 1684, 1633, 1645, 1662.  Without the direct
+  // writes: three.
   const size_t bytes = (size_t)p.BH * unit;
-  const int want = g_host_chunks > 0 ? g_host_chunks : (!direct ? 4 : (bytes < ((size_t)4 << 20) ? 1 : (bytes < ((size_t)14 << 20) ? 2 : 3)));
+  const int want = g_host_chunks > 0 ? g_host_chunks : (direct && bytes < ((size_t)4 << 20) ? 1 : (direct && bytes < ((size_t)14 << 20) ? 2 : 3));
   const int chunks = (unit % 16 == 0 && p.BH >= want) ? want : 1;
+  // Shares fall linearly where the last chunk's results have still to be copied back (4 x 4 x 4096: 645 us with
+  // four equal chunks, 627 with three falling ones; 16 x 16384 2240 and 2152); equal ones are as good or
+  // better where the kernel writes them.
+  auto first_unit = [&](int c) {
+    return (int)(direct ? (long long)p.BH * c / chunks : (long long)p.BH * c * (2 * chunks + 1 - c) / (chunks * (chunks + 1)));
+  };
   // one chunk: everything in order on the caller's stream
   cudaStream_t compute = chunks > 1 ? B.compute : st, back = chunks > 1 ? B.d2h : st;
   int launches = 0;
   for (int c = 0; c < chunks; ++c) {
-    const int u0 = (int)((long long)p.BH * c / chunks), u1 = (int)((long long)p.BH * (c + 1) / chunks);
+    const int u0 = first_unit(c), u1 = first_unit(c + 1);
     const size_t off = (size_t)u0 * unit, len = (size_t)(u1 - u0) * unit;
     if (cudaMemcpyAsync(s + off, (const char*)Qh + off, len, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(s + one + off, (const char*)Kh + off, len, cudaMemcpyHostToDevice, st) != cudaSuccess ||
