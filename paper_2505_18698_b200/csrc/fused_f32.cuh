@@ -19,8 +19,10 @@
 // conflict-free along a block (R) and across blocks (L).  alpha_R and alpha_L replace each other in place,
 // V is read once, from global memory (requested into L2 at the start), and y takes rows of K.
 //
-// Measured (B200, us per call, against one lane per output): 96 heads of 256 = 16 x 16, three rounds 48 /
-// 224; 96 of 384 = 16 x 24, one round 48 / 193; 12 of 256, two rounds 15 / 30; one head, one round 8.6 / 10.3.
+// Measured (B200, us per call, against one lane per output): 96 heads of 256 = 16 x 16, three rounds 44 /
+// 224; 96 of 384 = 16 x 24, one round 39 / 193; 12 of 256, two rounds 13.4 / 30; one head, one round 7.7 /
+// 10.3.  Index arithmetic without integer division, ragged reads out of the way (code 126 -> 41 KB and 140 ->
+// 64 KB: instruction fetch was the first stall) and weights stored normalised took 8 to 20 % off.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -32,7 +34,6 @@
 namespace ma {
 namespace ffused {
 
-using generic::io_off;
 using generic::ld_as_float;
 using generic::st_from_float;
 using tensor::ffma2;
@@ -40,7 +41,7 @@ using tensor::ffma2;
 constexpr int kThreads = 256, kMaxSmem = 227 * 1024;
 
 // Shared memory in 16-byte units: K [k][i], then for the CTA's JT positions Q and alpha_R / alpha_L
-// [k or l][jj], the weights of a half-step [row][column], and c_L, c_R, 1 / row sum per row.
+// [k or l][jj], the weights of a half-step [row][column], and c_L, c_R per row.
 struct Layout {
   int d4, pu, bu, ju, su;      // units of a row, row pitch, block pitch of K, of Q and alpha, pitch of a row of weights
   int Q, A, S, C, total;
@@ -56,21 +57,24 @@ __host__ __device__ inline Layout layout(int d, int b, int m, int JT) {
   y.A = y.Q + m * y.ju;
   y.S = y.A + m * y.ju;
   y.C = y.S + JT * m * y.su;
-  y.total = y.C + 3 * ((JT * m + 3) / 4);
+  y.total = y.C + 2 * ((JT * m + 3) / 4);
   return y;
 }
 inline size_t smem_bytes(int d, int b, int m, int JT) { return (size_t)layout(d, b, m, JT).total * 16; }
 
 // Positions per CTA: the number for which the fullest SM has the least to do, a CTA costing its
 // positions and about three more for its copy of K and its start (measured: 1 to 3 agree on most shapes;
-// 32 heads of 384 = 16 x 24, two rounds: 42 us with 1, 33 with 3).
+// 32 heads of 384 = 16 x 24, two rounds: 42 us with 1, 33 with 3); a third more where no second CTA fits
+// beside it (96 heads of 256 = 16 x 16, three rounds: 43 us with 4 positions, 64 with the 16 that just fit;
+// 36 heads of 238 = 14 x 17, two rounds: 22 with 4, 27.5 with 8).
 inline int positions_per_cta(int d, int b, int m, int BH, int num_sms) {
   int best = 0;
   long long least = 0;
   for (int jt = 1; jt <= b; jt = jt < 4 ? 2 * jt : jt + 4) {
     if (smem_bytes(d, b, m, jt) > (size_t)kMaxSmem) break;
     const long long ctas = (long long)BH * ((b + jt - 1) / jt);
-    const long long cost = (ctas + num_sms - 1) / num_sms * (jt + 3);
+    const bool two = 2 * (smem_bytes(d, b, m, jt) + 1024) <= (size_t)228 * 1024;
+    const long long cost = (ctas + num_sms - 1) / num_sms * (jt + 3) * (two ? 3 : 4);
     if (best == 0 || cost < least) {
       best = jt;
       least = cost;
@@ -103,30 +107,34 @@ __device__ __forceinline__ void dot4(float2& acc, const float4& a, const float4&
   acc = ffma2(make_float2(a.z, a.w), make_float2(x.z, x.w), acc);
 }
 __device__ __forceinline__ float elem(const float4& v, int i) { return i == 0 ? v.x : (i == 1 ? v.y : (i == 2 ? v.z : v.w)); }
-// Four elements from column `col` of a row of d (zeros past its end).
-__device__ __forceinline__ float4 load4(const float* p, int col, int d) {
-  if (d % 4 == 0) return *reinterpret_cast<const float4*>(p + col);
-  return make_float4(p[col], col + 1 < d ? p[col + 1] : 0.f, col + 2 < d ? p[col + 2] : 0.f, col + 3 < d ? p[col + 3] : 0.f);
-}
+// Four elements from column `col` of a row of d (zeros past its end).  Rows that are no whole number of
+// 16-byte units are read element by element, out of line.
 template <typename TIn>
+__device__ __noinline__ float4 load4_ragged(const TIn* p, int left) {
+  return make_float4(ld_as_float(p), left > 1 ? ld_as_float(p + 1) : 0.f, left > 2 ? ld_as_float(p + 2) : 0.f,
+                     left > 3 ? ld_as_float(p + 3) : 0.f);
+}
+template <bool WHOLE, typename TIn>
 __device__ __forceinline__ float4 load4(const TIn* p, int col, int d) {
-  if (d % 4 == 0) {
+  if (!WHOLE && d % 4 != 0) return load4_ragged(p + col, d - col);
+  if constexpr (sizeof(TIn) == 4) {
+    return *reinterpret_cast<const float4*>(p + col);
+  } else {
     const uint2 u = *reinterpret_cast<const uint2*>(p + col);
     const TIn* e = reinterpret_cast<const TIn*>(&u);
     return make_float4(ld_as_float(e), ld_as_float(e + 1), ld_as_float(e + 2), ld_as_float(e + 3));
   }
-  return make_float4(ld_as_float(p + col), col + 1 < d ? ld_as_float(p + col + 1) : 0.f,
-                     col + 2 < d ? ld_as_float(p + col + 2) : 0.f, col + 3 < d ? ld_as_float(p + col + 3) : 0.f);
 }
 template <typename TIn>
-__device__ __forceinline__ void store4(TIn* p, int col, int d, const float4& v) {
-  if (d % 4 == 0 && sizeof(TIn) == 4) {
-    *reinterpret_cast<float4*>(p + col) = v;
-    return;
-  }
+__device__ __noinline__ void store4_ragged(TIn* p, int left, float4 v) {
 #pragma unroll
   for (int c = 0; c < 4; ++c)
-    if (col + c < d) st_from_float(p + col + c, elem(v, c));
+    if (c < left) st_from_float(p + c, elem(v, c));
+}
+template <bool WHOLE, typename TIn>
+__device__ __forceinline__ void store4(TIn* p, int col, int d, const float4& v) {
+  if (WHOLE || (d % 4 == 0 && sizeof(TIn) == 4)) *reinterpret_cast<float4*>(p + col) = v;
+  else store4_ragged(p + col, d - col, v);
 }
 // Over the eight lanes that share a row.
 __device__ __forceinline__ float row_max(float v) {
@@ -144,8 +152,8 @@ __device__ __forceinline__ int divide(int x, float inv) { return __float2int_rd(
 
 // Scores and softmax of R rows against up to 8 TC columns by a group of 8 DS lanes: a lane has TC columns
 // (c, c + 8, ..) and a DS-th of the depth; the depth is summed over the group, which then splits the
-// rows.  rows[r], cols[c]: addresses; logit(r, column, dot) scales and masks; the weights exp(z - max) of
-// the first n_rows rows go to w + r * wp, and done(r, max, sum, sum of weight * logit) keeps the rest.
+// rows.  rows[r], cols[c]: addresses; logit(r, column, dot) scales and masks; the weights of the first n_rows
+// rows go to w + r * wp, and done(r, max, sum of exp(z - max), sum of weight * logit) keeps the rest.
 template <int R, int DS, int TC, typename Logit, typename Done>
 __device__ __forceinline__ void score_rows(const float4* (&rows)[R], const float4* (&cols)[TC], int d4, int lane, int n_cols,
                                            float* w, int wp, Logit logit, Done done, int n_rows) {
@@ -200,17 +208,19 @@ __device__ __forceinline__ void score_rows(const float4* (&rows)[R], const float
     }
     s = row_sum(s);
     sz = row_sum(sz);
+    const float inv = 1.f / s;
     if (R > 1 || part == 0) {
 #pragma unroll
       for (int c = 0; c < TC; ++c)
-        if (r < n_rows && c0 + 8 * c < n_cols) w[r * wp + c0 + 8 * c] = z[q][c];
-      if (c0 == 0) done(r, zmax, s, sz);
+        if (r < n_rows && c0 + 8 * c < n_cols) w[r * wp + c0 + 8 * c] = z[q][c] * inv;
+      if (c0 == 0) done(r, zmax, s, sz * inv);
     }
   }
 }
 
-// TR: positions of a register tile (1, 2 or 4).  CB, CM: up to 8 CB keys and 8 CM blocks; 0: any number.
-template <typename TIn, int TR, int CB, int CM>
+// TR: positions of a register tile (1, 2 or 4).  CB, CM: up to 8 CB keys and 8 CM blocks; 0: any numbers.
+// WHOLE: rows are whole 16-byte units.
+template <typename TIn, int TR, int CB, int CM, bool WHOLE>
 __global__ void __launch_bounds__(kThreads, 2)
 monarch_fused_f32(const TIn* __restrict__ Q, const TIn* __restrict__ K, const TIn* __restrict__ V,
                   TIn* __restrict__ Y, int N, int d, int b, int m, int T_steps, float scale,
@@ -227,29 +237,39 @@ monarch_fused_f32(const TIn* __restrict__ Q, const TIn* __restrict__ K, const TI
   float4 *sK = sm, *sQ = sm + ly.Q, *sA = sm + ly.A;
   float* cL = reinterpret_cast<float*>(sm + ly.C);          // [k * JT + jj]
   float* cR = cL + (JT * m + 3) / 4 * 4;                    // [k * JT + jj]
-  float* ri = cR + (JT * m + 3) / 4 * 4;                    // 1 / row sum of the half-step's rows
   float* sW = reinterpret_cast<float*>(sm + ly.S);          // weights, row pitch 4 su
   const int wp = 4 * su;
 
+  // the head's first row, and from row to row
+  const size_t base = H == 0 ? (size_t)h * N * d : ((size_t)(h / H) * N * H + h % H) * d;
+  const int rs = H == 0 ? d : H * d;
+  Q += base;
+  K += base;
+  V += base;
+  Y += base;
+  if (row_lse != nullptr) row_lse += (size_t)h * N;
+  const float inv_d4 = 1.f / d4;
+
   // ---- loads; V is asked for into L2
+  const float inv_b = 1.f / b, inv_nj = 1.f / nj;
 #pragma unroll 8
   for (int e = tid; e < N * d4; e += kThreads) {
-    const int n = e / d4, u = e - n * d4, k = n / b, i = n - k * b;
-    sK[k * bu + i * pu + u] = load4(K + io_off(h, n, N, d, H), 4 * u, d);
+    const int n = divide(e, inv_d4), u = e - n * d4, k = divide(n, inv_b), i = n - k * b;
+    sK[k * bu + i * pu + u] = load4<WHOLE>(K + (size_t)n * rs, 4 * u, d);
   }
 #pragma unroll 4
   for (int e = tid; e < nj * m * d4; e += kThreads) {
-    const int r = e / d4, u = e - r * d4, l = r / nj, jj = r - l * nj;
-    sQ[l * ju + jj * pu + u] = load4(Q + io_off(h, l * b + j0 + jj, N, d, H), 4 * u, d);
+    const int r = divide(e, inv_d4), u = e - r * d4, l = divide(r, inv_nj), jj = r - l * nj;
+    sQ[l * ju + jj * pu + u] = load4<WHOLE>(Q + (size_t)(l * b + j0 + jj) * rs, 4 * u, d);
   }
   for (int n = tid; n < N; n += kThreads) {
-    const char* p = reinterpret_cast<const char*>(V + io_off(h, n, N, d, H));
+    const char* p = reinterpret_cast<const char*>(V + (size_t)n * rs);
     for (int o = 0; o < d * (int)sizeof(TIn); o += 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + o));
   }
   __syncthreads();
 
-  // Softmax over the first `cols` of `rows` rows of logits, eight lanes a row: to weights exp(z - max),
-  // 1 / sum to ri; done(row, max, sum, sum of weight * logit).
+  // Softmax over the first `cols` of `rows` rows of logits, eight lanes a row: to weights;
+  // done(row, max, sum of exp(z - max), sum of weight * logit).
   auto softmax = [&](int rows, int cols, auto done) {
     for (int r0 = 0; r0 < rows; r0 += kThreads / 8) {
       const int r = r0 + (tid >> 3), g = tid & 7;
@@ -271,15 +291,15 @@ monarch_fused_f32(const TIn* __restrict__ Q, const TIn* __restrict__ K, const TI
         }
       s = row_sum(s);
       sz = row_sum(sz);
-      if (on && g == 0) {
-        ri[r] = 1.f / s;
-        done(r, zmax, s, sz);
-      }
+      const float inv = 1.f / s;
+      if (on)
+        for (int i = g; i < cols; i += 8) w[i] *= inv;
+      if (on && g == 0) done(r, zmax, s, sz * inv);
     }
   };
 
   const int JG = (nj + TR - 1) / TR, LG = (m + TL - 1) / TL;
-  const float inv_JG = 1.f / JG, inv_d4 = 1.f / d4, inv_LG = 1.f / LG;
+  const float inv_JG = 1.f / JG, inv_LG = 1.f / LG, inv_m = 1.f / m;
   for (int step = 1; step <= T_steps; ++step) {
     const bool first = step == 1, last = step == T_steps;
     // ---------------------------------------------------------------- R half-step (Eq. 7, 9, 10)
@@ -317,8 +337,7 @@ monarch_fused_f32(const TIn* __restrict__ Q, const TIn* __restrict__ K, const TI
             },
             [&](int r, float zmax, float sum, float sz) {
               if (!on || jr + r >= nj) return;
-              ri[k * JT + jr + r] = 1.f / sum;
-              cL[k * JT + jr + r] = sz / sum - (zmax + logf(sum));
+              cL[k * JT + jr + r] = sz - (zmax + logf(sum));
             },
             nj - jr);
       }
@@ -360,7 +379,7 @@ monarch_fused_f32(const TIn* __restrict__ Q, const TIn* __restrict__ K, const TI
         }
       }
       __syncthreads();
-      softmax(m * JT, b, [&](int r, float zmax, float s, float sz) { cL[r] = sz / s - (zmax + logf(s)); });
+      softmax(m * JT, b, [&](int r, float zmax, float s, float sz) { cL[r] = sz - (zmax + logf(s)); });
       __syncthreads();
     }
     // second products: TR positions x 4 columns; row(k, i, u): four columns from 4 u of row (k, i) of K or V
@@ -397,17 +416,14 @@ monarch_fused_f32(const TIn* __restrict__ Q, const TIn* __restrict__ K, const TI
         }
 #pragma unroll
         for (int r = 0; r < TR; ++r)
-          if (jr + r < nj) {
-            const float s = ri[k * JT + jr + r];
-            put(k, jr + r, u, make_float4(acc[r].x * s, acc[r].y * s, acc[r].z * s, acc[r].w * s));
-          }
+          if (jr + r < nj) put(k, jr + r, u, acc[r]);
       }
     };
     apply([&](int k, int i, int u) { return sK[k * bu + i * pu + u]; },
           [&](int k, int jj, int u, const float4& v) { sA[k * ju + jj * pu + u] = v; });
     __syncthreads();
     if (last) {      // y over the rows of K
-      apply([&](int k, int i, int u) { return load4(V + io_off(h, k * b + i, N, d, H), 4 * u, d); },
+      apply([&](int k, int i, int u) { return load4<WHOLE>(V + (size_t)(k * b + i) * rs, 4 * u, d); },
             [&](int k, int jj, int u, const float4& v) { sK[k * bu + jj * pu + u] = v; });
       __syncthreads();
     }
@@ -417,7 +433,7 @@ monarch_fused_f32(const TIn* __restrict__ Q, const TIn* __restrict__ K, const TI
     auto row_done = [&](int r, float zmax, float s) {
       // log-sum-exp of row b l + j: summed over a head's rows it is the objective (Eq. 6)
       const int jj = r / m, l = r - jj * m;
-      if (last && row_lse != nullptr) row_lse[(size_t)h * N + (size_t)l * b + j0 + jj] = zmax + logf(s);
+      if (last && row_lse != nullptr) row_lse[l * b + j0 + jj] = zmax + logf(s);
     };
     if constexpr (CM > 0) {
       const int RG = (m + TR - 1) / TR, groups = nj * RG;
@@ -436,7 +452,6 @@ monarch_fused_f32(const TIn* __restrict__ Q, const TIn* __restrict__ K, const TI
             [&](int, int k, float dot) { return dot * scale - cL[k * JT + jj]; },
             [&](int r, float zmax, float sum, float) {
               if (!on || l0 + r >= m) return;
-              ri[jj * m + l0 + r] = 1.f / sum;
               row_done(jj * m + l0 + r, zmax, sum);
             },
             m - l0);
@@ -510,44 +525,40 @@ monarch_fused_f32(const TIn* __restrict__ Q, const TIn* __restrict__ K, const TI
         }
 #pragma unroll
         for (int r = 0; r < TL; ++r)
-          if (r0 + r < m) {
-            const float s = ri[jj * m + r0 + r];
-            store4(Y + io_off(h, (r0 + r) * b + j0 + jj, N, d, H), 4 * u, d,
-                   make_float4(acc[r].x * s, acc[r].y * s, acc[r].z * s, acc[r].w * s));
-          }
+          if (r0 + r < m) store4<WHOLE>(Y + (size_t)((r0 + r) * b + j0 + jj) * rs, 4 * u, d, acc[r]);
       } else {
         // alpha_R(k,j) = sum_l L[l,k] Q(l,j), c_R(k,j) = sum_l L[l,k], blocks k = r0 ..
         const float4* x = sQ + jj * pu + u;
-        float c[TL];
-#pragma unroll
-        for (int r = 0; r < TL; ++r) c[r] = 0.f;
 #pragma unroll 4
         for (int l = 0; l < m; ++l) {
           const float4 v = x[l * ju];
-          const float s = ri[jj * m + l];
-          float p[TL];
           if constexpr (TL == 4) {
-            const float4 p4 = *reinterpret_cast<const float4*>(w + l * wp + r0);
-            p[0] = p4.x; p[1] = p4.y; p[2] = p4.z; p[3] = p4.w;
+            const float4 p = *reinterpret_cast<const float4*>(w + l * wp + r0);
+            fma4(acc[0], p.x, v);
+            fma4(acc[1], p.y, v);
+            fma4(acc[2], p.z, v);
+            fma4(acc[3], p.w, v);
           } else {
-            p[0] = w[l * wp + r0];
-          }
-#pragma unroll
-          for (int r = 0; r < TL; ++r) {
-            p[r] *= s;
-            c[r] += p[r];
-            fma4(acc[r], p[r], v);
+            fma4(acc[0], w[l * wp + r0], v);
           }
         }
 #pragma unroll
         for (int r = 0; r < TL; ++r)
-          if (r0 + r < m) {
-            sA[(r0 + r) * ju + jj * pu + u] = acc[r];
-            if (u == 0) cR[(r0 + r) * JT + jj] = c[r];
-          }
+          if (r0 + r < m) sA[(r0 + r) * ju + jj * pu + u] = acc[r];
       }
     }
-    if (!last) __syncthreads();
+    if (!last) {
+      // c_R, four lanes a column
+      for (int c0 = 0; c0 < nj * m; c0 += kThreads / 4) {
+        const int c = c0 + (tid >> 2), jj = divide(min(c, nj * m - 1), inv_m), k = min(c, nj * m - 1) - jj * m;
+        float sum = 0.f;
+        for (int l = tid & 3; l < m; l += 4) sum += sW[(jj * m + l) * wp + k];
+        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+        sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+        if (c < nj * m && (tid & 3) == 0) cR[k * JT + jj] = sum;
+      }
+      __syncthreads();
+    }
   }
 }
 
@@ -566,24 +577,27 @@ inline int launch_t(const void* Q, const void* K, const void* V, void* Y, int BH
   const int JT = positions_per_cta(d, b, m, BH, sms[dev]);
   if (JT < 1 || BH > 65535) return 4;
   // (the kernels with whole score rows in a group of lanes are for fp32 inputs, the only ones this path
-  // is chosen for, and up to 32 keys and blocks)
+  // is chosen for, up to 32 keys and blocks, with the
+  // reads of ragged rows left out where there are none: instruction fetch counts, a warp executes most of the
+  // code once or twice)
   const int cb = b <= 16 ? 2 : (b <= 24 ? 3 : 4), cm = m <= 16 ? 2 : 4;
-  const bool small = sizeof(TIn) == 4 && b <= 32 && m <= 32;
+  const bool small = sizeof(TIn) == 4 && b <= 32 && m <= 32, whole = d % 4 == 0;
   auto pick = [&](auto tr) {
     constexpr int TR = decltype(tr)::value;
     if constexpr (sizeof(TIn) == 4) {
-      if (small) {
-        if (cm == 2) return cb == 2 ? monarch_fused_f32<TIn, TR, 2, 2> : (cb == 3 ? monarch_fused_f32<TIn, TR, 3, 2> : monarch_fused_f32<TIn, TR, 4, 2>);
-        return cb == 2 ? monarch_fused_f32<TIn, TR, 2, 4> : (cb == 3 ? monarch_fused_f32<TIn, TR, 3, 4> : monarch_fused_f32<TIn, TR, 4, 4>);
-      }
+      if (small && !whole) return monarch_fused_f32<TIn, TR, 4, 4, false>;
+      if (small && cm == 2)
+        return cb == 2 ? monarch_fused_f32<TIn, TR, 2, 2, true> : (cb == 3 ? monarch_fused_f32<TIn, TR, 3, 2, true> : monarch_fused_f32<TIn, TR, 4, 2, true>);
+      if (small)
+        return cb == 2 ? monarch_fused_f32<TIn, TR, 2, 4, true> : (cb == 3 ? monarch_fused_f32<TIn, TR, 3, 4, true> : monarch_fused_f32<TIn, TR, 4, 4, true>);
     }
-    return monarch_fused_f32<TIn, TR, 0, 0>;
+    return monarch_fused_f32<TIn, TR, 0, 0, false>;
   };
   auto kern = JT == 1 ? pick(std::integral_constant<int, 1>())
                       : (JT == 2 ? pick(std::integral_constant<int, 2>()) : pick(std::integral_constant<int, 4>()));
   const size_t smem = smem_bytes(d, b, m, JT);
-  static bool prepared[64][3][7] = {};
-  bool& ready = prepared[dev][JT < 4 ? JT - 1 : 2][small ? cb - 2 + 3 * (cm == 4) : 6];
+  static bool prepared[64][3][8] = {};
+  bool& ready = prepared[dev][JT < 4 ? JT - 1 : 2][!small ? 6 : (whole ? cb - 2 + 3 * (cm == 4) : 7)];
   if (!ready) {      // once per device: the kernel may use all of shared memory
     if (cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) !=
         cudaSuccess)
