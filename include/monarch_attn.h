@@ -56,11 +56,11 @@ typedef enum {
                                 m = b in {64, 128}; the plain statement the persistent kernels are
                                 tested against */
   MA_PATH_FUSED_F32 = 5, /* fp32 arithmetic and fp32 states in shared memory, one launch for all T
-                            rounds: any dtype, any N = m*b whose K, V and one position's states fit
-                            shared memory (N <= ~430 at d = 64); a CTA owns a set of in-block
+                            rounds: any dtype, any N = m*b whose K and one position's states fit
+                            shared memory (N <= ~750 at d = 64); a CTA owns a set of in-block
                             positions of one head (the recursion is independent across them), so a
                             single small head is spread over up to b CTAs.  What AUTO takes for
-                            fp32 inputs of that size */
+                            fp32 inputs unless many long heads leave room for a position or two */
   MA_PATH_FUSED_JSPLIT = 6, /* N = 1024 as m = b = 32 (d = 64, f16/bf16, either layout, no mask, no
                               row_lse): all T rounds in one launch; a head is split over two or four
                               CTAs by in-block position (Eq. 7-10 never mix two positions j), each
@@ -71,7 +71,8 @@ typedef enum {
                              T > 1 (the states of a head must fit shared memory); f16 arithmetic.
                              For T >= 3 with m, b <= 16 and d <= 80 the states and the weights that
                              form them are hi + lo pairs of f16 (what AUTO takes there) */
-  MA_PATH_TILE_MMA = 8    /* warp-MMA kernels, one launch per half-step, f16 states in the workspace
+  MA_PATH_TILE_MMA = 8    /* tile kernels (tcgen05 for T <= 2, d <= 64 and enough tiles, else warp MMA), one
+                             launch per half-step, f16 states in the workspace
                              (hi + lo pairs of f16 from T = 3 on): f16/bf16, m and b <= 128 (m need
                              not equal b), d <= 128 a multiple of 8; the 16-bit path of the shapes no
                              other tensor-core kernel takes */
