@@ -283,10 +283,18 @@ static bool touches_workspace(int resolved) {
 // negative scales).  Where both apply the tcgen05 tiles pay for their set-up and longer chain once
 // there are tiles enough to keep several in flight on every SM: measured over N = 960 .. 10240 and 8
 // to 64 heads they are 1.0-1.9 x as fast from 448 tiles of 128 rows on (two rounds of blocks of
-// more than 32: from 160 on), and 0.65-0.97 x below.
+// more than 32: from 160 on), and 0.65-0.97 x below.  Their tiles hold whole blocks rounded up to 32, 64 or
+// 128 rows; the warp-MMA tiles are as wide as the block.  With blocks of up to 64 rows and so few of them
+// that the two half-steps take 5/3 of the tiles the rows would fill, the warp-MMA tiles win (8 blocks of 48
+// 44.6 against 52.4 us, 16 of 48 36.9 / 40.3, 12 of 64 40.9 / 42.8; 16 of 64 38.5 / 38.2, 17 of 48 42.3 / 39.5;
+// 8 of 128 59.1 / 51.4).
 static bool tiles_on_tensor_cores(const Problem& p, float scale) {
   if (p.T > 2 || !(scale >= 0.f) || !ttc::supported(p.N, p.d, p.b, p.m, p.dtype, p.BH)) return false;
   const long long tiles = (long long)p.BH * p.N / 128;
+  auto per_tile = [](int rows) { return rows <= 32 ? 4 : (rows <= 64 ? 2 : 1); };
+  const int pr = per_tile(p.b), pl = per_tile(p.m);
+  const int taken = (p.m + pr - 1) / pr + (p.b + pl - 1) / pl;
+  if (p.b <= 64 && 3 * 128 * taken >= 5 * 2 * p.N) return false;
   return tiles >= (p.T == 2 && p.b > 32 ? 160 : 448);
 }
 
