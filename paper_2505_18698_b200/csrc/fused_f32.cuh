@@ -37,7 +37,6 @@ namespace ffused {
 
 using generic::ld_as_float;
 using generic::st_from_float;
-using tensor::ffma2;
 
 constexpr int kThreads = 256, kMaxSmem = 227 * 1024;
 

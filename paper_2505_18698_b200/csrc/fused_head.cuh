@@ -81,8 +81,9 @@ __device__ __forceinline__ void load_5d(uint32_t dst, const CUtensorMap* tm, uin
 // Four 8 x 8 pieces of an accumulator pair (two 8-column tiles of 16 rows) as 16-bit rows.
 __device__ __forceinline__ void put(uint32_t addr, const float (&o)[2][4], float m0, float m1) {
   typedef Mma<__half> M;
-  stsm_x4(addr, M::pack(o[0][0] * m0, o[0][1] * m0), M::pack(o[0][2] * m1, o[0][3] * m1), M::pack(o[1][0] * m0, o[1][1] * m0),
-          M::pack(o[1][2] * m1, o[1][3] * m1));
+  const float2 a = both(m0), b = both(m1);
+  stsm_x4(addr, M::pack(fmul2(make_float2(o[0][0], o[0][1]), a)), M::pack(fmul2(make_float2(o[0][2], o[0][3]), b)),
+          M::pack(fmul2(make_float2(o[1][0], o[1][1]), a)), M::pack(fmul2(make_float2(o[1][2], o[1][3]), b)));
 }
 // Byte offset of a 16-byte chunk of a row under the 128-byte swizzle.
 __device__ __forceinline__ uint32_t at(uint32_t base, int row, int chunk) {
@@ -126,10 +127,24 @@ __device__ __forceinline__ void pack_a(uint32_t (&pa)[(NT + 1) / 2][4], const fl
   }
 }
 
-// Shared memory of a CTA: `bufs` x (Q, K, V), the state tile (more than one round), c_L ([position]
-// [nm * 8 blocks]), a dump for matrix-store rows past a block, barriers.
+// Two 8-column tiles of a product over KT 16-row steps.
+template <int KT>
+__device__ __forceinline__ void products(float (&o)[2][4], const uint32_t (&a)[KT][4], const uint32_t (&b)[KT][4]) {
+  typedef Mma<__half> M;
+#pragma unroll
+  for (int kk = 0; kk < KT; ++kk)
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+      if (kk == 0) M::first(o[v], a[kk], b[kk] + 2 * v);
+      else M::run(o[v], a[kk], b[kk] + 2 * v);
+    }
+}
+
+// Shared memory of a CTA: `bufs` x (Q, K, V), the state tile (more than one round), a dump for matrix-store rows past a
+// block (a line of its own: addresses step through a row by an exclusive or of bits 5 and 6), c_L ([position]
+// [nm * 8 blocks]), barriers.
 inline size_t smem_bytes(int tile, int bufs, bool multi, int b, int nm) {
-  return (size_t)tile * (3 * bufs + (multi ? 1 : 0)) + (size_t)b * nm * 8 * 4 + 128 + sizeof(Bars) + 1024 + 16;
+  return (size_t)tile * (3 * bufs + (multi ? 1 : 0)) + 128 + (size_t)b * nm * 8 * 4 + sizeof(Bars) + 1024;
 }
 
 // NB, NM: 8-column tiles that hold b keys / m blocks.
@@ -143,11 +158,11 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
   const int tile = P.tile, b = P.b, bp = P.bp;
   const uint32_t s0 = smem_u32(smem);
   const uint32_t sS = s0 + 3 * P.bufs * tile;              // state tile (MULTI)
-  float* sCL = reinterpret_cast<float*>(smem + (3 * P.bufs + (MULTI ? 1 : 0)) * tile);
-  uint8_t* tail = reinterpret_cast<uint8_t*>(sCL + b * NM * 8);
+  uint8_t* tail = smem + (3 * P.bufs + (MULTI ? 1 : 0)) * tile;
+  float* sCL = reinterpret_cast<float*>(tail + 128);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const uint32_t dump = smem_u32(tail) + (lane & 7) * 16;
-  Bars* bars = reinterpret_cast<Bars*>(tail + 128);
+  Bars* bars = reinterpret_cast<Bars*>(sCL + b * NM * 8);
   if (tid == 0) {
     for (int i = 0; i < P.bufs; ++i)
       for (int k = 0; k < P.m; ++k) mbar_init(&bars->full[i][k], 1);
@@ -221,17 +236,16 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
 #pragma unroll
           for (int rt = 0; rt < RB; ++rt) {
             float s[NB][4];
-#pragma unroll
-            for (int nt = 0; nt < NB; ++nt)
-#pragma unroll
-              for (int e = 0; e < 4; ++e) s[nt][e] = 0.f;
             const uint32_t ad = at(sA, r0 + min(16 * rt + a_row, b - 1), a_ch);
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks) {
               uint32_t a[4];
               ldsm_x4(a, ad ^ (ks << 5));
 #pragma unroll
-              for (int nt = 0; nt < NB; ++nt) M::run(s[nt], a, kb[nt][ks]);
+              for (int nt = 0; nt < NB; ++nt) {
+                if (ks == 0) M::first(s[nt], a, kb[nt][ks]);
+                else M::run(s[nt], a, kb[nt][ks]);
+              }
             }
             // rows j = 16 rt + g (c0, c1) and + 8 (c2, c3); columns i = 8 nt + 2 t, + 1.  Columns past the
             // block, in the last column tile, and padded keys of the last block: a score of weight 0.
@@ -252,19 +266,19 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
               for (int nt = 0; nt < NB; ++nt) mx = fmaxf(mx, fmaxf(s[nt][2 * hh], s[nt][2 * hh + 1]));
               mx = quad_max(mx);
               off[2 * rt + hh] = -mx * fl;
-              float sum = 0.f, sz = 0.f;
+              float2 sum = both(0.f), sz = both(0.f);
 #pragma unroll
-              for (int nt = 0; nt < NB; ++nt)
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                  const float x = s[nt][2 * hh + e];
-                  const float p = ex2(fmaf(x, fl, off[2 * rt + hh]));
-                  s[nt][2 * hh + e] = p;
-                  sum += p;
-                  sz = fmaf(p, x, sz);               // 0 times a finite number where masked (0 log 0 = 0)
-                }
-              red[2 * (2 * rt + hh)] = sum;
-              red[2 * (2 * rt + hh) + 1] = sz;
+              for (int nt = 0; nt < NB; ++nt) {
+                const float2 x = make_float2(s[nt][2 * hh], s[nt][2 * hh + 1]);
+                const float2 z = ffma2(x, both(fl), both(off[2 * rt + hh]));
+                const float2 p = make_float2(ex2(z.x), ex2(z.y));
+                s[nt][2 * hh] = p.x;
+                s[nt][2 * hh + 1] = p.y;
+                sum = nt ? fadd2(sum, p) : p;
+                sz = nt ? ffma2(p, x, sz) : fmul2(p, x);      // 0 times a finite number where masked (0 log 0 = 0)
+              }
+              red[2 * (2 * rt + hh)] = sum.x + sum.y;
+              red[2 * (2 * rt + hh) + 1] = sz.x + sz.y;
             }
             pack_a<NB>(pa[rt], s);
           }
@@ -291,36 +305,32 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
         uint32_t kt[RB], st[RB];
 #pragma unroll
         for (int kk = 0; kk < RB; ++kk) {
-          kt[kk] = at(0, r0 + min(16 * kk + a_row, b - 1), a_ch);
-          st[kk] = at(0, r0 + 16 * kk + a_row, a_ch);
+          kt[kk] = at(sK, r0 + min(16 * kk + a_row, b - 1), a_ch);
+          st[kk] = 16 * kk + a_row < b ? at(dst, r0 + 16 * kk + a_row, a_ch) : dump;
         }
+        // (from the K tile's addresses to the V tile's, from those of alpha_L to y's)
+        const uint32_t to_v = sV - sK;
+        uint32_t sy[RB];
+#pragma unroll
+        for (int kk = 0; kk < RB; ++kk) sy[kk] = 16 * kk + a_row < b ? st[kk] - dst + sV : dump;
 #pragma unroll
         for (int np = 0; np < 4; ++np) {
           uint32_t bk[RB][4], bv[RB][4];
 #pragma unroll
           for (int kk = 0; kk < RB; ++kk) {
-            ldsm_x4_trans(bk[kk], sK + (kt[kk] ^ (np << 5)));
-            if (last) ldsm_x4_trans(bv[kk], sV + (kt[kk] ^ (np << 5)));
+            const uint32_t ad = kt[kk] ^ (np << 5);
+            ldsm_x4_trans(bk[kk], ad);
+            if (last) ldsm_x4_trans(bv[kk], ad + to_v);
           }
           __syncwarp();
 #pragma unroll
           for (int rt = 0; rt < RB; ++rt) {
-            const bool on = 16 * rt + a_row < b;
-            float o[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-#pragma unroll
-            for (int kk = 0; kk < RB; ++kk) {
-              M::run(o[0], pa[rt][kk], bk[kk]);
-              M::run(o[1], pa[rt][kk], bk[kk] + 2);
-            }
-            put(on ? dst + (st[rt] ^ (np << 5)) : dump, o, inv[rt][0], inv[rt][1]);
+            float o[2][4];
+            products<RB>(o, pa[rt], bk);
+            put(st[rt] ^ (np << 5), o, inv[rt][0], inv[rt][1]);
             if (last) {
-              float y[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-#pragma unroll
-              for (int kk = 0; kk < RB; ++kk) {
-                M::run(y[0], pa[rt][kk], bv[kk]);
-                M::run(y[1], pa[rt][kk], bv[kk] + 2);
-              }
-              put(on ? sV + (st[rt] ^ (np << 5)) : dump, y, inv[rt][0], inv[rt][1]);
+              products<RB>(o, pa[rt], bv);
+              put(sy[rt] ^ (np << 5), o, inv[rt][0], inv[rt][1]);
             }
           }
         }
@@ -346,40 +356,38 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
 #pragma unroll
           for (int rt = 0; rt < RM; ++rt) {
             float s[NM][4];
-#pragma unroll
-            for (int nt = 0; nt < NM; ++nt)
-#pragma unroll
-              for (int e = 0; e < 4; ++e) s[nt][e] = 0.f;
             const uint32_t ad = at(sQ, min(16 * rt + a_row, m - 1) * bp + j, a_ch);
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks) {
               uint32_t a[4];
               ldsm_x4(a, ad ^ (ks << 5));
 #pragma unroll
-              for (int nt = 0; nt < NM; ++nt) M::run(s[nt], a, kb[nt][ks]);
+              for (int nt = 0; nt < NM; ++nt) {
+                if (ks == 0) M::first(s[nt], a, kb[nt][ks]);
+                else M::run(s[nt], a, kb[nt][ks]);
+              }
             }
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {
               float mx = kMasked;
 #pragma unroll
-              for (int nt = 0; nt < NM; ++nt)
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                  const float z = fmaf(s[nt][2 * hh + e], fl, c[nt][e]);
-                  s[nt][2 * hh + e] = z;
-                  mx = fmaxf(mx, z);
-                }
+              for (int nt = 0; nt < NM; ++nt) {
+                const float2 z = ffma2(make_float2(s[nt][2 * hh], s[nt][2 * hh + 1]), both(fl), make_float2(c[nt][0], c[nt][1]));
+                s[nt][2 * hh] = z.x;
+                s[nt][2 * hh + 1] = z.y;
+                mx = fmaxf(mx, fmaxf(z.x, z.y));
+              }
               mx = quad_max(mx);
-              float sum = 0.f;
+              float2 sum = both(0.f);
 #pragma unroll
-              for (int nt = 0; nt < NM; ++nt)
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                  const float p = ex2(s[nt][2 * hh + e] - mx);
-                  s[nt][2 * hh + e] = p;
-                  sum += p;
-                }
-              red[2 * rt + hh] = sum;
+              for (int nt = 0; nt < NM; ++nt) {
+                const float2 z = fadd2(make_float2(s[nt][2 * hh], s[nt][2 * hh + 1]), both(-mx));
+                const float2 p = make_float2(ex2(z.x), ex2(z.y));
+                s[nt][2 * hh] = p.x;
+                s[nt][2 * hh + 1] = p.y;
+                sum = nt ? fadd2(sum, p) : p;
+              }
+              red[2 * rt + hh] = sum.x + sum.y;
               mxs[2 * rt + hh] = mx;
             }
             if (last) {
@@ -409,8 +417,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
         uint32_t kt[RM], st[RM];
 #pragma unroll
         for (int kk = 0; kk < RM; ++kk) {
-          kt[kk] = at(0, min(16 * kk + a_row, m - 1) * bp + j, a_ch);
-          st[kk] = at(0, (16 * kk + a_row) * bp + j, a_ch);
+          kt[kk] = at(last ? sV : sQ, min(16 * kk + a_row, m - 1) * bp + j, a_ch);
+          st[kk] = 16 * kk + a_row < m ? at(last ? sQ : sS, (16 * kk + a_row) * bp + j, a_ch) : dump;
         }
         if (last) {
           // Y(l,j) = sum_k L[j,k,l] y(k,j), over the rows of Q the scores were formed from
@@ -418,16 +426,12 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
           for (int np = 0; np < 4; ++np) {
             uint32_t by[RM][4];
 #pragma unroll
-            for (int kk = 0; kk < RM; ++kk) ldsm_x4_trans(by[kk], sV + (kt[kk] ^ (np << 5)));
+            for (int kk = 0; kk < RM; ++kk) ldsm_x4_trans(by[kk], kt[kk] ^ (np << 5));
 #pragma unroll
             for (int rt = 0; rt < RM; ++rt) {
-              float o[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-#pragma unroll
-              for (int kk = 0; kk < RM; ++kk) {
-                M::run(o[0], pa[rt][kk], by[kk]);
-                M::run(o[1], pa[rt][kk], by[kk] + 2);
-              }
-              put(16 * rt + a_row < m ? sQ + (st[rt] ^ (np << 5)) : dump, o, inv[rt][0], inv[rt][1]);
+              float o[2][4];
+              products<RM>(o, pa[rt], by);
+              put(st[rt] ^ (np << 5), o, inv[rt][0], inv[rt][1]);
             }
           }
           __syncwarp();
@@ -456,12 +460,13 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
               // (rows past the last block: not in sums over rows)
               const float on = 16 * rt + g + 8 * hh < m ? inv[rt][hh] : 0.f;
 #pragma unroll
-              for (int nt = 0; nt < NM; ++nt)
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                  w[rt][nt][2 * hh + e] *= on;
-                  cms[2 * nt + e] = fmaxf(cms[2 * nt + e], w[rt][nt][2 * hh + e]);
-                }
+              for (int nt = 0; nt < NM; ++nt) {
+                const float2 v = fmul2(make_float2(w[rt][nt][2 * hh], w[rt][nt][2 * hh + 1]), both(on));
+                w[rt][nt][2 * hh] = v.x;
+                w[rt][nt][2 * hh + 1] = v.y;
+                cms[2 * nt] = fmaxf(cms[2 * nt], v.x);
+                cms[2 * nt + 1] = fmaxf(cms[2 * nt + 1], v.y);
+              }
             }
           const float cm = scatter_reduce<kCols, 16, 4>(cms, lane, warpmma::Max());
           const float gl = __uint_as_float((253u << 23) - (__float_as_uint(cm) & 0x7f800000u));
@@ -475,21 +480,22 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
             for (int rt = 0; rt < RM; ++rt)
 #pragma unroll
               for (int hh = 0; hh < 2; ++hh)
-                tp[rt][hh][nt] = movm_trans(M::pack(w[rt][nt][2 * hh] * gk[0], w[rt][nt][2 * hh + 1] * gk[1]));
+                tp[rt][hh][nt] = movm_trans(M::pack(fmul2(make_float2(w[rt][nt][2 * hh], w[rt][nt][2 * hh + 1]), make_float2(gk[0], gk[1]))));
           }
           const uint32_t ones[2] = {0x3C003C00u, 0x3C003C00u};
           uint32_t pk[RM][RM][4];    // A[k][l]: rows k = 16 kq .., contraction over l = 16 ls ..
           float c1 = 0.f;
 #pragma unroll
           for (int kq = 0; kq < RM; ++kq) {
-            float cr[4] = {0.f, 0.f, 0.f, 0.f};
+            float cr[4];
 #pragma unroll
             for (int ls = 0; ls < RM; ++ls) {
               pk[kq][ls][0] = tp[ls][0][2 * kq];
               pk[kq][ls][1] = 2 * kq + 1 < NM ? tp[ls][0][(2 * kq + 1) % NM] : 0u;
               pk[kq][ls][2] = tp[ls][1][2 * kq];
               pk[kq][ls][3] = 2 * kq + 1 < NM ? tp[ls][1][(2 * kq + 1) % NM] : 0u;
-              M::run(cr, pk[kq][ls], ones);
+              if (ls == 0) M::first(cr, pk[kq][ls], ones);
+              else M::run(cr, pk[kq][ls], ones);
             }
             if (t == 2 * kq) c1 = cr[0];      // a division a lane
             if (t == 2 * kq + 1) c1 = cr[2];
@@ -500,15 +506,12 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
             const float i0 = __shfl_sync(0xffffffffu, c1, (lane & ~3) + 2 * kq), i1 = __shfl_sync(0xffffffffu, c1, (lane & ~3) + 2 * kq + 1);
 #pragma unroll
             for (int np = 0; np < 4; ++np) {
-              float o[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+              float o[2][4];
+              uint32_t bq[RM][4];      // B[l][v] = Q(l,j)[v], read transposed
 #pragma unroll
-              for (int ls = 0; ls < RM; ++ls) {
-                uint32_t bq[4];      // B[l][v] = Q(l,j)[v], read transposed
-                ldsm_x4_trans(bq, sQ + (kt[ls] ^ (np << 5)));
-                M::run(o[0], pk[kq][ls], bq);
-                M::run(o[1], pk[kq][ls], bq + 2);
-              }
-              put(16 * kq + a_row < m ? sS + (st[kq] ^ (np << 5)) : dump, o, i0, i1);
+              for (int ls = 0; ls < RM; ++ls) ldsm_x4_trans(bq[ls], kt[ls] ^ (np << 5));
+              products<RM>(o, pk[kq], bq);
+              put(st[kq] ^ (np << 5), o, i0, i1);
             }
           }
         }

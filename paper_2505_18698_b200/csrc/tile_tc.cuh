@@ -49,9 +49,8 @@ constexpr int kSlot = kTileBytes;            // 16 KB
 constexpr int kSlots = 6;
 constexpr int kOffOnes = kSlots * kSlot;     // 2 KB of ones
 constexpr int kOffVec = kOffOnes + 2048;     // c_L of a tile's rows: three tiles of 128 floats
-constexpr int kOffCol = kOffVec + 3 * 512;   // per group: column maxima, then scales, of the non-final L weights
-constexpr int kOffScale = kOffCol + 2 * 512;
-constexpr int kOffBar = kOffScale + 2 * 512;
+constexpr int kOffCol = kOffVec + 3 * 512;   // per group, two sets in turn: column maxima of the non-final L weights
+constexpr int kOffBar = kOffCol + 4 * 512;
 constexpr int kSmem = kOffBar + 384 + 1024;  // + alignment slack
 static_assert(kCtasPerSm * (kSmem + 1024) <= 228 * 1024, "two CTAs per SM");
 
@@ -126,6 +125,25 @@ __device__ __forceinline__ void st_cols<32>(uint32_t taddr, const uint32_t* r) {
       "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
       "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
       : "memory");
+}
+// 32 rows x 32 columns of the warp's part of tensor memory as matrix fragments: v[16 h + 4 o + 2 q + e] is row
+// 16 h + 8 q + lane / 4, column 8 o + 2 (lane % 4) + e.
+__device__ __forceinline__ void ld_frag16(uint32_t taddr, float* v) {
+  uint32_t* r = reinterpret_cast<uint32_t*>(v);
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void ld_frag32(uint32_t taddr, float* v) {
+  ld_frag16(taddr, v);
+  ld_frag16(taddr + (16u << 16), v + 16);
+}
+__device__ __forceinline__ void stmatrix_x4(uint32_t saddr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(saddr), "r"(a), "r"(b), "r"(c), "r"(d)
+               : "memory");
 }
 __device__ __forceinline__ float ld_col(uint32_t taddr) {
   uint32_t r;
@@ -555,36 +573,54 @@ struct Kernel {
 #pragma unroll
     for (int i = 0; i < CH / 2; ++i) u[i] = pack2<TA>(v[2 * i], v[2 * i + 1]);
   }
-  // 16 weights of a row, times `on` and the column scales, to the shared-memory operand: `base` is the
-  // row's 128 bytes in the 64-column chunk, col its first column there (128-byte swizzle).
-  static __device__ __forceinline__ void emit16(const float* v, uint8_t* base, int col, float on, const float* scale, int row) {
-    const float2 on2 = make_float2(on, on);
-    const float4* g4 = reinterpret_cast<const float4*>(scale);
-    uint32_t u[8];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      float2 a = fmul2(make_float2(v[4 * i], v[4 * i + 1]), on2), b = fmul2(make_float2(v[4 * i + 2], v[4 * i + 3]), on2);
-      const float4 g = g4[i];
-      a = fmul2(a, make_float2(g.x, g.y));
-      b = fmul2(b, make_float2(g.z, g.w));
-      u[2 * i] = pack2<TA>(a.x, a.y);
-      u[2 * i + 1] = pack2<TA>(b.x, b.y);
-    }
-    const int c0 = col >> 3;
-    *reinterpret_cast<uint4*>(base + ((c0 ^ (row & 7)) << 4)) = make_uint4(u[0], u[1], u[2], u[3]);
-    *reinterpret_cast<uint4*>(base + (((c0 + 1) ^ (row & 7)) << 4)) = make_uint4(u[4], u[5], u[6], u[7]);
+  // Scale of a column of the non-final L weights: 2^-(exponent of its largest weight).
+  static __device__ __forceinline__ float column_scale(unsigned mx) { return __uint_as_float((253u << 23) - (mx & 0x7f800000u)); }
+  // A pair of a lane's weights in fragments (`x` of ld_frag32): column octet o, its i-th row.
+  static __device__ __forceinline__ float2 frag_pair(const float* x, int o, int i) {
+    const float* p = x + 16 * (i >> 1) + 4 * o + 2 * (i & 1);
+    return make_float2(p[0], p[1]);
   }
-  // Maxima of 32 columns over the warp's rows, to the shared maxima.
-  static __device__ __forceinline__ void fold_columns(const float* v, float on, unsigned* sMax, int lane) {
-    unsigned keep = 0u;
+  // Maxima of 32 columns over the warp's rows, to the shared maxima (weights are not negative: their bits are in
+  // their order).  In fragments a lane has four rows of eight columns, and three exchanges finish it: one exchange for every
+  // 4.6 columns instead of a warp-wide reduction for each.
+  static __device__ __forceinline__ void fold_columns(const float* x, const float* on, unsigned* sMax, int lane) {
+    unsigned a[8];
 #pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(v[i] * on));
-      if (lane == i) keep = w;
+    for (int o = 0; o < 4; ++o) {
+      a[2 * o] = a[2 * o + 1] = 0u;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 v = fmul2(frag_pair(x, o, i), make_float2(on[i], on[i]));
+        a[2 * o] = max(a[2 * o], __float_as_uint(v.x));
+        a[2 * o + 1] = max(a[2 * o + 1], __float_as_uint(v.y));
+      }
     }
-    atomicMax(sMax + lane, keep);
+#pragma unroll
+    for (int n = 4, m = 16; n >= 1; n >>= 1, m >>= 1)
+#pragma unroll
+      for (int i = 0; i < n; ++i) {
+        const unsigned keep = lane & m ? a[i + n] : a[i], send = lane & m ? a[i] : a[i + n];
+        a[i] = max(keep, __shfl_xor_sync(0xffffffffu, send, m));
+      }
+    atomicMax(sMax + 8 * (lane >> 3) + 2 * (lane & 3) + ((lane >> 2) & 1), a[0]);
   }
-
+  // The same 32 columns to the shared-memory operand, normalised and scaled.  row_at: the lane's row of the 64-column chunk
+  // (128-byte swizzle); c0: the first of the four 16-byte pieces.
+  static __device__ __forceinline__ void emit_columns(const float* x, const float* on, const unsigned* sMax, uint32_t row_at, int c0,
+                                                      int row, int lane) {
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      const uint2 mx = *reinterpret_cast<const uint2*>(sMax + 8 * o + 2 * (lane & 3));
+      const float2 g = make_float2(column_scale(mx.x), column_scale(mx.y));
+      uint32_t u[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 v = fmul2(fmul2(frag_pair(x, o, i), make_float2(on[i], on[i])), g);
+        u[i] = pack2<TA>(v.x, v.y);
+      }
+      stmatrix_x4(row_at + (((c0 + o) ^ (row & 7)) << 4), u[0], u[1], u[2], u[3]);
+    }
+  }
 
   static __device__ __forceinline__ void compute(const Params& P, uint8_t* smem, Shared* sh, uint32_t tmem, int w) {
     const int row = threadIdx.x & 127, warp = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
@@ -593,7 +629,7 @@ struct Kernel {
     int i3 = w;
     // Parities: load (round of three tiles), one phase per tile of the group, and the barriers that
     // only some tiles use.
-    uint32_t par_l = 0, par = 0, par_t = 0, par_1 = 0, par_c = 0, par_o = 1;
+    uint32_t par_l = 0, par = 0, par_t = 0, par_1 = 0, par_o = 1;
 #define MA_WAIT(BAR, PAR, WHERE) \
   if (!__all_sync(0xffffffffu, wait_bar(&(BAR), PAR, sh, P, WHERE))) return
     // Staged rows (or the end) to the store thread, once it has taken the word of the one before.
@@ -701,35 +737,32 @@ struct Kernel {
           // so they are normalised before they are rounded, and go through shared memory (over
           // alpha_L, which the score MMA has read; at B = 128 with a slot of their own for one half).
           const float on = FULL || r_pos < mv ? mul : 0.f;     // rows past the last block: weight 0
-          float* scale = reinterpret_cast<float*>(smem + kOffScale) + 128 * w;
-          {
-            // column k times 2^-(exponent of its largest weight)
-            unsigned* sMax = reinterpret_cast<unsigned*>(smem + kOffCol) + 128 * w;
-            float x[32];
-#pragma unroll 1
-            for (int cc = 0; cc < B / 32; ++cc) {
-              tmem_ld32(tS + 32 * cc, x);
-              tmem_ld_wait();
-              fold_columns(x, on, sMax + B * r_blk + 32 * cc, lane);
-            }
-            arrive(&sh->cols[w]);
-            MA_WAIT(sh->cols[w], par_c, 34);
-            scale[row] = __uint_as_float((253u << 23) - (sMax[row] & 0x7f800000u));
-            sMax[row] = 0u;
-            arrive(&sh->cols[w]);
-            MA_WAIT(sh->cols[w], par_c ^ 1, 35);
+          float onr[4];                          // of the lane's rows in fragments
+#pragma unroll
+          for (int i = 0; i < 4; ++i) onr[i] = __shfl_sync(0xffffffffu, on, 8 * i + (lane >> 2));
+          // column k times 2^-(exponent of its largest weight)
+          unsigned* sMax = reinterpret_cast<unsigned*>(smem + kOffCol) + 128 * (2 * w + par);
+          float x[32];
+#pragma unroll
+          for (int cc = 0; cc < B / 32; ++cc) {
+            ld_frag32(tS + 32 * cc, x);
+            tmem_ld_wait();
+            fold_columns(x, onr, sMax + B * r_blk + 32 * cc, lane);
           }
-          float x[2][16];
-          tmem_ld16(tS, x[0]);
+          arrive(&sh->cols[w]);
+          ld_frag32(tS, x);
+          MA_WAIT(sh->cols[w], par, 34);
+          // (the set of the tile before: all warps are done with it, and none begins the next tile before all have come by)
+          reinterpret_cast<unsigned*>(smem + kOffCol)[128 * (2 * w + (par ^ 1)) + row] = 0u;
           const int e2 = wrap(e1 + 1);
           uint8_t* p_lo = smem + (B == 128 ? min(e1, e2) : e1) * kSlot + row * 128;
           uint8_t* p_hi = smem + (B == 128 ? max(e1, e2) : e1) * kSlot + row * 128;
           const int win = B == 32 ? 32 * (r_blk & 1) : 0;
 #pragma unroll
-          for (int cc = 0; cc < B / 16; ++cc) {
+          for (int cc = 0; cc < B / 32; ++cc) {
+            if (cc > 0) ld_frag32(tS + 32 * cc, x);
             tmem_ld_wait();
-            if (cc < B / 16 - 1) tmem_ld16(tS + 16 * (cc + 1), x[(cc + 1) & 1]);
-            emit16(x[cc & 1], cc < 4 ? p_lo : p_hi, win + (16 * cc & 63), on, scale + B * r_blk + 16 * cc, row);
+            emit_columns(x, onr, sMax + B * r_blk + 32 * cc, smem_u32(cc < 2 ? p_lo : p_hi), (win >> 3) + (4 * cc & 7), row, lane);
           }
           if constexpr (B == 32) {               // zeros beside the window
             const int c0 = (32 - win) >> 3;
@@ -834,7 +867,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) monarch_tiles(const __gr
     *reinterpret_cast<uint4*>(smem + kOffOnes + tid * 16) = make_uint4(one2, one2, one2, one2);
   }
   for (int i = tid; i < 3 * 128; i += kThreads) reinterpret_cast<float*>(smem + kOffVec)[i] = 0.f;
-  if (tid < 256) reinterpret_cast<unsigned*>(smem + kOffCol)[tid] = 0u;
+  for (int i = tid; i < 4 * 128; i += kThreads) reinterpret_cast<unsigned*>(smem + kOffCol)[i] = 0u;
   if (warp == 8) tmem_alloc(&sh->tmem, 256);
   fence_proxy_async();
   tc_fence_before();
