@@ -58,6 +58,9 @@ using warpmma::ex2;
 using warpmma::kLog2e;
 using warpmma::ldsm_x4;
 using warpmma::ldsm_x4_trans;
+using warpmma::mma;
+using warpmma::put_pair;
+using warpmma::row_pair;
 using warpmma::lg2;
 using warpmma::movm_trans;
 using warpmma::quad_max;
@@ -210,7 +213,7 @@ monarch_jsplit32(const __grid_constant__ CUtensorMap tmQ,    // Q as rows of d, 
       float inv[NT][2], red[4 * NT], mxs[2 * NT];
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) {
-        float s[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+        float s[2][4];
         const uint32_t row = first ? rq(k, 8 * nt + (lane & 7)) : rs(k, 8 * nt + (lane & 7));
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
@@ -219,26 +222,28 @@ monarch_jsplit32(const __grid_constant__ CUtensorMap tmQ,    // Q as rows of d, 
 #pragma unroll
           for (int k2 = 0; k2 < 2; ++k2)
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt) M::run(s[mt], kf[mt][2 * half + k2], bq + 2 * k2);
+            for (int mt = 0; mt < 2; ++mt) mma<__half>(half + k2 == 0, s[mt], kf[mt][2 * half + k2], bq + 2 * k2);
         }
         // column j = 8 nt + 2 t + e holds rows i = 16 mt + g (+ 8): softmax over i
+        float2 mx, sum = both(0.f), sz = both(0.f);        // of the lane's two columns
+        mx.x = col_max(fmaxf(fmaxf(s[0][0], s[0][2]), fmaxf(s[1][0], s[1][2])) * fl);
+        mx.y = col_max(fmaxf(fmaxf(s[0][1], s[0][3]), fmaxf(s[1][1], s[1][3])) * fl);
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const float mx = col_max(fmaxf(fmaxf(s[0][e], s[0][e + 2]), fmaxf(s[1][e], s[1][e + 2])) * fl);
-          float sum = 0.f, sz = 0.f;
+        for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-          for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-              const float p = ex2(fmaf(s[mt][e + 2 * hh], fl, -mx));
-              sum += p;
-              sz = fmaf(p, s[mt][e + 2 * hh], sz);
-              s[mt][e + 2 * hh] = p;
-            }
-          mxs[2 * nt + e] = mx;
-          red[2 * (2 * nt + e)] = sum;
-          red[2 * (2 * nt + e) + 1] = sz;
-        }
+          for (int hh = 0; hh < 2; ++hh) {
+            const float2 x = row_pair(s[mt], hh), z = ffma2(x, both(fl), make_float2(-mx.x, -mx.y));
+            const float2 p = make_float2(ex2(z.x), ex2(z.y));
+            sum = mt + hh ? fadd2(sum, p) : p;
+            sz = mt + hh ? ffma2(p, x, sz) : fmul2(p, x);
+            put_pair(s[mt], hh, p);
+          }
+        mxs[2 * nt] = mx.x;
+        mxs[2 * nt + 1] = mx.y;
+        red[4 * nt] = sum.x;
+        red[4 * nt + 1] = sz.x;
+        red[4 * nt + 2] = sum.y;
+        red[4 * nt + 3] = sz.y;
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt) {
           pb[nt][mt][0] = movm_trans(M::pack(s[mt][0], s[mt][1]));
@@ -270,26 +275,20 @@ monarch_jsplit32(const __grid_constant__ CUtensorMap tmQ,    // Q as rows of d, 
       for (int vp = 0; vp < 2; ++vp) {
         float o[NT][2][4];
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-          for (int v2 = 0; v2 < 2; ++v2)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) o[nt][v2][e] = 0.f;
-#pragma unroll
         for (int v2 = 0; v2 < 2; ++v2)
 #pragma unroll
           for (int is = 0; is < 2; ++is) {
             const uint32_t* f = kf[is][2 * vp + v2];
             const uint32_t a[4] = {movm_trans(f[0]), movm_trans(f[2]), movm_trans(f[1]), movm_trans(f[3])};
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt) M::run(o[nt][v2], a, pb[nt][is]);
+            for (int nt = 0; nt < NT; ++nt) mma<__half>(is == 0, o[nt][v2], a, pb[nt][is]);
           }
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
-          const float i0 = inv[nt][0], i1 = inv[nt][1];
-          stsm_x4_trans(swz(rs(k, 8 * nt + (lane & 7)), 4 * vp + (lane >> 3)), M::pack(o[nt][0][0] * i0, o[nt][0][1] * i1),
-                        M::pack(o[nt][0][2] * i0, o[nt][0][3] * i1), M::pack(o[nt][1][0] * i0, o[nt][1][1] * i1),
-                        M::pack(o[nt][1][2] * i0, o[nt][1][3] * i1));
+          const float2 i2 = make_float2(inv[nt][0], inv[nt][1]);
+          stsm_x4_trans(swz(rs(k, 8 * nt + (lane & 7)), 4 * vp + (lane >> 3)), M::pack(fmul2(row_pair(o[nt][0], 0), i2)),
+                        M::pack(fmul2(row_pair(o[nt][0], 1), i2)), M::pack(fmul2(row_pair(o[nt][1], 0), i2)),
+                        M::pack(fmul2(row_pair(o[nt][1], 1), i2)));
         }
       }
       if (last) {
@@ -299,21 +298,18 @@ monarch_jsplit32(const __grid_constant__ CUtensorMap tmQ,    // Q as rows of d, 
         for (int vt = 0; vt < 4; ++vt) {
           float o[NT][4];
 #pragma unroll
-          for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) o[nt][e] = 0.f;
-#pragma unroll
           for (int is = 0; is < 2; ++is) {
             uint32_t a[4];
             ldsm_x4_trans(a, swz(slot + (16 * is + (lane & 7) + 8 * (lane >> 4)) * 128, 2 * vt + ((lane >> 3) & 1)));
             convert_frag(a);
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt) M::run(o[nt], a, pb[nt][is]);
+            for (int nt = 0; nt < NT; ++nt) mma<__half>(is == 0, o[nt], a, pb[nt][is]);
           }
 #pragma unroll
           for (int nt = 0; nt < NT; ++nt) {
-            yk[u][nt][vt][0] = M::pack(o[nt][0] * inv[nt][0], o[nt][1] * inv[nt][1]);
-            yk[u][nt][vt][1] = M::pack(o[nt][2] * inv[nt][0], o[nt][3] * inv[nt][1]);
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh)
+              yk[u][nt][vt][hh] = M::pack(fmul2(row_pair(o[nt], hh), make_float2(inv[nt][0], inv[nt][1])));
           }
         }
         if (u + 1 < NB) request(&tmK, k + NW);
@@ -347,12 +343,6 @@ monarch_jsplit32(const __grid_constant__ CUtensorMap tmQ,    // Q as rows of d, 
       }
       float s[LT][4][4], inv[LT][2], rsum[2 * LT];
 #pragma unroll
-      for (int lt = 0; lt < LT; ++lt)
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) s[lt][nt][e] = 0.f;
-#pragma unroll
       for (int ks = 0; ks < 4; ++ks) {
         uint32_t bf[2][4];
 #pragma unroll
@@ -363,7 +353,7 @@ monarch_jsplit32(const __grid_constant__ CUtensorMap tmQ,    // Q as rows of d, 
           uint32_t a[4];
           ldsm_x4(a, swz(rq(l0 + 16 * lt + (lane & 15), jj), 2 * ks + (lane >> 4)));
 #pragma unroll
-          for (int nt = 0; nt < 4; ++nt) M::run(s[lt][nt], a, bf[nt >> 1] + 2 * (nt & 1));
+          for (int nt = 0; nt < 4; ++nt) mma<__half>(ks == 0, s[lt][nt], a, bf[nt >> 1] + 2 * (nt & 1));
         }
       }
 #pragma unroll
@@ -372,24 +362,21 @@ monarch_jsplit32(const __grid_constant__ CUtensorMap tmQ,    // Q as rows of d, 
         for (int hh = 0; hh < 2; ++hh) {
           float mx = -INFINITY;
 #pragma unroll
-          for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              const float z = fmaf(s[lt][nt][2 * hh + e], fl, c[nt][e]);
-              s[lt][nt][2 * hh + e] = z;
-              mx = fmaxf(mx, z);
-            }
+          for (int nt = 0; nt < 4; ++nt) {
+            const float2 z = ffma2(row_pair(s[lt][nt], hh), both(fl), make_float2(c[nt][0], c[nt][1]));
+            put_pair(s[lt][nt], hh, z);
+            mx = fmaxf(mx, fmaxf(z.x, z.y));
+          }
           mx = quad_max(mx);
-          float sum = 0.f;
+          float2 sum = both(0.f);
 #pragma unroll
-          for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              const float p = ex2(s[lt][nt][2 * hh + e] - mx);
-              s[lt][nt][2 * hh + e] = p;
-              sum += p;
-            }
-          rsum[2 * lt + hh] = sum;
+          for (int nt = 0; nt < 4; ++nt) {
+            const float2 z = fadd2(row_pair(s[lt][nt], hh), both(-mx));
+            const float2 p = make_float2(ex2(z.x), ex2(z.y));
+            put_pair(s[lt][nt], hh, p);
+            sum = nt ? fadd2(sum, p) : p;
+          }
+          rsum[2 * lt + hh] = sum.x + sum.y;
         }
       const float ri = 1.f / scatter_reduce<2 * LT, 2, 1>(rsum, lane, warpmma::Add());
 #pragma unroll
@@ -415,16 +402,16 @@ monarch_jsplit32(const __grid_constant__ CUtensorMap tmQ,    // Q as rows of d, 
           for (int k2 = 0; k2 < 2; ++k2) ldsm_x4_trans(bf[k2], swz(ry(16 * k2 + (lane & 15), jj), 2 * vp + (lane >> 4)));
 #pragma unroll
           for (int lt = 0; lt < LT; ++lt) {
-            float o[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+            float o[2][4];
 #pragma unroll
             for (int k2 = 0; k2 < 2; ++k2) {
-              M::run(o[0], pa[lt][k2], bf[k2]);
-              M::run(o[1], pa[lt][k2], bf[k2] + 2);
+              mma<__half>(k2 == 0, o[0], pa[lt][k2], bf[k2]);
+              mma<__half>(k2 == 0, o[1], pa[lt][k2], bf[k2] + 2);
             }
-            const float i0 = inv[lt][0], i1 = inv[lt][1];
-            stsm_x4(swz(rq(l0 + 16 * lt + (lane & 15), jj), 2 * vp + (lane >> 4)), M::pack(o[0][0] * i0, o[0][1] * i0),
-                    M::pack(o[0][2] * i1, o[0][3] * i1), M::pack(o[1][0] * i0, o[1][1] * i0),
-                    M::pack(o[1][2] * i1, o[1][3] * i1));
+            const float2 i0 = both(inv[lt][0]), i1 = both(inv[lt][1]);
+            stsm_x4(swz(rq(l0 + 16 * lt + (lane & 15), jj), 2 * vp + (lane >> 4)), M::pack(fmul2(row_pair(o[0], 0), i0)),
+                    M::pack(fmul2(row_pair(o[0], 1), i1)), M::pack(fmul2(row_pair(o[1], 0), i0)),
+                    M::pack(fmul2(row_pair(o[1], 1), i1)));
           }
         }
         __syncwarp();
@@ -448,18 +435,18 @@ monarch_jsplit32(const __grid_constant__ CUtensorMap tmQ,    // Q as rows of d, 
         // each forms 16 of the rows k.
         float cms[8];
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
+        for (int nt = 0; nt < 4; ++nt) {
+          cms[2 * nt] = cms[2 * nt + 1] = 0.f;
 #pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            cms[2 * nt + e] = 0.f;
+          for (int lt = 0; lt < LT; ++lt)
 #pragma unroll
-            for (int lt = 0; lt < LT; ++lt)
-#pragma unroll
-              for (int hh = 0; hh < 2; ++hh) {
-                s[lt][nt][2 * hh + e] *= inv[lt][hh];
-                cms[2 * nt + e] = fmaxf(cms[2 * nt + e], s[lt][nt][2 * hh + e]);
-              }
-          }
+            for (int hh = 0; hh < 2; ++hh) {
+              const float2 v = fmul2(row_pair(s[lt][nt], hh), both(inv[lt][hh]));
+              put_pair(s[lt][nt], hh, v);
+              cms[2 * nt] = fmaxf(cms[2 * nt], v.x);
+              cms[2 * nt + 1] = fmaxf(cms[2 * nt + 1], v.y);
+            }
+        }
         float cm = scatter_reduce<8, 16, 4>(cms, lane, warpmma::Max());     // of column 8 (g / 2) + 2 t + g % 2
         if constexpr (W == 2) {
           float* xm = reinterpret_cast<float*>(smem + L::X + jj * 256);
@@ -477,7 +464,7 @@ monarch_jsplit32(const __grid_constant__ CUtensorMap tmQ,    // Q as rows of d, 
 #pragma unroll
           for (int lt = 0; lt < LT; ++lt)
 #pragma unroll
-            for (int hh = 0; hh < 2; ++hh) w[lt][hh][nt] = M::pack(s[lt][nt][2 * hh] * gk[0], s[lt][nt][2 * hh + 1] * gk[1]);
+            for (int hh = 0; hh < 2; ++hh) w[lt][hh][nt] = M::pack(fmul2(row_pair(s[lt][nt], hh), make_float2(gk[0], gk[1])));
         }
         uint32_t pk[LT][2][4];     // A[k][l], the weights transposed: row tile kt, contraction step ls
         if constexpr (W == 2) {
@@ -501,9 +488,9 @@ monarch_jsplit32(const __grid_constant__ CUtensorMap tmQ,    // Q as rows of d, 
         float ic[LT][2], c1 = 0.f;
 #pragma unroll
         for (int kt = 0; kt < LT; ++kt) {
-          float cr[4] = {0.f, 0.f, 0.f, 0.f};
+          float cr[4];
 #pragma unroll
-          for (int ls = 0; ls < 2; ++ls) M::run(cr, pk[kt][ls], ones);
+          for (int ls = 0; ls < 2; ++ls) mma<__half>(ls == 0, cr, pk[kt][ls], ones);
           if (t == 2 * kt) c1 = cr[0];            // a division a lane
           if (t == 2 * kt + 1) c1 = cr[2];
         }
@@ -517,16 +504,16 @@ monarch_jsplit32(const __grid_constant__ CUtensorMap tmQ,    // Q as rows of d, 
           for (int ls = 0; ls < 2; ++ls) ldsm_x4_trans(bf[ls], swz(rq(16 * ls + (lane & 15), jj), 2 * vp + (lane >> 4)));
 #pragma unroll
           for (int kt = 0; kt < LT; ++kt) {
-            float o[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+            float o[2][4];
 #pragma unroll
             for (int ls = 0; ls < 2; ++ls) {
-              M::run(o[0], pk[kt][ls], bf[ls]);
-              M::run(o[1], pk[kt][ls], bf[ls] + 2);
+              mma<__half>(ls == 0, o[0], pk[kt][ls], bf[ls]);
+              mma<__half>(ls == 0, o[1], pk[kt][ls], bf[ls] + 2);
             }
             // alpha_R rows (k, j) over the alpha_L rows (whose readers have formed their scores)
-            stsm_x4(swz(rs(l0 + 16 * kt + (lane & 15), jj), 2 * vp + (lane >> 4)), M::pack(o[0][0] * ic[kt][0], o[0][1] * ic[kt][0]),
-                    M::pack(o[0][2] * ic[kt][1], o[0][3] * ic[kt][1]), M::pack(o[1][0] * ic[kt][0], o[1][1] * ic[kt][0]),
-                    M::pack(o[1][2] * ic[kt][1], o[1][3] * ic[kt][1]));
+            stsm_x4(swz(rs(l0 + 16 * kt + (lane & 15), jj), 2 * vp + (lane >> 4)), M::pack(fmul2(row_pair(o[0], 0), both(ic[kt][0]))),
+                    M::pack(fmul2(row_pair(o[0], 1), both(ic[kt][1]))), M::pack(fmul2(row_pair(o[1], 0), both(ic[kt][0]))),
+                    M::pack(fmul2(row_pair(o[1], 1), both(ic[kt][1]))));
           }
         }
       }

@@ -40,6 +40,9 @@ using warpmma::kLn2;
 using warpmma::kLog2e;
 using warpmma::ldsm_x4;
 using warpmma::ldsm_x4_trans;
+using warpmma::mma;
+using warpmma::put_pair;
+using warpmma::row_pair;
 using warpmma::lg2;
 using warpmma::movm_trans;
 using warpmma::quad_max;
@@ -48,6 +51,7 @@ using warpmma::scatter_reduce;
 constexpr int kThreads = 256, kWarps = 8, kRowBytes = 128, kMaxSmem = 227 * 1024;
 // where stmatrix rows past the end of a block go: eight rows of 16 bytes (nothing reads them)
 constexpr size_t kDumpBytes = 128;
+constexpr float kMasked = -3.0e38f;      // finite, and far below any logit
 
 // Four 8x8 16-bit matrices from accumulator-layout registers; lane L gives the address of row L & 7
 // of matrix L >> 3.
@@ -59,13 +63,9 @@ __device__ __forceinline__ void stsm_x4(uint32_t saddr, uint32_t r0, uint32_t r1
 
 // x rounded to f16 (hi) and the f16 rounding of what is left (lo): hi + lo carries 22 bits of x.
 template <bool HILO>
-__device__ __forceinline__ void split_hilo(float x0, float x1, uint32_t& hi, uint32_t& lo) {
-  hi = Mma<__half>::pack(x0, x1);
-  lo = 0u;
-  if (HILO) {
-    const float2 h = Mma<__half>::unpack(hi);
-    lo = Mma<__half>::pack(x0 - h.x, x1 - h.y);
-  }
+__device__ __forceinline__ void split_hilo(float2 x, uint32_t& hi, uint32_t& lo) {
+  hi = Mma<__half>::pack(x);
+  lo = HILO ? Mma<__half>::pack(ffma2(Mma<__half>::unpack(hi), both(-1.f), x)) : 0u;
 }
 
 // Tile layouts.  KS = number of 16-column steps a row holds (4: d <= 64, 5: d <= 80, 8: d <= 128).
@@ -244,10 +244,6 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
           const int j0 = 16 * rt;
           if (j0 >= b) continue;
           float s[BP / 8][4];
-#pragma unroll
-          for (int nt = 0; nt < BP / 8; ++nt)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) s[nt][e] = 0.f;
           const uint32_t a_u =
               sA_u + rowx<KS>(k, min(j0 + (lane & 7) + ((lane >> 3) & 1) * 8, b - 1), b, lane >> 4);
           uint32_t b_u[BP / 16];
@@ -263,8 +259,8 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
             for (int cp = 0; cp < BP / 16; ++cp) {
               uint32_t bf[4];
               ldsm_x4(bf, stp<KS>(b_u[cp], ks));
-              Mma<T>::run(s[2 * cp], a, bf);
-              Mma<T>::run(s[2 * cp + 1], a, bf + 2);
+              mma<T>(ks == 0, s[2 * cp], a, bf);
+              mma<T>(ks == 0, s[2 * cp + 1], a, bf + 2);
               if (HILO && !first) {      // + <alpha_R lo, K>
                 Mma<T>::run(s[2 * cp], al, bf);
                 Mma<T>::run(s[2 * cp + 1], al, bf + 2);
@@ -272,34 +268,35 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
             }
           }
           // rows j = j0 + g (c0, c1) and j0 + g + 8 (c2, c3); columns i = 8 nt + 2t, +1
+          // (columns past the block, which only the last two column tiles have, and keys past n_valid: a finite
+          // logit of weight 0, so that 0 log 0 = 0)
           float red[4], mxs[2];      // sum of the weights and of weight times logit, by row
+          const int lim = min(b, n_valid - k * b) - 2 * t;
 #pragma unroll
           for (int hh = 0; hh < 2; ++hh) {
-            float mx = -INFINITY;
+            float mx = kMasked;
 #pragma unroll
-            for (int nt = 0; nt < BP / 8; ++nt)
-#pragma unroll
-              for (int e = 0; e < 2; ++e) {
-                const int i = 8 * nt + 2 * t + e;
-                const bool valid = i < b && k * b + i < n_valid;
-                const float z = valid ? s[nt][2 * hh + e] * fl : -INFINITY;
-                s[nt][2 * hh + e] = z;
-                mx = fmaxf(mx, z);
+            for (int nt = 0; nt < BP / 8; ++nt) {
+              float2 z = fmul2(row_pair(s[nt], hh), both(fl));
+              if (nt >= BP / 8 - 2 || lim + 2 * t <= BP - 16) {
+                z.x = 8 * nt < lim ? z.x : kMasked;
+                z.y = 8 * nt + 1 < lim ? z.y : kMasked;
               }
+              put_pair(s[nt], hh, z);
+              mx = fmaxf(mx, fmaxf(z.x, z.y));
+            }
             mx = quad_max(mx);
-            float sum = 0.f, sz = 0.f;
+            float2 sum = both(0.f), sz = both(0.f);
 #pragma unroll
-            for (int nt = 0; nt < BP / 8; ++nt)
-#pragma unroll
-              for (int e = 0; e < 2; ++e) {
-                const float z = s[nt][2 * hh + e];
-                const float p = ex2(z - mx);                 // 0 for masked columns
-                s[nt][2 * hh + e] = p;
-                sum += p;
-                if (z > -INFINITY) sz = fmaf(p, z, sz);      // 0 log 0 = 0
-              }
-            red[2 * hh] = sum;
-            red[2 * hh + 1] = sz;
+            for (int nt = 0; nt < BP / 8; ++nt) {
+              const float2 z = row_pair(s[nt], hh), e = fadd2(z, both(-mx));
+              const float2 p = make_float2(ex2(e.x), ex2(e.y));
+              put_pair(s[nt], hh, p);
+              sum = nt ? fadd2(sum, p) : p;
+              sz = nt ? ffma2(p, z, sz) : fmul2(p, z);
+            }
+            red[2 * hh] = sum.x + sum.y;
+            red[2 * hh + 1] = sz.x + sz.y;
             mxs[hh] = mx;
           }
           {
@@ -322,9 +319,8 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
             if (HILO) {                // what the f16 rounding of the weights left out
 #pragma unroll
               for (int q = 0; q < 4; ++q) {
-                const float2 hi = Mma<T>::unpack(pa[rt][kk][q]);
-                const int nt = 2 * kk + (q >> 1), e0 = 2 * (q & 1);
-                pal[rt][kk][q] = Mma<T>::pack(s[nt][e0] - hi.x, s[nt][e0 + 1] - hi.y);
+                uint32_t hi;
+                split_hilo<HILO>(row_pair(s[2 * kk + (q >> 1)], q & 1), hi, pal[rt][kk][q]);
               }
             }
           }
@@ -348,35 +344,32 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
 #pragma unroll
           for (int rt = 0; rt < BP / 16; ++rt) {
             if (16 * rt >= b) continue;
-            float o[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-            float y[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+            float o[2][4], y[2][4];
 #pragma unroll
             for (int kk = 0; kk < BP / 16; ++kk) {
-              Mma<T>::run(o[0], pa[rt][kk], bk[kk]);
-              Mma<T>::run(o[1], pa[rt][kk], bk[kk] + 2);
+              mma<T>(kk == 0, o[0], pa[rt][kk], bk[kk]);
+              mma<T>(kk == 0, o[1], pa[rt][kk], bk[kk] + 2);
               if (HILO) {
                 Mma<T>::run(o[0], pal[rt][kk], bk[kk]);
                 Mma<T>::run(o[1], pal[rt][kk], bk[kk] + 2);
               }
               if (last) {
-                Mma<T>::run(y[0], pa[rt][kk], bv[kk]);
-                Mma<T>::run(y[1], pa[rt][kk], bv[kk] + 2);
+                mma<T>(kk == 0, y[0], pa[rt][kk], bv[kk]);
+                mma<T>(kk == 0, y[1], pa[rt][kk], bv[kk] + 2);
               }
             }
             const int j = 16 * rt + st_row;
             const uint32_t off = stp<KS>(rowx<KS>(k, j, b, st_nt), np);
-            const float i0 = inv_s[rt][0], i1 = inv_s[rt][1];
             uint32_t hi[4], lo[4];
-            split_hilo<HILO>(o[0][0] * i0, o[0][1] * i0, hi[0], lo[0]);
-            split_hilo<HILO>(o[0][2] * i1, o[0][3] * i1, hi[1], lo[1]);
-            split_hilo<HILO>(o[1][0] * i0, o[1][1] * i0, hi[2], lo[2]);
-            split_hilo<HILO>(o[1][2] * i1, o[1][3] * i1, hi[3], lo[3]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) split_hilo<HILO>(fmul2(row_pair(o[q >> 1], q & 1), both(inv_s[rt][q & 1])), hi[q], lo[q]);
             stsm_x4(j < b ? dstL_u + off : dump_u, hi[0], hi[1], hi[2], hi[3]);
             if (HILO) stsm_x4(j < b ? sALlo_u + off : dump_u, lo[0], lo[1], lo[2], lo[3]);
-            if (last)
-              stsm_x4(j < b ? sV_u + off : dump_u, Mma<T>::pack(y[0][0] * i0, y[0][1] * i0),
-                      Mma<T>::pack(y[0][2] * i1, y[0][3] * i1), Mma<T>::pack(y[1][0] * i0, y[1][1] * i0),
-                      Mma<T>::pack(y[1][2] * i1, y[1][3] * i1));
+            if (last) {
+#pragma unroll
+              for (int q = 0; q < 4; ++q) hi[q] = Mma<T>::pack(fmul2(row_pair(y[q >> 1], q & 1), both(inv_s[rt][q & 1])));
+              stsm_x4(j < b ? sV_u + off : dump_u, hi[0], hi[1], hi[2], hi[3]);
+            }
           }
         }
       }
@@ -394,7 +387,7 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
         for (int nt = 0; nt < MP / 8; ++nt)
 #pragma unroll
           for (int e = 0; e < 2; ++e)
-            c[nt][e] = sCL[min(8 * nt + 2 * t + e, m - 1) * b + j];
+            c[nt][e] = 8 * nt + 2 * t + e < m ? sCL[(8 * nt + 2 * t + e) * b + j] : kMasked;
         float pn[MP / 16][2][MP / 8][2];           // normalised weights [row tile][half][nt][e]
 #pragma unroll
         for (int rt = 0; rt < MP / 16; ++rt) {
@@ -407,10 +400,6 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
             continue;
           }
           float s[MP / 8][4];
-#pragma unroll
-          for (int nt = 0; nt < MP / 8; ++nt)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) s[nt][e] = 0.f;
           const uint32_t a_u =
               sQ_u + rowx<KS>(min(l0 + (lane & 7) + ((lane >> 3) & 1) * 8, m - 1), j, b, lane >> 4);
           uint32_t b_u[MP / 16];
@@ -425,8 +414,8 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
             for (int cp = 0; cp < MP / 16; ++cp) {
               uint32_t bf[4];
               ldsm_x4(bf, stp<KS>(b_u[cp], ks));
-              Mma<T>::run(s[2 * cp], a, bf);
-              Mma<T>::run(s[2 * cp + 1], a, bf + 2);
+              mma<T>(ks == 0, s[2 * cp], a, bf);
+              mma<T>(ks == 0, s[2 * cp + 1], a, bf + 2);
               if (HILO) {      // + <Q, alpha_L lo>
                 ldsm_x4(bf, stp<KS>(b_u[cp] - sAL_u + sALlo_u, ks));
                 Mma<T>::run(s[2 * cp], a, bf);
@@ -437,27 +426,23 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
           float inv_s[2], red[2], mxs[2];
 #pragma unroll
           for (int hh = 0; hh < 2; ++hh) {
-            float mx = -INFINITY;
+            float mx = kMasked;
 #pragma unroll
-            for (int nt = 0; nt < MP / 8; ++nt)
-#pragma unroll
-              for (int e = 0; e < 2; ++e) {
-                const float z = (8 * nt + 2 * t + e < m) ? fmaf(s[nt][2 * hh + e], fl, c[nt][e])
-                                                         : -INFINITY;
-                s[nt][2 * hh + e] = z;
-                mx = fmaxf(mx, z);
-              }
+            for (int nt = 0; nt < MP / 8; ++nt) {       // (blocks past m: c is kMasked, next to which the score is nothing)
+              const float2 z = ffma2(row_pair(s[nt], hh), both(fl), make_float2(c[nt][0], c[nt][1]));
+              put_pair(s[nt], hh, z);
+              mx = fmaxf(mx, fmaxf(z.x, z.y));
+            }
             mx = quad_max(mx);
-            float sum = 0.f;
+            float2 sum = both(0.f);
 #pragma unroll
-            for (int nt = 0; nt < MP / 8; ++nt)
-#pragma unroll
-              for (int e = 0; e < 2; ++e) {
-                const float p = ex2(s[nt][2 * hh + e] - mx);
-                s[nt][2 * hh + e] = p;
-                sum += p;
-              }
-            red[hh] = sum;
+            for (int nt = 0; nt < MP / 8; ++nt) {
+              const float2 e = fadd2(row_pair(s[nt], hh), both(-mx));
+              const float2 p = make_float2(ex2(e.x), ex2(e.y));
+              put_pair(s[nt], hh, p);
+              sum = nt ? fadd2(sum, p) : p;
+            }
+            red[hh] = sum.x + sum.y;
             mxs[hh] = mx;
           }
           {
@@ -492,18 +477,18 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
             __syncwarp();
 #pragma unroll
             for (int np = 0; np < ksteps; ++np) {
-              float o[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+              float o[2][4];
 #pragma unroll
               for (int kk = 0; kk < MP / 16; ++kk) {
                 uint32_t bf[4];
                 ldsm_x4_trans(bf, stp<KS>(y_u[kk], np));
-                Mma<T>::run(o[0], pa[kk], bf);
-                Mma<T>::run(o[1], pa[kk], bf + 2);
+                mma<T>(kk == 0, o[0], pa[kk], bf);
+                mma<T>(kk == 0, o[1], pa[kk], bf + 2);
               }
-              stsm_x4(l < m ? stp<KS>(row_u, np) : dump_u, Mma<T>::pack(o[0][0] * inv_s[0], o[0][1] * inv_s[0]),
-                      Mma<T>::pack(o[0][2] * inv_s[1], o[0][3] * inv_s[1]),
-                      Mma<T>::pack(o[1][0] * inv_s[0], o[1][1] * inv_s[0]),
-                      Mma<T>::pack(o[1][2] * inv_s[1], o[1][3] * inv_s[1]));
+              uint32_t u[4];
+#pragma unroll
+              for (int q = 0; q < 4; ++q) u[q] = Mma<T>::pack(fmul2(row_pair(o[q >> 1], q & 1), both(inv_s[q & 1])));
+              stsm_x4(l < m ? stp<KS>(row_u, np) : dump_u, u[0], u[1], u[2], u[3]);
             }
             __syncwarp();
           } else {
@@ -511,10 +496,11 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
             for (int hh = 0; hh < 2; ++hh) {
               const bool row_ok = l0 + g + 8 * hh < m;     // rows past the block must not count
 #pragma unroll
-              for (int nt = 0; nt < MP / 8; ++nt)
-#pragma unroll
-                for (int e = 0; e < 2; ++e)
-                  pn[rt][hh][nt][e] = row_ok ? s[nt][2 * hh + e] * inv_s[hh] : 0.f;
+              for (int nt = 0; nt < MP / 8; ++nt) {
+                const float2 v = fmul2(row_pair(s[nt], hh), both(inv_s[hh]));
+                pn[rt][hh][nt][0] = row_ok ? v.x : 0.f;
+                pn[rt][hh][nt][1] = row_ok ? v.y : 0.f;
+              }
             }
           }
         }
@@ -555,26 +541,23 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
             for (int e = 0; e < 2; ++e) gk[e] = __shfl_sync(0xffffffffu, gl, (2 * nt + e) * kColStep + t);
             // column sums of the weights AS ROUNDED to 16 bit: numerator (the MMA below) and
             // denominator of the weighted mean must see the same weights
-            float c0 = 0.f, c1 = 0.f;
+            float2 c2 = both(0.f);
 #pragma unroll
             for (int rt = 0; rt < MP / 16; ++rt)
 #pragma unroll
               for (int hh = 0; hh < 2; ++hh) {
-                const uint32_t u = Mma<T>::pack(pn[rt][hh][nt][0] * gk[0], pn[rt][hh][nt][1] * gk[1]);
+                uint32_t u, ul;
+                split_hilo<HILO>(fmul2(make_float2(pn[rt][hh][nt][0], pn[rt][hh][nt][1]), make_float2(gk[0], gk[1])), u, ul);
                 tp[rt][hh][nt] = u;
                 float2 f = Mma<T>::unpack(u);
                 if (HILO) {      // the pair carries the weight to 22 bits; c_R sums what the MMAs will see
-                  const uint32_t ul = Mma<T>::pack(pn[rt][hh][nt][0] * gk[0] - f.x, pn[rt][hh][nt][1] * gk[1] - f.y);
                   tpl[rt][hh][nt] = ul;
-                  const float2 fl2 = Mma<T>::unpack(ul);
-                  f.x += fl2.x;
-                  f.y += fl2.y;
+                  f = fadd2(f, Mma<T>::unpack(ul));
                 }
-                c0 += f.x;
-                c1 += f.y;
+                c2 = rt + hh ? fadd2(c2, f) : f;
               }
-            cs[2 * nt] = c0;
-            cs[2 * nt + 1] = c1;
+            cs[2 * nt] = c2.x;
+            cs[2 * nt + 1] = c2.y;
           }
           const float cr = scatter_reduce<kCols, 16, 4>(cs, lane, warpmma::Add());
           const float icl = cr > 1e-30f ? 1.f / cr : 0.f;
@@ -607,23 +590,21 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
             const uint32_t row_u = sAR_u + rowx<KS>(kr, j, b, st_nt);
 #pragma unroll
             for (int np = 0; np < ksteps; ++np) {
-              float o[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+              float o[2][4];
 #pragma unroll
               for (int ls = 0; ls < MP / 16; ++ls) {
                 uint32_t bf[4];   // B[kk = l][n = v] = Q(l,j)[v], read transposed; two 8-column tiles
                 ldsm_x4_trans(bf, stp<KS>(q_u[ls], np));
-                Mma<T>::run(o[0], pa[ls], bf);
-                Mma<T>::run(o[1], pa[ls], bf + 2);
+                mma<T>(ls == 0, o[0], pa[ls], bf);
+                mma<T>(ls == 0, o[1], pa[ls], bf + 2);
                 if (HILO) {
                   Mma<T>::run(o[0], pal[ls], bf);
                   Mma<T>::run(o[1], pal[ls], bf + 2);
                 }
               }
               uint32_t hi[4], lo[4];
-              split_hilo<HILO>(o[0][0] * ic[0], o[0][1] * ic[0], hi[0], lo[0]);
-              split_hilo<HILO>(o[0][2] * ic[1], o[0][3] * ic[1], hi[1], lo[1]);
-              split_hilo<HILO>(o[1][0] * ic[0], o[1][1] * ic[0], hi[2], lo[2]);
-              split_hilo<HILO>(o[1][2] * ic[1], o[1][3] * ic[1], hi[3], lo[3]);
+#pragma unroll
+              for (int q = 0; q < 4; ++q) split_hilo<HILO>(fmul2(row_pair(o[q >> 1], q & 1), both(ic[q & 1])), hi[q], lo[q]);
               stsm_x4(kr < m ? stp<KS>(row_u, np) : dump_u, hi[0], hi[1], hi[2], hi[3]);
               if (HILO) stsm_x4(kr < m ? stp<KS>(row_u - sAR_u + sARlo_u, np) : dump_u, lo[0], lo[1], lo[2], lo[3]);
             }

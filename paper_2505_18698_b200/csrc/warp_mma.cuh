@@ -59,6 +59,19 @@ template <> struct Mma<__nv_bfloat16> {
   }
 };
 
+// c = a b where `fresh`, else c += a b.
+template <typename T>
+__device__ __forceinline__ void mma(bool fresh, float* c, const uint32_t* a, const uint32_t* b) {
+  if (fresh) Mma<T>::first(c, a, b);
+  else Mma<T>::run(c, a, b);
+}
+// The two rows of an accumulator tile, as pairs.
+__device__ __forceinline__ float2 row_pair(const float* c, int hh) { return make_float2(c[2 * hh], c[2 * hh + 1]); }
+__device__ __forceinline__ void put_pair(float* c, int hh, float2 v) {
+  c[2 * hh] = v.x;
+  c[2 * hh + 1] = v.y;
+}
+
 // Lets a kernel use up to `bytes` of dynamic shared memory: once per kernel and device (the call
 // costs most of a microsecond of host time).
 struct SmemOptIn {
