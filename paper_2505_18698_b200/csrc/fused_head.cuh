@@ -26,6 +26,8 @@
 #pragma once
 #include <cuda.h>
 
+#include <algorithm>
+
 #include "status_word.cuh"
 #include "tensor_path.cuh"
 #include "warp_mma.cuh"
@@ -47,7 +49,7 @@ using warpmma::movm_trans;
 using warpmma::quad_max;
 using warpmma::scatter_reduce;
 
-constexpr int kMaxThreads = 512, kMaxSmem = 227 * 1024, kMaxBlocks = 32;
+constexpr int kMaxSmem = 227 * 1024, kMaxBlocks = 32;
 constexpr float kMasked = -3.0e38f;      // finite, and far below any score
 
 struct Params {
@@ -63,7 +65,7 @@ struct Params {
   float scale;
 };
 struct __align__(16) Bars {
-  uint64_t full[2][kMaxBlocks];      // by buffer and block
+  uint64_t full[2][kMaxBlocks];      // by buffer (V over the states: the second set is V's) and block
 };
 
 __device__ __forceinline__ void stsm_x4(uint32_t saddr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
@@ -77,6 +79,11 @@ __device__ __forceinline__ void load_5d(uint32_t dst, const CUtensorMap* tm, uin
           dst),
       "l"((uint64_t)tm), "r"(smem_u32(bar)), "r"(0), "r"(blk), "r"(h0), "r"(h1)
       : "memory");
+}
+__device__ __forceinline__ void prefetch_5d(const CUtensorMap* tm, int blk, int h0, int h1) {
+  asm volatile("cp.async.bulk.prefetch.tensor.5d.L2.global [%0, {%1, %1, %2, %3, %4}];" ::"l"((uint64_t)tm), "r"(0), "r"(blk), "r"(h0),
+               "r"(h1)
+               : "memory");
 }
 // Four 8 x 8 pieces of an accumulator pair (two 8-column tiles of 16 rows) as 16-bit rows.
 __device__ __forceinline__ void put(uint32_t addr, const float (&o)[2][4], float m0, float m1) {
@@ -140,31 +147,40 @@ __device__ __forceinline__ void products(float (&o)[2][4], const uint32_t (&a)[K
     }
 }
 
+// What a kernel is for: one round; more, with a state tile beside Q, K and V; more, with V over the states once the last round
+// has read them (three tiles a head).
+enum Rounds { kOne = 0, kMore = 1, kMoreVLast = 2 };
+// Warps an SM has room for.  Two 8-column tiles either way fit 64 registers (nothing is spilled), 24 warps' 80 the other one-round
+// kernels and 24 x 16 (at most 16 bytes), the rest take 128.
+constexpr int max_warps(int nb, int nm, int rounds) { return nb == 2 && nm == 2 ? 32 : (rounds == kOne || (nb == 3 && nm == 2) ? 24 : 16); }
+
 // Shared memory of a CTA: `bufs` x (Q, K, V), the state tile (more than one round), a dump for matrix-store rows past a
 // block (a line of its own: addresses step through a row by an exclusive or of bits 5 and 6), c_L ([position]
 // [nm * 8 blocks]), barriers.
-inline size_t smem_bytes(int tile, int bufs, bool multi, int b, int nm) {
-  return (size_t)tile * (3 * bufs + (multi ? 1 : 0)) + 128 + (size_t)b * nm * 8 * 4 + sizeof(Bars) + 1024;
+inline size_t smem_bytes(int tile, int bufs, int rounds, int b, int nm) {
+  return (size_t)tile * (rounds == kMoreVLast ? 3 : 3 * bufs + (rounds == kMore ? 1 : 0)) + 128 + (size_t)b * nm * 8 * 4 + sizeof(Bars) + 1024;
 }
 
 // NB, NM: 8-column tiles that hold b keys / m blocks.
-template <typename TIn, int NB, int NM, bool MULTI>
-__global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __grid_constant__ Params P) {
+template <typename TIn, int NB, int NM, int ROUNDS>
+__global__ void __launch_bounds__(32 * max_warps(NB, NM, ROUNDS), 1) monarch_fused_head(const __grid_constant__ Params P) {
   typedef Mma<__half> M;
+  constexpr bool MULTI = ROUNDS != kOne, V_LAST = ROUNDS == kMoreVLast;
   constexpr int RB = (NB + 1) / 2, RM = (NM + 1) / 2;      // 16-row tiles
   extern __shared__ uint8_t smem_raw[];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const int tile = P.tile, b = P.b, bp = P.bp;
   const uint32_t s0 = smem_u32(smem);
-  const uint32_t sS = s0 + 3 * P.bufs * tile;              // state tile (MULTI)
-  uint8_t* tail = smem + (3 * P.bufs + (MULTI ? 1 : 0)) * tile;
+  const int tiles = V_LAST ? 3 : 3 * P.bufs + (MULTI ? 1 : 0);
+  const uint32_t sS = s0 + (tiles - 1) * tile;             // state tile (MULTI)
+  uint8_t* tail = smem + tiles * tile;
   float* sCL = reinterpret_cast<float*>(tail + 128);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const uint32_t dump = smem_u32(tail) + (lane & 7) * 16;
   Bars* bars = reinterpret_cast<Bars*>(sCL + b * NM * 8);
   if (tid == 0) {
-    for (int i = 0; i < P.bufs; ++i)
+    for (int i = 0; i < (V_LAST ? 2 : P.bufs); ++i)
       for (int k = 0; k < P.m; ++k) mbar_init(&bars->full[i][k], 1);
     tensor::fence_barrier_init();
   }
@@ -186,19 +202,39 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
     for (int k = warp; k < m; k += nw) {
       uint64_t* bar = &bars->full[buf][k];
       const uint32_t dst = s0 + 3 * buf * tile + k * bp * 128;
-      mbar_expect_tx(bar, 3 * bp * 128);
+      mbar_expect_tx(bar, (V_LAST ? 2 : 3) * bp * 128);
       load_5d(dst, &P.q, bar, k, h0, h1);
       load_5d(dst + tile, &P.k, bar, k, h0, h1);
-      load_5d(dst + 2 * tile, &P.v, bar, k, h0, h1);
+      if (!V_LAST) load_5d(dst + 2 * tile, &P.v, bar, k, h0, h1);
+      else prefetch_5d(&P.v, k, h0, h1);
+    }
+  };
+  // bf16: to f16 in place, `n` operands of a block, a tile apart.
+  auto convert = [&](uint32_t block, int n) {
+    if (Mma<TIn>::is_f16) return;
+    for (int e = lane; e < b * 8; e += 32) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        if (a >= n) break;
+        uint4* p = reinterpret_cast<uint4*>(smem + (block - s0) + a * tile + e * 16);
+        *p = warpmma::to_f16x8(*p, (const TIn*)nullptr);
+      }
     }
   };
   request(blockIdx.x, 0);
   int buf = 0;
   uint32_t par = 0;                 // bit 16 buf + r: parity of the warp's r-th block in that buffer
   constexpr uint32_t kDead = 1u << 31;      // in `par`: a wait ran out; the warp waits no more and leaves after this head
+  auto landed = [&](uint64_t* bar, int bit) {
+    if (!(par & kDead) && !tensor::mbar_wait(bar, (par >> bit) & 1)) {
+      tensor::report_timeout(P.status, 2);
+      par |= kDead;
+    }
+    par ^= 1u << bit;
+  };
   for (int h = blockIdx.x; h < P.BH; h += gridDim.x) {
-    if (P.bufs == 2) request(h + gridDim.x, buf ^ 1);
-    const uint32_t sQ = s0 + 3 * buf * tile, sK = sQ + tile, sV = sK + tile;
+    if (!V_LAST && P.bufs == 2) request(h + gridDim.x, buf ^ 1);
+    const uint32_t sQ = s0 + 3 * buf * tile, sK = sQ + tile, sV = V_LAST ? sS : sK + tile;
     const int n_valid = valid_of(h);
     const int m = P.seq_len != nullptr ? (n_valid + b - 1) / b : P.m;
     const size_t head_base = P.H == 0 ? (size_t)h * P.N * P.d : ((size_t)(h / P.H) * P.N * P.H + (h % P.H)) * P.d;
@@ -207,26 +243,14 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
       const bool first = !MULTI || step == 1, last = !MULTI || step == P.T;
       // ================================================================ R half-step (Eq. 7, 9, 10)
       for (int k = warp, r = 0; k < m; k += nw, ++r) {
+        const int r0 = k * bp;
         if (first) {
-          if (!(par & kDead) && !tensor::mbar_wait(&bars->full[buf][k], (par >> (16 * buf + r)) & 1)) {
-            tensor::report_timeout(P.status, 2);
-            par |= kDead;
-          }
-          par ^= 1u << (16 * buf + r);
-          if (!Mma<TIn>::is_f16) {      // bf16: to f16 in place, the block's three operands
-            for (int e = lane; e < b * 8; e += 32) {
-#pragma unroll
-              for (int a = 0; a < 3; ++a) {
-                uint4* p = reinterpret_cast<uint4*>(smem + (sQ - s0) + a * tile + (k * bp) * 128 + e * 16);
-                *p = warpmma::to_f16x8(*p, (const TIn*)nullptr);
-              }
-            }
-          }
+          landed(&bars->full[buf][k], 16 * buf + r);
+          convert(sQ + r0 * 128, V_LAST ? 2 : 3);
           __syncwarp();
         }
         const uint32_t sA = first ? sQ : sS;                 // alpha_R (= Q rows while L is the identity)
-        const uint32_t dst = MULTI ? sS : sK;                // alpha_L
-        const int r0 = k * bp;
+        const uint32_t dst = !MULTI || (V_LAST && last) ? sK : sS;      // alpha_L
         const int lim = min(b, n_valid - k * b);             // keys of this block that count
         uint32_t pa[RB][RB][4];                              // unnormalised weights: the largest is exactly 1
         float inv[RB][2], off[2 * RB], red[4 * RB];          // red: sum of the weights, sum of weight times score
@@ -300,6 +324,14 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
           // -c_L log2 e = log2 sum + max - sum R z (Eq. 10), the addend of the L logits
           if ((RB == 2 || (t & 1)) && j < b) sCL[j * NM * 8 + k] = lg2(so) - mo - fl * (sz * io);
         }
+        if (V_LAST && last) {      // the block's rows of alpha_R have been read, V takes their place
+          tensor::fence_proxy_async();
+          __syncwarp();
+          if (lane == 0 && !(par & kDead)) {
+            mbar_expect_tx(&bars->full[1][k], bp * 128);
+            load_5d(sV + r0 * 128, &P.v, &bars->full[1][k], k, P.H ? h % P.H : h, P.H ? h / P.H : 0);
+          }
+        }
         __syncwarp();
         // second products, 16 columns at a time; a warp alone reads and writes the rows of its block
         uint32_t kt[RB], st[RB];
@@ -320,7 +352,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
           for (int kk = 0; kk < RB; ++kk) {
             const uint32_t ad = kt[kk] ^ (np << 5);
             ldsm_x4_trans(bk[kk], ad);
-            if (last) ldsm_x4_trans(bv[kk], ad + to_v);
+            if (!V_LAST && last) ldsm_x4_trans(bv[kk], ad + to_v);
           }
           __syncwarp();
 #pragma unroll
@@ -328,7 +360,25 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
             float o[2][4];
             products<RB>(o, pa[rt], bk);
             put(st[rt] ^ (np << 5), o, inv[rt][0], inv[rt][1]);
-            if (last) {
+            if (!V_LAST && last) {
+              products<RB>(o, pa[rt], bv);
+              put(sy[rt] ^ (np << 5), o, inv[rt][0], inv[rt][1]);
+            }
+          }
+        }
+        if (V_LAST && last) {
+          landed(&bars->full[1][k], 16 + r);
+          convert(sV + r0 * 128, 1);
+          __syncwarp();
+#pragma unroll
+          for (int np = 0; np < 4; ++np) {
+            uint32_t bv[RB][4];
+#pragma unroll
+            for (int kk = 0; kk < RB; ++kk) ldsm_x4_trans(bv[kk], (kt[kk] ^ (np << 5)) + to_v);
+            __syncwarp();
+#pragma unroll
+            for (int rt = 0; rt < RB; ++rt) {
+              float o[2][4];
               products<RB>(o, pa[rt], bv);
               put(sy[rt] ^ (np << 5), o, inv[rt][0], inv[rt][1]);
             }
@@ -339,7 +389,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
 
       // ================================================================ L half-step (Eq. 8, 9 / Eq. 4)
       for (int j = warp; j < b; j += nw) {
-        const uint32_t sA = MULTI ? sS : sK;                 // alpha_L
+        const uint32_t sA = !MULTI || (V_LAST && last) ? sK : sS;       // alpha_L
         float c[NM][2];
 #pragma unroll
         for (int nt = 0; nt < NM; ++nt) {
@@ -525,7 +575,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) monarch_fused_head(const __gri
       tensor::let_copies_land();
       return;
     }
-    if (P.bufs == 2) buf ^= 1;
+    if (!V_LAST && P.bufs == 2) buf ^= 1;
     else request(h + gridDim.x, 0);
   }
 }
@@ -534,42 +584,51 @@ inline bool shape_ok(int d, int b, int m, int dtype) {
   return (dtype == 1 || dtype == 2) && d % 8 == 0 && d <= 64 && b > 8 && b <= 32 && m > 8 && m <= 32;
 }
 struct Plan {
-  int bp, tile, bufs, warps, ctas;      // ctas: per SM
+  int bp, tile, bufs, warps, ctas, rounds;      // ctas: per SM
   size_t smem;
 };
 inline bool plan(int b, int m, int T, int BH, int num_sms, Plan* p) {
-  const int nm = (m + 7) / 8;
-  const bool multi = T > 1;
+  const int nb = (b + 7) / 8, nm = (m + 7) / 8, rounds = T > 1 ? kMore : kOne;
   // The odd pitch where it fits; without it the L half-step's rows conflict (8-way for b = 16, 24, 32,
   // which the general kernel then serves faster: N = 576 as 24 x 24, 768 heads, 120 against 125 us).
   for (int odd = 1; odd >= (b % 8 != 0 ? 0 : 1); --odd) {
     p->bp = odd ? (b | 1) : b;
     p->tile = (m * p->bp * 128 + 1023) / 1024 * 1024;
-    const size_t one = smem_bytes(p->tile, 1, multi, b, nm), two = smem_bytes(p->tile, 2, multi, b, nm);
-    if (one > (size_t)kMaxSmem) continue;
-    const int fit = (int)((size_t)(227 * 1024) / (one + 1024));      // CTAs per SM by shared memory
-    // At most one head per SM: one CTA with as many warps as a half-step has tiles.  More: the 16 warps
-    // an SM holds (128 registers) go to as many CTAs as fit, up to three, each with a head of its own
-    // (768 heads of 130 = 13 x 10, two rounds: 34.6 us with three, 39.8 with two); except that where no
-    // third fits and there are heads left for a second turn, one CTA of all 16 with the next head's
-    // loads under way is faster (768 heads of 256 = 16 x 16: 25.6 against 27.4 us).
-    p->ctas = BH <= num_sms ? 1 : (fit < 3 ? fit : 3);
+    p->rounds = rounds;
     p->bufs = 1;
-    if (p->ctas <= 2 && BH > p->ctas * num_sms && two <= (size_t)kMaxSmem) {
-      p->ctas = 1;
-      p->bufs = 2;
+    const size_t two = smem_bytes(p->tile, 2, rounds, b, nm);
+    p->smem = smem_bytes(p->tile, 1, rounds, b, nm);
+    if (p->smem > (size_t)kMaxSmem) continue;
+    auto fit = [](size_t bytes) { return (int)((size_t)(227 * 1024) / (bytes + 1024)); };      // CTAs per SM by shared memory
+    // At most one head per SM: one CTA with as many warps as a half-step has tiles.  More: the warps an SM holds go to
+    // as many CTAs as fit, up to three, each with a head of its own (768 heads of 130 = 13 x 10, two rounds: 34.6 us with
+    // three, 39.8 with two).  Where no third fits and there are heads left for a second turn, one CTA of all warps
+    // with the next head's loads under way is faster with 16 warps an SM (it has the same work in flight), with 32 two
+    // CTAs are, and V goes over the states where that makes room for the second.
+    p->ctas = BH <= num_sms ? 1 : std::min(fit(p->smem), 3);
+    const int most = max_warps(nb, nm, rounds);
+    if (p->ctas <= 2 && BH > p->ctas * num_sms) {
+      const size_t v_last = smem_bytes(p->tile, 1, kMoreVLast, b, nm);
+      if (most == 32 && p->ctas == 2) {
+      } else if (most == 32 && rounds == kMore && fit(v_last) >= 2) {
+        p->ctas = 2;
+        p->rounds = kMoreVLast;
+        p->smem = v_last;
+      } else if (two <= (size_t)kMaxSmem) {
+        p->ctas = 1;
+        p->bufs = 2;
+        p->smem = two;
+      }
     }
-    const int most = 16 / p->ctas;
     // the fewest warps that take the fewest rounds of tiles over both half-steps
     int best = 1 << 30;
-    for (int w = 1; w <= most; ++w) {
-      const int rounds = (m + w - 1) / w + (b + w - 1) / w;
-      if (rounds < best) {
-        best = rounds;
+    for (int w = 1; w <= most / p->ctas; ++w) {
+      const int turns = (m + w - 1) / w + (b + w - 1) / w;
+      if (turns < best) {
+        best = turns;
         p->warps = w;
       }
     }
-    p->smem = p->bufs == 2 ? two : one;
     return true;
   }
   return false;
@@ -639,9 +698,9 @@ inline bool get_maps(Params* P, const Args& a, const Plan& p, int dev) {
   P->v = c.maps[e][2];
   return true;
 }
-template <typename TIn, int NB, int NM, bool MULTI>
+template <typename TIn, int NB, int NM, int ROUNDS>
 inline int launch_k(const Params& P, const Plan& p, int num_sms, cudaStream_t st) {
-  auto kern = monarch_fused_head<TIn, NB, NM, MULTI>;
+  auto kern = monarch_fused_head<TIn, NB, NM, ROUNDS>;
   static warpmma::SmemOptIn opt_in;
   if (!opt_in.done((const void*)kern, kMaxSmem)) return 7;
   cudaLaunchAttribute attr;
@@ -657,14 +716,19 @@ inline int launch_k(const Params& P, const Plan& p, int num_sms, cudaStream_t st
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, P) == cudaSuccess ? 0 : 7;
 }
-template <typename TIn, bool MULTI>
+template <typename TIn, int ROUNDS>
 inline int launch_n(const Params& P, const Plan& p, int num_sms, cudaStream_t st) {
   const int nb = (P.b + 7) / 8, nm = (P.m + 7) / 8;
 #define MA_FH(B)                                            \
-  (nm == 2 ? launch_k<TIn, B, 2, MULTI>(P, p, num_sms, st)  \
-           : (nm == 3 ? launch_k<TIn, B, 3, MULTI>(P, p, num_sms, st) : launch_k<TIn, B, 4, MULTI>(P, p, num_sms, st)))
+  (nm == 2 ? launch_k<TIn, B, 2, ROUNDS>(P, p, num_sms, st) \
+           : (nm == 3 ? launch_k<TIn, B, 3, ROUNDS>(P, p, num_sms, st) : launch_k<TIn, B, 4, ROUNDS>(P, p, num_sms, st)))
   return nb == 2 ? MA_FH(2) : (nb == 3 ? MA_FH(3) : MA_FH(4));
 #undef MA_FH
+}
+template <typename TIn>
+inline int launch_t(const Params& P, const Plan& p, int num_sms, cudaStream_t st) {
+  if (p.rounds == kMoreVLast) return launch_k<TIn, 2, 2, kMoreVLast>(P, p, num_sms, st);
+  return p.rounds == kMore ? launch_n<TIn, kMore>(P, p, num_sms, st) : launch_n<TIn, kOne>(P, p, num_sms, st);
 }
 int launch(const Args& a, cudaStream_t st) {
   static int sms[64] = {};
@@ -679,8 +743,7 @@ int launch(const Args& a, cudaStream_t st) {
   P.BH = a.BH; P.N = a.N; P.d = a.d; P.b = a.b; P.m = a.m; P.T = a.T; P.H = a.H; P.heads = a.heads; P.n_valid = a.n_valid;
   P.bp = p.bp; P.tile = p.tile; P.bufs = p.bufs;
   P.scale = a.scale;
-  if (a.dtype == 1) return a.T > 1 ? launch_n<__half, true>(P, p, sms[dev], st) : launch_n<__half, false>(P, p, sms[dev], st);
-  return a.T > 1 ? launch_n<__nv_bfloat16, true>(P, p, sms[dev], st) : launch_n<__nv_bfloat16, false>(P, p, sms[dev], st);
+  return a.dtype == 1 ? launch_t<__half>(P, p, sms[dev], st) : launch_t<__nv_bfloat16>(P, p, sms[dev], st);
 }
 #endif  // MA_TU_FUSED_HEAD
 
