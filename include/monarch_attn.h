@@ -101,9 +101,9 @@ size_t monarch_attn_workspace_bytes(int batch, int heads, int N, int d, int b, i
  *
  * Concurrency.  A workspace serves one call at a time: calls that may overlap on the GPU (different
  * streams, no dependency) need a workspace each, and monarch_attn_fwd's library-owned workspace
- * serves one call in flight per device.  The persistent kernels (MA_PATH_TENSOR,
- * MA_PATH_TENSOR_TMEM; what AUTO picks for d = 64, m = b in {32, 64, 128}) deal their tiles out
- * statically over one CTA per SM and the CTAs wait for each other's results, so such a launch only
+ * serves one call in flight per device.  The persistent kernels (MA_PATH_TENSOR, from 1024 tiles of 128 rows at b = 64 on
+ * excepted: those take tiles as they come to them; MA_PATH_TENSOR_TMEM; what AUTO picks for d = 64, m = b in {32, 64, 128}) deal
+ * their tiles out statically over one CTA per SM and the CTAs wait for each other's results, so such a launch only
  * makes progress with every CTA resident: it needs the whole GPU.  The library chains these
  * launches per device with an event, so two of them never share the SMs whatever streams they are
  * on; a foreign kernel that holds SMs for longer than the bound of the device-side waits (about a

@@ -32,8 +32,8 @@ int monarch_attn_set_trace_buffer(void* device_buffer, size_t bytes);
 int monarch_attn_debug_knob(int knob, long long value);
 
 /* Which set of kernels served the last successful call on this host thread: "generic", "fused_small", "fused_head",
- * "fused_f32", "jsplit", "tile_mma", "tile_tc", "tensor_decoupled", "tensor_tmem", "tensor_basic" ("" before the first).
- * Two of the paths of monarch_attn.h have two sets each, chosen by size. */
+ * "fused_f32", "jsplit", "tile_mma", "tile_tc", "tensor_decoupled", "tensor_chain", "tensor_tmem", "tensor_basic" ("" before the first).
+ * Three of the paths of monarch_attn.h have two sets each, chosen by size. */
 const char* monarch_attn_last_kernels(void);
 
 #ifdef __cplusplus

@@ -347,7 +347,7 @@ static int launch_resolved(const void* Q, const void* K, const void* V, void* Y,
     kernels = "tensor_basic";
     rc = tensor::launch(Q, K, V, Y, p.BH, p.N, p.d, p.b, p.T, p.dtype, scale, ws, status.report, st, &launches);
   } else {
-    kernels = resolved == MA_PATH_TENSOR_TMEM ? "tensor_tmem" : "tensor_decoupled";
+    kernels = resolved == MA_PATH_TENSOR_TMEM ? "tensor_tmem" : (tp::chain_chosen(p.BH, p.N, p.b) ? "tensor_chain" : "tensor_decoupled");
     rc = tp::launch(Q, K, V, Y, p.BH, p.N, p.b, p.T, p.dtype, scale, ws, st, &launches,
                     resolved == MA_PATH_TENSOR_TMEM ? 1 : 0,
                     ws_armed, status.report, p.H, p.lse, p.n_valid < p.N ? p.n_valid : 0);

@@ -18,11 +18,12 @@
 // other in place in a state tile.  Arithmetic is f16 whatever the input type (see fused_small.cuh).
 //
 // Measured (B200, us per call, against the general per-head kernel): 768 heads of 256 = 16 x 16, one
-// round 25.2 / 27.7 (61 % of the copy bandwidth); 768 of 210 = 15 x 14, two rounds 41.5 / 47.7; 384 of
-// lengths up to 384 = 16 x 24 23.4 / 28.9; 720 of 396 = 22 x 18 64 / 97; 24 of 210 5 / 7.  Row and column
+// round 23.8 / 27.7 (65 % of the copy bandwidth); 768 of 210 = 15 x 14, two rounds 36.3 / 47.7; 384 of
+// lengths up to 384 = 16 x 24 24.1 / 28.9; 720 of 396 = 22 x 18 64 / 97; 24 of 210 5 / 7.  Row and column
 // reductions that halve the values a lane carries, with one division a lane, took 3 % (16 x 16) to 11 %
-// (10 x 24, two rounds) off.  What is left is instruction issue and shared-memory latency at four warps
-// per scheduler, and the last of six turns of heads, which few SMs take.
+// (10 x 24, two rounds) off.  The tiles wait on latencies: 32 warps with two heads at work, where two 8-column tiles either way
+// fit 64 registers, took 41 to 36.3 us (15 x 14, two rounds) and 24.8 to 23.8 (16 x 16, one).  What is left is latency at four to eight
+// warps per scheduler, and the last turn of heads, which few SMs take.
 #pragma once
 #include <cuda.h>
 

@@ -11,8 +11,9 @@
 // This header holds what the kernels share: the parameter block (tensor maps, state arrays,
 // counters), the tile iterator, bounded waits and small PTX wrappers, and the host-side set-up
 // (workspace layout, tensor maps cached per problem, launch).  The kernels themselves are in
-// tensor_decoupled.cuh (operand rings in shared memory, P through shared memory) and
-// tensor_tmem.cuh (P handed to the apply MMA through tensor memory).
+// tensor_decoupled.cuh (operand rings in shared memory, P through shared memory),
+// tensor_tmem.cuh (P handed to the apply MMA through tensor memory) and tensor_chain.cuh (many tiles in flight, taken from the
+// list as CTAs come to them, so that it does not need the whole GPU).
 #pragma once
 #include <mutex>
 
@@ -189,6 +190,14 @@ template <typename T, int B, int SB>
 cudaError_t launch_decoupled(const Params& P, int grid, cudaStream_t st);
 template <typename T, int B>
 cudaError_t launch_tmem(const Params& P, int grid, cudaStream_t st);
+//   launch_chain:     tensor_chain.cuh, SB == B == 64
+template <typename T>
+cudaError_t launch_chain(const Params& P, int grid, cudaStream_t st);
+// Whether MA_PATH_TENSOR runs the kernel of tensor_chain.cuh and not that of tensor_decoupled.cuh (by size alone: either layout
+// gives the same bits).  Measured over heads of 4096 in loops of tenths of a second, us (this one / that one): two
+// rounds: 16 heads 39.4 / 37.0, 24 43.7 / 44.4, 32 48.6 / 50.8, 64 82 / 90, one round: 32 31.3 / 30.8, 48 39.0 / 41.0; two rounds in the other
+// layout or masked, where that one is a fifth slower: 36 57.9 / 68.4, 48 68.0 / 76.7.
+inline bool chain_chosen(int BH, int N, int b) { return b == 64 && (long long)BH * N / kRows >= 1024; }      // tiles of a half-step
 
 // mode 0: kernel of tensor_decoupled.cuh; mode 1: kernel of tensor_tmem.cuh (m = b in {64, 128},
 // plain calls only: no [batch][N][heads][d] layout, no row log-sum-exp, no padding mask).
@@ -249,6 +258,17 @@ struct PersistentChain {      // one event per device: the end of the last persi
   }
   bool recorded() const { const int d = dev(); return d >= 0 && rec[d]; }
   void set_recorded() { const int d = dev(); if (d >= 0) rec[d] = true; }
+  // A launch that does not need the whole GPU goes after one that does and has not finished: a steady stream of them might
+  // otherwise keep that one's CTAs, which take a whole SM, from coming in.
+  bool let_pending_pass(cudaStream_t st) {
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (!recorded()) return true;
+    if (cudaStreamIsCapturing(st, &capturing) != cudaSuccess) return false;
+    if (capturing != cudaStreamCaptureStatusNone) return true;
+    const cudaError_t e = cudaEventQuery(event());
+    if (e == cudaErrorNotReady) return cudaStreamWaitEvent(st, event(), 0) == cudaSuccess;
+    return e == cudaSuccess;
+  }
 };
 inline PersistentChain& persistent_chain() {
   static PersistentChain c;
@@ -262,11 +282,13 @@ inline int launch_t(const void* Q, const void* K, const void* V, void* Y, int BH
   if (mode == 1 && (SB != B || !tmem_kernel_supported(SB, H, lse, n_valid))) return 4;
   // the padding mask only where a tile row owns a whole key block
   if (n_valid != 0 && SB != B) return 4;
-  const Ws w = ws_layout(ws, BH, N);
-  int* counters = (int*)((char*)ws + w.bytes);
+  // status block, counters (cleared together), states
+  int* counters = (int*)((char*)ws + kWsStatusBytes);
+  Ws w = ws_layout((char*)ws + counters_bytes(BH, T_steps), BH, N);
+  w.status = (int*)ws;
   const int m = N / SB;            // = SB on this path
   const uint64_t rows = (uint64_t)BH * N;
-  void* aLlo = (char*)counters + counters_bytes(BH, T_steps);   // used when uses_hilo(dtype, SB)
+  void* aLlo = (char*)ws + w.bytes + counters_bytes(BH, T_steps);   // used when uses_hilo(dtype, SB)
   Params P;
   {
     MapCache& c = map_cache();
@@ -310,6 +332,7 @@ inline int launch_t(const void* Q, const void* K, const void* V, void* Y, int BH
   // long done when its turn comes (measured: C5, 1024 tiles of 128 x 128 per group and half-step,
   // same time and 118 MB instead of 217 MB of DRAM traffic; C4, 1024 tiles of two 64 x 64 blocks,
   // 3 % slower, hence the higher bar for the faster small tiles)
+  const bool chained = mode == 0 && P.trace == nullptr && chain_chosen(BH, N, SB);
   const int min_tiles = B == 128 ? 1024 : 2048;
   P.head_groups = 1;
   while (BH % (2 * P.head_groups) == 0 && P.tiles_per_phase / (2 * P.head_groups) >= min_tiles) P.head_groups *= 2;
@@ -318,24 +341,31 @@ inline int launch_t(const void* Q, const void* K, const void* V, void* Y, int BH
   P.n_counters = 2 * T_steps * BH;
   P.wait_cycles = knobs().wait_cycles;
   if (!ws_armed) {   // status block and counters start at zero; the kernel leaves them that way
-    if (cudaMemsetAsync(ws, 0, kWsStatusBytes, st) != cudaSuccess) return 7;
-    if (cudaMemsetAsync(counters, 0, counters_bytes(BH, T_steps), st) != cudaSuccess) return 7;
+    if (cudaMemsetAsync(ws, 0, kWsStatusBytes + counters_bytes(BH, T_steps), st) != cudaSuccess) return 7;
   }
   const int num_sms = sm_count();
   if (num_sms <= 0) return 7;
+  const int total = 2 * T_steps * P.tiles_per_phase;
+  // one launch, dependencies tracked by counters
+  P.g_begin = knobs().skip_first_half_step ? P.tiles_per_phase : 0; P.g_end = total; P.check_deps = 1;
+  PersistentChain& chain = persistent_chain();
+  std::lock_guard<std::mutex> chain_lock(chain.mu);
+  if constexpr (SB == 64) {
+    if (chained) {      // its tiles are taken by CTAs that run, whichever they are
+      if (!chain.let_pending_pass(st)) return 7;
+      if (launch_chain<T>(P, total < 2 * num_sms ? total : 2 * num_sms, st) != cudaSuccess) return 7;
+      *launches = 1;
+      return 0;
+    }
+  }
   // The grid only makes progress if every CTA is resident (tiles are dealt out statically and wait
   // on each other's results), i.e. if it has the GPU to itself.  Two such launches on different
   // streams could split the SMs between them and starve each other, so launches of this family are
   // chained per device with an event: a later one starts when the earlier one has finished,
   // whatever streams they are on.
-  PersistentChain& chain = persistent_chain();
-  std::lock_guard<std::mutex> chain_lock(chain.mu);
   cudaEvent_t ev = chain.event();
   if (ev == nullptr) return 7;
   if (chain.recorded() && cudaStreamWaitEvent(st, ev, 0) != cudaSuccess) return 7;
-  const int total = 2 * T_steps * P.tiles_per_phase;
-  // one launch, dependencies tracked by counters
-  P.g_begin = knobs().skip_first_half_step ? P.tiles_per_phase : 0; P.g_end = total; P.check_deps = 1;
   const int grid = total < num_sms ? total : num_sms;
   cudaError_t e;
   if constexpr (SB == B) {
