@@ -27,8 +27,7 @@
 #pragma once
 #include <cuda.h>
 
-#include <algorithm>
-
+#include "head_plan.h"
 #include "status_word.cuh"
 #include "tensor_path.cuh"
 #include "warp_mma.cuh"
@@ -50,7 +49,6 @@ using warpmma::movm_trans;
 using warpmma::quad_max;
 using warpmma::scatter_reduce;
 
-constexpr int kMaxSmem = 227 * 1024, kMaxBlocks = 32;
 constexpr float kMasked = -3.0e38f;      // finite, and far below any score
 
 struct Params {
@@ -64,9 +62,6 @@ struct Params {
   int tile;                 // bytes of a tile
   int bufs;                 // heads in shared memory
   float scale;
-};
-struct __align__(16) Bars {
-  uint64_t full[2][kMaxBlocks];      // by buffer (V over the states: the second set is V's) and block
 };
 
 __device__ __forceinline__ void stsm_x4(uint32_t saddr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
@@ -146,20 +141,6 @@ __device__ __forceinline__ void products(float (&o)[2][4], const uint32_t (&a)[K
       if (kk == 0) M::first(o[v], a[kk], b[kk] + 2 * v);
       else M::run(o[v], a[kk], b[kk] + 2 * v);
     }
-}
-
-// What a kernel is for: one round; more, with a state tile beside Q, K and V; more, with V over the states once the last round
-// has read them (three tiles a head).
-enum Rounds { kOne = 0, kMore = 1, kMoreVLast = 2 };
-// Warps an SM has room for.  Two 8-column tiles either way fit 64 registers (nothing is spilled), 24 warps' 80 the other one-round
-// kernels and 24 x 16 (at most 16 bytes), the rest take 128.
-constexpr int max_warps(int nb, int nm, int rounds) { return nb == 2 && nm == 2 ? 32 : (rounds == kOne || (nb == 3 && nm == 2) ? 24 : 16); }
-
-// Shared memory of a CTA: `bufs` x (Q, K, V), the state tile (more than one round), a dump for matrix-store rows past a
-// block (a line of its own: addresses step through a row by an exclusive or of bits 5 and 6), c_L ([position]
-// [nm * 8 blocks]), barriers.
-inline size_t smem_bytes(int tile, int bufs, int rounds, int b, int nm) {
-  return (size_t)tile * (rounds == kMoreVLast ? 3 : 3 * bufs + (rounds == kMore ? 1 : 0)) + 128 + (size_t)b * nm * 8 * 4 + sizeof(Bars) + 1024;
 }
 
 // NB, NM: 8-column tiles that hold b keys / m blocks.
@@ -584,56 +565,6 @@ __global__ void __launch_bounds__(32 * max_warps(NB, NM, ROUNDS), 1) monarch_fus
 inline bool shape_ok(int d, int b, int m, int dtype) {
   return (dtype == 1 || dtype == 2) && d % 8 == 0 && d <= 64 && b > 8 && b <= 32 && m > 8 && m <= 32;
 }
-struct Plan {
-  int bp, tile, bufs, warps, ctas, rounds;      // ctas: per SM
-  size_t smem;
-};
-inline bool plan(int b, int m, int T, int BH, int num_sms, Plan* p) {
-  const int nb = (b + 7) / 8, nm = (m + 7) / 8, rounds = T > 1 ? kMore : kOne;
-  // The odd pitch where it fits; without it the L half-step's rows conflict (8-way for b = 16, 24, 32,
-  // which the general kernel then serves faster: N = 576 as 24 x 24, 768 heads, 120 against 125 us).
-  for (int odd = 1; odd >= (b % 8 != 0 ? 0 : 1); --odd) {
-    p->bp = odd ? (b | 1) : b;
-    p->tile = (m * p->bp * 128 + 1023) / 1024 * 1024;
-    p->rounds = rounds;
-    p->bufs = 1;
-    const size_t two = smem_bytes(p->tile, 2, rounds, b, nm);
-    p->smem = smem_bytes(p->tile, 1, rounds, b, nm);
-    if (p->smem > (size_t)kMaxSmem) continue;
-    auto fit = [](size_t bytes) { return (int)((size_t)(227 * 1024) / (bytes + 1024)); };      // CTAs per SM by shared memory
-    // At most one head per SM: one CTA with as many warps as a half-step has tiles.  More: the warps an SM holds go to
-    // as many CTAs as fit, up to three, each with a head of its own (768 heads of 130 = 13 x 10, two rounds: 34.6 us with
-    // three, 39.8 with two).  Where no third fits and there are heads left for a second turn, one CTA of all warps
-    // with the next head's loads under way is faster with 16 warps an SM (it has the same work in flight), with 32 two
-    // CTAs are, and V goes over the states where that makes room for the second.
-    p->ctas = BH <= num_sms ? 1 : std::min(fit(p->smem), 3);
-    const int most = max_warps(nb, nm, rounds);
-    if (p->ctas <= 2 && BH > p->ctas * num_sms) {
-      const size_t v_last = smem_bytes(p->tile, 1, kMoreVLast, b, nm);
-      if (most == 32 && p->ctas == 2) {
-      } else if (most == 32 && rounds == kMore && fit(v_last) >= 2) {
-        p->ctas = 2;
-        p->rounds = kMoreVLast;
-        p->smem = v_last;
-      } else if (two <= (size_t)kMaxSmem) {
-        p->ctas = 1;
-        p->bufs = 2;
-        p->smem = two;
-      }
-    }
-    // the fewest warps that take the fewest rounds of tiles over both half-steps
-    int best = 1 << 30;
-    for (int w = 1; w <= most / p->ctas; ++w) {
-      const int turns = (m + w - 1) / w + (b + w - 1) / w;
-      if (turns < best) {
-        best = turns;
-        p->warps = w;
-      }
-    }
-    return true;
-  }
-  return false;
-}
 inline bool supported(int N, int d, int b, int m, int dtype, int T) {
   (void)N;
   Plan p;
@@ -703,7 +634,7 @@ template <typename TIn, int NB, int NM, int ROUNDS>
 inline int launch_k(const Params& P, const Plan& p, int num_sms, cudaStream_t st) {
   auto kern = monarch_fused_head<TIn, NB, NM, ROUNDS>;
   static warpmma::SmemOptIn opt_in;
-  if (!opt_in.done((const void*)kern, kMaxSmem)) return 7;
+  if (!opt_in.done((const void*)kern, (int)kMaxSmem)) return 7;
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;

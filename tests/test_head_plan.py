@@ -1,0 +1,40 @@
+"""How the per-head kernel shares an SM between heads, compiled for the host and checked without a GPU."""
+import os
+import subprocess
+
+HERE = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+HEADER = os.path.join(HERE, "paper_2505_18698_b200", "csrc", "head_plan.h")
+
+
+def test_every_plan_can_be_launched(tmp_path):
+    """All shapes the kernel is made for, one round and more, from one head to many turns of the GPU: at least a CTA and a warp,
+    the CTAs of an SM fit its shared memory and registers, the blocks of a warp fit the bits it keeps for them."""
+    src = tmp_path / "t.cpp"
+    src.write_text(f"""
+#include <cstdio>
+#include "{HEADER}"
+using namespace ma::fhead;
+int main() {{
+  for (int b = 9; b <= 32; ++b)
+    for (int m = 9; m <= 32; ++m)
+      for (int T = 1; T <= 2; ++T)
+        for (int BH : {{1, 12, 148, 149, 160, 296, 297, 444, 445, 768, 100000}}) {{
+          Plan p;
+          if (plan(b, m, T, BH, 148, &p))
+            printf("%d %d %d %d %d %d %d %d %zu %d\\n", b, m, T, BH, p.ctas, p.warps, p.bufs, p.rounds, p.smem, max_warps((b + 7) / 8, (m + 7) / 8, p.rounds));
+        }}
+}}""")
+    exe = str(tmp_path / "t")
+    subprocess.run(["g++", "-O1", "-std=c++17", "-Wall", "-Werror", "-o", exe, str(src)], check=True)
+    seen, whole = set(), set()
+    for line in subprocess.run([exe], check=True, capture_output=True, text=True).stdout.splitlines():
+        b, m, T, BH, ctas, warps, bufs, rounds, smem, most = map(int, line.split())
+        assert 1 <= ctas <= 3 and 1 <= warps and ctas * warps <= most and 32 * warps <= 1024, line
+        assert smem <= 227 * 1024 and ctas * (smem + 1024) <= 228 * 1024, line
+        assert bufs in (1, 2) and -(-m // warps) <= 15, line      # (bit 31 of the parities says that a wait ran out)
+        assert (rounds == 0) == (T == 1), line
+        seen.add((b, m, T))
+        if smem > 226 * 1024 and BH > 148:
+            whole.add((b, m))
+    assert {(31, 19), (30, 19), (28, 21), (20, 28), (21, 28)} <= whole      # one CTA takes all there is
+    assert len(seen) > 700
