@@ -850,6 +850,14 @@ inline EncodeTiledFn encode_fn() {
             cudaSuccess && q == cudaDriverEntryPointSuccess)
       fn = (EncodeTiledFn)p;
   }
+  // The encoder wants a current context, which a thread that has not yet used the device does not have.
+  static thread_local int bound = -1;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+  if (bound != dev) {
+    if (cudaSetDevice(dev) != cudaSuccess) return nullptr;
+    bound = dev;
+  }
   return fn;
 }
 // 2D view [rows][64] of a contiguous 16-bit array, box = 128 rows.
