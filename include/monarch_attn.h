@@ -101,12 +101,13 @@ size_t monarch_attn_workspace_bytes(int batch, int heads, int N, int d, int b, i
  *
  * Concurrency.  A workspace serves one call at a time: calls that may overlap on the GPU (different
  * streams, no dependency) need a workspace each, and monarch_attn_fwd's library-owned workspace
- * serves one call in flight per device.  The persistent kernels (MA_PATH_TENSOR, from 1024 tiles of 128 rows at b = 64 on
- * excepted: those take tiles as they come to them; MA_PATH_TENSOR_TMEM; what AUTO picks for d = 64, m = b in {32, 64, 128}) deal
+ * serves one call in flight per device.  The persistent kernels (MA_PATH_TENSOR, MA_PATH_TENSOR_TMEM; what
+ * AUTO picks for d = 64, m = b in {32, 64, 128}), except the one of MA_PATH_TENSOR for b = 64 from 1024 tiles of 128 rows on, deal
  * their tiles out statically over one CTA per SM and the CTAs wait for each other's results, so such a launch only
- * makes progress with every CTA resident: it needs the whole GPU.  The library chains these
- * launches per device with an event, so two of them never share the SMs whatever streams they are
- * on; a foreign kernel that holds SMs for longer than the bound of the device-side waits (about a
+ * makes progress with every CTA resident: it needs the whole GPU.  The library chains all persistent
+ * launches per device with an event, so two of them never share the SMs whatever streams they are on; captured
+ * launches wait for and record that event too, as external nodes, so replays take their turn.  What the library cannot order is
+ * foreign: a kernel that holds SMs for longer than the bound of the device-side waits (about a
  * second) while one of them runs makes the waits run out: the call then ends with undefined output
  * and monarch_attn_device_status reports MA_ERR_TIMEOUT. */
 int monarch_attn_fwd_ex(const void* Q, const void* K, const void* V, void* Y,

@@ -241,33 +241,35 @@ inline int sm_count() {   // of the current device
   return sms[dev];
 }
 
-struct PersistentChain {      // one event per device: the end of the last persistent launch
+// Orders the persistent launches of a device, whatever streams they are on: each waits for an event that the one before recorded
+// (no measurable time where both are on one stream).  A captured launch does so through external event nodes, so that every
+// replay of its graph takes its turn too; an event recorded by plain capture could not be waited for by anything outside the graph.
+struct PersistentChain {
   std::mutex mu;
-  cudaEvent_t ev[64] = {};
-  bool rec[64] = {};
-  int dev() const {
-    int d = 0;
-    return (cudaGetDevice(&d) == cudaSuccess && d >= 0 && d < 64) ? d : -1;
-  }
+  cudaEvent_t ev[64] = {};      // by device: the end of the last persistent launch
   cudaEvent_t event() {
-    const int d = dev();
-    if (d < 0) return nullptr;
-    if (ev[d] == nullptr && cudaEventCreateWithFlags(&ev[d], cudaEventDisableTiming) != cudaSuccess)
-      ev[d] = nullptr;
+    int d = 0;
+    if (cudaGetDevice(&d) != cudaSuccess || d < 0 || d >= 64) return nullptr;
+    if (ev[d] == nullptr) {
+      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+      if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return nullptr;
+      if (cudaEventCreateWithFlags(&ev[d], cudaEventDisableTiming) != cudaSuccess) ev[d] = nullptr;
+      cudaThreadExchangeStreamCaptureMode(&mode);
+    }
     return ev[d];
   }
-  bool recorded() const { const int d = dev(); return d >= 0 && rec[d]; }
-  void set_recorded() { const int d = dev(); if (d >= 0) rec[d] = true; }
-  // A launch that does not need the whole GPU goes after one that does and has not finished: a steady stream of them might
-  // otherwise keep that one's CTAs, which take a whole SM, from coming in.
-  bool let_pending_pass(cudaStream_t st) {
-    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-    if (!recorded()) return true;
-    if (cudaStreamIsCapturing(st, &capturing) != cudaSuccess) return false;
-    if (capturing != cudaStreamCaptureStatusNone) return true;
-    const cudaError_t e = cudaEventQuery(event());
-    if (e == cudaErrorNotReady) return cudaStreamWaitEvent(st, event(), 0) == cudaSuccess;
-    return e == cudaSuccess;
+  // Runs `launch` in its turn.
+  template <typename F>
+  bool in_turn(cudaStream_t st, F launch) {
+    std::lock_guard<std::mutex> lock(mu);
+    const cudaEvent_t e = event();
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (e == nullptr || cudaStreamIsCapturing(st, &capture) != cudaSuccess) return false;
+    const bool plain = capture == cudaStreamCaptureStatusNone;
+    if (cudaStreamWaitEvent(st, e, plain ? cudaEventWaitDefault : cudaEventWaitExternal) != cudaSuccess) return false;
+    const bool ok = launch() == cudaSuccess;
+    // (the event is recorded in any case: the set-up of a launch that failed is ordered by it too)
+    return cudaEventRecordWithFlags(e, st, plain ? cudaEventRecordDefault : cudaEventRecordExternal) == cudaSuccess && ok;
   }
 };
 inline PersistentChain& persistent_chain() {
@@ -340,42 +342,30 @@ inline int launch_t(const void* Q, const void* K, const void* V, void* Y, int BH
   P.negate = scale < 0.f ? kNegateA : 0u;
   P.n_counters = 2 * T_steps * BH;
   P.wait_cycles = knobs().wait_cycles;
-  if (!ws_armed) {   // status block and counters start at zero; the kernel leaves them that way
-    if (cudaMemsetAsync(ws, 0, kWsStatusBytes + counters_bytes(BH, T_steps), st) != cudaSuccess) return 7;
-  }
   const int num_sms = sm_count();
   if (num_sms <= 0) return 7;
   const int total = 2 * T_steps * P.tiles_per_phase;
   // one launch, dependencies tracked by counters
   P.g_begin = knobs().skip_first_half_step ? P.tiles_per_phase : 0; P.g_end = total; P.check_deps = 1;
-  PersistentChain& chain = persistent_chain();
-  std::lock_guard<std::mutex> chain_lock(chain.mu);
-  if constexpr (SB == 64) {
-    if (chained) {      // its tiles are taken by CTAs that run, whichever they are
-      if (!chain.let_pending_pass(st)) return 7;
-      if (launch_chain<T>(P, total < 2 * num_sms ? total : 2 * num_sms, st) != cudaSuccess) return 7;
-      *launches = 1;
-      return 0;
+  // The grids of tensor_decoupled.cuh and tensor_tmem.cuh only make progress if every CTA is resident (tiles are dealt out
+  // statically and wait on each other's results), i.e. if they have the GPU to themselves: two of them could split the SMs
+  // between them and starve each other, and a steady stream of monarch_chain launches, whose CTAs take half an SM, could keep theirs
+  // from coming in.  So all launches of this family take turns.
+  auto go = [&]() -> cudaError_t {
+    if (!ws_armed) {   // status block and counters start at zero; the kernel leaves them that way
+      const cudaError_t e = cudaMemsetAsync(ws, 0, kWsStatusBytes + counters_bytes(BH, T_steps), st);
+      if (e != cudaSuccess) return e;
     }
-  }
-  // The grid only makes progress if every CTA is resident (tiles are dealt out statically and wait
-  // on each other's results), i.e. if it has the GPU to itself.  Two such launches on different
-  // streams could split the SMs between them and starve each other, so launches of this family are
-  // chained per device with an event: a later one starts when the earlier one has finished,
-  // whatever streams they are on.
-  cudaEvent_t ev = chain.event();
-  if (ev == nullptr) return 7;
-  if (chain.recorded() && cudaStreamWaitEvent(st, ev, 0) != cudaSuccess) return 7;
-  const int grid = total < num_sms ? total : num_sms;
-  cudaError_t e;
-  if constexpr (SB == B) {
-    e = mode == 1 ? launch_tmem<T, B>(P, grid, st) : launch_decoupled<T, B, SB>(P, grid, st);
-  } else {
-    e = launch_decoupled<T, B, SB>(P, grid, st);
-  }
-  if (e != cudaSuccess) return 7;
-  if (cudaEventRecord(ev, st) != cudaSuccess) return 7;
-  chain.set_recorded();
+    if constexpr (SB == 64) {
+      if (chained) return launch_chain<T>(P, total < 2 * num_sms ? total : 2 * num_sms, st);      // taken by CTAs that run, whichever
+    }
+    const int grid = total < num_sms ? total : num_sms;
+    if constexpr (SB == B) {
+      if (mode == 1) return launch_tmem<T, B>(P, grid, st);
+    }
+    return launch_decoupled<T, B, SB>(P, grid, st);
+  };
+  if (!persistent_chain().in_turn(st, go)) return 7;
   *launches = 1;
   return 0;
 }
