@@ -246,6 +246,7 @@ struct DeviceBuffers {
   void* ws = nullptr;
   size_t ws_bytes = 0;
   long long armed_key = -1;   // problem whose status block / counters the workspace is armed for
+  bool captured = false;   // a graph holds calls that use the workspace: replays write it unseen, and it is never freed
   void* stage = nullptr;   // Q, K, V, Y staging for the host entry point
   size_t stage_bytes = 0;
   // host entry point: kernels and the copy back run on streams of their own, so that the compute
@@ -259,11 +260,14 @@ constexpr int kHostChunks = 8;
 static int g_host_chunks = 0;   // chunks a host call is cut into (<= kHostChunks); 0: by size
 static DeviceBuffers g_dev[kMaxDevices];
 
-static int grow(void** ptr, size_t* have, size_t need) {
+// `keep`: what there was stays allocated (a graph may still use it).
+static int grow(void** ptr, size_t* have, size_t need, bool keep = false) {
   if (*have >= need) return MA_OK;
   if (*ptr) {
-    if (cudaDeviceSynchronize() != cudaSuccess) return MA_ERR_CUDA;
-    cudaFree(*ptr);
+    if (!keep) {
+      if (cudaDeviceSynchronize() != cudaSuccess) return MA_ERR_CUDA;
+      cudaFree(*ptr);
+    }
     *ptr = nullptr;
     *have = 0;
   }
@@ -452,12 +456,17 @@ static int run_call(const Call& c) {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return MA_ERR_CUDA;
   DeviceBuffers& B = g_dev[dev];
   const size_t had = B.ws_bytes;
-  rc = grow(&B.ws, &B.ws_bytes, workspace_bytes_for(p, r));
+  rc = grow(&B.ws, &B.ws_bytes, workspace_bytes_for(p, r), B.captured);
   if (rc != MA_OK) return rc;
+  if (touches_workspace(r) && !B.captured) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) return MA_ERR_CUDA;
+    B.captured = capture != cudaStreamCaptureStatusNone;
+  }
   // The persistent kernel leaves its status block and counters zeroed, so the library's own
-  // workspace is cleared only when the problem (hence the layout) changes.
+  // workspace is cleared only when the problem (hence the layout) changes; or each time, once a graph may write it in between.
   const long long key = ((long long)r << 56) ^ ((long long)p.T << 48) ^ ((long long)p.BH << 24) ^ p.N;
-  const bool armed = (r == MA_PATH_TENSOR) && had == B.ws_bytes && B.armed_key == key;
+  const bool armed = (r == MA_PATH_TENSOR) && !B.captured && had == B.ws_bytes && B.armed_key == key;
   rc = fwd_ex(c.Q, c.K, c.V, c.Y, p, 1.0f / sqrtf((float)c.d), r, B.ws, B.ws_bytes, status, st, armed);
   B.armed_key = (rc == MA_OK && r == MA_PATH_TENSOR) ? key : -1;
   return rc;
