@@ -146,7 +146,10 @@ struct Chain {
     for (uint32_t q = 0;; ++q) {
       const int g = P.g_begin + claim;
       uint64_t *bar = &sh->full[w][q & 1], *bar3 = &sh->third[w][q & 1];
-      if (g >= P.g_end) {                    // (once all threads are through the last tile: the word and the barrier are free then)
+      // The end: once all threads are through the last two tiles, the word and the barrier are free.  One after the other: a parity
+      // alone does not tell tile q - 1 from q - 3 (which is through, since q - 1 has got its first slot).
+      if (g >= P.g_end) {
+        if (q > 1 && !wait_bar(&sh->o_free[w], q & 1, sh, P, 12)) return;
         if (q > 0 && !wait_bar(&sh->o_free[w], (q - 1) & 1, sh, P, 12)) return;
         sh->tile[w][q & 1] = make_int4(-1, 0, 0, 0);
         mbar_arrive(bar);
