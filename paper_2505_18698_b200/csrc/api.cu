@@ -314,7 +314,7 @@ struct Status {
 static int launch_resolved(const void* Q, const void* K, const void* V, void* Y, const Problem& p,
                            float scale, int resolved, void* ws, const Status& status, cudaStream_t st, bool ws_armed) {
   int rc, launches = 1;
-  const char* kernels;
+  const char* kernels = "";
   if (resolved == MA_PATH_GENERIC) {
     kernels = "generic";
     rc = launch_generic(p, Q, K, V, Y, scale, ws, st);
@@ -351,10 +351,9 @@ static int launch_resolved(const void* Q, const void* K, const void* V, void* Y,
     kernels = "tensor_basic";
     rc = tensor::launch(Q, K, V, Y, p.BH, p.N, p.d, p.b, p.T, p.dtype, scale, ws, status.report, st, &launches);
   } else {
-    kernels = resolved == MA_PATH_TENSOR_TMEM ? "tensor_tmem" : (tp::chain_chosen(p.BH, p.N, p.b) ? "tensor_chain" : "tensor_decoupled");
     rc = tp::launch(Q, K, V, Y, p.BH, p.N, p.b, p.T, p.dtype, scale, ws, st, &launches,
                     resolved == MA_PATH_TENSOR_TMEM ? 1 : 0,
-                    ws_armed, status.report, p.H, p.lse, p.n_valid < p.N ? p.n_valid : 0);
+                    ws_armed, status.report, &kernels, p.H, p.lse, p.n_valid < p.N ? p.n_valid : 0);
   }
   if (rc == MA_OK) {
     g_last_launches = launches;

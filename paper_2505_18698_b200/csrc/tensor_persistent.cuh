@@ -199,11 +199,11 @@ cudaError_t launch_chain(const Params& P, int grid, cudaStream_t st);
 // layout or masked, where that one is a fifth slower: 36 57.9 / 68.4, 48 68.0 / 76.7.
 inline bool chain_chosen(int BH, int N, int b) { return b == 64 && (long long)BH * N / kRows >= 1024; }      // tiles of a half-step
 
-// mode 0: kernel of tensor_decoupled.cuh; mode 1: kernel of tensor_tmem.cuh (m = b in {64, 128},
-// plain calls only: no [batch][N][heads][d] layout, no row log-sum-exp, no padding mask).
+// mode 0: kernel of tensor_decoupled.cuh or tensor_chain.cuh; mode 1: kernel of tensor_tmem.cuh (m = b in {64, 128},
+// plain calls only: no [batch][N][heads][d] layout, no row log-sum-exp, no padding mask).  *kernels: which it was.
 int launch(const void* Q, const void* K, const void* V, void* Y, int BH, int N, int b, int T,
            int dtype, float scale, void* ws, cudaStream_t st, int* launches, int mode,
-           bool ws_armed, int* report, int H = 0, float* lse = nullptr, int n_valid = 0);
+           bool ws_armed, int* report, const char** kernels, int H = 0, float* lse = nullptr, int n_valid = 0);
 inline bool tmem_kernel_supported(int b, int H, const float* lse, int n_valid) {
   return (b == 64 || b == 128) && H == 0 && lse == nullptr && n_valid == 0;
 }
@@ -280,7 +280,7 @@ inline PersistentChain& persistent_chain() {
 template <typename T, int B, int SB>
 inline int launch_t(const void* Q, const void* K, const void* V, void* Y, int BH, int N, int T_steps,
                     int dtype, float scale, void* ws, cudaStream_t st, int* launches, int mode,
-                    bool ws_armed, int* report, int H, float* lse, int n_valid) {
+                    bool ws_armed, int* report, const char** kernels, int H, float* lse, int n_valid) {
   if (mode == 1 && (SB != B || !tmem_kernel_supported(SB, H, lse, n_valid))) return 4;
   // the padding mask only where a tile row owns a whole key block
   if (n_valid != 0 && SB != B) return 4;
@@ -366,14 +366,15 @@ inline int launch_t(const void* Q, const void* K, const void* V, void* Y, int BH
     return launch_decoupled<T, B, SB>(P, grid, st);
   };
   if (!persistent_chain().in_turn(st, go)) return 7;
+  *kernels = chained ? "tensor_chain" : (mode == 1 ? "tensor_tmem" : "tensor_decoupled");
   *launches = 1;
   return 0;
 }
 
 int launch(const void* Q, const void* K, const void* V, void* Y, int BH, int N, int b, int T,
            int dtype, float scale, void* ws, cudaStream_t st, int* launches, int mode,
-           bool ws_armed, int* report, int H, float* lse, int n_valid) {
-#define MA_TP_ARGS Q, K, V, Y, BH, N, T, dtype, scale, ws, st, launches, mode, ws_armed, report, H, lse, n_valid
+           bool ws_armed, int* report, const char** kernels, int H, float* lse, int n_valid) {
+#define MA_TP_ARGS Q, K, V, Y, BH, N, T, dtype, scale, ws, st, launches, mode, ws_armed, report, kernels, H, lse, n_valid
   if (dtype == 1) {
     if (b == 128) return launch_t<__half, 128, 128>(MA_TP_ARGS);
     if (b == 64) return launch_t<__half, 64, 64>(MA_TP_ARGS);
