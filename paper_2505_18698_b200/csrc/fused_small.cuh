@@ -51,7 +51,7 @@ using warpmma::scatter_reduce;
 constexpr int kThreads = 256, kWarps = 8, kRowBytes = 128, kMaxSmem = 227 * 1024;
 // where stmatrix rows past the end of a block go: eight rows of 16 bytes (nothing reads them)
 constexpr size_t kDumpBytes = 128;
-constexpr float kMasked = -3.0e38f;      // finite, and far below any logit
+constexpr float kLowest = -3.4028234e38f;
 
 // Four 8x8 16-bit matrices from accumulator-layout registers; lane L gives the address of row L & 7
 // of matrix L >> 3.
@@ -268,19 +268,19 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
             }
           }
           // rows j = j0 + g (c0, c1) and j0 + g + 8 (c2, c3); columns i = 8 nt + 2t, +1
-          // (columns past the block, which only the last two column tiles have, and keys past n_valid: a finite
-          // logit of weight 0, so that 0 log 0 = 0)
+          // (columns past the block, which only the last two column tiles have, and keys past n_valid: a logit of minus
+          // infinity, which a large scale's may be too; times its weight of 0 it counts as a finite one, so that 0 log 0 = 0)
           float red[4], mxs[2];      // sum of the weights and of weight times logit, by row
           const int lim = min(b, n_valid - k * b) - 2 * t;
 #pragma unroll
           for (int hh = 0; hh < 2; ++hh) {
-            float mx = kMasked;
+            float mx = -INFINITY;
 #pragma unroll
             for (int nt = 0; nt < BP / 8; ++nt) {
               float2 z = fmul2(row_pair(s[nt], hh), both(fl));
               if (nt >= BP / 8 - 2 || lim + 2 * t <= BP - 16) {
-                z.x = 8 * nt < lim ? z.x : kMasked;
-                z.y = 8 * nt + 1 < lim ? z.y : kMasked;
+                z.x = 8 * nt < lim ? z.x : -INFINITY;
+                z.y = 8 * nt + 1 < lim ? z.y : -INFINITY;
               }
               put_pair(s[nt], hh, z);
               mx = fmaxf(mx, fmaxf(z.x, z.y));
@@ -289,10 +289,11 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
             float2 sum = both(0.f), sz = both(0.f);
 #pragma unroll
             for (int nt = 0; nt < BP / 8; ++nt) {
-              const float2 z = row_pair(s[nt], hh), e = fadd2(z, both(-mx));
-              const float2 p = make_float2(ex2(e.x), ex2(e.y));
+              float2 z = row_pair(s[nt], hh);
+              const float2 e = fadd2(z, both(-mx)), p = make_float2(ex2(e.x), ex2(e.y));
               put_pair(s[nt], hh, p);
               sum = nt ? fadd2(sum, p) : p;
+              z = make_float2(fmaxf(z.x, kLowest), fmaxf(z.y, kLowest));
               sz = nt ? ffma2(p, z, sz) : fmul2(p, z);
             }
             red[2 * hh] = sum.x + sum.y;
@@ -387,7 +388,7 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
         for (int nt = 0; nt < MP / 8; ++nt)
 #pragma unroll
           for (int e = 0; e < 2; ++e)
-            c[nt][e] = 8 * nt + 2 * t + e < m ? sCL[(8 * nt + 2 * t + e) * b + j] : kMasked;
+            c[nt][e] = 8 * nt + 2 * t + e < m ? sCL[(8 * nt + 2 * t + e) * b + j] : -INFINITY;
         float pn[MP / 16][2][MP / 8][2];           // normalised weights [row tile][half][nt][e]
 #pragma unroll
         for (int rt = 0; rt < MP / 16; ++rt) {
@@ -426,9 +427,9 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
           float inv_s[2], red[2], mxs[2];
 #pragma unroll
           for (int hh = 0; hh < 2; ++hh) {
-            float mx = kMasked;
+            float mx = -INFINITY;
 #pragma unroll
-            for (int nt = 0; nt < MP / 8; ++nt) {       // (blocks past m: c is kMasked, next to which the score is nothing)
+            for (int nt = 0; nt < MP / 8; ++nt) {       // (blocks past m: the addend is minus infinity)
               const float2 z = ffma2(row_pair(s[nt], hh), both(fl), make_float2(c[nt][0], c[nt][1]));
               put_pair(s[nt], hh, z);
               mx = fmaxf(mx, fmaxf(z.x, z.y));
