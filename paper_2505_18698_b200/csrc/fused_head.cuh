@@ -18,8 +18,8 @@
 // other in place in a state tile.  Arithmetic is f16 whatever the input type (see fused_small.cuh).
 //
 // Measured (B200, us per call, against the general per-head kernel): 768 heads of 256 = 16 x 16, one
-// round 23.8 / 27.7 (65 % of the copy bandwidth); 768 of 210 = 15 x 14, two rounds 36.3 / 47.7; 384 of
-// lengths up to 384 = 16 x 24 24.1 / 28.9; 720 of 396 = 22 x 18 64 / 97; 24 of 210 5 / 7.  Row and column
+// round 23.7 / 27.7 (65 % of the copy bandwidth); 768 of 210 = 15 x 14, two rounds 36.4 / 47.7; 384 of
+// lengths up to 384 = 16 x 24 23.6 / 28.9.  24 of 210 4.4, two rounds 7.0; 720 of 396 = 22 x 18 53, 94.  Row and column
 // reductions that halve the values a lane carries, with one division a lane, took 3 % (16 x 16) to 11 %
 // (10 x 24, two rounds) off.  The tiles wait on latencies: 32 warps with two heads at work, where two 8-column tiles either way
 // fit 64 registers, took 41 to 36.3 us (15 x 14, two rounds) and 24.8 to 23.8 (16 x 16, one).  What is left is latency at four to eight
@@ -143,9 +143,9 @@ __device__ __forceinline__ void products(float (&o)[2][4], const uint32_t (&a)[K
     }
 }
 
-// NB, NM: 8-column tiles that hold b keys / m blocks.
-template <typename TIn, int NB, int NM, int ROUNDS>
-__global__ void __launch_bounds__(32 * max_warps(NB, NM, ROUNDS), 1) monarch_fused_head(const __grid_constant__ Params P) {
+// NB, NM: 8-column tiles that hold b keys / m blocks.  WARPS: on an SM.
+template <typename TIn, int NB, int NM, int ROUNDS, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, 1) monarch_fused_head(const __grid_constant__ Params P) {
   typedef Mma<__half> M;
   constexpr bool MULTI = ROUNDS != kOne, V_LAST = ROUNDS == kMoreVLast;
   constexpr int RB = (NB + 1) / 2, RM = (NM + 1) / 2;      // 16-row tiles
@@ -630,9 +630,9 @@ inline bool get_maps(Params* P, const Args& a, const Plan& p, int dev) {
   P->v = c.maps[e][2];
   return true;
 }
-template <typename TIn, int NB, int NM, int ROUNDS>
+template <typename TIn, int NB, int NM, int ROUNDS, int WARPS = max_warps(NB, NM, ROUNDS)>
 inline int launch_k(const Params& P, const Plan& p, int num_sms, cudaStream_t st) {
-  auto kern = monarch_fused_head<TIn, NB, NM, ROUNDS>;
+  auto kern = monarch_fused_head<TIn, NB, NM, ROUNDS, WARPS>;
   static warpmma::SmemOptIn opt_in;
   if (!opt_in.done((const void*)kern, (int)kMaxSmem)) return 7;
   cudaLaunchAttribute attr;
@@ -651,6 +651,7 @@ inline int launch_k(const Params& P, const Plan& p, int num_sms, cudaStream_t st
 template <typename TIn, int ROUNDS>
 inline int launch_n(const Params& P, const Plan& p, int num_sms, cudaStream_t st) {
   const int nb = (P.b + 7) / 8, nm = (P.m + 7) / 8;
+  if (p.bound == 16 && nb == 2 && nm == 2) return launch_k<TIn, 2, 2, ROUNDS, 16>(P, p, num_sms, st);
 #define MA_FH(B)                                            \
   (nm == 2 ? launch_k<TIn, B, 2, ROUNDS>(P, p, num_sms, st) \
            : (nm == 3 ? launch_k<TIn, B, 3, ROUNDS>(P, p, num_sms, st) : launch_k<TIn, B, 4, ROUNDS>(P, p, num_sms, st)))

@@ -20,9 +20,14 @@ struct alignas(16) Bars {
 // What a kernel is for: one round; more, with a state tile beside Q, K and V; more, with V over the states once the last round
 // has read them (three tiles a head).
 enum Rounds { kOne = 0, kMore = 1, kMoreVLast = 2 };
-// Warps an SM has room for.  Two 8-column tiles either way fit 64 registers (nothing is spilled), 24 warps' 80 the other one-round
-// kernels and 24 x 16 (at most 16 bytes), the rest take 128.
-constexpr int max_warps(int nb, int nm, int rounds) { return nb == 2 && nm == 2 ? 32 : (rounds == kOne || (nb == 3 && nm == 2) ? 24 : 16); }
+// Warps an SM has room for, that is, the registers that a kernel is compiled for (65536 / 32 / warps).  More warps pay where a half-step then
+// takes fewer turns or a second head is at work, and cost where they make the compiler spill.  Two 8-column tiles either way fit 64
+// registers (nothing is spilled): 32 warps.  Up to three either way fit 80 in the one-round kernels (up to 12 bytes spilled): 24 warps take 17 to
+// 24 rows or blocks in one turn instead of two (us with 24 / with 16: 768 heads of 20 x 20 59.1 / 62.4 in f16, 66.9 / 74.3 in bf16, 12 heads
+// 9.0 / 10.3; 24 x 16 48.0 / 47.9, 56.3 / 56.3, 12 heads 6.9 / 7.1; 10 x 18 29.9 / 30.1, 35.4 / 36.2; 14 x 22 41.9 / 40.8, 50.0 / 50.0).
+// 25 to 32 take two turns either way and 80 registers spill 20 to 52 bytes (12 x 32 47.5 / 46.0, 32 x 11 48.1 / 45.9, 32 x 17 79.6 / 71.6, bf16 92.5 / 89.2,
+// 26 x 22 bf16 100.3 / 98.1, though 28 x 20 bf16 88.5 / 90.5); so do more rounds (24 x 16 81.5 / 77.6, bf16 88.5 / 85.4, 20 x 12 61.0 / 58.9): 16.
+constexpr int max_warps(int nb, int nm, int rounds) { return nb == 2 && nm == 2 ? 32 : (rounds == kOne && nb <= 3 && nm <= 3 ? 24 : 16); }
 
 // Shared memory of a CTA: `bufs` x (Q, K, V), the state tile (more than one round), a dump for matrix-store rows past a
 // block (a line of its own: addresses step through a row by an exclusive or of bits 5 and 6), c_L ([position]
@@ -32,7 +37,7 @@ inline size_t smem_bytes(int tile, int bufs, int rounds, int b, int nm) {
 }
 
 struct Plan {
-  int bp, tile, bufs, warps, ctas, rounds;      // ctas: per SM
+  int bp, tile, bufs, warps, ctas, rounds, bound;      // ctas: per SM; bound: warps an SM that the kernel is compiled for
   size_t smem;
 };
 inline bool plan(int b, int m, int T, int BH, int num_sms, Plan* p) {
@@ -77,6 +82,9 @@ inline bool plan(int b, int m, int T, int BH, int num_sms, Plan* p) {
         p->warps = w;
       }
     }
+    // Where an SM does not get more than 16 warps (a head an SM or fewer), 64 registers only make the chain longer (us with up to 128 / with
+    // 64): two rounds, 12 heads of 12 x 15 6.7 / 7.6, 48 6.7 / 8.7, 148 of 16 x 16 7.6 / 8.3; one round, 48 of 16 x 16 4.6 / 5.3, 100 of 12 x 16 in bf16 5.2 / 7.8.
+    p->bound = most == 32 && p->ctas * p->warps <= 16 ? 16 : most;
     return true;
   }
   return false;

@@ -21,7 +21,7 @@ int main() {{
         for (int BH : {{1, 12, 148, 149, 160, 296, 297, 444, 445, 768, 100000}}) {{
           Plan p;
           if (plan(b, m, T, BH, 148, &p))
-            printf("%d %d %d %d %d %d %d %d %zu %d\\n", b, m, T, BH, p.ctas, p.warps, p.bufs, p.rounds, p.smem, max_warps((b + 7) / 8, (m + 7) / 8, p.rounds));
+            printf("%d %d %d %d %d %d %d %d %zu %d\\n", b, m, T, BH, p.ctas, p.warps, p.bufs, p.rounds, p.smem, p.bound);
         }}
 }}""")
     exe = str(tmp_path / "t")
@@ -33,6 +33,8 @@ int main() {{
         assert smem <= 227 * 1024 and ctas * (smem + 1024) <= 228 * 1024, line
         assert bufs in (1, 2) and -(-m // warps) <= 15, line      # (bit 31 of the parities says that a wait ran out)
         assert (rounds == 0) == (T == 1), line
+        if BH <= 148 and max(b, m) <= 16:
+            assert most == 16, line                               # few heads: all the registers a warp can use
         seen.add((b, m, T))
         if smem > 226 * 1024 and BH > 148:
             whole.add((b, m))
