@@ -48,7 +48,9 @@ typedef enum {
                           {32, 64, 128}: one persistent launch for all 2T half-steps, softmax
                           weights handed to the second MMA through shared memory; bf16 with b = 32
                           keeps alpha_L as a hi + lo pair of bf16 arrays (one more workspace
-                          array).  Needs the whole GPU: see monarch_attn_fwd_ex */
+                          array).  b = 64 from 1024 tiles of 128 rows on: a kernel with four tiles
+                          at work per SM and the weights in tensor memory.  The others need the
+                          whole GPU: see monarch_attn_fwd_ex */
   MA_PATH_TENSOR_TMEM = 3, /* the same tiles and order with the softmax weights handed over in
                               tensor memory and deeper operand rings: f16/bf16, d = 64, m = b in
                               {64, 128}.  Needs the whole GPU as well */
@@ -138,7 +140,7 @@ int monarch_attn_fwd_host(const void* Q_host, const void* K_host, const void* V_
  * half-step has that number for each row anyway and writes it out:
  *   row_lse: DEVICE pointer, [batch][heads][N] floats (natural logarithm), row b l + j of a head;
  *   f of a head = sum of its N entries (the caller reduces; 4-byte aligned).
- * `path`: MA_PATH_AUTO, MA_PATH_TENSOR (second-generation kernel), MA_PATH_FUSED_SMALL, MA_PATH_FUSED_F32,
+ * `path`: MA_PATH_AUTO, MA_PATH_TENSOR, MA_PATH_FUSED_SMALL, MA_PATH_FUSED_F32,
  * MA_PATH_TILE_MMA or MA_PATH_GENERIC.  Y, workspace
  * and everything else as monarch_attn_fwd_ex.  Asynchronous on `stream`. */
 int monarch_attn_fwd_objective(const void* Q, const void* K, const void* V, void* Y, int batch,
@@ -150,7 +152,7 @@ int monarch_attn_fwd_objective(const void* Q, const void* K, const void* V, void
  * its QKV projection, before any transpose); the paper's method is per head (Sec. 3), so only the
  * addressing changes.  Q, K, V, Y: DEVICE pointers to contiguous [batch][N][heads][d] arrays of
  * `dtype`, 16-byte aligned, Y not overlapping an input.  `path`: MA_PATH_AUTO, MA_PATH_TENSOR (the
- * second-generation kernel: the head becomes a column offset in the TMA tensor maps),
+ * tcgen05 kernels: the head becomes a column offset in the TMA tensor maps),
  * MA_PATH_FUSED_JSPLIT (likewise), MA_PATH_FUSED_SMALL, MA_PATH_FUSED_F32, MA_PATH_TILE_MMA or
  * MA_PATH_GENERIC; other paths give MA_ERR_UNSUPPORTED.  Workspace as for monarch_attn_fwd_ex with
  * the same path (monarch_attn_workspace_bytes does not depend on the layout).  Everything else as
@@ -172,7 +174,7 @@ int monarch_attn_fwd_bshd(const void* Q, const void* K, const void* V, void* Y, 
  * n_valid must satisfy N - b < n_valid <= N (less than one block of padding, so that every key
  * block keeps a valid key; anything else is MA_ERR_SHAPE).  n_valid == N is the unpadded pass.
  * Runs on the per-head kernels (MA_PATH_FUSED_SMALL) where they support the shape and dtype,
- * on the second-generation tensor kernel (MA_PATH_TENSOR) for f16/bf16 with d = 64 and
+ * on the tensor kernels (MA_PATH_TENSOR) for f16/bf16 with d = 64 and
  * m = b in {64, 128}, on the tile kernels (MA_PATH_TILE_MMA) for other 16-bit shapes they
  * support, on the fused fp32 kernel (MA_PATH_FUSED_F32) for short fp32 sequences, else on the generic kernels (any
  * dtype, m need not equal b).  Workspace: the

@@ -194,9 +194,10 @@ cudaError_t launch_tmem(const Params& P, int grid, cudaStream_t st);
 template <typename T>
 cudaError_t launch_chain(const Params& P, int grid, cudaStream_t st);
 // Whether MA_PATH_TENSOR runs the kernel of tensor_chain.cuh and not that of tensor_decoupled.cuh (by size alone: either layout
-// gives the same bits).  Measured over heads of 4096 in loops of tenths of a second, us (this one / that one): two
-// rounds: 16 heads 39.4 / 37.0, 24 43.7 / 44.4, 32 48.6 / 50.8, 64 82 / 90, one round: 32 31.3 / 30.8, 48 39.0 / 41.0; two rounds in the other
-// layout or masked, where that one is a fifth slower: 36 57.9 / 68.4, 48 68.0 / 76.7.
+// gives the same bits; for one round both kernels do).  Measured over heads of 4096 in loops of tenths of a second, us (this one / that one):
+// two rounds: 16 heads 39.4 / 37.0, 24 43.7 / 44.4, 32 48.4 / 50.2 (on another GPU 49.8 / 49.3), 33 48.7 / 51.9, 36 49.8 / 55.0, 64 82 / 89; one round: 32
+// 30.8 / 30.9 (on the other 31.2 / 30.9), 33 30.9 / 32.6, 35 32.4 / 32.9, 38 33.1 / 34.9, 48 37.8 / 41.1, 64 51 / 53; masked or in the other layout, where
+// that one is a fifth slower: one round 32 34.4 / 35.3 and 34.4 / 37.7, two rounds 32 55.1 / 58.1, 48 66.2 / 78.6.
 inline bool chain_chosen(int BH, int N, int b) { return b == 64 && (long long)BH * N / kRows >= 1024; }      // tiles of a half-step
 
 // mode 0: kernel of tensor_decoupled.cuh or tensor_chain.cuh; mode 1: kernel of tensor_tmem.cuh (m = b in {64, 128},
