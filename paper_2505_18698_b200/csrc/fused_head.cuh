@@ -8,7 +8,7 @@
 // instruction stream is short enough.  Hence
 //   * an SM works on as many heads at a time as its shared memory holds: three or two small CTAs, or one CTA that
 //     starts on a head by requesting the next (every warp asks TMA for the Q, K and V rows of the blocks it will own
-//     there, zero-filled past d); `plan` chooses.  A head of 16 x 24 takes 157 KB: one, with its loads exposed;
+//     there, zero-filled past d); `plan` (head_plan.h) chooses.  A head of 16 x 24 takes 157 KB: one, with its loads exposed;
 //   * rows of a tile lie k bp + i with an odd block pitch bp = b | 1: under the 128-byte swizzle of the TMA
 //     eight rows are then free of bank conflicts along a block (R half-step) and across blocks
 //     (L half-step), so the permutation between the half-steps is only a choice of rows;
@@ -652,6 +652,7 @@ template <typename TIn, int ROUNDS>
 inline int launch_n(const Params& P, const Plan& p, int num_sms, cudaStream_t st) {
   const int nb = (P.b + 7) / 8, nm = (P.m + 7) / 8;
   if (p.bound == 16 && nb == 2 && nm == 2) return launch_k<TIn, 2, 2, ROUNDS, 16>(P, p, num_sms, st);
+  if (p.bound == 24 && nb == 3 && nm == 2) return launch_k<TIn, 3, 2, ROUNDS, 24>(P, p, num_sms, st);
 #define MA_FH(B)                                            \
   (nm == 2 ? launch_k<TIn, B, 2, ROUNDS>(P, p, num_sms, st) \
            : (nm == 3 ? launch_k<TIn, B, 3, ROUNDS>(P, p, num_sms, st) : launch_k<TIn, B, 4, ROUNDS>(P, p, num_sms, st)))

@@ -26,7 +26,7 @@ enum Rounds { kOne = 0, kMore = 1, kMoreVLast = 2 };
 // 24 rows or blocks in one turn instead of two (us with 24 / with 16: 768 heads of 20 x 20 59.1 / 62.4 in f16, 66.9 / 74.3 in bf16, 12 heads
 // 9.0 / 10.3; 24 x 16 48.0 / 47.9, 56.3 / 56.3, 12 heads 6.9 / 7.1; 10 x 18 29.9 / 30.1, 35.4 / 36.2; 14 x 22 41.9 / 40.8, 50.0 / 50.0).
 // 25 to 32 take two turns either way and 80 registers spill 20 to 52 bytes (12 x 32 47.5 / 46.0, 32 x 11 48.1 / 45.9, 32 x 17 79.6 / 71.6, bf16 92.5 / 89.2,
-// 26 x 22 bf16 100.3 / 98.1, though 28 x 20 bf16 88.5 / 90.5); so do more rounds (24 x 16 81.5 / 77.6, bf16 88.5 / 85.4, 20 x 12 61.0 / 58.9): 16.
+// 26 x 22 bf16 100.3 / 98.1, though 28 x 20 bf16 88.5 / 90.5); so do more rounds (24 x 16 81.5 / 77.6, bf16 88.5 / 85.4, 20 x 12 61.0 / 58.9), a head an SM: 16.
 constexpr int max_warps(int nb, int nm, int rounds) { return nb == 2 && nm == 2 ? 32 : (rounds == kOne && nb <= 3 && nm <= 3 ? 24 : 16); }
 
 // Shared memory of a CTA: `bufs` x (Q, K, V), the state tile (more than one round), a dump for matrix-store rows past a
@@ -54,25 +54,35 @@ inline bool plan(int b, int m, int T, int BH, int num_sms, Plan* p) {
     if (p->smem > kMaxSmem) continue;
     auto fit = [](size_t bytes) { return (int)(kSmSmem / (bytes + kCtaReserve)); };      // CTAs per SM by shared memory
     // At most one head per SM: one CTA with as many warps as a half-step has tiles.  More: the warps an SM holds go to
-    // as many CTAs as fit, up to three, each with a head of its own (768 heads of 130 = 13 x 10, two rounds: 34.6 us with
-    // three, 39.8 with two).  Where no third fits and there are heads left for a second turn, one CTA of all warps
-    // with the next head's loads under way is faster with 16 warps an SM (it has the same work in flight), with 32 two
-    // CTAs are, and V goes over the states where that makes room for the second.
-    p->ctas = BH <= num_sms ? 1 : std::min(fit(p->smem), 3);
-    const int most = max_warps(nb, nm, rounds);
+    // as many CTAs as fit, up to three and up to the heads an SM gets, each with a head of its own (768 heads of 130 = 13 x 10, two rounds:
+    // 34.6 us with three, 39.8 with two; 216 of 187 = 11 x 17, one round 8.9 with two, 12.0 with three, 280 of 17 x 9 8.6 / 12.1).  Where no third fits
+    // and there are heads left for a second turn, one CTA of all warps with the next head's loads under way is faster with 16 warps an
+    // SM (it has the same work in flight), with 32 two CTAs are, and V goes over the states where that makes room for the second.
+    p->ctas = std::min({fit(p->smem), 3, (BH + num_sms - 1) / num_sms});
+    int most = max_warps(nb, nm, rounds);
     if (p->ctas <= 2 && BH > p->ctas * num_sms) {
       const size_t v_last = smem_bytes(p->tile, 1, kMoreVLast, b, nm);
-      if (most == 32 && p->ctas == 2) {
-      } else if (most == 32 && rounds == kMore && fit(v_last) >= 2) {
+      // But a turn of two heads an SM takes 1.6 to 1.7 times a turn of one, also where it is less than full, because which SMs the last
+      // heads meet is chance (up to half a head an SM it takes 1.1).  So one CTA where that makes fewer of it (us, one CTA / two): 16 x 16, one round
+      // 360 heads 14.0 / 13.2, 380 14.1 / 15.2, 440 14.4 / 16.1, 460 17.3 / 16.1, 740 21.9 / 22.7, 768 24.8 / 22.7, 1000 29.0 / 29.1; 14 x 15, two
+      // rounds 380 21.4 / 21.9, 440 21.5 / 24.6, 592 27.9 / 25.2, 740 34.0 / 35.9, 768 39.5 / 35.8.
+      const bool ahead = two <= kMaxSmem;
+      const int left = BH % (2 * num_sms), one_each = 10 * ((BH + num_sms - 1) / num_sms);
+      const int two_each = 17 * (BH / (2 * num_sms)) + (left == 0 ? 0 : (2 * left <= num_sms ? 11 : 17));
+      const bool pairs = most == 32 && (!ahead || two_each < one_each);
+      if (pairs && p->ctas == 2) {
+      } else if (pairs && rounds == kMore && fit(v_last) >= 2) {
         p->ctas = 2;
         p->rounds = kMoreVLast;
         p->smem = v_last;
-      } else if (two <= kMaxSmem) {
+      } else if (ahead) {
         p->ctas = 1;
         p->bufs = 2;
         p->smem = two;
       }
     }
+    // (24 x 16 and the like, more rounds: 24 warps where they are two heads: 216 heads of 20 x 10 16.0 us, with 16 17.4)
+    if (nb == 3 && nm == 2 && rounds == kMore && p->ctas == 2) most = 24;
     // the fewest warps that take the fewest rounds of tiles over both half-steps
     int best = 1 << 30;
     for (int w = 1; w <= most / p->ctas; ++w) {

@@ -18,7 +18,7 @@ int main() {{
   for (int b = 9; b <= 32; ++b)
     for (int m = 9; m <= 32; ++m)
       for (int T = 1; T <= 2; ++T)
-        for (int BH : {{1, 12, 148, 149, 160, 296, 297, 444, 445, 768, 100000}}) {{
+        for (int BH : {{1, 12, 148, 149, 160, 296, 297, 370, 371, 444, 445, 740, 768, 100000}}) {{
           Plan p;
           if (plan(b, m, T, BH, 148, &p))
             printf("%d %d %d %d %d %d %d %d %zu %d\\n", b, m, T, BH, p.ctas, p.warps, p.bufs, p.rounds, p.smem, p.bound);
