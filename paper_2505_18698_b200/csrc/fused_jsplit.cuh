@@ -118,7 +118,7 @@ monarch_jsplit32(const __grid_constant__ CUtensorMap tmQ,    // Q as rows of d, 
   constexpr int NT = PJ / 8;                    // 8-position tiles
   extern __shared__ uint8_t smem_raw[];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem = align_smem<1024>(smem_raw);
   const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(smem);
   float* sCL = reinterpret_cast<float*>(smem + L::C);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::Bar);      // by warp: what it asked for has landed in its slot

@@ -174,7 +174,7 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, Ba
 template <typename T, int B, int SB, bool EXTRA>
 __global__ void __launch_bounds__(kThreads, 1) monarch_decoupled(const __grid_constant__ Params P) {
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem = align_smem<1024>(smem_raw);
   constexpr bool HILO = std::is_same<T, __nv_bfloat16>::value && SB == 32;
   using Lay = tp2::Lay<B, HILO>;
   using C = Cfg<B, HILO>;

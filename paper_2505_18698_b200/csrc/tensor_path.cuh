@@ -30,6 +30,7 @@
 #include <stdint.h>
 
 #include "f32x2.cuh"
+#include "shared_align.cuh"
 
 namespace ma {
 namespace tensor {
@@ -534,7 +535,7 @@ r_step_tc(const __grid_constant__ CUtensorMap tmA,      // aR (or Q when FIRST):
           const __grid_constant__ CUtensorMap tmYs,     // y store:  3D (64, m, BH*b)
           const float* __restrict__ cR, float* __restrict__ cL, int* status, int m, float scale) {
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem = align_smem<1024>(smem_raw);
   Barriers* bars = reinterpret_cast<Barriers*>(smem + SmemLayout::Bars);
   const int t = threadIdx.x, warp = t >> 5;
   constexpr int kTiles = Geo<B>::kTiles;
@@ -665,7 +666,7 @@ l_step_tc(const __grid_constant__ CUtensorMap tmQs,     // Q strided view: 3D (6
           const __grid_constant__ CUtensorMap tmOut,    // aR (or Y when FINAL) strided view: 3D
           const float* __restrict__ cL, float* __restrict__ cR, int* status, int m, float scale) {
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem = align_smem<1024>(smem_raw);
   Barriers* bars = reinterpret_cast<Barriers*>(smem + SmemLayout::Bars);
   float* cvec = reinterpret_cast<float*>(smem + SmemLayout::Vec);   // [tile][k] : cL * log2e
   const int t = threadIdx.x, warp = t >> 5;

@@ -251,7 +251,7 @@ __device__ __forceinline__ void store_packed_row64(uint8_t* tile, int srow, cons
 template <typename T, int B, bool TRACE>
 __global__ void __launch_bounds__(kThreads, 1) monarch_tmem(const __grid_constant__ Params P) {
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem = align_smem<1024>(smem_raw);
   using Lay = tp3::Lay<B>;
   using C = Cfg<B>;
   constexpr int kRingE = C::kRingE, kRingL = C::kRingL, kRingV = C::kRingV;

@@ -839,7 +839,7 @@ struct Kernel {
 template <typename TIn, int B, bool FULL, int MODE>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm) monarch_tiles(const __grid_constant__ Params P) {
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem = align_smem<1024>(smem_raw);
   Shared* sh = reinterpret_cast<Shared*>(smem + kOffBar);
   const int tid = threadIdx.x, warp = tid >> 5;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
