@@ -5,8 +5,9 @@
 // kernel is how many chains an SM has in flight and what the states cost on their way through L2.  So, against the one chain with
 // a stage per warpgroup of tensor_decoupled.cuh:
 //   * two CTAs per SM with two compute groups of four warps each; a group (thread = score row) takes a tile from its scores
-//     to its staged rows, and its first warp issues the tile's MMAs itself: nobody polls, a hand-over is a barrier
-//     of the group;
+//     to its staged rows, and its first warp issues the tile's MMAs itself.  That warp alone looks at mbarriers, which means trying again
+//     and again; the others and the store warp wait in hardware barriers (64 heads of 4096, T = 2: 77.8 us with every warp
+//     at the mbarriers, 76.7 with one; trying in a tighter loop, a quarter more branches in all, cost 4 %);
 //   * three 16 KB slots a group.  Which of them a tile's operands take follows from the order in which the tile before gives
 //     its slots up (Slots), so that loads of the next tile run under the softmax of this one;
 //   * the weights go back to tensor memory over the scores and are the A operand of the apply MMA; in the non-final L
@@ -14,7 +15,7 @@
 //     more columns, of a tile of ones;
 //   * alpha_R is stored divided by c_R: no c_R vector.  f16: the weights of that half-step carry 2^14 (the quotient does not change), so
 //     that columns of small weights keep their bits.
-// Service warps: a producer and a store thread per group.
+// Service warps: a producer thread and a store warp per group.
 //
 // Measured (B200, us per call in loops of tenths of a second, against tensor_decoupled.cuh): 64 heads of 4096, T = 2 82 / 91 (bursts: 74 / 88;
 // the loop runs into the power limit, at 1765 MHz), 48 heads masked 68 / 77. A tile takes 3.8 to 5.7 us, of which its group waits
@@ -56,7 +57,8 @@ static_assert(kCtasPerSm * (kSmem + 1024) <= 228 * 1024, "two CTAs per SM");
 struct __align__(16) Shared {
   uint64_t full[2][2], third[2][2];                   // by group, tiles in turn: first two operands, third slot
   uint64_t empty[kSlots];
-  uint64_t mma1[2], weights[2], first[2], oread[2], mma2[2], o_free[2], staged[2], out_free[2];
+  uint64_t mma1[2], first[2], mma2[2], o_free[2], out_free[2];
+  int go[2];                                          // whether the group goes on: its first warp's word before every release
   int4 tile[2][2];                                    // {half-step, head, first block or position} of a tile, or {-1, ..}
   int4 out[2];                                        // {head or -1, first block or position, slot | Rows << 4 | last << 8, half-step}
   uint32_t tmem;
@@ -82,7 +84,9 @@ struct Slots {
   }
 };
 
-// Bounded wait: after a timeout (status word and abort flag set) every wait of the CTA returns at once.
+// Bounded wait: after a timeout (status word and abort flag set) every wait of the CTA returns at once (HEED: but for those that
+// come to an end by themselves).
+template <bool HEED = true>
 __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Shared* sh, const Params& P, int where) {
   const uint32_t addr = smem_u32(bar);
   long long t0 = 0;
@@ -96,7 +100,7 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Shared*
         : "r"(addr), "r"(parity)
         : "memory");
     if (done) return true;
-    if (sh->abort_flag) return false;
+    if (HEED && sh->abort_flag) return false;
     if (n == 0) {
       t0 = clock64();
     } else if (clock64() - t0 > P.wait_cycles) {
@@ -106,6 +110,12 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Shared*
     }
   }
 }
+
+// Barriers in hardware, by group: the first warp lets the others go on, it waits for them, the store warp waits for staged
+// rows.
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+enum BarId { kRelease = 1, kCollect = 3, kStaged = 5 };
 
 // Tile p, h, idx0 as its roles see it.
 __device__ __forceinline__ Tile tile_of(const Params& P, int p, int h, int idx0) {
@@ -217,30 +227,35 @@ struct Chain {
     }
   }
 
-  // ================================================================ store thread of group w
+  // ================================================================ store warp of group w (its first lane)
   static __device__ __forceinline__ void store(const Params& P, uint8_t* smem, Shared* sh, int w) {
     const uint64_t pol_first = policy_evict_first();
-    for (uint32_t par = 0;; par ^= 1) {
-      if (!wait_bar(&sh->staged[w], par, sh, P, 40)) break;
+    const bool lane0 = (threadIdx.x & 31) == 0;
+    for (;;) {
+      bar_sync(kStaged + w, 160);
       const int4 o = sh->out[w];
-      mbar_arrive(&sh->out_free[w]);
+      __syncwarp();
+      if (lane0) mbar_arrive(&sh->out_free[w]);
       if (o.x < 0) break;
-      const int slot = o.z & 15, rows = (o.z >> 4) & 15;
-      const uint8_t* s = smem + slot * kSlot;
-      if (rows == kAlphaL) tma_store_3d(&P.tmALs, s, 0, o.x * B, o.y);
-      else if (rows == kY) tma_store_3d(&P.tmYs, s, 0, o.x * B, o.y);
-      else if (rows == kAlphaR) tma_store_3d(&P.tmARs, s, 0, o.x * P.m, o.y);
-      else tma_store_3d_hint(&P.tmOut, s, (EXTRA && P.H) ? (o.x % P.H) * kD : 0, ((EXTRA && P.H) ? o.x / P.H : o.x) * P.m, o.y, pol_first);
-      tma_store_commit();
-      tma_store_wait_read();
-      mbar_arrive(&sh->empty[slot]);
-      if (o.z >> 8) {                        // the tile's last rows: counted once they (and c_L) are in global memory
-        tma_store_wait_all();
-        asm volatile("fence.proxy.async.global;" ::: "memory");
-        asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(P.counters + o.w * P.BH + o.x) : "memory");
+      if (lane0) {
+        const int slot = o.z & 15, rows = (o.z >> 4) & 15;
+        const uint8_t* s = smem + slot * kSlot;
+        if (rows == kAlphaL) tma_store_3d(&P.tmALs, s, 0, o.x * B, o.y);
+        else if (rows == kY) tma_store_3d(&P.tmYs, s, 0, o.x * B, o.y);
+        else if (rows == kAlphaR) tma_store_3d(&P.tmARs, s, 0, o.x * P.m, o.y);
+        else tma_store_3d_hint(&P.tmOut, s, (EXTRA && P.H) ? (o.x % P.H) * kD : 0, ((EXTRA && P.H) ? o.x / P.H : o.x) * P.m, o.y, pol_first);
+        tma_store_commit();
+        tma_store_wait_read();
+        mbar_arrive(&sh->empty[slot]);
+        if (o.z >> 8) {                        // the tile's last rows: counted once they (and c_L) are in global memory
+          tma_store_wait_all();
+          asm volatile("fence.proxy.async.global;" ::: "memory");
+          asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(P.counters + o.w * P.BH + o.x) : "memory");
+        }
       }
+      __syncwarp();
     }
-    tma_store_wait_all();
+    if (lane0) tma_store_wait_all();
   }
 
   // ================================================================ MMAs (one thread of the group's first warp)
@@ -285,35 +300,70 @@ struct Chain {
     Slots x(w);
     uint32_t par_o = 1, par_1 = 0;
     uint32_t par_3 = 0;                        // bit i: parity of third[w][i]
-#define MA_WAIT(BAR, PAR, WHERE) \
-  if (!__all_sync(0xffffffffu, wait_bar(&(BAR), PAR, sh, P, WHERE))) return
+    bool ok = true;                            // (first warp) no wait has run out
+    // The first warp alone looks at mbarriers and lets the others go on once it has seen one: four warps that try and try again take
+    // issue slots from those at work.  A wait that ran out reaches the others with the same release.
+    auto await = [&](uint64_t* bar, uint32_t parity, int where) { ok = __all_sync(0xffffffffu, wait_bar(bar, parity, sh, P, where)) && ok; };
+    auto release = [&](bool on) {              // of the group; false: no more tiles
+      if (t_row == 0) sh->go[w] = on;
+      tc_fence_before();
+      bar_sync(kRelease + w, 128);
+      tc_fence_after();
+      return *(volatile int*)&sh->go[w] != 0;
+    };
+    auto collect = [&]() {                     // all warps have come by: the first one waits
+      tc_fence_before();
+      if (warp == 0) {
+        bar_sync(kCollect + w, 128);
+        tc_fence_after();
+      } else {
+        bar_arrive(kCollect + w, 128);
+      }
+    };
+    // An accumulator is done, and the store warp has taken the word of the rows before: nobody comes by at kStaged a second time
+    // before the store warp has.
+    auto await_rows = [&](uint64_t* bar, uint32_t parity, int where) {
+      if (warp == 0) {
+        await(bar, parity, where);
+        if (ok) await(&sh->out_free[w], par_o, 38);
+        if (ok) par_o ^= 1;
+      }
+      return release(ok);
+    };
     auto hand_over = [&](int h, int idx0, int what, int p) {
-      const bool ok = wait_bar(&sh->out_free[w], par_o, sh, P, 38);
-      par_o ^= 1;
       if (t_row == 0) sh->out[w] = make_int4(h, idx0, what, p);
-      mbar_arrive(&sh->staged[w]);
-      return __all_sync(0xffffffffu, ok);
+      __syncwarp();
+      bar_arrive(kStaged + w, 160);
     };
     for (uint32_t q = 0;; ++q) {
       const uint32_t par = q & 1;
       const uint32_t a0 = sm + x.x0 * kSlot, a1 = sm + x.x1 * kSlot, a2 = sm + x.x2 * kSlot;
-      MA_WAIT(sh->full[w][q & 1], (q >> 1) & 1, 30);
-      const int4 it = sh->tile[w][q & 1];
-      if (it.x < 0) break;
-      const Tile t = tile_of(P, it.x, it.y, it.z);
+      bool more = true;
       if (warp == 0) {
-        MA_WAIT(sh->o_free[w], par ^ 1, 29);   // every row of the tile before has left tensor memory
-        tc_fence_after();
-        if (elect_one()) {
-          issue_scores<B, FT>(d, a0, a1, P.negate);
-          umma_commit(&sh->mma1[w]);
-          if (t.isR || t.final_) umma_commit(&sh->empty[x.x0]);
-          if (t.final_) umma_commit(&sh->empty[x.x1]);
+        if (q > 0) {                           // every row of the tile before has left tensor memory
+          bar_sync(kCollect + w, 128);
+          tc_fence_after();
+          if (t_row == 0) mbar_arrive(&sh->o_free[w]);
         }
-        __syncwarp();
+        await(&sh->full[w][q & 1], (q >> 1) & 1, 30);
+        const int4 it = sh->tile[w][q & 1];
+        more = ok && it.x >= 0;
+        if (more) {
+          const Tile t = tile_of(P, it.x, it.y, it.z);
+          if (elect_one()) {
+            issue_scores<B, FT>(d, a0, a1, P.negate);
+            umma_commit(&sh->mma1[w]);
+            if (t.isR || t.final_) umma_commit(&sh->empty[x.x0]);
+            if (t.final_) umma_commit(&sh->empty[x.x1]);
+          }
+          __syncwarp();
+          await(&sh->mma1[w], par, 31);
+          more = ok;
+        }
       }
-      MA_WAIT(sh->mma1[w], par, 31);
-      tc_fence_after();
+      if (!release(more)) break;
+      const int4 it = sh->tile[w][q & 1];
+      const Tile t = tile_of(P, it.x, it.y, it.z);
       // the state rows the score MMA consumed are read exactly once: drop them from L2
       if (!t.isR) discard_line(P.aL + ((size_t)(t.h * B + t.idx0) * m + t_row) * 128);
       else if (!t.first) discard_line(P.aR + ((size_t)(t.h * m + t.idx0) * B + t_row) * 128);
@@ -451,16 +501,11 @@ struct Chain {
           fence_proxy_async();
         }
       }
-      tc_fence_before();
-      mbar_arrive(&sh->weights[w]);
+      collect();
       const bool third = Slots::uses_third(t);
       if (warp == 0) {
-        MA_WAIT(sh->weights[w], par, 35);
-        if (t.final_) {
-          MA_WAIT(sh->third[w][q & 1], (par_3 >> (q & 1)) & 1, 36);
-        }
-        tc_fence_after();
-        if (elect_one()) {
+        if (t.final_) await(&sh->third[w][q & 1], (par_3 >> (q & 1)) & 1, 36);
+        if (ok && elect_one()) {
           if (t.isR) {
             apply(d, a1);
             umma_commit(t.withV ? &sh->first[w] : &sh->mma2[w]);
@@ -478,19 +523,15 @@ struct Chain {
       // ============================================================== rows
       float o[64];
       if (t.isR && t.withV) {                  // alpha_L, over K; then y = R V through the same columns, over V
-        MA_WAIT(sh->first[w], par_1, 32);
+        if (!await_rows(&sh->first[w], par_1, 32)) break;
         par_1 ^= 1;
-        tc_fence_after();
         tmem_ld32(tS + 64, o);
         tmem_ld32(tS + 96, o + 32);
         tmem_ld_wait();
-        tc_fence_before();
-        mbar_arrive(&sh->oread[w]);
+        collect();
         if (warp == 0) {
-          MA_WAIT(sh->oread[w], par_1 ^ 1, 37);
-          MA_WAIT(sh->third[w][q & 1], (par_3 >> (q & 1)) & 1, 36);
-          tc_fence_after();
-          if (elect_one()) {
+          await(&sh->third[w][q & 1], (par_3 >> (q & 1)) & 1, 36);
+          if (ok && elect_one()) {
             apply(d, a2);
             umma_commit(&sh->mma2[w]);
           }
@@ -499,10 +540,9 @@ struct Chain {
         store_row32<T>(smem + x.x1 * kSlot, srow, 0, o, mul);
         store_row32<T>(smem + x.x1 * kSlot, srow, 32, o + 32, mul);
         fence_proxy_async();
-        if (!hand_over(t.h, t.idx0, x.x1 | kAlphaL << 4, t.p)) return;
+        hand_over(t.h, t.idx0, x.x1 | kAlphaL << 4, t.p);
       }
-      MA_WAIT(sh->mma2[w], par, 33);
-      tc_fence_after();
+      if (!await_rows(&sh->mma2[w], par, 33)) break;
       if (t.final_) discard_line(P.y + ((size_t)(t.h * B + t.idx0) * m + t_row) * 128);
       const bool turned = !t.isR && !t.final_;
       float cr = 1.f;
@@ -512,18 +552,20 @@ struct Chain {
       tmem_ld32(tO + 32, o + 32);
       tmem_ld_wait();
       tc_fence_before();
-      mbar_arrive(&sh->o_free[w]);
+      if (warp != 0) bar_arrive(kCollect + w, 128);        // (the first warp waits for it before the next tile's scores)
       if (turned) mul = cr > 1e-30f ? 1.f / cr : 0.f;
       const int slot = t.isR ? (t.withV ? x.x2 : x.x1) : (t.final_ ? x.x2 : x.x0);
       store_row32<T>(smem + slot * kSlot, srow, 0, o, mul);
       store_row32<T>(smem + slot * kSlot, srow, 32, o + 32, mul);
       fence_proxy_async();
-      if (!hand_over(t.h, t.idx0, slot | (t.isR ? (t.withV ? kY : kAlphaL) : (t.final_ ? kOut : kAlphaR)) << 4 | 1 << 8, t.p)) return;
+      hand_over(t.h, t.idx0, slot | (t.isR ? (t.withV ? kY : kAlphaL) : (t.final_ ? kOut : kAlphaR)) << 4 | 1 << 8, t.p);
       if (third) par_3 ^= 1u << (q & 1);
       x.next(t);
     }
+    // (aborted or not: rows handed over before are on their way, and the store warp comes back for this word)
+    if (warp == 0) __all_sync(0xffffffffu, wait_bar<false>(&sh->out_free[w], par_o, sh, P, 38));
+    release(false);
     hand_over(-1, 0, 0, 0);
-#undef MA_WAIT
   }
 };
 
@@ -545,10 +587,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) monarch_chain(const __gr
       mbar_init(&sh->first[w], 1);
       mbar_init(&sh->mma2[w], 1);
       mbar_init(&sh->out_free[w], 1);
-      mbar_init(&sh->weights[w], 128);
-      mbar_init(&sh->oread[w], 128);
-      mbar_init(&sh->o_free[w], 128);
-      mbar_init(&sh->staged[w], 128);
+      mbar_init(&sh->o_free[w], 1);
     }
     sh->abort_flag = 0;
     fence_barrier_init();
@@ -568,10 +607,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) monarch_chain(const __gr
   // registers: 384 threads at the launch's 80; 128 x 48 + 256 x 96 make use of all of them
   if (warp >= 8) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
-    if (elect_one()) {
-      if (warp < 10) C::produce(P, smem, sh, warp - 8);
-      else C::store(P, smem, sh, warp - 10);
-    }
+    if (warp >= 10) C::store(P, smem, sh, warp - 10);
+    else if (elect_one()) C::produce(P, smem, sh, warp - 8);
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 96;");
     C::compute(P, smem, sh, tmem, warp >> 2);
