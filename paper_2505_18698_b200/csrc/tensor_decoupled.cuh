@@ -166,15 +166,15 @@ __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, Ba
   }
 }
 
-// EXTRA: the rarely used hooks (inputs laid out [batch][N][heads][d], row log-sum-exp output, time
-// stamps for the trace buffer) are
-// compiled into a second instantiation: in the plain one they cost 4 % even when switched off (the
-// producer's instruction stream is on the critical path and the compiler predicates the head
-// index division instead of branching around it).
-template <typename T, int B, int SB, bool EXTRA>
+// EXTRA: what plain calls do without is compiled into instantiations of its own: 1: inputs laid out [batch][N][heads][d], row log-sum-exp
+// output (in the plain one they cost 4 % even when switched off: the producer's instruction stream is on the critical path and the
+// compiler predicates the head index division instead of branching around it); 2: the padding mask and the time stamps of the trace
+// buffer too (their selects cost the other layout 10 to 15 %: 8 heads of 16384, T = 2 74 / 62 us, 4 49 / 44).
+template <typename T, int B, int SB, int EXTRA>
 __global__ void __launch_bounds__(kThreads, 1) monarch_decoupled(const __grid_constant__ Params P) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem<1024>(smem_raw);
+  constexpr bool ALL = EXTRA == 2;
   constexpr bool HILO = std::is_same<T, __nv_bfloat16>::value && SB == 32;
   using Lay = tp2::Lay<B, HILO>;
   using C = Cfg<B, HILO>;
@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(kThreads, 1) monarch_decoupled(const __grid_co
               // one box: kBlocks blocks (positions j) of SB rows (l) each, block after block
               tma_load_3d(sL, &P.tmQs, &bars->fullL[eL], xin, hin * m, t.idx0);
             }
-            if (EXTRA) stamp(P, nE, 0);
+            if (ALL) stamp(P, nE, 0);
             ++nE;
             rE.advance();
             rL.advance();
@@ -376,7 +376,7 @@ __global__ void __launch_bounds__(kThreads, 1) monarch_decoupled(const __grid_co
             if (needV) { umma_commit(&bars->emptyV[eV]); rV.advance(); }
             umma_commit(&bars->p_free[c]);
             umma_commit(&bars->o_ready[o2]);
-            if (EXTRA) stamp(P, i2, 4);
+            if (ALL) stamp(P, i2, 4);
             ++i2;
             it2.next();
             r2L.advance();
@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(kThreads, 1) monarch_decoupled(const __grid_co
           if (HILO && !t.isR) issue_scores<B, FT, FT, true>(tmem + s1 * B, sL, sE + kSlot, P.negate);
           umma_commit(&bars->emptyE[eE]);
           umma_commit(&bars->s_ready[s1]);
-          if (EXTRA) stamp(P, i1, 1);
+          if (ALL) stamp(P, i1, 1);
           ++i1;
           it1.next();
           r1E.advance();
@@ -456,7 +456,7 @@ __global__ void __launch_bounds__(kThreads, 1) monarch_decoupled(const __grid_co
           // for the round trip to the counter's home in L2 as it would with a fence and an atomic)
           asm volatile("fence.proxy.async.global;" ::: "memory");
           asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(P.counters + t.p * P.BH + t.h) : "memory");
-          if (EXTRA) stamp(P, n, 7);
+          if (ALL) stamp(P, n, 7);
           round += nr;
         }
       }
@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(kThreads, 1) monarch_decoupled(const __grid_co
       const uint32_t tS = tmem + s * B + ((uint32_t)(sub * 32) << 16);
       wait_or_abort(&bars->s_ready[s], (n / kStagesS) & 1, bars, P.report, 30);
       tc_fence_after();
-      if (EXTRA && stamper) stamp(P, n, 2);
+      if (ALL && stamper) stamp(P, n, 2);
       // the state tile MMA 1 consumed is read exactly once: drop its lines from L2
       if (t.isR) {
         if (!t.first) discard_line(P.aR + ((size_t)(t.h * m + t.idx0) * SB + t_row) * 128);
@@ -508,7 +508,7 @@ __global__ void __launch_bounds__(kThreads, 1) monarch_decoupled(const __grid_co
         // Padding mask (App. C.3): in the last key block the columns from `lim` on are keys past
         // n_valid; they take no part in the maximum and get weight 0.
         int lim = B;
-        if (EXTRA && SB == B && P.n_valid != 0 && t.idx0 + blk == m - 1) lim = P.n_valid - (m - 1) * SB;
+        if (ALL && SB == B && P.n_valid != 0 && t.idx0 + blk == m - 1) lim = P.n_valid - (m - 1) * SB;
         if constexpr (SB == B) {
           // Every row owns all B columns: 16-column chunks, the load of the next chunk in flight
           // while the current one is worked on (TMEM reads compete with the MMAs' accumulator
@@ -524,7 +524,7 @@ __global__ void __launch_bounds__(kThreads, 1) monarch_decoupled(const __grid_co
             float* nxt = (cc & 1) ? b0 : b1;
             tmem_ld_wait();
             tmem_ld16(tS + 16 * ((cc + 1) % NC16), nxt);     // wraps to the first chunk of pass 2
-            if (EXTRA && lim < B) {
+            if (ALL && lim < B) {
 #pragma unroll
               for (int i = 0; i < 16; ++i)
                 if (16 * cc + i >= lim) cur[i] = -INFINITY;
@@ -545,13 +545,13 @@ __global__ void __launch_bounds__(kThreads, 1) monarch_decoupled(const __grid_co
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
               float2 x = make_float2(cur[2 * i], cur[2 * i + 1]);
-              if (EXTRA && lim < B) {      // masked keys: score 0 (any finite value), weight 0 below
+              if (ALL && lim < B) {      // masked keys: score 0 (any finite value), weight 0 below
                 if (16 * cc + 2 * i >= lim) x.x = 0.f;
                 if (16 * cc + 2 * i + 1 >= lim) x.y = 0.f;
               }
               const float2 zz = ffma2(x, f2, off2);
               float2 pp = exp2_pair(zz, i);
-              if (EXTRA && lim < B) {
+              if (ALL && lim < B) {
                 if (16 * cc + 2 * i >= lim) pp.x = 0.f;
                 if (16 * cc + 2 * i + 1 >= lim) pp.y = 0.f;
               }
@@ -768,7 +768,7 @@ __global__ void __launch_bounds__(kThreads, 1) monarch_decoupled(const __grid_co
       fence_proxy_async();
       tc_fence_before();
       mbar_arrive(&bars->p_ready[c]);
-      if (EXTRA && stamper) stamp(P, n, 3);
+      if (ALL && stamper) stamp(P, n, 3);
     }
   } else {
     // ------------------------------------------------------------------ epilogue group: O -> rows
@@ -789,7 +789,7 @@ __global__ void __launch_bounds__(kThreads, 1) monarch_decoupled(const __grid_co
       const uint32_t tO = tO0 + o * 128;
       wait_or_abort(&bars->o_ready[o], (n / kStagesO) & 1, bars, P.report, 31);
       tc_fence_after();
-      if (EXTRA && stamper) stamp(P, n, 5);
+      if (ALL && stamper) stamp(P, n, 5);
       const float inv_s = stat[(n & 3) * 128 + t_row];
       if (t.final_) discard_line(P.y + ((size_t)(t.h * SB + t.idx0) * m + t_row) * 128);
       const int nr = rounds_of(t);
@@ -828,7 +828,7 @@ __global__ void __launch_bounds__(kThreads, 1) monarch_decoupled(const __grid_co
         mbar_arrive(&bars->stage_ready[n & 1]);
       }
       if (!scaled) P.cR[((size_t)t.h * m + rb) * SB + t.idx0 + blk] = c1;
-      if (EXTRA && stamper) stamp(P, n, 6);
+      if (ALL && stamper) stamp(P, n, 6);
       round += nr;
     }
   }
@@ -850,7 +850,7 @@ __global__ void __launch_bounds__(kThreads, 1) monarch_decoupled(const __grid_co
   }
 }
 
-template <typename T, int B, int SB, bool EXTRA>
+template <typename T, int B, int SB, int EXTRA>
 inline cudaError_t launch_kernel_x(const Params& P, int grid, cudaStream_t st) {
   const void* fn = (const void*)monarch_decoupled<T, B, SB, EXTRA>;
   constexpr int kSmem = Lay<B, std::is_same<T, __nv_bfloat16>::value && SB == 32>::kSmem;
@@ -861,9 +861,9 @@ inline cudaError_t launch_kernel_x(const Params& P, int grid, cudaStream_t st) {
 }
 template <typename T, int B, int SB>
 inline cudaError_t launch_kernel(const Params& P, int grid, cudaStream_t st) {
-  if (P.H != 0 || P.lse != nullptr || P.trace != nullptr || P.n_valid != 0)
-    return launch_kernel_x<T, B, SB, true>(P, grid, st);
-  return launch_kernel_x<T, B, SB, false>(P, grid, st);
+  if (P.trace != nullptr || P.n_valid != 0) return launch_kernel_x<T, B, SB, 2>(P, grid, st);
+  if (P.H != 0 || P.lse != nullptr) return launch_kernel_x<T, B, SB, 1>(P, grid, st);
+  return launch_kernel_x<T, B, SB, 0>(P, grid, st);
 }
 
 }  // namespace tp2
