@@ -1,4 +1,4 @@
-// Persistent tensor-core kernel for m = b = 64 with tiles enough to fill the GPU (MA_PATH_TENSOR): tiles, order,
+// Persistent tensor-core kernel for m = b = 64 or 128 with tiles enough to fill the GPU (MA_PATH_TENSOR): tiles, order,
 // tensor maps and dependency counters as described in tensor_persistent.cuh.
 //
 // What bounds a tile is its chain load -> score MMA -> softmax -> apply MMA -> rows -> store, nearly all of it latency; what bounds the
@@ -21,8 +21,8 @@
 // the loop runs into the power limit, at 1765 MHz), 48 heads masked 68 / 77. A tile takes 3.8 to 5.7 us, of which its group waits
 // for operands 0.2 to 0.8.  Measured and not kept: tiles dealt out in advance (81 against 78 us in bursts: SMs differ in speed), a row of scores
 // in registers instead of read twice (44 bytes spilled: 80 against 74), heads in groups that stay in L2 (more tiles are in work and
-// requested, twice 592, than a half-step of 1024 leaves room for: 91 against 82), b = 128 (16 heads of 16384, T = 2: bursts 95 / 102.5, but
-// 105.3 / 105.2 at the power limit, and T = 1 63.0 / 61.2).
+// requested, twice 592, than a half-step of 1024 leaves room for: 91 against 82).
+// Blocks of 128 (16 heads of 16384, T = 2, loops): 95 / 99.5; the weights of a non-final L half-step then take two of the three slots.
 #pragma once
 #include <type_traits>
 
@@ -33,7 +33,6 @@ namespace ma {
 namespace tp3 {
 
 using namespace ma::tensor;
-constexpr int B = 64;
 using ma::tp::Params;
 using ma::tp::Tile;
 using ma::tp::bulk_load_1d;
@@ -69,8 +68,9 @@ enum Rows { kAlphaL = 0, kY = 1, kAlphaR = 2, kOut = 3 };
 
 // A group's slots as the operands of its current tile; next(): in the order in which the tile gives them up.
 //   R:            first  alpha_R (Q), free after the score MMA; second K, alpha_L staged over it; third, last round, V and y over it
-//   L, not last:  first  Q(.,j), alpha_R staged over it; second alpha_L, then weights, free after the apply MMA
+//   L, not last:  first  Q(.,j), alpha_R staged over it; second alpha_L, then weights, free after the apply MMA (128 columns: and third)
 //   L, last:      first  Q(.,j), second alpha_L, both free after the score MMA; third y, Y staged over it
+template <int B>
 struct Slots {
   int x0, x1, x2;
   __device__ __forceinline__ explicit Slots(int w) : x0(3 * w), x1(3 * w + 1), x2(3 * w + 2) {}
@@ -78,6 +78,12 @@ struct Slots {
   __device__ __forceinline__ void next(const Tile& t) {
     const int a = x0, b = x1, c = x2;
     if (uses_third(t)) return;
+    if (B == 128 && !t.isR) {
+      x0 = b;
+      x1 = c;
+      x2 = a;
+      return;
+    }
     x0 = c;
     x1 = t.isR ? a : b;
     x2 = t.isR ? b : a;
@@ -130,9 +136,11 @@ __device__ __forceinline__ Tile tile_of(const Params& P, int p, int h, int idx0)
   return t;
 }
 
-// EXTRA: inputs laid out [batch][N][heads][d], row log-sum-exp output, padding mask.
-template <typename T, bool EXTRA>
+// EXTRA 1: inputs laid out [batch][N][heads][d], row log-sum-exp output; 2: the padding mask too, whose selects every tile pays for (40 heads
+// of 4096 in the other layout 58.8 us with them, 56.0 without).
+template <typename T, int B, int EXTRA>
 struct Chain {
+  static constexpr bool MASK = EXTRA == 2;
   static constexpr int FT = Fmt<T>::code, kBlocks = kRows / B;
   static constexpr float kWeightScale = std::is_same<T, __half>::value ? 16384.f : 1.f;      // of the non-final L weights
 
@@ -141,7 +149,7 @@ struct Chain {
   // out in advance the slowest set the time (a sixth of it).
   static __device__ __forceinline__ void produce(const Params& P, uint8_t* smem, Shared* sh, int w) {
     const int tpg = P.tiles_per_phase / P.head_groups, per_group = 2 * P.T * tpg, hpg = P.BH / P.head_groups;
-    Slots x(w);
+    Slots<B> x(w);
     uint32_t busy = 0, par = 0;              // by slot: a use is to be waited for; parity of that wait
     auto take = [&](int s) {
       const uint32_t bit = 1u << s;
@@ -221,6 +229,9 @@ struct Chain {
           if (!take(x.x2)) return;
           mbar_expect_tx(bar3, kSlot);
           tma_load_2d(s2, &P.tmY, bar3, 0, row0);
+        } else if (B == 128) {                 // weights alone
+          if (!take(x.x2)) return;
+          mbar_arrive(bar3);
         }
       }
       x.next(t);
@@ -275,9 +286,9 @@ struct Chain {
   }
   // Rows k of sum_l P[l, k] [Q(l, .) | 1]: the ones are a second 64-column chunk of the B operand, whose distance shrinks as
   // the address walks down the rows of Q.
-  static __device__ __forceinline__ void apply_transposed(uint32_t d, uint32_t sP, uint32_t sQ, uint32_t sOnes) {
+  static __device__ __forceinline__ void apply_transposed(uint32_t d, uint32_t sP, uint32_t chunk, uint32_t sQ, uint32_t sOnes) {
     constexpr uint32_t id = instr_desc(B, 80, FT, 1, 1);
-    const uint64_t dP = smem_desc(sP, kSlot, 1024);
+    const uint64_t dP = smem_desc(sP, chunk, 1024);
 #pragma unroll
     for (int t = 0; t < Geo<B>::kTiles; ++t)
 #pragma unroll
@@ -297,10 +308,10 @@ struct Chain {
     const uint32_t sm = smem_u32(smem);
     const int m = P.m;
     constexpr int NC = B / 16;
-    Slots x(w);
+    Slots<B> x(w);
     uint32_t par_o = 1, par_1 = 0;
     uint32_t par_3 = 0;                        // bit i: parity of third[w][i]
-    bool ok = true;                            // (first warp) no wait has run out
+    bool ok = true;                            // (the first warp's decides) no wait has run out
     // The first warp alone looks at mbarriers and lets the others go on once it has seen one: four warps that try and try again take
     // issue slots from those at work.  A wait that ran out reaches the others with the same release.
     auto await = [&](uint64_t* bar, uint32_t parity, int where) { ok = __all_sync(0xffffffffu, wait_bar(bar, parity, sh, P, where)) && ok; };
@@ -375,7 +386,7 @@ struct Chain {
       if (t.isR) {
         // Z_R = scale S (Eq. 7; alpha_R arrives divided by c_R), -c_L log2 e = log2 sum + max - sum R z (Eq. 10)
         int lim = B;                           // keys of the block that count (App. C.3)
-        if (EXTRA && P.n_valid != 0 && t.idx0 + blk == m - 1) lim = P.n_valid - (m - 1) * B;
+        if (MASK && P.n_valid != 0 && t.idx0 + blk == m - 1) lim = P.n_valid - (m - 1) * B;
         float2 z2[2] = {both(0.f), both(0.f)};
         tmem_ld16(tS, c[0]);
 #pragma unroll
@@ -383,7 +394,7 @@ struct Chain {
           float* cur = c[cc & 1];
           tmem_ld_wait();
           tmem_ld16(tS + 16 * ((cc + 1) % NC), c[(cc + 1) & 1]);      // wraps to the first chunk of pass 2
-          if (EXTRA && lim < B) {
+          if (MASK && lim < B) {
 #pragma unroll
             for (int i = 0; i < 16; ++i)
               if (16 * cc + i >= lim) cur[i] = -INFINITY;
@@ -402,13 +413,13 @@ struct Chain {
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             float2 v = make_float2(cur[2 * i], cur[2 * i + 1]);
-            if (EXTRA && lim < B) {            // masked keys: score 0 (any finite value), weight 0 below
+            if (MASK && lim < B) {            // masked keys: score 0 (any finite value), weight 0 below
               if (16 * cc + 2 * i >= lim) v.x = 0.f;
               if (16 * cc + 2 * i + 1 >= lim) v.y = 0.f;
             }
             const float2 e = ffma2(v, f2, off2);
             float2 p = make_float2(fast_exp2(e.x), fast_exp2(e.y));
-            if (EXTRA && lim < B) {
+            if (MASK && lim < B) {
               if (16 * cc + 2 * i >= lim) p.x = 0.f;
               if (16 * cc + 2 * i + 1 >= lim) p.y = 0.f;
             }
@@ -481,7 +492,10 @@ struct Chain {
         if (!t.final_) {
           // the contraction runs over the rows of the weights: normalised in fp32, rounded once, to shared memory
           const float2 n2 = both(mul * kWeightScale);
-          uint8_t* base = smem + x.x1 * kSlot + srow * 128;
+          // (128 columns: the slot of the second half is free.  Every warp looks for itself, two releases in a row would share their word.)
+          if (B == 128) await(&sh->third[w][q & 1], (par_3 >> (q & 1)) & 1, 36);
+          uint8_t* lower = smem + (B == 128 ? min(x.x1, x.x2) : x.x1) * kSlot + srow * 128;
+          uint8_t* upper = smem + max(x.x1, x.x2) * kSlot + srow * 128;
           tmem_ld16(tS, c[0]);
 #pragma unroll
           for (int cc = 0; cc < NC; ++cc) {
@@ -494,7 +508,8 @@ struct Chain {
               const float2 v = fmul2(make_float2(cur[2 * i], cur[2 * i + 1]), n2);
               u[i] = pack2<T>(v.x, v.y);
             }
-            const int c0 = 2 * cc;
+            const int c0 = 2 * cc & 7;
+            uint8_t* base = cc < 4 ? lower : upper;
             *reinterpret_cast<uint4*>(base + ((c0 ^ (srow & 7)) << 4)) = make_uint4(u[0], u[1], u[2], u[3]);
             *reinterpret_cast<uint4*>(base + (((c0 + 1) ^ (srow & 7)) << 4)) = make_uint4(u[4], u[5], u[6], u[7]);
           }
@@ -502,7 +517,7 @@ struct Chain {
         }
       }
       collect();
-      const bool third = Slots::uses_third(t);
+      const bool third = Slots<B>::uses_third(t) || (B == 128 && !t.isR);
       if (warp == 0) {
         if (t.final_) await(&sh->third[w][q & 1], (par_3 >> (q & 1)) & 1, 36);
         if (ok && elect_one()) {
@@ -513,9 +528,12 @@ struct Chain {
             apply(d, a2);
             umma_commit(&sh->mma2[w]);
           } else {
-            apply_transposed(d, a1, a0, sm + kOffOnes);
+            // (128 columns of weights: the first 64 in the lower of the two slots)
+            if (B == 128) apply_transposed(d, min(a1, a2), max(a1, a2) - min(a1, a2), a0, sm + kOffOnes);
+            else apply_transposed(d, a1, kSlot, a0, sm + kOffOnes);
             umma_commit(&sh->mma2[w]);
             umma_commit(&sh->empty[x.x1]);
+            if (B == 128) umma_commit(&sh->empty[x.x2]);
           }
         }
         __syncwarp();
@@ -569,7 +587,7 @@ struct Chain {
   }
 };
 
-template <typename T, bool EXTRA>
+template <typename T, int B, int EXTRA>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm) monarch_chain(const __grid_constant__ Params P) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem<1024>(smem_raw);
@@ -603,7 +621,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) monarch_chain(const __gr
   tc_fence_after();
   const uint32_t tmem = sh->tmem;
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  using C = Chain<T, EXTRA>;
+  using C = Chain<T, B, EXTRA>;
   // registers: 384 threads at the launch's 80; 128 x 48 + 256 x 96 make use of all of them
   if (warp >= 8) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
@@ -630,9 +648,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) monarch_chain(const __gr
   }
 }
 
-template <typename T, bool EXTRA>
+template <typename T, int B, int EXTRA>
 inline cudaError_t launch_kernel(const Params& P, int grid, cudaStream_t st) {
-  auto kern = monarch_chain<T, EXTRA>;
+  auto kern = monarch_chain<T, B, EXTRA>;
   static bool prepared[64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -659,14 +677,17 @@ inline cudaError_t launch_kernel(const Params& P, int grid, cudaStream_t st) {
 }  // namespace tp3
 
 namespace tp {
-template <typename T>
+template <typename T, int B>
 cudaError_t launch_chain(const Params& P, int grid, cudaStream_t st) {
-  if (P.H != 0 || P.lse != nullptr || P.n_valid != 0) return tp3::launch_kernel<T, true>(P, grid, st);
-  return tp3::launch_kernel<T, false>(P, grid, st);
+  if (P.n_valid != 0) return tp3::launch_kernel<T, B, 2>(P, grid, st);
+  if (P.H != 0 || P.lse != nullptr) return tp3::launch_kernel<T, B, 1>(P, grid, st);
+  return tp3::launch_kernel<T, B, 0>(P, grid, st);
 }
 #ifdef MA_TU_TENSOR_CHAIN
-template cudaError_t launch_chain<__half>(const Params&, int, cudaStream_t);
-template cudaError_t launch_chain<__nv_bfloat16>(const Params&, int, cudaStream_t);
+template cudaError_t launch_chain<__half, 64>(const Params&, int, cudaStream_t);
+template cudaError_t launch_chain<__half, 128>(const Params&, int, cudaStream_t);
+template cudaError_t launch_chain<__nv_bfloat16, 64>(const Params&, int, cudaStream_t);
+template cudaError_t launch_chain<__nv_bfloat16, 128>(const Params&, int, cudaStream_t);
 #endif
 }  // namespace tp
 }  // namespace ma

@@ -191,14 +191,20 @@ cudaError_t launch_decoupled(const Params& P, int grid, cudaStream_t st);
 template <typename T, int B>
 cudaError_t launch_tmem(const Params& P, int grid, cudaStream_t st);
 //   launch_chain:     tensor_chain.cuh, SB == B == 64
-template <typename T>
+template <typename T, int B>
 cudaError_t launch_chain(const Params& P, int grid, cudaStream_t st);
 // Whether MA_PATH_TENSOR runs the kernel of tensor_chain.cuh and not that of tensor_decoupled.cuh (by size alone: either layout
 // gives the same bits; for one round both kernels do).  Measured over heads of 4096 in loops of tenths of a second, us (this one / that one):
 // two rounds: 16 heads 39.4 / 37.0, 24 43.7 / 44.4, 32 48.4 / 50.2 (on another GPU 49.8 / 49.3), 33 48.7 / 51.9, 36 49.8 / 55.0, 64 82 / 89; one round: 32
 // 30.8 / 30.9 (on the other 31.2 / 30.9), 33 30.9 / 32.6, 35 32.4 / 32.9, 38 33.1 / 34.9, 48 37.8 / 41.1, 64 51 / 53; masked or in the other layout, where
 // that one is a fifth slower: one round 32 34.4 / 35.3 and 34.4 / 37.7, two rounds 32 55.1 / 58.1, 48 66.2 / 78.6.
-inline bool chain_chosen(int BH, int N, int b) { return b == 64 && (long long)BH * N / kRows >= 1024; }      // tiles of a half-step
+// Blocks of 128 (bf16 T = 2, f16 T = 1; loops): 8 heads of 16384 55.3 / 54.9 and 32.3 / 32.9 (replayed graphs 59.9 / 57.5 and 37.1 / 35.3), 9 59.8 / 60.0 and
+// 35.4 / 35.6, 12 74.3 / 79.9 and 44.4 / 46.2, 16 95.0 / 99.5 and 58.6 / 59.5; other layout 8 59 / 62 and 35 / 37, 12 78 / 86 and 46 / 50; masked 6 57 / 54, 8
+// 66.8 / 66.4, 12 81 / 93.
+inline bool chain_chosen(int BH, int N, int b) {      // by tiles of a half-step
+  const long long tiles = (long long)BH * N / kRows;
+  return b == 64 ? tiles >= 1024 : b == 128 && tiles >= 1152;
+}
 
 // mode 0: kernel of tensor_decoupled.cuh or tensor_chain.cuh; mode 1: kernel of tensor_tmem.cuh (m = b in {64, 128},
 // plain calls only: no [batch][N][heads][d] layout, no row log-sum-exp, no padding mask).  *kernels: which it was.
@@ -334,9 +340,10 @@ inline int launch_t(const void* Q, const void* K, const void* V, void* Y, int BH
   // head groups: as many as keep a group's half-step long enough that a tile's dependencies are
   // long done when its turn comes (measured: C5, 1024 tiles of 128 x 128 per group and half-step,
   // same time and 118 MB instead of 217 MB of DRAM traffic; C4, 1024 tiles of two 64 x 64 blocks,
-  // 3 % slower, hence the higher bar for the faster small tiles)
+  // 3 % slower, hence the higher bar for the faster small tiles; monarch_chain has 1184 tiles in work or requested: 16 heads of
+  // 16384 take it 104 us in groups of 1024, 95 in one, 24 149 in one, 141 in two of 1536)
   const bool chained = mode == 0 && P.trace == nullptr && chain_chosen(BH, N, SB);
-  const int min_tiles = B == 128 ? 1024 : 2048;
+  const int min_tiles = B == 128 ? (chained ? 1536 : 1024) : 2048;
   P.head_groups = 1;
   while (BH % (2 * P.head_groups) == 0 && P.tiles_per_phase / (2 * P.head_groups) >= min_tiles) P.head_groups *= 2;
   P.scale = fabsf(scale);
@@ -357,8 +364,8 @@ inline int launch_t(const void* Q, const void* K, const void* V, void* Y, int BH
       const cudaError_t e = cudaMemsetAsync(ws, 0, kWsStatusBytes + counters_bytes(BH, T_steps), st);
       if (e != cudaSuccess) return e;
     }
-    if constexpr (SB == 64) {
-      if (chained) return launch_chain<T>(P, total < 2 * num_sms ? total : 2 * num_sms, st);      // taken by CTAs that run, whichever
+    if constexpr (SB == B) {
+      if (chained) return launch_chain<T, B>(P, total < 2 * num_sms ? total : 2 * num_sms, st);      // taken by CTAs that run, whichever
     }
     const int grid = total < num_sms ? total : num_sms;
     if constexpr (SB == B) {
