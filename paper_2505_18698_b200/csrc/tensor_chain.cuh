@@ -56,7 +56,8 @@ static_assert(kCtasPerSm * (kSmem + 1024) <= 228 * 1024, "two CTAs per SM");
 struct __align__(16) Shared {
   uint64_t full[2][2], third[2][2];                   // by group, tiles in turn: first two operands, third slot
   uint64_t empty[kSlots];
-  uint64_t mma1[2], first[2], mma2[2], o_free[2], out_free[2];
+  uint64_t mma1[2], first[2], mma2[2], out_free[2];
+  int through[2];                                     // tiles of a group that have left tensor memory
   int go[2];                                          // whether the group goes on: its first warp's word before every release
   int4 tile[2][2];                                    // {half-step, head, first block or position} of a tile, or {-1, ..}
   int4 out[2];                                        // {head or -1, first block or position, slot | Rows << 4 | last << 8, half-step}
@@ -122,6 +123,25 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Shared*
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 __device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 enum BarId { kRelease = 1, kCollect = 3, kStaged = 5 };
+// Tiles that a group is through with: its first warp says so once all warps have come by, the producer waits for it (bounded).
+__device__ __forceinline__ void say_through(Shared* sh, int w, uint32_t tiles) {
+  __threadfence_block();
+  *(volatile int*)&sh->through[w] = (int)tiles;
+}
+__device__ __forceinline__ bool wait_through(Shared* sh, int w, uint32_t tiles, const Params& P) {
+  const long long t0 = clock64();
+  while (*(volatile int*)&sh->through[w] < (int)tiles) {
+    if (sh->abort_flag) return false;
+    if (clock64() - t0 > P.wait_cycles) {
+      report_timeout(P.report, 12);
+      sh->abort_flag = 1;
+      return false;
+    }
+    __nanosleep(100);
+  }
+  __threadfence_block();
+  return true;
+}
 
 // Tile p, h, idx0 as its roles see it.
 __device__ __forceinline__ Tile tile_of(const Params& P, int p, int h, int idx0) {
@@ -164,11 +184,10 @@ struct Chain {
     for (uint32_t q = 0;; ++q) {
       const int g = P.g_begin + claim;
       uint64_t *bar = &sh->full[w][q & 1], *bar3 = &sh->third[w][q & 1];
-      // The end: once all threads are through the last two tiles, the word and the barrier are free.  One after the other: a parity
-      // alone does not tell tile q - 1 from q - 3 (which is through, since q - 1 has got its first slot).
+      // The end: once all threads are through all tiles, the word and the barrier are free.  (A count: by the parity of a barrier a
+      // producer that comes late cannot tell the last tile from the one before the last but one.)
       if (g >= P.g_end) {
-        if (q > 1 && !wait_bar(&sh->o_free[w], q & 1, sh, P, 12)) return;
-        if (q > 0 && !wait_bar(&sh->o_free[w], (q - 1) & 1, sh, P, 12)) return;
+        if (!wait_through(sh, w, q, P)) return;
         sh->tile[w][q & 1] = make_int4(-1, 0, 0, 0);
         mbar_arrive(bar);
         return;
@@ -354,7 +373,7 @@ struct Chain {
         if (q > 0) {                           // every row of the tile before has left tensor memory
           bar_sync(kCollect + w, 128);
           tc_fence_after();
-          if (t_row == 0) mbar_arrive(&sh->o_free[w]);
+          if (t_row == 0) say_through(sh, w, q);
         }
         await(&sh->full[w][q & 1], (q >> 1) & 1, 30);
         const int4 it = sh->tile[w][q & 1];
@@ -605,7 +624,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) monarch_chain(const __gr
       mbar_init(&sh->first[w], 1);
       mbar_init(&sh->mma2[w], 1);
       mbar_init(&sh->out_free[w], 1);
-      mbar_init(&sh->o_free[w], 1);
+      sh->through[w] = 0;
     }
     sh->abort_flag = 0;
     fence_barrier_init();
