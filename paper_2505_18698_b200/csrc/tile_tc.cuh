@@ -4,11 +4,13 @@
 // rounds where there are tiles enough to fill the GPU (the rule is in api.cu).
 //
 // What bounds a tile.  Its chain load -> score MMA -> softmax -> apply MMA -> epilogue -> store is mostly
-// latency (a launch with less than a tile a compute group takes 10 us, 3.5 turns of tiles 31), while its pipe time is
+// latency (a launch with less than a tile a compute group takes 9 us), while its pipe time is
 // half a microsecond (128 x 128 exponentials at 16 per clock and SM).  So as many chains as possible have to be in flight with as few hand-overs as
-// possible: two CTAs share an SM, each with two compute groups of four warps (thread = score row,
-// one tile per group: softmax and epilogue) over one ring of six 16 KB operand slots, and four service
-// threads (producer, MMA issuer, one store thread per group) that serve only that CTA.
+// possible: two CTAs share an SM, each with two compute groups of four warps (thread = score row, one tile per group: softmax and
+// epilogue).  A group has three 16 KB slots, a producer thread and a store warp of its own; its first warp issues its MMAs, and
+// hand-overs inside a group are hardware barriers.  The producers ask for inputs (Q, K, V) before the half-step before has ended.
+// (With a ring of slots and a polling MMA thread shared by the groups, and loads that all waited: 8 heads of 7600, T = 2 39.5 us, now
+// 35.3; 48 of 47 x 64 83.4 / 75.6; 16 of 94 x 128, T = 1 54.2 / 56.4, the only one that lost: a whole tile was requested ahead there.)
 //
 // One tile shape for everything: 128 score rows = 128 / B blocks of B rows (B = b or m rounded up
 // to 32, 64 or 128; rows past the block are zero-filled by TMA), one M = N = 128 score MMA, of which a
@@ -18,10 +20,6 @@
 // over the rows of the weights, passes them through shared memory.
 //   TMEM columns of a group: scores 0-127; weights (16-bit pairs) 0-63; apply accumulator 64-127; in
 //   the non-final L half-step sixteen copies of c_R in 0-15.
-//   Slots of a tile: the first operand (alpha_R or Q(.,j)), the second (K or alpha_L).  A third operand
-//   (V, y) lands over the first once the score MMA has read it, under the softmax; the weights of the
-//   non-final L half-step go over alpha_L (at B = 128 their second half takes a slot of its own); rows
-//   are staged for their store over an operand that is dead by then.
 //
 // Arithmetic and states are f16 (bf16 inputs are converted in shared memory: the rounding of alpha_L
 // is the dominant error of a 16-bit pipeline and f16 has three more bits).  alpha_R is stored divided
@@ -29,7 +27,7 @@
 // rounded (the quotient is invariant), so that a column of small weights keeps its bits however small
 // c_R is; c_R sums the weights as rounded.
 //
-// Measured (B200, us per call, against the warp-MMA tiles that served these shapes): 8 heads of N =
+// Measured when they came (B200, us per call, against the warp-MMA tiles that served these shapes): 8 heads of N =
 // 7600 in blocks of 128, d = 48, two rounds 43.9 / 61.9; 32 heads of N = 8192 as 128 blocks of 64, one
 // round (bf16) 64 / 95, two rounds (f16) 119 / 214; 64 heads of 60 blocks of 64, two rounds 102 / 150.
 #pragma once
@@ -48,8 +46,8 @@ constexpr int kCtasPerSm = 2;
 constexpr int kSlot = kTileBytes;            // 16 KB
 constexpr int kSlots = 6;
 constexpr int kOffOnes = kSlots * kSlot;     // 2 KB of ones
-constexpr int kOffVec = kOffOnes + 2048;     // c_L of a tile's rows: three tiles of 128 floats
-constexpr int kOffCol = kOffVec + 3 * 512;   // per group, two sets in turn: column maxima of the non-final L weights
+constexpr int kOffVec = kOffOnes + 2048;     // c_L of a tile's rows: two tiles of 128 floats a group
+constexpr int kOffCol = kOffVec + 4 * 512;   // per group, two sets in turn: column maxima of the non-final L weights
 constexpr int kOffBar = kOffCol + 4 * 512;
 constexpr int kSmem = kOffBar + 384 + 1024;  // + alignment slack
 static_assert(kCtasPerSm * (kSmem + 1024) <= 228 * 1024, "two CTAs per SM");
@@ -75,14 +73,69 @@ struct Params {
 };
 
 struct __align__(16) Shared {
-  uint64_t load[3], empty[kSlots];                     // by tile, by slot
-  uint64_t mma1[2], weights[2], first[2], mma2[2];     // by group from here on
-  uint64_t third[2], prep[2], oread[2], o_free[2], staged[2], out_free[2], cols[2];
+  uint64_t full[2][2], third[2][2];                    // by group, tiles in turn: first two operands, third slot
+  uint64_t empty[kSlots];
+  uint64_t mma1[2], first[2], mma2[2], out_free[2];      // by group from here on
+  int4 tile[2][2];           // {head or -1, first block or position, keys that count}
+  int4 out[2];               // {head or -1, first block or position, slot, is y}
+  int through[2];            // tiles of a group that have left tensor memory
+  int go[2];                 // whether the group goes on: its first warp's word before every release
+  int taken;                 // tiles of the CTA that its groups have taken
   uint32_t tmem;
   volatile int abort_flag;
-  int4 tile[3], out[2];      // {head or -1, first block or position, slot, keys that count}, {head or -1, first .., slot, is y}
 };
 static_assert(sizeof(Shared) <= 384, "barrier block");
+
+// A group's slots as the operands of its current tile; next(): in the order in which the tile gives them up.
+//   R:            first  alpha_R (Q), free after the score MMA; second K, alpha_L staged over it; third, last round, V and y over it
+//   L, not last:  first  Q(.,j), alpha_R staged over it; second alpha_L, then weights, free after the apply MMA (128 columns: and third)
+//   L, last:      first  Q(.,j), second alpha_L, both free after the score MMA; third y, Y staged over it
+template <int B, bool R>
+struct Slots {
+  int x0, x1, x2;
+  __device__ __forceinline__ explicit Slots(int w) : x0(3 * w), x1(3 * w + 1), x2(3 * w + 2) {}
+  __device__ __forceinline__ void next(bool last) {
+    const int a = x0, b = x1, c = x2;
+    if (last) return;
+    if (B == 128 && !R) {
+      x0 = b;
+      x1 = c;
+      x2 = a;
+      return;
+    }
+    x0 = c;
+    x1 = R ? a : b;
+    x2 = R ? b : a;
+  }
+};
+
+// Barriers in hardware, by group: the first warp lets the others go on, it waits for them, the store warp waits for staged
+// rows.
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+enum BarId { kRelease = 1, kCollect = 3, kStaged = 5 };
+// Tiles that a group is through with: its first warp says so once all warps have come by, the producer waits for it (bounded).
+__device__ __forceinline__ void say_through(Shared* sh, int w, uint32_t tiles) {
+  __threadfence_block();
+  *(volatile int*)&sh->through[w] = (int)tiles;
+}
+__device__ __forceinline__ bool wait_through(Shared* sh, int w, uint32_t tiles, const Params& P) {
+  const long long t0 = clock64();
+  while (*(volatile int*)&sh->through[w] < (int)tiles) {
+    if (sh->abort_flag) return false;
+    if (clock64() - t0 > P.wait_cycles) {
+      report_timeout(P.status, 12);
+      sh->abort_flag = 1;
+      return false;
+    }
+    __nanosleep(100);
+  }
+  __threadfence_block();
+  return true;
+}
+
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ------------------------------------------------------------------------------------ PTX helpers
 __device__ __forceinline__ void load_5d(void* dst, const CUtensorMap* tm, uint64_t* bar, int r, int blk, int h0, int h1) {
@@ -159,8 +212,9 @@ __device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64
       : "memory");
 }
 
-// Bounded wait: after a timeout (status word and abort flag set) every wait of the CTA returns at
-// once, the tile ends with garbage and the CTA leaves at the tile's last barrier.
+// Bounded wait: after a timeout (status word and abort flag set) every wait of the CTA returns at once (HEED: but for those that
+// come to an end by themselves), and its groups stop.
+template <bool HEED = true>
 __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Shared* sh, const Params& P, int where) {
   const uint32_t addr = smem_u32(bar);
   uint32_t done = 0;
@@ -174,7 +228,7 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Shared*
         : "r"(addr), "r"(parity)
         : "memory");
     if (done) return true;
-    if (sh->abort_flag) return false;
+    if (HEED && sh->abort_flag) return false;
     if (n == 0) {
       t0 = clock64();
     } else if (clock64() - t0 > P.wait_cycles) {
@@ -188,18 +242,6 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Shared*
 __device__ __forceinline__ void arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ bool test_bar(uint64_t* bar, uint32_t parity) {
-  uint32_t done;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(done)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return done != 0;
-}
-
 // ------------------------------------------------------------------------------------ kernel
 // MODE 0: R tiles, 1: L tiles of blocks (rows of blocks) padded to B.  FULL: nothing is padded or masked.
 template <typename TIn, int B, bool FULL, int MODE>
@@ -211,203 +253,159 @@ struct Kernel {
   static constexpr int FT = Fmt<TA>::code;
   static constexpr uint32_t kIdScore = instr_desc(128, 128, FT, 0, 0), kIdApply = instr_desc(128, 64, FT, 0, 1);
 
-  // Slots of a tile: two, and a third for the weights of a non-final L tile of 128 columns.
-  static __device__ __forceinline__ int slots(const Params& P) { return B == 128 && !R && !P.last ? 3 : 2; }
-  static __device__ __forceinline__ int wrap(int s) { return s >= kSlots ? s - kSlots : s; }
   static __device__ __forceinline__ bool prepares(const Params& P) { return kConvert || (!FULL && P.seq_len != nullptr); }
 
-  // ================================================================ producer (one thread)
-  // Requests the first two operands of the CTA's tiles.
-  static __device__ __forceinline__ void produce(const Params& P, uint8_t* smem, Shared* sh) {
-    int q = 0, i3 = 0, ends = 0;
-    uint32_t par_e = (1u << kSlots) - 1;      // per slot: parity of its next "empty"
-    const int ns = slots(P);
-    for (int g = blockIdx.x;; g += gridDim.x) {
-      const bool end = g >= P.tiles;
-      const int h = end ? -1 : g / P.per_head, idx0 = end ? 0 : (g - h * P.per_head) * kBlocks;
-      int n_valid = P.n_valid;
-      if (!FULL && !end && P.seq_len != nullptr) {
-        n_valid = min(max(P.seq_len[h / P.heads], 1), P.N);
-        if (R && idx0 * P.b >= n_valid) continue;      // key blocks that are absent from a shorter sequence
-      }
-      for (int s = 0; s < ns; ++s) {
-        const int e = wrap(q + s);
-        if (!wait_bar(&sh->empty[e], (par_e >> e) & 1, sh, P, 11)) return;
-        par_e ^= 1u << e;
-      }
-      uint64_t* bar = &sh->load[i3];
-      sh->tile[i3] = make_int4(h, idx0, q, n_valid);
-      if (end) {                              // once for each group
-        arrive(bar);
-        if (++ends == 2) return;
-      } else {
-        const int h0 = P.H ? h % P.H : h, h1 = P.H ? h / P.H : 0;
-        uint8_t *s0 = smem + q * kSlot, *s1 = smem + wrap(q + 1) * kSlot;
-        if (R) {
-          mbar_expect_tx(bar, 2 * kSlot);
-          if (P.first) load_5d(s0, &P.rQ, bar, 0, idx0, h0, h1);
-          else load_5d(s0, &P.rAR, bar, 0, idx0, h, 0);
-          load_5d(s1, &P.rK, bar, 0, idx0, h0, h1);
-        } else {
-          float* sC = reinterpret_cast<float*>(smem + kOffVec) + i3 * 128;
-          const int nj = min(kBlocks, P.b - idx0);
-          mbar_expect_tx(bar, 2 * kSlot + nj * P.mp * 4);
-          load_5d(s0, &P.lQ, bar, 0, idx0, h0, h1);
-          load_5d(s1, &P.lAL, bar, 0, idx0, h, 0);
-          const float* c = P.cL + ((size_t)h * P.b + idx0) * P.mp;
-          for (int jj = 0; jj < nj; ++jj) bulk_1d(sC + jj * B, c + (size_t)jj * P.mp, P.mp * 4, bar);
-        }
-      }
-      q = wrap(q + ns);
-      i3 = i3 == 2 ? 0 : i3 + 1;
+  // ================================================================ producer of group w (one thread)
+  // The groups of a CTA take its tiles in turn, each when it has slots for one.  Q, K, V and the lengths are asked for before the end of the
+  // half-step before (the first launch of a call lets the next ones start only once it has waited for whatever wrote them).
+  static __device__ __forceinline__ void produce(const Params& P, uint8_t* smem, Shared* sh, int w) {
+    const bool last = P.last != 0;
+    bool waited = R && P.first;
+    if (waited) {
+      grid_wait();
+      grid_launch_dependents();
     }
-  }
-
-  // ================================================================ issuer (one thread): all MMAs
-  // Polls: what is ready first, the scores of the next tile or the apply MMA of an earlier one, is
-  // issued first.
-  static __device__ __forceinline__ void issue(const Params& P, uint8_t* smem, Shared* sh, uint32_t tmem) {
-    const bool prep = prepares(P), last = P.last != 0;
-    auto apply = [&](uint32_t d, const uint8_t* x, uint64_t* done) {     // weights (TMEM) times the rows of a slot
-      const uint64_t dX = smem_desc(smem_u32(x), 16, 1024);
-      umma_ts<false>(d + 64, d, dX, kIdApply);
-#pragma unroll
-      for (int ks = 1; ks < 8; ++ks) umma_ts<true>(d + 64, d + 8 * ks, dX + 128 * ks, kIdApply);
-      umma_commit(done);
+    Slots<B, R> x(w);
+    uint32_t busy = 0, par = 0;               // by slot: a use is to be waited for; parity of that wait
+    auto take = [&](int s) {
+      const uint32_t bit = 1u << s;
+      if ((busy & bit) && !wait_bar(&sh->empty[s], (par & bit) != 0, sh, P, 11)) return false;
+      if (busy & bit) par ^= bit;
+      busy |= bit;
+      return true;
     };
-    int n1 = 0, n2 = 0, i1 = 0, i2 = 0;       // tiles and load barriers of the two MMAs
-    uint32_t par1 = 0, par_t = 0, par_r = 0;                 // (bit w: group w)
-    bool second = false, end = false, idle = false;
-    long long t0 = 0;
-    while (!end || n2 < n1) {
-      bool did = false;
-      const int w1 = n1 & 1, w2 = n2 & 1;
-      const uint32_t d1 = tmem + 128 * w1, d2 = tmem + 128 * w2;
-      if (n2 < n1) {
-        if (!second && test_bar(&sh->weights[w2], (n2 >> 1) & 1)) {
-          if (R || !last || prep || test_bar(&sh->third[w2], (par_t >> w2) & 1)) {
-            const int q2 = sh->tile[i2].z;
-            uint8_t *s0 = smem + q2 * kSlot, *s1 = smem + wrap(q2 + 1) * kSlot;
-            tc_fence_after();
-            if (R) {
-              apply(d2, s1, last ? &sh->first[w2] : &sh->mma2[w2]);
-              second = last;
-            } else if (last) {
-              par_t ^= 1u << w2;
-              apply(d2, s0, &sh->mma2[w2]);
-              umma_commit(&sh->empty[q2]);
-            } else {
-              const uint64_t dQ = smem_desc(smem_u32(s0), 16, 1024), dO = smem_desc(smem_u32(smem + kOffOnes), 16, 1024);
-              if constexpr (B == 128) {
-                const int e1 = wrap(q2 + 1), e2 = wrap(q2 + 2);
-                const uint32_t lo = smem_u32(smem) + min(e1, e2) * kSlot, hi = smem_u32(smem) + max(e1, e2) * kSlot;
-                const uint64_t dP = smem_desc(lo, hi - lo, 1024);
-                constexpr uint32_t id = instr_desc(128, 64, FT, 1, 1), id1 = instr_desc(128, 16, FT, 1, 0);
-                umma_c<false>(d2 + 64, dP, dQ, id);
-                umma_c<false>(d2, dP, dO, id1);
-#pragma unroll
-                for (int ks = 1; ks < 8; ++ks) {
-                  umma_c<true>(d2 + 64, dP + 128 * ks, dQ + 128 * ks, id);
-                  umma_c<true>(d2, dP + 128 * ks, dO, id1);
-                }
-                umma_commit(&sh->empty[e2]);
-              } else {
-                // two groups of 64 rows; their accumulators take the lower and upper 16 lanes of
-                // every warp's part of tensor memory
-                const uint64_t dP = smem_desc(smem_u32(s1), 16, 1024);
-                constexpr uint32_t id = instr_desc(64, 64, FT, 1, 1), id1 = instr_desc(64, 16, FT, 1, 0);
-#pragma unroll
-                for (int g = 0; g < 2; ++g) {
-                  const uint32_t d = d2 + ((uint32_t)(16 * g) << 16);
-#pragma unroll
-                  for (int ks = 0; ks < 4; ++ks) {
-                    const uint64_t off = 512 * g + 128 * ks;
-                    if (ks == 0) {
-                      umma_c<false>(d + 64, dP + off, dQ + off, id);
-                      umma_c<false>(d, dP + off, dO, id1);
-                    } else {
-                      umma_c<true>(d + 64, dP + off, dQ + off, id);
-                      umma_c<true>(d, dP + off, dO, id1);
-                    }
-                  }
-                }
-              }
-              umma_commit(&sh->mma2[w2]);
-              umma_commit(&sh->empty[wrap(q2 + 1)]);
-            }
-            if (!second) {
-              i2 = i2 == 2 ? 0 : i2 + 1;
-              ++n2;
-            }
-            did = true;
-          }
-        } else if (second && test_bar(&sh->oread[w2], (par_r >> w2) & 1) &&
-                   (prep || test_bar(&sh->third[w2], (par_t >> w2) & 1))) {
-          par_r ^= 1u << w2;              // alpha_L is out: y = R V through the same columns
-          par_t ^= 1u << w2;
-          tc_fence_after();
-          apply(d2, smem + sh->tile[i2].z * kSlot, &sh->mma2[w2]);
-          second = false;
-          i2 = i2 == 2 ? 0 : i2 + 1;
-          ++n2;
-          did = true;
-        }
-      }
-      if (!end && n1 < n2 + 2 && test_bar(&sh->load[i1], par1) && (n1 < 2 || test_bar(&sh->o_free[w1], ((n1 >> 1) & 1) ^ 1))) {
-        const int4 t = sh->tile[i1];
-        if (t.x < 0) {
-          end = true;
-        } else if (!prep || test_bar(&sh->prep[w1], (n1 >> 1) & 1)) {
-          const int q1 = t.z;
-          tc_fence_after();
-          const uint64_t da = smem_desc(smem_u32(smem + q1 * kSlot), 16, 1024);
-          const uint64_t db = smem_desc(smem_u32(smem + wrap(q1 + 1) * kSlot), 16, 1024);
-          umma_c<false>(d1, da, db, kIdScore);
-          umma_c<true>(d1, da + 2, db + 2, kIdScore);
-          umma_c<true>(d1, da + 4, db + 4, kIdScore);
-          umma_c<true>(d1, da + 6, db + 6, kIdScore);
-          umma_commit(&sh->mma1[w1]);
-          if (R && !last) umma_commit(&sh->empty[q1]);
-          if (++i1 == 3) {
-            i1 = 0;
-            par1 ^= 1;
-          }
-          ++n1;
-          did = true;
-        }
-      }
-      if (did) {
-        idle = false;
-      } else if (!idle) {
-        idle = true;
-        t0 = clock64();
-      } else if (sh->abort_flag) {
-        return;
-      } else if (clock64() - t0 > P.wait_cycles) {
-        report_timeout(P.status, 20);
-        sh->abort_flag = 1;
+    for (uint32_t q = 0;; ++q) {
+      uint64_t *bar = &sh->full[w][q & 1], *bar3 = &sh->third[w][q & 1];
+      int h, idx0, n_valid = P.n_valid;
+      bool end;
+      do {
+        const int g = blockIdx.x + atomicAdd(&sh->taken, 1) * gridDim.x;
+        end = g >= P.tiles;
+        h = end ? -1 : g / P.per_head;
+        idx0 = end ? 0 : (g - h * P.per_head) * kBlocks;
+        if (!FULL && !end && P.seq_len != nullptr) n_valid = min(max(P.seq_len[h / P.heads], 1), P.N);
+      } while (!FULL && R && !end && P.seq_len != nullptr && idx0 * P.b >= n_valid);      // key blocks that a shorter sequence does not have
+      // The end: once all threads are through all tiles, the word and the barrier are free.  (A count: by the parity of a barrier a
+      // producer that comes late cannot tell the last tile from the one before the last but one.)
+      if (end) {
+        if (!wait_through(sh, w, q, P)) return;
+        sh->tile[w][q & 1] = make_int4(-1, 0, 0, 0);
+        arrive(bar);
         return;
       }
+      if (!take(x.x0) || !take(x.x1)) return;
+      sh->tile[w][q & 1] = make_int4(h, idx0, n_valid, 0);
+      const int h0 = P.H ? h % P.H : h, h1 = P.H ? h / P.H : 0;
+      uint8_t *s0 = smem + x.x0 * kSlot, *s1 = smem + x.x1 * kSlot, *s2 = smem + x.x2 * kSlot;
+      if (R) {
+        const bool v_first = last && !waited;      // (its slot is free then)
+        auto load_v = [&]() {
+          if (!take(x.x2)) return false;
+          mbar_expect_tx(bar3, kSlot);
+          load_5d(s2, &P.rV, bar3, 0, idx0, h0, h1);
+          return true;
+        };
+        mbar_expect_tx(bar, 2 * kSlot);
+        load_5d(s1, &P.rK, bar, 0, idx0, h0, h1);
+        if (v_first && !load_v()) return;
+        if (!waited) grid_wait();
+        if (P.first) load_5d(s0, &P.rQ, bar, 0, idx0, h0, h1);
+        else load_5d(s0, &P.rAR, bar, 0, idx0, h, 0);
+        if (last && !v_first && !load_v()) return;
+      } else {
+        float* sC = reinterpret_cast<float*>(smem + kOffVec) + (2 * w + (q & 1)) * 128;
+        const int nj = min(kBlocks, P.b - idx0);
+        mbar_expect_tx(bar, 2 * kSlot + nj * P.mp * 4);
+        load_5d(s0, &P.lQ, bar, 0, idx0, h0, h1);
+        if (!waited) grid_wait();
+        load_5d(s1, &P.lAL, bar, 0, idx0, h, 0);
+        const float* c = P.cL + ((size_t)h * P.b + idx0) * P.mp;
+        for (int jj = 0; jj < nj; ++jj) bulk_1d(sC + jj * B, c + (size_t)jj * P.mp, P.mp * 4, bar);
+        if (last || B == 128) {
+          if (!take(x.x2)) return;
+          if (last) {
+            mbar_expect_tx(bar3, kSlot);
+            load_5d(s2, &P.lY, bar3, 0, idx0, h, 0);
+          } else {
+            arrive(bar3);                     // for weights
+          }
+        }
+      }
+      waited = true;
+      x.next(last);
     }
   }
 
-  // ================================================================ store thread of group w
+  // ================================================================ store warp of group w (its first lane)
   // Stores what the group has staged; sh->out[w] says what and where.
   static __device__ __forceinline__ void store(const Params& P, uint8_t* smem, Shared* sh, int w) {
-    for (uint32_t par = 0;; par ^= 1) {
-      if (!wait_bar(&sh->staged[w], par, sh, P, 40)) break;
+    const bool lane0 = (threadIdx.x & 31) == 0;
+    for (;;) {
+      bar_sync(kStaged + w, 160);
       const int4 o = sh->out[w];          // head, first block or position, slot, y?
-      arrive(&sh->out_free[w]);
+      __syncwarp();
+      if (lane0) arrive(&sh->out_free[w]);
       if (o.x < 0) break;
-      const uint8_t* s = smem + o.z * kSlot;
-      if (R) store_5d(o.w ? &P.rY : &P.rAL, s, o.y, o.x, 0);
-      else if (!P.last) store_5d(&P.lAR, s, o.y, o.x, 0);
-      else store_5d(&P.lOut, s, o.y, P.H ? o.x % P.H : o.x, P.H ? o.x / P.H : 0);
-      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-      asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-      arrive(&sh->empty[o.z]);
+      if (lane0) {
+        const uint8_t* s = smem + o.z * kSlot;
+        if (R) store_5d(o.w ? &P.rY : &P.rAL, s, o.y, o.x, 0);
+        else if (!P.last) store_5d(&P.lAR, s, o.y, o.x, 0);
+        else store_5d(&P.lOut, s, o.y, P.H ? o.x % P.H : o.x, P.H ? o.x / P.H : 0);
+        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        arrive(&sh->empty[o.z]);
+      }
+      __syncwarp();
     }
-    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    if (lane0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+  }
+
+  // ================================================================ MMAs (one thread of the group's first warp)
+  static __device__ __forceinline__ void scores(uint32_t d, const uint8_t* s0, const uint8_t* s1) {
+    const uint64_t da = smem_desc(smem_u32(s0), 16, 1024), db = smem_desc(smem_u32(s1), 16, 1024);
+    umma_c<false>(d, da, db, kIdScore);
+    umma_c<true>(d, da + 2, db + 2, kIdScore);
+    umma_c<true>(d, da + 4, db + 4, kIdScore);
+    umma_c<true>(d, da + 6, db + 6, kIdScore);
+  }
+  static __device__ __forceinline__ void apply(uint32_t d, const uint8_t* x) {     // weights (TMEM) times the rows of a slot
+    const uint64_t dX = smem_desc(smem_u32(x), 16, 1024);
+    umma_ts<false>(d + 64, d, dX, kIdApply);
+#pragma unroll
+    for (int ks = 1; ks < 8; ++ks) umma_ts<true>(d + 64, d + 8 * ks, dX + 128 * ks, kIdApply);
+  }
+  // Rows k of sum_l P[l, k] Q(l, .), and the sums of the weights against ones.  chunk: from the first 64 columns of P to the others.
+  static __device__ __forceinline__ void apply_transposed(uint32_t d, const uint8_t* p, uint32_t chunk, const uint8_t* q, const uint8_t* ones) {
+    const uint64_t dP = smem_desc(smem_u32(p), chunk, 1024), dQ = smem_desc(smem_u32(q), 16, 1024), dO = smem_desc(smem_u32(ones), 16, 1024);
+    if constexpr (B == 128) {
+      constexpr uint32_t id = instr_desc(128, 64, FT, 1, 1), id1 = instr_desc(128, 16, FT, 1, 0);
+      umma_c<false>(d + 64, dP, dQ, id);
+      umma_c<false>(d, dP, dO, id1);
+#pragma unroll
+      for (int ks = 1; ks < 8; ++ks) {
+        umma_c<true>(d + 64, dP + 128 * ks, dQ + 128 * ks, id);
+        umma_c<true>(d, dP + 128 * ks, dO, id1);
+      }
+    } else {
+      // two groups of 64 rows; their accumulators take the lower and upper 16 lanes of
+      // every warp's part of tensor memory
+      constexpr uint32_t id = instr_desc(64, 64, FT, 1, 1), id1 = instr_desc(64, 16, FT, 1, 0);
+#pragma unroll
+      for (int g = 0; g < 2; ++g) {
+        const uint32_t dg = d + ((uint32_t)(16 * g) << 16);
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) {
+          const uint64_t off = 512 * g + 128 * ks;
+          if (ks == 0) {
+            umma_c<false>(dg + 64, dP + off, dQ + off, id);
+            umma_c<false>(dg, dP + off, dO, id1);
+          } else {
+            umma_c<true>(dg + 64, dP + off, dQ + off, id);
+            umma_c<true>(dg, dP + off, dO, id1);
+          }
+        }
+      }
+    }
   }
 
   // ================================================================ compute warps (thread = score row)
@@ -624,60 +622,93 @@ struct Kernel {
 
   static __device__ __forceinline__ void compute(const Params& P, uint8_t* smem, Shared* sh, uint32_t tmem, int w) {
     const int row = threadIdx.x & 127, warp = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
-    const uint32_t t_row = tmem + 128 * w + ((uint32_t)(warp * 32) << 16);     // this warp's TMEM lanes
+    const uint32_t d = tmem + 128 * w, t_row = d + ((uint32_t)(warp * 32) << 16);     // the group's columns, this warp's lanes
     const bool prep = prepares(P), last = P.last != 0;
-    int i3 = w;
-    // Parities: load (round of three tiles), one phase per tile of the group, and the barriers that
-    // only some tiles use.
-    uint32_t par_l = 0, par = 0, par_t = 0, par_1 = 0, par_o = 1;
-#define MA_WAIT(BAR, PAR, WHERE) \
-  if (!__all_sync(0xffffffffu, wait_bar(&(BAR), PAR, sh, P, WHERE))) return
-    // Staged rows (or the end) to the store thread, once it has taken the word of the one before.
-    auto hand_over = [&](int h, int idx0, int slot, int is_y) {
-      const bool ok = wait_bar(&sh->out_free[w], par_o, sh, P, 38);
-      par_o ^= 1;
-      if (row == 0) sh->out[w] = make_int4(h, idx0, slot, is_y);
-      arrive(&sh->staged[w]);
-      return ok;
+    Slots<B, R> x(w);
+    uint32_t par_o = 1;
+    bool ok = true;                            // (the first warp's decides) no wait has run out
+    // The first warp alone looks at mbarriers and lets the others go on once it has seen one: four warps that try and try again take
+    // issue slots from those at work.  A wait that ran out reaches the others with the same release.
+    auto await = [&](uint64_t* bar, uint32_t parity, int where) { ok = __all_sync(0xffffffffu, wait_bar(bar, parity, sh, P, where)) && ok; };
+    auto release = [&](bool on) {              // of the group; false: no more tiles.  (A collect comes between any two: they share the word.)
+      if (row == 0) sh->go[w] = on;
+      tc_fence_before();
+      bar_sync(kRelease + w, 128);
+      tc_fence_after();
+      return *(volatile int*)&sh->go[w] != 0;
     };
-    for (;; par ^= 1) {
-      MA_WAIT(sh->load[i3], par_l, 30);
-      const int4 t = sh->tile[i3];               // head, first block or position, slot, keys that count
-      if (t.x < 0) {
-        hand_over(-1, 0, 0, 0);
-        return;
-      }
-      const float* sC = reinterpret_cast<const float*>(smem + kOffVec) + i3 * 128;
-      if (i3 == 0) {
-        i3 = 2;
+    auto collect = [&]() {                     // all warps have come by: the first one waits
+      tc_fence_before();
+      if (warp == 0) {
+        bar_sync(kCollect + w, 128);
+        tc_fence_after();
       } else {
-        i3 -= 1;
-        par_l ^= 1;
+        bar_arrive(kCollect + w, 128);
       }
-      const int h = t.x, idx0 = t.y, e0 = t.z, e1 = wrap(e0 + 1);
-      uint8_t *s0 = smem + e0 * kSlot, *s1 = smem + e1 * kSlot;
+    };
+    // An accumulator is done, and the store warp has taken the word of the rows before: nobody comes by at kStaged a second time
+    // before the store warp has.
+    auto await_rows = [&](uint64_t* bar, uint32_t parity, int where) {
+      if (warp == 0) {
+        await(bar, parity, where);
+        if (ok) await(&sh->out_free[w], par_o, 38);
+        if (ok) par_o ^= 1;
+      }
+      return release(ok);
+    };
+    auto hand_over = [&](int h, int idx0, int slot, int is_y) {
+      if (row == 0) sh->out[w] = make_int4(h, idx0, slot, is_y);
+      __syncwarp();
+      bar_arrive(kStaged + w, 160);
+    };
+    for (uint32_t q = 0;; ++q) {
+      const uint32_t par = q & 1, par2 = (q >> 1) & 1;
+      uint8_t *s0 = smem + x.x0 * kSlot, *s1 = smem + x.x1 * kSlot, *s2 = smem + x.x2 * kSlot;
       const int r_blk = row / B, r_pos = row % B;   // block of the tile, row in it
-      const int mv = FULL ? P.m : (t.w + P.b - 1) / P.b;                            // blocks that are present
+      auto score = [&]() {                     // first warp
+        if (elect_one()) {
+          scores(d, s0, s1);
+          umma_commit(&sh->mma1[w]);
+          if (R || last) umma_commit(&sh->empty[x.x0]);
+          if (!R && last) umma_commit(&sh->empty[x.x1]);
+        }
+        __syncwarp();
+        await(&sh->mma1[w], par, 31);
+        if (prep && last) await(&sh->third[w][par], par2, 36);
+      };
+      bool more = true;
+      if (warp == 0) {
+        if (q > 0) {                           // every row of the tile before has left tensor memory
+          bar_sync(kCollect + w, 128);
+          tc_fence_after();
+          if (row == 0) say_through(sh, w, q);
+        }
+        await(&sh->full[w][par], par2, 30);
+        more = ok && sh->tile[w][par].x >= 0;
+        if (more && !prep) {
+          score();
+          more = ok;
+        }
+      }
+      if (!release(more)) break;
+      const int4 t = sh->tile[w][par];         // head, first block or position, keys that count
+      const int h = t.x, idx0 = t.y;
+      const int mv = FULL ? P.m : (t.z + P.b - 1) / P.b;                            // blocks that are present
       if (prep) {
         prepare(P, s0, !R || P.first, idx0, mv, row);      // Q, but not alpha_R
         prepare(P, s1, R, idx0, mv, row);                   // K, but not alpha_L
-        arrive(&sh->prep[w]);
+        collect();
+        if (warp == 0) score();
+        if (!release(ok)) break;
       }
-      MA_WAIT(sh->mma1[w], par, 31);
-      tc_fence_after();
-      if (last && warp == 0 && elect_one()) {    // the third operand, over the first: the score MMA has read it
-        mbar_expect_tx(&sh->third[w], kSlot);
-        if (R) load_5d(s0, &P.rV, &sh->third[w], 0, idx0, P.H ? h % P.H : h, P.H ? h / P.H : 0);
-        else load_5d(s0, &P.lY, &sh->third[w], 0, idx0, h, 0);
-      }
-      __syncwarp();
+      const float* sC = reinterpret_cast<const float*>(smem + kOffVec) + (2 * w + par) * 128;
       if (FULL && P.discard) {     // the state rows the score MMA consumed are read exactly once: drop them from L2
         if (!R) discard_line(P.aL + ((size_t)(h * P.b + idx0) * P.m + row) * 128);
         else if (!P.first) discard_line(P.aR + ((size_t)(h * P.m + idx0) * P.b + row) * 128);
       }
       float mul;                                 // of the accumulator rows in the epilogue
       if constexpr (R) {
-        mul = r_softmax(P, h, idx0 + r_blk, t.w, t_row, r_blk, r_pos);
+        mul = r_softmax(P, h, idx0 + r_blk, t.z, t_row, r_blk, r_pos);
       } else {
         // ============================================================ L: softmax over the blocks
         const float f = P.scale * kLog2e;
@@ -689,13 +720,13 @@ struct Kernel {
         float mx;
         {
           // logits back over the scores, then weights (final: 16-bit, as the MMA's operand)
-          float x[2][16];
-          tmem_ld16(tS, x[0]);
+          float v[2][16];
+          tmem_ld16(tS, v[0]);
 #pragma unroll
           for (int cc = 0; cc < B / 16; ++cc) {
-            float* cur = x[cc & 1];
+            float* cur = v[cc & 1];
             tmem_ld_wait();
-            if (cc < B / 16 - 1) tmem_ld16(tS + 16 * (cc + 1), x[(cc + 1) & 1]);
+            if (cc < B / 16 - 1) tmem_ld16(tS + 16 * (cc + 1), v[(cc + 1) & 1]);
             l_logits<16>(cur, cv + 16 * cc, f);
             mask<16>(cur, 16 * cc, lim);
             fold_max<16>(cur, m4);
@@ -703,12 +734,12 @@ struct Kernel {
           }
           mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
           tmem_st_wait();
-          tmem_ld16(tS, x[0]);
+          tmem_ld16(tS, v[0]);
 #pragma unroll
           for (int cc = 0; cc < B / 16; ++cc) {
-            float* cur = x[cc & 1];
+            float* cur = v[cc & 1];
             tmem_ld_wait();
-            if (cc < B / 16 - 1) tmem_ld16(tS + 16 * (cc + 1), x[(cc + 1) & 1]);
+            if (cc < B / 16 - 1) tmem_ld16(tS + 16 * (cc + 1), v[(cc + 1) & 1]);
             l_weights<16>(cur, mx, a2);
             if (last) {
               uint32_t u[8];
@@ -742,27 +773,27 @@ struct Kernel {
           for (int i = 0; i < 4; ++i) onr[i] = __shfl_sync(0xffffffffu, on, 8 * i + (lane >> 2));
           // column k times 2^-(exponent of its largest weight)
           unsigned* sMax = reinterpret_cast<unsigned*>(smem + kOffCol) + 128 * (2 * w + par);
-          float x[32];
+          float v[32];
 #pragma unroll
           for (int cc = 0; cc < B / 32; ++cc) {
-            ld_frag32(tS + 32 * cc, x);
+            ld_frag32(tS + 32 * cc, v);
             tmem_ld_wait();
-            fold_columns(x, onr, sMax + B * r_blk + 32 * cc, lane);
+            fold_columns(v, onr, sMax + B * r_blk + 32 * cc, lane);
           }
-          arrive(&sh->cols[w]);
-          ld_frag32(tS, x);
-          MA_WAIT(sh->cols[w], par, 34);
+          ld_frag32(tS, v);
+          // (128 columns: the slot of the second half is free.  Every warp looks for itself, a release would share its word with the last.)
+          if (B == 128) await(&sh->third[w][par], par2, 36);
+          bar_sync(kRelease + w, 128);
           // (the set of the tile before: all warps are done with it, and none begins the next tile before all have come by)
           reinterpret_cast<unsigned*>(smem + kOffCol)[128 * (2 * w + (par ^ 1)) + row] = 0u;
-          const int e2 = wrap(e1 + 1);
-          uint8_t* p_lo = smem + (B == 128 ? min(e1, e2) : e1) * kSlot + row * 128;
-          uint8_t* p_hi = smem + (B == 128 ? max(e1, e2) : e1) * kSlot + row * 128;
+          uint8_t* p_lo = smem + (B == 128 ? min(x.x1, x.x2) : x.x1) * kSlot + row * 128;
+          uint8_t* p_hi = smem + (B == 128 ? max(x.x1, x.x2) : x.x1) * kSlot + row * 128;
           const int win = B == 32 ? 32 * (r_blk & 1) : 0;
 #pragma unroll
           for (int cc = 0; cc < B / 32; ++cc) {
-            if (cc > 0) ld_frag32(tS + 32 * cc, x);
+            if (cc > 0) ld_frag32(tS + 32 * cc, v);
             tmem_ld_wait();
-            emit_columns(x, onr, sMax + B * r_blk + 32 * cc, smem_u32(cc < 2 ? p_lo : p_hi), (win >> 3) + (4 * cc & 7), row, lane);
+            emit_columns(v, onr, sMax + B * r_blk + 32 * cc, smem_u32(cc < 2 ? p_lo : p_hi), (win >> 3) + (4 * cc & 7), row, lane);
           }
           if constexpr (B == 32) {               // zeros beside the window
             const int c0 = (32 - win) >> 3;
@@ -772,32 +803,53 @@ struct Kernel {
           fence_proxy_async();
         }
       }
-      if (last && prep) {
-        MA_WAIT(sh->third[w], par_t, 36);
-        par_t ^= 1;
-        prepare(P, s0, R, idx0, mv, row);                   // V, but not y
+      if (last && prep) prepare(P, s2, R, idx0, mv, row);   // V, but not y
+      collect();
+      if (warp == 0) {
+        if (!R && last && !prep) await(&sh->third[w][par], par2, 36);
+        if (ok && elect_one()) {
+          if (R) {
+            apply(d, s1);
+            umma_commit(last ? &sh->first[w] : &sh->mma2[w]);
+          } else if (last) {
+            apply(d, s2);
+            umma_commit(&sh->mma2[w]);
+          } else {
+            // (128 columns of weights: the first 64 in the lower of the two slots)
+            const uint8_t* lower = B == 128 ? smem + min(x.x1, x.x2) * kSlot : s1;
+            apply_transposed(d, lower, B == 128 ? (max(x.x1, x.x2) - min(x.x1, x.x2)) * kSlot : 16, s0, smem + kOffOnes);
+            umma_commit(&sh->mma2[w]);
+            umma_commit(&sh->empty[x.x1]);
+            if (B == 128) umma_commit(&sh->empty[x.x2]);
+          }
+        }
+        __syncwarp();
       }
-      tc_fence_before();
-      arrive(&sh->weights[w]);
       // ============================================================== epilogue
       float o[32];
       if (R && last) {                           // alpha_L, over K; then y, over V
-        MA_WAIT(sh->first[w], par_1, 32);
-        par_1 ^= 1;
-        tc_fence_after();
+        if (!await_rows(&sh->first[w], par, 32)) break;
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
           tmem_ld32(t_row + 64 + 32 * hf, o);
           tmem_ld_wait();
+          if (hf == 1) {
+            collect();
+            if (warp == 0) {
+              if (!prep) await(&sh->third[w][par], par2, 36);
+              if (ok && elect_one()) {
+                apply(d, s2);
+                umma_commit(&sh->mma2[w]);
+              }
+              __syncwarp();
+            }
+          }
           store_row32<TA>(s1, row, 32 * hf, o, mul);
         }
-        tc_fence_before();
-        arrive(&sh->oread[w]);
         fence_proxy_async();
-        if (!__all_sync(0xffffffffu, hand_over(h, idx0, e1, 0))) return;
+        hand_over(h, idx0, x.x1, 0);
       }
-      MA_WAIT(sh->mma2[w], par, 33);
-      tc_fence_after();
+      if (!await_rows(&sh->mma2[w], par, 33)) break;
       int out_row = row;
       if (!R && !last) {
         if constexpr (!R && B < 128) out_row = ((lane >> 4) << 6) + 16 * warp + (lane & 15);
@@ -806,16 +858,16 @@ struct Kernel {
         mul = cr > 1e-30f ? 1.f / cr : 0.f;
       }
       if (FULL && P.discard && !R && last) discard_line(P.y + ((size_t)(h * P.b + idx0) * P.m + row) * 128);
-      // rows go: alpha_L over K, y over V (first slot), alpha_R over Q (first), Y over alpha_L (second)
-      const bool to_first = R ? last : !last;
-      uint8_t* dst = to_first ? s0 : s1;
+      // rows go: alpha_L over K, y over V, alpha_R over Q, Y over y
+      const int slot = last ? x.x2 : (R ? x.x1 : x.x0);
+      uint8_t* dst = smem + slot * kSlot;
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf) {
         tmem_ld32(t_row + 64 + 32 * hf, o);
         tmem_ld_wait();
-        if (hf == 1) {                           // the next tile's scores may come
+        if (hf == 1) {                           // the next tile's scores may come (the first warp waits for it before them)
           tc_fence_before();
-          arrive(&sh->o_free[w]);
+          if (warp != 0) bar_arrive(kCollect + w, 128);
         }
         if (R && last && !(mul == mul)) {      // NaN weights, and c_L is: the final L tiles hold several positions
           zero_row(dst, row);
@@ -830,9 +882,13 @@ struct Kernel {
         }
       }
       fence_proxy_async();
-      if (!__all_sync(0xffffffffu, hand_over(h, idx0, to_first ? e0 : e1, R && last))) return;
+      hand_over(h, idx0, slot, R && last);
+      x.next(last);
     }
-#undef MA_WAIT
+    // (aborted or not: rows handed over before are on their way, and the store warp comes back for this word)
+    if (warp == 0) __all_sync(0xffffffffu, wait_bar<false>(&sh->out_free[w], par_o, sh, P, 38));
+    release(false);
+    hand_over(-1, 0, 0, 0);
   }
 };
 
@@ -842,23 +898,22 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) monarch_tiles(const __gr
   uint8_t* smem = align_smem<1024>(smem_raw);
   Shared* sh = reinterpret_cast<Shared*>(smem + kOffBar);
   const int tid = threadIdx.x, warp = tid >> 5;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const bool starts = MODE == 0 && P.first;      // the first launch of a call
+  if (!starts) grid_launch_dependents();
   if (tid == 0) {
-    for (int i = 0; i < 3; ++i) mbar_init(&sh->load[i], 1);
     for (int i = 0; i < kSlots; ++i) mbar_init(&sh->empty[i], 1);
     for (int w = 0; w < 2; ++w) {
+      for (int i = 0; i < 2; ++i) {
+        mbar_init(&sh->full[w][i], 1);
+        mbar_init(&sh->third[w][i], 1);
+      }
       mbar_init(&sh->mma1[w], 1);
       mbar_init(&sh->first[w], 1);
       mbar_init(&sh->mma2[w], 1);
-      mbar_init(&sh->third[w], 1);
+      sh->through[w] = 0;
       mbar_init(&sh->out_free[w], 1);
-      mbar_init(&sh->prep[w], 128);
-      mbar_init(&sh->weights[w], 128);
-      mbar_init(&sh->oread[w], 128);
-      mbar_init(&sh->o_free[w], 128);
-      mbar_init(&sh->staged[w], 128);
-      mbar_init(&sh->cols[w], 128);
     }
+    sh->taken = 0;
     sh->abort_flag = 0;
     fence_barrier_init();
   }
@@ -866,7 +921,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) monarch_tiles(const __gr
     const uint32_t one2 = pack2<__half>(1.f, 1.f);
     *reinterpret_cast<uint4*>(smem + kOffOnes + tid * 16) = make_uint4(one2, one2, one2, one2);
   }
-  for (int i = tid; i < 3 * 128; i += kThreads) reinterpret_cast<float*>(smem + kOffVec)[i] = 0.f;
+  for (int i = tid; i < 4 * 128; i += kThreads) reinterpret_cast<float*>(smem + kOffVec)[i] = 0.f;
   for (int i = tid; i < 4 * 128; i += kThreads) reinterpret_cast<unsigned*>(smem + kOffCol)[i] = 0u;
   if (warp == 8) tmem_alloc(&sh->tmem, 256);
   fence_proxy_async();
@@ -874,19 +929,23 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) monarch_tiles(const __gr
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sh->tmem;
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (MODE == 0 && P.first) clear_status(P.clear);
   using K = Kernel<TIn, B, FULL, MODE>;
   // registers: 384 threads at the launch's 80; 128 x 48 + 256 x 96 make use of all of them
   if (warp >= 8) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
-    if (elect_one()) {
-      if (warp == 8) K::produce(P, smem, sh);
-      else if (warp == 9) K::issue(P, smem, sh, tmem);
-      else K::store(P, smem, sh, warp - 10);
+    if (warp < 10) {
+      if (elect_one()) K::produce(P, smem, sh, warp - 8);
+    } else {
+      grid_wait();
+      K::store(P, smem, sh, warp - 10);
     }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 96;");
+    grid_wait();
+    if (starts) {
+      grid_launch_dependents();
+      clear_status(P.clear);
+    }
     K::compute(P, smem, sh, tmem, warp >> 2);
   }
   __syncwarp();
