@@ -296,6 +296,9 @@ static bool touches_workspace(int resolved) {
 // that the two half-steps take 5/3 of the tiles the rows would fill, the warp-MMA tiles win (8 blocks of 48
 // 44.6 against 52.4 us, 16 of 48 36.9 / 40.3, 12 of 64 40.9 / 42.8; 16 of 64 38.5 / 38.2, 17 of 48 42.3 / 39.5;
 // 8 of 128 59.1 / 51.4).
+// One round (us, warp-MMA / tcgen05 tiles): blocks of 64 and more from 64 tiles on, 3 heads of 47 x 64 14.2 / 10.9, 9 15.7 / 13.1, bf16 5 16.6 / 14.5, 7 of
+// 60 x 128 25.4 / 17.4, one 13.6 / 11.7, bf16 one of 90 x 128 16.1 / 16.0; smaller ones in f16 from 128 on, 14 of 30 x 48 13.3 / 12.5, 16 of 40 x 32 12.8 / 12.2, 27 of
+// 60 x 32 18.1 / 15.6; in bf16, which these tiles convert first, 20 of 60 x 32 15.5 / 16.5, 30 of 40 x 32 16.5 / 17.3: from 448 on.
 static bool tiles_on_tensor_cores(const Problem& p, float scale) {
   if (p.T > 2 || !(scale >= 0.f) || !ttc::supported(p.N, p.d, p.b, p.m, p.dtype, p.BH)) return false;
   const long long tiles = (long long)p.BH * p.N / 128;
@@ -303,7 +306,8 @@ static bool tiles_on_tensor_cores(const Problem& p, float scale) {
   const int pr = per_tile(p.b), pl = per_tile(p.m);
   const int taken = (p.m + pr - 1) / pr + (p.b + pl - 1) / pl;
   if (p.b <= 64 && 3 * 128 * taken >= 5 * 2 * p.N) return false;
-  return tiles >= (p.T == 2 && p.b > 32 ? 160 : 448);
+  if (p.T == 2) return tiles >= (p.b > 32 ? 160 : 448);
+  return tiles >= (p.d < 48 ? 448 : (p.b >= 64 ? 64 : (p.dtype == MA_F16 ? 128 : 448)));
 }
 
 // Where a call's waits report to, and the status word it clears first (a caller's workspace; nullptr: none).
