@@ -58,7 +58,6 @@ struct __align__(16) Shared {
   uint64_t empty[kSlots];
   uint64_t mma1[2], first[2], mma2[2], out_free[2];
   int through[2];                                     // tiles of a group that have left tensor memory
-  int go[2];                                          // whether the group goes on: its first warp's word before every release
   int4 tile[2][2];                                    // {half-step, head, first block or position} of a tile, or {-1, ..}
   int4 out[2];                                        // {head or -1, first block or position, slot | Rows << 4 | last << 8, half-step}
   uint32_t tmem;
@@ -122,6 +121,16 @@ __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Shared*
 // rows.
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 __device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+// The same with a vote: whether it is true for all of them.
+__device__ __forceinline__ bool bar_all(int id, int n, bool on) {
+  uint32_t all;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %3, 0;\n\tbarrier.cta.red.and.pred q, %1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(all)
+      : "r"(id), "r"(n), "r"((uint32_t)on)
+      : "memory");
+  return all != 0;
+}
 enum BarId { kRelease = 1, kCollect = 3, kStaged = 5 };
 // Tiles that a group is through with: its first warp says so once all warps have come by, the producer waits for it (bounded).
 __device__ __forceinline__ void say_through(Shared* sh, int w, uint32_t tiles) {
@@ -320,8 +329,8 @@ struct Chain {
   }
 
   // ================================================================ compute group w (thread = score row)
-  static __device__ __forceinline__ void compute(const Params& P, uint8_t* smem, Shared* sh, uint32_t tmem, int w) {
-    const int t_row = threadIdx.x & 127, warp = (threadIdx.x >> 5) & 3;
+  static __device__ __forceinline__ void compute(const Params& P, uint8_t* smem, Shared* sh, uint32_t tmem, int warp_of_cta) {
+    const int t_row = threadIdx.x & 127, warp = warp_of_cta & 3, w = warp_of_cta >> 2;
     const int blk = Geo<B>::tile(t_row), r = Geo<B>::row(t_row), srow = blk * B + r;
     const uint32_t d = tmem + 128 * w, tS = d + ((uint32_t)(warp * 32) << 16);
     const uint32_t sm = smem_u32(smem);
@@ -335,11 +344,10 @@ struct Chain {
     // issue slots from those at work.  A wait that ran out reaches the others with the same release.
     auto await = [&](uint64_t* bar, uint32_t parity, int where) { ok = __all_sync(0xffffffffu, wait_bar(bar, parity, sh, P, where)) && ok; };
     auto release = [&](bool on) {              // of the group; false: no more tiles
-      if (t_row == 0) sh->go[w] = on;
       tc_fence_before();
-      bar_sync(kRelease + w, 128);
+      const bool go = bar_all(kRelease + w, 128, on);
       tc_fence_after();
-      return *(volatile int*)&sh->go[w] != 0;
+      return go;
     };
     auto collect = [&]() {                     // all warps have come by: the first one waits
       tc_fence_before();
@@ -511,7 +519,7 @@ struct Chain {
         if (!t.final_) {
           // the contraction runs over the rows of the weights: normalised in fp32, rounded once, to shared memory
           const float2 n2 = both(mul * kWeightScale);
-          // (128 columns: the slot of the second half is free.  Every warp looks for itself, two releases in a row would share their word.)
+          // (128 columns: the slot of the second half is free; every warp looks for itself)
           if (B == 128) await(&sh->third[w][q & 1], (par_3 >> (q & 1)) & 1, 36);
           uint8_t* lower = smem + (B == 128 ? min(x.x1, x.x2) : x.x1) * kSlot + srow * 128;
           uint8_t* upper = smem + max(x.x1, x.x2) * kSlot + srow * 128;
@@ -611,7 +619,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) monarch_chain(const __gr
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem<1024>(smem_raw);
   Shared* sh = reinterpret_cast<Shared*>(smem + kOffBar);
-  const int tid = threadIdx.x, warp = tid >> 5;
+  // (by a shuffle, so that the compiler knows it to be the same in a warp: descriptors and addresses of tensor memory then stay in uniform
+  // registers)
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid == 0) {
     for (int i = 0; i < kSlots; ++i) mbar_init(&sh->empty[i], 1);
@@ -638,17 +648,17 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) monarch_chain(const __gr
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = sh->tmem;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, sh->tmem, 0);
   asm volatile("griddepcontrol.wait;" ::: "memory");
   using C = Chain<T, B, EXTRA>;
-  // registers: 384 threads at the launch's 80; 128 x 48 + 256 x 96 make use of all of them
+  // registers: 384 threads at the launch's 80; 128 x 64 + 256 x 88 make use of all of them (nothing is spilled; with 48 the producers spill)
   if (warp >= 8) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
     if (warp >= 10) C::store(P, smem, sh, warp - 10);
     else if (elect_one()) C::produce(P, smem, sh, warp - 8);
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 96;");
-    C::compute(P, smem, sh, tmem, warp >> 2);
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 88;");
+    C::compute(P, smem, sh, tmem, warp);
   }
   __syncwarp();
   tc_fence_before();
