@@ -79,7 +79,6 @@ struct __align__(16) Shared {
   int4 tile[2][2];           // {head or -1, first block or position, keys that count}
   int4 out[2];               // {head or -1, first block or position, slot, is y}
   int through[2];            // tiles of a group that have left tensor memory
-  int go[2];                 // whether the group goes on: its first warp's word before every release
   int taken;                 // tiles of the CTA that its groups have taken
   uint32_t tmem;
   volatile int abort_flag;
@@ -113,6 +112,16 @@ struct Slots {
 // rows.
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 __device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+// The same with a vote: whether it is true for all of them.
+__device__ __forceinline__ bool bar_all(int id, int n, bool on) {
+  uint32_t all;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %3, 0;\n\tbarrier.cta.red.and.pred q, %1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(all)
+      : "r"(id), "r"(n), "r"((uint32_t)on)
+      : "memory");
+  return all != 0;
+}
 enum BarId { kRelease = 1, kCollect = 3, kStaged = 5 };
 // Tiles that a group is through with: its first warp says so once all warps have come by, the producer waits for it (bounded).
 __device__ __forceinline__ void say_through(Shared* sh, int w, uint32_t tiles) {
@@ -620,8 +629,8 @@ struct Kernel {
     }
   }
 
-  static __device__ __forceinline__ void compute(const Params& P, uint8_t* smem, Shared* sh, uint32_t tmem, int w) {
-    const int row = threadIdx.x & 127, warp = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
+  static __device__ __forceinline__ void compute(const Params& P, uint8_t* smem, Shared* sh, uint32_t tmem, int warp_of_cta) {
+    const int row = threadIdx.x & 127, warp = warp_of_cta & 3, w = warp_of_cta >> 2, lane = threadIdx.x & 31;
     const uint32_t d = tmem + 128 * w, t_row = d + ((uint32_t)(warp * 32) << 16);     // the group's columns, this warp's lanes
     const bool prep = prepares(P), last = P.last != 0;
     Slots<B, R> x(w);
@@ -630,12 +639,11 @@ struct Kernel {
     // The first warp alone looks at mbarriers and lets the others go on once it has seen one: four warps that try and try again take
     // issue slots from those at work.  A wait that ran out reaches the others with the same release.
     auto await = [&](uint64_t* bar, uint32_t parity, int where) { ok = __all_sync(0xffffffffu, wait_bar(bar, parity, sh, P, where)) && ok; };
-    auto release = [&](bool on) {              // of the group; false: no more tiles.  (A collect comes between any two: they share the word.)
-      if (row == 0) sh->go[w] = on;
+    auto release = [&](bool on) {              // of the group; false: no more tiles
       tc_fence_before();
-      bar_sync(kRelease + w, 128);
+      const bool go = bar_all(kRelease + w, 128, on);
       tc_fence_after();
-      return *(volatile int*)&sh->go[w] != 0;
+      return go;
     };
     auto collect = [&]() {                     // all warps have come by: the first one waits
       tc_fence_before();
@@ -781,7 +789,7 @@ struct Kernel {
             fold_columns(v, onr, sMax + B * r_blk + 32 * cc, lane);
           }
           ld_frag32(tS, v);
-          // (128 columns: the slot of the second half is free.  Every warp looks for itself, a release would share its word with the last.)
+          // (128 columns: the slot of the second half is free; every warp looks for itself)
           if (B == 128) await(&sh->third[w][par], par2, 36);
           bar_sync(kRelease + w, 128);
           // (the set of the tile before: all warps are done with it, and none begins the next tile before all have come by)
@@ -897,7 +905,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) monarch_tiles(const __gr
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem<1024>(smem_raw);
   Shared* sh = reinterpret_cast<Shared*>(smem + kOffBar);
-  const int tid = threadIdx.x, warp = tid >> 5;
+  // (by a shuffle, so that the compiler knows it to be the same in a warp: descriptors and addresses of tensor memory then stay in uniform
+  // registers)
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const bool starts = MODE == 0 && P.first;      // the first launch of a call
   if (!starts) grid_launch_dependents();
   if (tid == 0) {
@@ -928,11 +938,11 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) monarch_tiles(const __gr
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = sh->tmem;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, sh->tmem, 0);
   using K = Kernel<TIn, B, FULL, MODE>;
-  // registers: 384 threads at the launch's 80; 128 x 48 + 256 x 96 make use of all of them
+  // registers: 384 threads at the launch's 80; 128 x 64 + 256 x 88 make use of all of them
   if (warp >= 8) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
     if (warp < 10) {
       if (elect_one()) K::produce(P, smem, sh, warp - 8);
     } else {
@@ -940,13 +950,13 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) monarch_tiles(const __gr
       K::store(P, smem, sh, warp - 10);
     }
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 96;");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 88;");
     grid_wait();
     if (starts) {
       grid_launch_dependents();
       clear_status(P.clear);
     }
-    K::compute(P, smem, sh, tmem, warp >> 2);
+    K::compute(P, smem, sh, tmem, warp);
   }
   __syncwarp();
   tc_fence_before();
