@@ -151,14 +151,14 @@ __global__ void __launch_bounds__(32 * WARPS, 1) monarch_fused_head(const __grid
   constexpr int RB = (NB + 1) / 2, RM = (NM + 1) / 2;      // 16-row tiles
   extern __shared__ uint8_t smem_raw[];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint8_t* smem = align_smem<1024>(smem_raw);
   const int tile = P.tile, b = P.b, bp = P.bp;
   const uint32_t s0 = smem_u32(smem);
   const int tiles = V_LAST ? 3 : 3 * P.bufs + (MULTI ? 1 : 0);
   const uint32_t sS = s0 + (tiles - 1) * tile;             // state tile (MULTI)
   uint8_t* tail = smem + tiles * tile;
   float* sCL = reinterpret_cast<float*>(tail + 128);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int tid = threadIdx.x, warp = warp_of_cta(), lane = tid & 31, g = lane >> 2, t = lane & 3;
   const uint32_t dump = smem_u32(tail) + (lane & 7) * 16;
   Bars* bars = reinterpret_cast<Bars*>(sCL + b * NM * 8);
   if (tid == 0) {

@@ -28,6 +28,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "shared_align.cuh"
 #include "status_word.cuh"
 #include "warp_mma.cuh"
 
@@ -133,8 +134,7 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
     n_valid = min(max(seq_len[blockIdx.x / heads], 1), N);
     m = (n_valid + b - 1) / b;
   }
-  constexpr uintptr_t kAlign = KS == 4 ? 1024 : 128;
-  uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + kAlign - 1) & ~(kAlign - 1));
+  uint8_t* smem = align_smem<KS == 4 ? 1024 : 128>(smem_raw);
   const int tile = KS == 4 ? N * kRowBytes : (N / b) * block_bytes<KS>(b);
   uint8_t* sQ = smem;
   // then K, then V (loaded when the last round starts) ...
@@ -155,7 +155,7 @@ monarch_fused_small(const TIn* __restrict__ Q, const TIn* __restrict__ K, const 
   const uint32_t sS_u = sQ_u + 3 * tile, sALlo_u = sQ_u + 4 * tile, sARlo_u = sALlo_u;   // HILO only
   const bool v_early = HILO || T_steps == 1;      // V comes in with the first round's loads
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_of_cta(), lane = tid & 31;
   const int nw = blockDim.x >> 5;    // 8 warps, or 16 where only one CTA fits an SM (16 x 16 blocks)
   const int g = lane >> 2, t = lane & 3;
   const int h_idx = blockIdx.x;

@@ -7,7 +7,9 @@
 //   * two CTAs per SM with two compute groups of four warps each; a group (thread = score row) takes a tile from its scores
 //     to its staged rows, and its first warp issues the tile's MMAs itself.  That warp alone looks at mbarriers, which means trying again
 //     and again; the others and the store warp wait in hardware barriers (64 heads of 4096, T = 2: 77.8 us with every warp
-//     at the mbarriers, 76.7 with one; trying in a tighter loop, a quarter more branches in all, cost 4 %);
+//     at the mbarriers, 76.7 with one; trying in a tighter loop, a quarter more branches in all, cost 4 %).  Issuing a tile's eight score MMAs took
+//     a thread about 1000 cycles and a release 500 (clock stamps) while the warp's number came from threadIdx and the release's word
+//     went through shared memory: 74.0 us, 70.7 with uniform descriptors and a vote in the barrier;
 //   * three 16 KB slots a group.  Which of them a tile's operands take follows from the order in which the tile before gives
 //     its slots up (Slots), so that loads of the next tile run under the softmax of this one;
 //   * the weights go back to tensor memory over the scores and are the A operand of the apply MMA; in the non-final L
@@ -619,9 +621,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) monarch_chain(const __gr
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem<1024>(smem_raw);
   Shared* sh = reinterpret_cast<Shared*>(smem + kOffBar);
-  // (by a shuffle, so that the compiler knows it to be the same in a warp: descriptors and addresses of tensor memory then stay in uniform
-  // registers)
-  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const int tid = threadIdx.x, warp = warp_of_cta();
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid == 0) {
     for (int i = 0; i < kSlots; ++i) mbar_init(&sh->empty[i], 1);

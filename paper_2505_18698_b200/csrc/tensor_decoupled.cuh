@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(kThreads, 1) monarch_decoupled(const __grid_co
   constexpr int kBlocks = kRows / SB;         // blocks (k of an R tile, j of an L tile) per CTA
   constexpr int NSUB = B / SB;                // blocks per MMA tile
   constexpr int FT = Fmt<T>::code;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_of_cta(), lane = tid & 31;
   const int m = P.m;
 
   if (tid == 0) {
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kThreads, 1) monarch_decoupled(const __grid_co
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = bars->tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, bars->tmem_slot, 0);
   const uint32_t tmem_o = tmem + kStagesS * B;   // O stage o at tmem_o + 128 o
 
   const int first_g = P.g_begin + blockIdx.x;

@@ -20,6 +20,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "shared_align.cuh"
 #include "status_word.cuh"
 #include "warp_mma.cuh"
 #include "fused_small.cuh"
@@ -167,7 +168,7 @@ r_tile_kernel(const TIn* __restrict__ Q, const TIn* __restrict__ K, const TIn* _
     n_valid = min(max(seq_len[h / heads], 1), N);
     if (k * b >= n_valid) return;
   }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int warp = warp_of_cta(), lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int rb = round16(b);
   uint8_t* sA = smem;
   uint8_t* sK = sA + (size_t)rb * kPitch;
@@ -365,7 +366,7 @@ l_tile_kernel(const TIn* __restrict__ Q, const __half* __restrict__ aL, const fl
   // 0 .. ceil(length / b) - 1 only; rows of Y in blocks past them are written as zeros.
   const int m_alloc = m;
   if (seq_len != nullptr) m = (min(max(seq_len[h / heads], 1), N) + b - 1) / b;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int warp = warp_of_cta(), lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int rm = round16(m);
   uint8_t* sQ = smem;
   uint8_t* sL = sQ + (size_t)rm * kPitch;

@@ -905,9 +905,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) monarch_tiles(const __gr
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align_smem<1024>(smem_raw);
   Shared* sh = reinterpret_cast<Shared*>(smem + kOffBar);
-  // (by a shuffle, so that the compiler knows it to be the same in a warp: descriptors and addresses of tensor memory then stay in uniform
-  // registers)
-  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const int tid = threadIdx.x, warp = warp_of_cta();
   const bool starts = MODE == 0 && P.first;      // the first launch of a call
   if (!starts) grid_launch_dependents();
   if (tid == 0) {
