@@ -13,7 +13,8 @@
 //     eight rows are then free of bank conflicts along a block (R half-step) and across blocks
 //     (L half-step), so the permutation between the half-steps is only a choice of rows;
 //   * a warp owns a block (R) or a position (L) and holds its scores and weights in registers, in as many
-//     8-column tiles as b or m need.
+//     8-column tiles as b or m need;
+//   * few heads of more than 16 rows a block go to two CTAs each, by in-block position (`plan`).
 // One round: alpha_L goes over K, y over V, Y over Q.  More rounds: alpha_R and alpha_L replace each
 // other in place in a state tile.  Arithmetic is f16 whatever the input type (see fused_small.cuh).
 //
@@ -61,6 +62,7 @@ struct Params {
   int bp;                   // block pitch in rows
   int tile;                 // bytes of a tile
   int bufs;                 // heads in shared memory
+  int part;                 // positions of a CTA (a head to two CTAs)
   float scale;
 };
 
@@ -143,12 +145,14 @@ __device__ __forceinline__ void products(float (&o)[2][4], const uint32_t (&a)[K
     }
 }
 
-// NB, NM: 8-column tiles that hold b keys / m blocks.  WARPS: on an SM.
-template <typename TIn, int NB, int NM, int ROUNDS, int WARPS>
+// NB, NM: 8-column tiles that hold b keys / m blocks.  WARPS: on an SM.  RT: 16-row tiles of a block's positions that a CTA has: all of
+// them, or one where a head goes to two CTAs (nothing couples two positions but K and V, which both read).
+template <typename TIn, int NB, int NM, int ROUNDS, int WARPS, int RT = (NB + 1) / 2>
 __global__ void __launch_bounds__(32 * WARPS, 1) monarch_fused_head(const __grid_constant__ Params P) {
   typedef Mma<__half> M;
   constexpr bool MULTI = ROUNDS != kOne, V_LAST = ROUNDS == kMoreVLast;
   constexpr int RB = (NB + 1) / 2, RM = (NM + 1) / 2;      // 16-row tiles
+  constexpr bool SPLIT = RT < RB;
   extern __shared__ uint8_t smem_raw[];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   uint8_t* smem = align_smem<1024>(smem_raw);
@@ -203,7 +207,9 @@ __global__ void __launch_bounds__(32 * WARPS, 1) monarch_fused_head(const __grid
       }
     }
   };
-  request(blockIdx.x, 0);
+  const int first_head = SPLIT ? (int)blockIdx.x >> 1 : (int)blockIdx.x, step_heads = SPLIT ? P.BH : (int)gridDim.x;
+  const int j0 = SPLIT && (blockIdx.x & 1) ? P.part : 0, j1 = SPLIT ? min(j0 + P.part, b) : b;      // the CTA's positions
+  request(first_head, 0);
   int buf = 0;
   uint32_t par = 0;                 // bit 16 buf + r: parity of the warp's r-th block in that buffer
   constexpr uint32_t kDead = 1u << 31;      // in `par`: a wait ran out; the warp waits no more and leaves after this head
@@ -214,8 +220,8 @@ __global__ void __launch_bounds__(32 * WARPS, 1) monarch_fused_head(const __grid
     }
     par ^= 1u << bit;
   };
-  for (int h = blockIdx.x; h < P.BH; h += gridDim.x) {
-    if (!V_LAST && P.bufs == 2) request(h + gridDim.x, buf ^ 1);
+  for (int h = first_head; h < P.BH; h += step_heads) {
+    if (!V_LAST && P.bufs == 2) request(h + step_heads, buf ^ 1);
     const uint32_t sQ = s0 + 3 * buf * tile, sK = sQ + tile, sV = V_LAST ? sS : sK + tile;
     const int n_valid = valid_of(h);
     const int m = P.seq_len != nullptr ? (n_valid + b - 1) / b : P.m;
@@ -234,15 +240,15 @@ __global__ void __launch_bounds__(32 * WARPS, 1) monarch_fused_head(const __grid
         const uint32_t sA = first ? sQ : sS;                 // alpha_R (= Q rows while L is the identity)
         const uint32_t dst = !MULTI || (V_LAST && last) ? sK : sS;      // alpha_L
         const int lim = min(b, n_valid - k * b);             // keys of this block that count
-        uint32_t pa[RB][RB][4];                              // unnormalised weights: the largest is exactly 1
-        float inv[RB][2], off[2 * RB], red[4 * RB];          // red: sum of the weights, sum of weight times score
+        uint32_t pa[RT][RB][4];                              // unnormalised weights: the largest is exactly 1
+        float inv[RT][2], off[2 * RT], red[4 * RT];          // red: sum of the weights, sum of weight times score
         {
           uint32_t kb[NB][4][2];
           load_b<NB>(kb, sK, lane, [&](int i) { return r0 + min(i, b - 1); });
 #pragma unroll
-          for (int rt = 0; rt < RB; ++rt) {
+          for (int rt = 0; rt < RT; ++rt) {
             float s[NB][4];
-            const uint32_t ad = at(sA, r0 + min(16 * rt + a_row, b - 1), a_ch);
+            const uint32_t ad = at(sA, r0 + min(j0 + 16 * rt + a_row, b - 1), a_ch);
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks) {
               uint32_t a[4];
@@ -253,7 +259,7 @@ __global__ void __launch_bounds__(32 * WARPS, 1) monarch_fused_head(const __grid
                 else M::run(s[nt], a, kb[nt][ks]);
               }
             }
-            // rows j = 16 rt + g (c0, c1) and + 8 (c2, c3); columns i = 8 nt + 2 t, + 1.  Columns past the
+            // rows j = j0 + 16 rt + g (c0, c1) and + 8 (c2, c3); columns i = 8 nt + 2 t, + 1.  Columns past the
             // block, in the last column tile, and padded keys of the last block: a score of weight 0.
 #pragma unroll
             for (int e = 0; e < 4; ++e)
@@ -290,21 +296,21 @@ __global__ void __launch_bounds__(32 * WARPS, 1) monarch_fused_head(const __grid
           }
           // a lane ends up with both sums of row q = t (two row tiles), or with one of them: one division a
           // lane, the reciprocals then go to the row's four lanes
-          const float r = scatter_reduce<4 * RB, 2, 1>(red, lane, warpmma::Add());
+          const float r = scatter_reduce<4 * RT, 2, 1>(red, lane, warpmma::Add());
           const float ri = 1.f / r;
-          const int q = RB == 2 ? t : t >> 1, j = 16 * (q >> 1) + g + 8 * (q & 1);
+          const int q = RT == 2 ? t : t >> 1, j = j0 + 16 * (q >> 1) + g + 8 * (q & 1);
 #pragma unroll
-          for (int i = 0; i < 2 * RB; ++i) inv[i >> 1][i & 1] = __shfl_sync(0xffffffffu, ri, (lane & ~3) + i * (2 / RB));
+          for (int i = 0; i < 2 * RT; ++i) inv[i >> 1][i & 1] = __shfl_sync(0xffffffffu, ri, (lane & ~3) + i * (2 / RT));
           float so = r, sz = red[1], io = ri, mo = off[0];
-          if (RB == 1) {
+          if (RT == 1) {
             sz = r;
             so = __shfl_xor_sync(0xffffffffu, r, 1);
             io = __shfl_xor_sync(0xffffffffu, ri, 1);
           }
 #pragma unroll
-          for (int i = 1; i < 2 * RB; ++i) mo = q == i ? off[i] : mo;
+          for (int i = 1; i < 2 * RT; ++i) mo = q == i ? off[i] : mo;
           // -c_L log2 e = log2 sum + max - sum R z (Eq. 10), the addend of the L logits
-          if ((RB == 2 || (t & 1)) && j < b) sCL[j * NM * 8 + k] = lg2(so) - mo - fl * (sz * io);
+          if ((RT == 2 || (t & 1)) && j < j1) sCL[j * NM * 8 + k] = lg2(so) - mo - fl * (sz * io);
         }
         if (V_LAST && last) {      // the block's rows of alpha_R have been read, V takes their place
           tensor::fence_proxy_async();
@@ -316,17 +322,16 @@ __global__ void __launch_bounds__(32 * WARPS, 1) monarch_fused_head(const __grid
         }
         __syncwarp();
         // second products, 16 columns at a time; a warp alone reads and writes the rows of its block
-        uint32_t kt[RB], st[RB];
+        uint32_t kt[RB], st[RT];
 #pragma unroll
-        for (int kk = 0; kk < RB; ++kk) {
-          kt[kk] = at(sK, r0 + min(16 * kk + a_row, b - 1), a_ch);
-          st[kk] = 16 * kk + a_row < b ? at(dst, r0 + 16 * kk + a_row, a_ch) : dump;
-        }
+        for (int kk = 0; kk < RB; ++kk) kt[kk] = at(sK, r0 + min(16 * kk + a_row, b - 1), a_ch);
+#pragma unroll
+        for (int rt = 0; rt < RT; ++rt) st[rt] = j0 + 16 * rt + a_row < j1 ? at(dst, r0 + j0 + 16 * rt + a_row, a_ch) : dump;
         // (from the K tile's addresses to the V tile's, from those of alpha_L to y's)
         const uint32_t to_v = sV - sK;
-        uint32_t sy[RB];
+        uint32_t sy[RT];
 #pragma unroll
-        for (int kk = 0; kk < RB; ++kk) sy[kk] = 16 * kk + a_row < b ? st[kk] - dst + sV : dump;
+        for (int rt = 0; rt < RT; ++rt) sy[rt] = j0 + 16 * rt + a_row < j1 ? st[rt] - dst + sV : dump;
 #pragma unroll
         for (int np = 0; np < 4; ++np) {
           uint32_t bk[RB][4], bv[RB][4];
@@ -338,7 +343,7 @@ __global__ void __launch_bounds__(32 * WARPS, 1) monarch_fused_head(const __grid
           }
           __syncwarp();
 #pragma unroll
-          for (int rt = 0; rt < RB; ++rt) {
+          for (int rt = 0; rt < RT; ++rt) {
             float o[2][4];
             products<RB>(o, pa[rt], bk);
             put(st[rt] ^ (np << 5), o, inv[rt][0], inv[rt][1]);
@@ -359,7 +364,7 @@ __global__ void __launch_bounds__(32 * WARPS, 1) monarch_fused_head(const __grid
             for (int kk = 0; kk < RB; ++kk) ldsm_x4_trans(bv[kk], (kt[kk] ^ (np << 5)) + to_v);
             __syncwarp();
 #pragma unroll
-            for (int rt = 0; rt < RB; ++rt) {
+            for (int rt = 0; rt < RT; ++rt) {
               float o[2][4];
               products<RB>(o, pa[rt], bv);
               put(sy[rt] ^ (np << 5), o, inv[rt][0], inv[rt][1]);
@@ -370,7 +375,7 @@ __global__ void __launch_bounds__(32 * WARPS, 1) monarch_fused_head(const __grid
       __syncthreads();
 
       // ================================================================ L half-step (Eq. 8, 9 / Eq. 4)
-      for (int j = warp; j < b; j += nw) {
+      for (int j = j0 + warp; j < j1; j += nw) {
         const uint32_t sA = !MULTI || (V_LAST && last) ? sK : sS;       // alpha_L
         float c[NM][2];
 #pragma unroll
@@ -558,7 +563,7 @@ __global__ void __launch_bounds__(32 * WARPS, 1) monarch_fused_head(const __grid
       return;
     }
     if (!V_LAST && P.bufs == 2) buf ^= 1;
-    else request(h + gridDim.x, 0);
+    else request(h + step_heads, 0);
   }
 }
 
@@ -630,17 +635,17 @@ inline bool get_maps(Params* P, const Args& a, const Plan& p, int dev) {
   P->v = c.maps[e][2];
   return true;
 }
-template <typename TIn, int NB, int NM, int ROUNDS, int WARPS = max_warps(NB, NM, ROUNDS)>
+template <typename TIn, int NB, int NM, int ROUNDS, int WARPS = max_warps(NB, NM, ROUNDS), int RT = (NB + 1) / 2>
 inline int launch_k(const Params& P, const Plan& p, int num_sms, cudaStream_t st) {
-  auto kern = monarch_fused_head<TIn, NB, NM, ROUNDS, WARPS>;
+  auto kern = monarch_fused_head<TIn, NB, NM, ROUNDS, WARPS, RT>;
   static warpmma::SmemOptIn opt_in;
   if (!opt_in.done((const void*)kern, (int)kMaxSmem)) return 7;
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
-  const int slots = p.ctas * num_sms;
-  cfg.gridDim = dim3(P.BH < slots ? P.BH : slots);
+  const int slots = p.ctas * num_sms, parts = p.parts * P.BH;
+  cfg.gridDim = dim3(parts < slots ? parts : slots);
   cfg.blockDim = dim3(32 * p.warps);
   cfg.dynamicSmemBytes = p.smem;
   cfg.stream = st;
@@ -653,6 +658,13 @@ inline int launch_n(const Params& P, const Plan& p, int num_sms, cudaStream_t st
   const int nb = (P.b + 7) / 8, nm = (P.m + 7) / 8;
   if (p.bound == 16 && nb == 2 && nm == 2) return launch_k<TIn, 2, 2, ROUNDS, 16>(P, p, num_sms, st);
   if (p.bound == 24 && nb == 3 && nm == 2) return launch_k<TIn, 3, 2, ROUNDS, 24>(P, p, num_sms, st);
+  if (p.parts == 2) {
+#define MA_FH(B)                                                   \
+  (nm == 2 ? launch_k<TIn, B, 2, ROUNDS, 16, 1>(P, p, num_sms, st) \
+           : (nm == 3 ? launch_k<TIn, B, 3, ROUNDS, 16, 1>(P, p, num_sms, st) : launch_k<TIn, B, 4, ROUNDS, 16, 1>(P, p, num_sms, st)))
+    return nb == 3 ? MA_FH(3) : MA_FH(4);
+#undef MA_FH
+  }
 #define MA_FH(B)                                            \
   (nm == 2 ? launch_k<TIn, B, 2, ROUNDS>(P, p, num_sms, st) \
            : (nm == 3 ? launch_k<TIn, B, 3, ROUNDS>(P, p, num_sms, st) : launch_k<TIn, B, 4, ROUNDS>(P, p, num_sms, st)))
@@ -675,7 +687,7 @@ int launch(const Args& a, cudaStream_t st) {
   if (!get_maps(&P, a, p, dev)) return 7;
   P.Y = a.Y; P.lse = a.lse; P.seq_len = a.seq_len; P.status = a.status; P.clear = a.clear;
   P.BH = a.BH; P.N = a.N; P.d = a.d; P.b = a.b; P.m = a.m; P.T = a.T; P.H = a.H; P.heads = a.heads; P.n_valid = a.n_valid;
-  P.bp = p.bp; P.tile = p.tile; P.bufs = p.bufs;
+  P.bp = p.bp; P.tile = p.tile; P.bufs = p.bufs; P.part = (a.b + 1) / 2;
   P.scale = a.scale;
   return a.dtype == 1 ? launch_t<__half>(P, p, sms[dev], st) : launch_t<__nv_bfloat16>(P, p, sms[dev], st);
 }

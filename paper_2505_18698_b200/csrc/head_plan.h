@@ -38,6 +38,7 @@ inline size_t smem_bytes(int tile, int bufs, int rounds, int b, int nm) {
 
 struct Plan {
   int bp, tile, bufs, warps, ctas, rounds, bound;      // ctas: per SM; bound: warps an SM that the kernel is compiled for
+  int parts;      // CTAs a head goes to
   size_t smem;
 };
 inline bool plan(int b, int m, int T, int BH, int num_sms, Plan* p) {
@@ -83,10 +84,15 @@ inline bool plan(int b, int m, int T, int BH, int num_sms, Plan* p) {
     }
     // (24 x 16 and the like, more rounds: 24 warps where they are two heads: 216 heads of 20 x 10 16.0 us, with 16 17.4)
     if (nb == 3 && nm == 2 && rounds == kMore && p->ctas == 2) most = 24;
+    // More than 16 positions and SMs enough for two CTAs a head: half of the positions each, so that a block is one 16-row tile instead of two
+    // and a position has a warp to itself (us, one CTA / two: 12 heads of 16 x 24, one round 6.9 / 4.8, two 11.7 / 7.6, 36 of 19 x 22 9.0 / 6.3, 48 of 12 x 20, two
+    // rounds 10.0 / 6.8, 72 of 23 x 17 9.6 / 7.3, 24 of 14 x 30 7.6 / 5.1).
+    p->parts = nb > 2 && 2 * BH <= num_sms ? 2 : 1;
+    if (p->parts == 2) most = 16;
     // the fewest warps that take the fewest rounds of tiles over both half-steps
     int best = 1 << 30;
     for (int w = 1; w <= most / p->ctas; ++w) {
-      const int turns = (m + w - 1) / w + (b + w - 1) / w;
+      const int turns = (m + w - 1) / w + ((b + p->parts - 1) / p->parts + w - 1) / w;
       if (turns < best) {
         best = turns;
         p->warps = w;
