@@ -290,12 +290,16 @@ static bool touches_workspace(int resolved) {
 // d <= 64) and warp-MMA tiles (tile_mma.cuh: hi + lo states for three or more rounds, wider heads,
 // negative scales).  Where both apply the tcgen05 tiles pay for their set-up and longer chain once
 // there are tiles enough to keep several in flight on every SM: measured over N = 960 .. 10240 and 8
-// to 64 heads they are 1.0-1.9 x as fast from 448 tiles of 128 rows on (two rounds of blocks of
-// more than 32: from 160 on), and 0.65-0.97 x below.  Their tiles hold whole blocks rounded up to 32, 64 or
+// to 64 heads they were 1.0-1.9 x as fast from 448 tiles of 128 rows on (two rounds of blocks of
+// more than 32: from 160 on); since a group issues its own MMAs the lines below hold.  Their tiles hold whole blocks rounded up to 32, 64 or
 // 128 rows; the warp-MMA tiles are as wide as the block.  With blocks of up to 64 rows and so few of them
 // that the two half-steps take 5/3 of the tiles the rows would fill, the warp-MMA tiles win (8 blocks of 48
 // 44.6 against 52.4 us, 16 of 48 36.9 / 40.3, 12 of 64 40.9 / 42.8; 16 of 64 38.5 / 38.2, 17 of 48 42.3 / 39.5;
 // 8 of 128 59.1 / 51.4).
+// Two rounds (us, warp-MMA / tcgen05 tiles; graphs): 8 heads of 60 x 32 in bf16 29.5 / 24.6, 16 of 47 x 32 28.3 / 23.7, 24 of 55 x 32 39.6 / 26.3, 12 of 64 x 32 27.4 /
+// 21.7, 25 of 32 x 32, masked 24.0 / 22.1, 6 of 47 x 64 32.6 / 24.0, 8 of 33 x 64 31.6 / 24.3, 1 of 70 x 128 32.0 / 26.9: 1.04 to 1.5 x over 150 sizes of these kinds, but
+// 13 of 60 x 32 in bf16 (26.4 / 26.9, d = 48 24.8 / 26.5), which the other tiles happen to fill the GPU with, as 4 of 47 x 64 (19.1 / 21.8; 3 of them 30.9 / 21.3),
+// hence 128 there; below 64 tiles 1 head of 34 x 32 15.7 / 18.1, bf16 1 of 47 x 32 17.1 / 21.2, but 1 of 64 x 32 16.5 / 16.8, 2 in bf16 23.6 / 19.3, 1 of 128 x 32 29.4 / 22.4.
 // One round (us, warp-MMA / tcgen05 tiles): blocks of 64 and more from 64 tiles on, 3 heads of 47 x 64 14.2 / 10.9, 9 15.7 / 13.1, bf16 5 16.6 / 14.5, 7 of
 // 60 x 128 25.4 / 17.4, one 13.6 / 11.7, bf16 one of 90 x 128 16.1 / 16.0; smaller ones in f16 from 128 on, 14 of 30 x 48 13.3 / 12.5, 16 of 40 x 32 12.8 / 12.2, 27 of
 // 60 x 32 18.1 / 15.6; in bf16, which these tiles convert first, 20 of 60 x 32 15.5 / 16.5, 30 of 40 x 32 16.5 / 17.3: from 448 on.
@@ -306,7 +310,11 @@ static bool tiles_on_tensor_cores(const Problem& p, float scale) {
   const int pr = per_tile(p.b), pl = per_tile(p.m);
   const int taken = (p.m + pr - 1) / pr + (p.b + pl - 1) / pl;
   if (p.b <= 64 && 3 * 128 * taken >= 5 * 2 * p.N) return false;
-  if (p.T == 2) return tiles >= (p.b > 32 ? 160 : 448);
+  if (p.T == 2) {
+    if (p.d < 48 || p.b < 32) return tiles >= (p.b > 32 ? 160 : 448);
+    if (p.b == 32) return p.m >= 64 || tiles >= (p.m > 32 || p.d == 64 ? 64 : 448);
+    return tiles >= (p.b > 64 ? 64 : (p.m > 32 ? 128 : 160));
+  }
   return tiles >= (p.d < 48 ? 448 : (p.b >= 64 ? 64 : (p.dtype == MA_F16 ? 128 : 448)));
 }
 

@@ -19,12 +19,11 @@
 //     that columns of small weights keep their bits.
 // Service warps: a producer thread and a store warp per group.
 //
-// Measured (B200, us per call in loops of tenths of a second, against tensor_decoupled.cuh): 64 heads of 4096, T = 2 82 / 91 (bursts: 74 / 88;
-// the loop runs into the power limit, at 1765 MHz), 48 heads masked 68 / 77. A tile takes 3.8 to 5.7 us, of which its group waits
-// for operands 0.2 to 0.8.  Measured and not kept: tiles dealt out in advance (81 against 78 us in bursts: SMs differ in speed), a row of scores
-// in registers instead of read twice (44 bytes spilled: 80 against 74), heads in groups that stay in L2 (more tiles are in work and
-// requested, twice 592, than a half-step of 1024 leaves room for: 91 against 82).
-// Blocks of 128 (16 heads of 16384, T = 2, loops): 95 / 99.5; the weights of a non-final L half-step then take two of the three slots.
+// Measured (B200, us per call in loops of tenths of a second, against tensor_decoupled.cuh): 64 heads of 4096, T = 2 71 / 87, 16 of 16384 (the weights
+// of a non-final L half-step then take two of the three slots) 88 / 98, 12 of 16300 masked 76 / 93.  GPUs differ by 5 %.  Measured and not kept:
+// tiles dealt out in advance (81 against 78 us in bursts at the time: SMs differ in speed), a row of 64 scores in registers instead of read
+// twice (no difference, masked 5 % slower), heads in groups that stay in L2 (more tiles are in work and
+// requested, twice 592, than a half-step of 1024 leaves room for: 91 against 82), waits that do not suspend (2 % slower).
 #pragma once
 #include <type_traits>
 
