@@ -89,6 +89,9 @@ inline bool plan(int b, int m, int T, int BH, int num_sms, Plan* p) {
     // rounds 10.0 / 6.8, 72 of 23 x 17 9.6 / 7.3, 24 of 14 x 30 7.6 / 5.1).
     p->parts = nb > 2 && 2 * BH <= num_sms ? 2 : 1;
     if (p->parts == 2) most = 16;
+    // A CTA an SM: so much shared memory that the next call's CTAs do not come to an SM at work (us in loops, without / with: 144 heads of 11 x 12
+    // 6.8 / 5.0, of 10 x 10 6.0 / 4.7, 108 of 10 x 10, two rounds 8.1 / 6.5, 72 of 10 x 17 5.6 / 4.6; never slower by more than 2 %).
+    if (p->parts * BH <= num_sms) p->smem = std::max(p->smem, (size_t)114 * 1024);
     // the fewest warps that take the fewest rounds of tiles over both half-steps
     int best = 1 << 30;
     for (int w = 1; w <= most / p->ctas; ++w) {
