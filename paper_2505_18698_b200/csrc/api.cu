@@ -38,6 +38,7 @@ struct Problem {
   int H;         // 0: [batch][heads][N][d]; heads: [batch][N][heads][d]
   float* lse;    // optional output [batch*heads][N]: row log-sum-exp of the final L half-step
   const int* seq_len;   // optional DEVICE array [batch]: valid length of every sequence (App. C.3)
+  int whole;     // heads whose number chooses between kernels that round differently: BH, or those of the call that this is a part of
 };
 
 static int validate_shape(int batch, int heads, int N, int d, int b, int T, int dtype, Problem* p) {
@@ -45,7 +46,7 @@ static int validate_shape(int batch, int heads, int N, int d, int b, int T, int 
   if (batch <= 0 || heads <= 0 || N <= 0 || d <= 0 || b <= 0 || T < 1) return MA_ERR_SHAPE;
   if (N % b != 0) return MA_ERR_SHAPE;
   if ((long long)batch * heads > 0x7fffffffLL / 2) return MA_ERR_SHAPE;
-  *p = Problem{batch, heads, N, d, b, T, dtype, N / b, batch * heads, N, 0, nullptr, nullptr};
+  *p = Problem{batch, heads, N, d, b, T, dtype, N / b, batch * heads, N, 0, nullptr, nullptr, batch * heads};
   return MA_OK;
 }
 
@@ -196,7 +197,7 @@ static int resolve_path(const Problem& p, int path, bool plain = true) {
     if (p.b <= 32 && fsmall::supported(p.N, p.d, p.b, p.m, p.dtype, p.T)) return MA_PATH_FUSED_SMALL;
     if (tile::supported(p.N, p.d, p.b, p.m, p.dtype, p.BH)) return MA_PATH_TILE_MMA;
     // fp32 inputs: short sequences in one launch with the states in shared memory
-    if (p.dtype == MA_F32 && p.BH <= 65535 && ffused::chosen(p.N, p.d, p.b, p.m, p.BH, kSmsB200)) return MA_PATH_FUSED_F32;
+    if (p.dtype == MA_F32 && p.BH <= 65535 && ffused::chosen(p.N, p.d, p.b, p.m, p.whole, kSmsB200)) return MA_PATH_FUSED_F32;
     if (generic_supported(p)) return MA_PATH_GENERIC;
     return f32_in_one_launch(p) ? MA_PATH_FUSED_F32 : -1;
   }
@@ -305,7 +306,7 @@ static bool touches_workspace(int resolved) {
 // 60 x 32 18.1 / 15.6; in bf16, which these tiles convert first, 20 of 60 x 32 15.5 / 16.5, 30 of 40 x 32 16.5 / 17.3: from 448 on.
 static bool tiles_on_tensor_cores(const Problem& p, float scale) {
   if (p.T > 2 || !(scale >= 0.f) || !ttc::supported(p.N, p.d, p.b, p.m, p.dtype, p.BH)) return false;
-  const long long tiles = (long long)p.BH * p.N / 128;
+  const long long tiles = (long long)p.whole * p.N / 128;
   auto per_tile = [](int rows) { return rows <= 32 ? 4 : (rows <= 64 ? 2 : 1); };
   const int pr = per_tile(p.b), pl = per_tile(p.m);
   const int taken = (p.m + pr - 1) / pr + (p.b + pl - 1) / pl;
@@ -365,7 +366,7 @@ static int launch_resolved(const void* Q, const void* K, const void* V, void* Y,
   } else {
     rc = tp::launch(Q, K, V, Y, p.BH, p.N, p.b, p.T, p.dtype, scale, ws, st, &launches,
                     resolved == MA_PATH_TENSOR_TMEM ? 1 : 0,
-                    ws_armed, status.report, &kernels, p.H, p.lse, p.n_valid < p.N ? p.n_valid : 0);
+                    ws_armed, status.report, &kernels, p.H, p.lse, p.n_valid < p.N ? p.n_valid : 0, p.whole);
   }
   if (rc == MA_OK) {
     g_last_launches = launches;
@@ -432,6 +433,7 @@ static int run_call(const Call& c) {
   Problem p;
   int rc = validate_shape(c.batch, c.heads, c.N, c.d, c.b, c.T, c.dtype, &p);
   if (rc != MA_OK) return rc;
+  if (c.whole > 0) p.whole = c.whole;
   // less than one block of padding: every key block keeps at least one valid key
   if (c.entry == Entry::kPadded && (c.n_valid > c.N || c.n_valid <= c.N - c.b)) return MA_ERR_SHAPE;
   rc = check_ptrs(c.Q, c.K, c.V, c.Y, p);
@@ -509,7 +511,7 @@ static bool pinned_range(const void* host, hostcall::Pinned* r) {
 struct HostOps {
   DeviceBuffers& B;
   cudaStream_t caller, compute, back;
-  int N, d, b, T, dtype;
+  int N, d, b, T, dtype, heads;
   int launches;
   static int status(cudaError_t e) { return e == cudaSuccess ? MA_OK : MA_ERR_CUDA; }
   static int order(cudaStream_t later, cudaStream_t earlier, cudaEvent_t ev) {
@@ -524,7 +526,7 @@ struct HostOps {
   int join_back() { return order(caller, back, B.all_back); }
   int forward(const void* Q, const void* K, const void* V, void* Y, int units) {
     const int rc = run_call(Call{Entry::kFwd, Q, K, V, Y, 1, units, N, d, b, T, dtype, 0.f, MA_PATH_AUTO, 0, nullptr, nullptr,
-                                 nullptr, 0, compute, nullptr, nullptr});
+                                 nullptr, 0, compute, nullptr, nullptr, heads});
     launches += rc == MA_OK ? g_last_launches : 0;
     return rc;
   }
@@ -551,14 +553,14 @@ int monarch_attn_fwd_ex(const void* Q, const void* K, const void* V, void* Y, in
                         int N, int d, int b, int T, int dtype, float softmax_scale, int path,
                         void* workspace, size_t workspace_bytes, void* stream) {
   return run_call(Call{Entry::kEx, Q, K, V, Y, batch, heads, N, d, b, T, dtype, softmax_scale, path, 0, nullptr,
-                       nullptr, workspace, workspace_bytes, stream, nullptr, nullptr});
+                       nullptr, workspace, workspace_bytes, stream, nullptr, nullptr, 0});
 }
 
 int monarch_attn_fwd_padded(const void* Q, const void* K, const void* V, void* Y, int batch,
                             int heads, int N, int d, int b, int T, int dtype, float softmax_scale,
                             int n_valid, void* workspace, size_t workspace_bytes, void* stream) {
   return run_call(Call{Entry::kPadded, Q, K, V, Y, batch, heads, N, d, b, T, dtype, softmax_scale, MA_PATH_AUTO,
-                       n_valid, nullptr, nullptr, workspace, workspace_bytes, stream, nullptr, nullptr});
+                       n_valid, nullptr, nullptr, workspace, workspace_bytes, stream, nullptr, nullptr, 0});
 }
 
 int monarch_attn_fwd_varlen(const void* Q, const void* K, const void* V, void* Y, int batch,
@@ -566,7 +568,7 @@ int monarch_attn_fwd_varlen(const void* Q, const void* K, const void* V, void* Y
                             const int* seq_len, void* workspace, size_t workspace_bytes,
                             void* stream) {
   return run_call(Call{Entry::kVarlen, Q, K, V, Y, batch, heads, N, d, b, T, dtype, softmax_scale, MA_PATH_AUTO, 0,
-                       seq_len, nullptr, workspace, workspace_bytes, stream, nullptr, nullptr});
+                       seq_len, nullptr, workspace, workspace_bytes, stream, nullptr, nullptr, 0});
 }
 
 int monarch_attn_fwd_objective(const void* Q, const void* K, const void* V, void* Y, int batch,
@@ -574,20 +576,20 @@ int monarch_attn_fwd_objective(const void* Q, const void* K, const void* V, void
                                float softmax_scale, int path, float* row_lse, void* workspace,
                                size_t workspace_bytes, void* stream) {
   return run_call(Call{Entry::kObjective, Q, K, V, Y, batch, heads, N, d, b, T, dtype, softmax_scale, path, 0,
-                       nullptr, row_lse, workspace, workspace_bytes, stream, nullptr, nullptr});
+                       nullptr, row_lse, workspace, workspace_bytes, stream, nullptr, nullptr, 0});
 }
 
 int monarch_attn_fwd_bshd(const void* Q, const void* K, const void* V, void* Y, int batch, int N,
                           int heads, int d, int b, int T, int dtype, float softmax_scale, int path,
                           void* workspace, size_t workspace_bytes, void* stream) {
   return run_call(Call{Entry::kBshd, Q, K, V, Y, batch, heads, N, d, b, T, dtype, softmax_scale, path, 0, nullptr,
-                       nullptr, workspace, workspace_bytes, stream, nullptr, nullptr});
+                       nullptr, workspace, workspace_bytes, stream, nullptr, nullptr, 0});
 }
 
 int monarch_attn_fwd(const void* Q, const void* K, const void* V, void* Y, int batch, int heads,
                      int N, int d, int b, int T, int dtype, void* stream) {
   return run_call(Call{Entry::kFwd, Q, K, V, Y, batch, heads, N, d, b, T, dtype, 0.f, MA_PATH_AUTO, 0, nullptr,
-                       nullptr, nullptr, 0, stream, nullptr, nullptr});
+                       nullptr, nullptr, 0, stream, nullptr, nullptr, 0});
 }
 
 int monarch_attn_fwd_host(const void* Qh, const void* Kh, const void* Vh, void* Yh, int batch,
@@ -633,7 +635,7 @@ int monarch_attn_fwd_host(const void* Qh, const void* Kh, const void* Vh, void* 
   const size_t bytes = (size_t)p.BH * unit;
   const int want = g_host_chunks > 0 ? g_host_chunks : (direct && bytes < ((size_t)4 << 20) ? 1 : (direct && bytes < ((size_t)14 << 20) ? 2 : 3));
   const int chunks = (unit % 16 == 0 && p.BH >= want) ? want : 1;
-  HostOps ops{B, st, chunks > 1 ? B.compute : st, chunks > 1 ? B.d2h : st, N, d, b, T, dtype, 0};
+  HostOps ops{B, st, chunks > 1 ? B.compute : st, chunks > 1 ? B.d2h : st, N, d, b, T, dtype, p.BH, 0};
   rc = hostcall::run({(const char*)Qh, (const char*)Kh, (const char*)Vh, (char*)Yh, (char*)B.stage, direct, one, unit}, p.BH,
                      chunks, ops);
   if (rc == MA_OK) g_last_launches = ops.launches;

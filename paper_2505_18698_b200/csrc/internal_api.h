@@ -24,6 +24,7 @@ struct Call {
   void* stream;
   void* (*alloc)(void* ctx, size_t bytes);
   void* ctx;
+  int whole;            // heads of the call that this one is a part of, whose kernels it then takes; 0: it is no part
 };
 
 }  // namespace ma

@@ -207,10 +207,11 @@ inline bool chain_chosen(int BH, int N, int b) {      // by tiles of a half-step
 }
 
 // mode 0: kernel of tensor_decoupled.cuh or tensor_chain.cuh; mode 1: kernel of tensor_tmem.cuh (m = b in {64, 128},
-// plain calls only: no [batch][N][heads][d] layout, no row log-sum-exp, no padding mask).  *kernels: which it was.
+// plain calls only: no [batch][N][heads][d] layout, no row log-sum-exp, no padding mask).  *kernels: which it was.  whole:
+// heads whose number chooses between the kernels of mode 0, BH of them or more.
 int launch(const void* Q, const void* K, const void* V, void* Y, int BH, int N, int b, int T,
            int dtype, float scale, void* ws, cudaStream_t st, int* launches, int mode,
-           bool ws_armed, int* report, const char** kernels, int H = 0, float* lse = nullptr, int n_valid = 0);
+           bool ws_armed, int* report, const char** kernels, int H, float* lse, int n_valid, int whole);
 inline bool tmem_kernel_supported(int b, int H, const float* lse, int n_valid) {
   return (b == 64 || b == 128) && H == 0 && lse == nullptr && n_valid == 0;
 }
@@ -287,7 +288,7 @@ inline PersistentChain& persistent_chain() {
 template <typename T, int B, int SB>
 inline int launch_t(const void* Q, const void* K, const void* V, void* Y, int BH, int N, int T_steps,
                     int dtype, float scale, void* ws, cudaStream_t st, int* launches, int mode,
-                    bool ws_armed, int* report, const char** kernels, int H, float* lse, int n_valid) {
+                    bool ws_armed, int* report, const char** kernels, int H, float* lse, int n_valid, int whole) {
   if (mode == 1 && (SB != B || !tmem_kernel_supported(SB, H, lse, n_valid))) return 4;
   // the padding mask only where a tile row owns a whole key block
   if (n_valid != 0 && SB != B) return 4;
@@ -342,7 +343,7 @@ inline int launch_t(const void* Q, const void* K, const void* V, void* Y, int BH
   // same time and 118 MB instead of 217 MB of DRAM traffic; C4, 1024 tiles of two 64 x 64 blocks,
   // 3 % slower, hence the higher bar for the faster small tiles; monarch_chain has 1184 tiles in work or requested: 16 heads of
   // 16384 take it 104 us in groups of 1024, 95 in one, 24 149 in one, 141 in two of 1536)
-  const bool chained = mode == 0 && P.trace == nullptr && chain_chosen(BH, N, SB);
+  const bool chained = mode == 0 && P.trace == nullptr && chain_chosen(whole, N, SB);
   const int min_tiles = B == 128 ? (chained ? 1536 : 1024) : 2048;
   P.head_groups = 1;
   while (BH % (2 * P.head_groups) == 0 && P.tiles_per_phase / (2 * P.head_groups) >= min_tiles) P.head_groups *= 2;
@@ -381,8 +382,8 @@ inline int launch_t(const void* Q, const void* K, const void* V, void* Y, int BH
 
 int launch(const void* Q, const void* K, const void* V, void* Y, int BH, int N, int b, int T,
            int dtype, float scale, void* ws, cudaStream_t st, int* launches, int mode,
-           bool ws_armed, int* report, const char** kernels, int H, float* lse, int n_valid) {
-#define MA_TP_ARGS Q, K, V, Y, BH, N, T, dtype, scale, ws, st, launches, mode, ws_armed, report, kernels, H, lse, n_valid
+           bool ws_armed, int* report, const char** kernels, int H, float* lse, int n_valid, int whole) {
+#define MA_TP_ARGS Q, K, V, Y, BH, N, T, dtype, scale, ws, st, launches, mode, ws_armed, report, kernels, H, lse, n_valid, whole
   if (dtype == 1) {
     if (b == 128) return launch_t<__half, 128, 128>(MA_TP_ARGS);
     if (b == 64) return launch_t<__half, 64, 64>(MA_TP_ARGS);
