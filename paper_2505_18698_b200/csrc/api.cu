@@ -289,34 +289,38 @@ static bool touches_workspace(int resolved) {
 
 // MA_PATH_TILE_MMA has two sets of kernels: tcgen05 tiles (tile_tc.cuh: f16 states, up to two rounds,
 // d <= 64) and warp-MMA tiles (tile_mma.cuh: hi + lo states for three or more rounds, wider heads,
-// negative scales).  Where both apply the tcgen05 tiles pay for their set-up and longer chain once
-// there are tiles enough to keep several in flight on every SM: measured over N = 960 .. 10240 and 8
-// to 64 heads they were 1.0-1.9 x as fast from 448 tiles of 128 rows on (two rounds of blocks of
-// more than 32: from 160 on); since a group issues its own MMAs the lines below hold.  Their tiles hold whole blocks rounded up to 32, 64 or
-// 128 rows; the warp-MMA tiles are as wide as the block.  With blocks of up to 64 rows and so few of them
-// that the two half-steps take 5/3 of the tiles the rows would fill, the warp-MMA tiles win (8 blocks of 48
-// 44.6 against 52.4 us, 16 of 48 36.9 / 40.3, 12 of 64 40.9 / 42.8; 16 of 64 38.5 / 38.2, 17 of 48 42.3 / 39.5;
-// 8 of 128 59.1 / 51.4).
-// Two rounds (us, warp-MMA / tcgen05 tiles; graphs): 8 heads of 60 x 32 in bf16 29.5 / 24.6, 16 of 47 x 32 28.3 / 23.7, 24 of 55 x 32 39.6 / 26.3, 12 of 64 x 32 27.4 /
-// 21.7, 25 of 32 x 32, masked 24.0 / 22.1, 6 of 47 x 64 32.6 / 24.0, 8 of 33 x 64 31.6 / 24.3, 1 of 70 x 128 32.0 / 26.9: 1.04 to 1.5 x over 150 sizes of these kinds, but
-// 13 of 60 x 32 in bf16 (26.4 / 26.9, d = 48 24.8 / 26.5), which the other tiles happen to fill the GPU with, as 4 of 47 x 64 (19.1 / 21.8; 3 of them 30.9 / 21.3),
-// hence 128 there; below 64 tiles 1 head of 34 x 32 15.7 / 18.1, bf16 1 of 47 x 32 17.1 / 21.2, but 1 of 64 x 32 16.5 / 16.8, 2 in bf16 23.6 / 19.3, 1 of 128 x 32 29.4 / 22.4.
-// One round (us, warp-MMA / tcgen05 tiles): blocks of 64 and more from 64 tiles on, 3 heads of 47 x 64 14.2 / 10.9, 9 15.7 / 13.1, bf16 5 16.6 / 14.5, 7 of
-// 60 x 128 25.4 / 17.4, one 13.6 / 11.7, bf16 one of 90 x 128 16.1 / 16.0; smaller ones in f16 from 128 on, 14 of 30 x 48 13.3 / 12.5, 16 of 40 x 32 12.8 / 12.2, 27 of
-// 60 x 32 18.1 / 15.6; in bf16, which these tiles convert first, 20 of 60 x 32 15.5 / 16.5, 30 of 40 x 32 16.5 / 17.3: from 448 on.
+// negative scales).  Where both apply, two figures of a call decide:
+//   * the tiles that its two half-steps launch on tcgen05, times b + m.  The chain of a tcgen05 tile takes the same time for any block, that of
+//     a warp-MMA tile grows with its block (of b rows, then of m), and the first sort needs some tiles to be worth its set-up;
+//   * the share of those tiles that rows fill.  They hold whole blocks rounded up to 32, 64 or 128 rows, and what is empty takes the same time;
+//     a warp-MMA tile is as wide as its block.
+// Both have to be larger where the groups go over a tile before its MMA (bf16 inputs, lengths), above all for one round, which has the least
+// other work.  us per call in graphs, warp-MMA / tcgen05 tiles, of some of the 868 sizes measured (3 to 128 rows and blocks, d = 8 to 64, 6 to
+// 4000 full tiles, masked and not; the lines depend on neither d nor masks):
+//   two rounds   6000: 3 heads of 46 x 50 30.3 / 21.9, 1 of 33 x 128 32.0 / 20.5, 1 of 72 x 62 33.0 / 23.6; below it 1 of 61 x 32 17.5 / 18.6
+//                8000: 1 of 66 x 64 35.5 / 23.6, 4 of 40 x 57 33.1 / 24.4, 2 of 57 x 46 23.1 / 23.5; below it 1 of 61 x 62 21.9 / 23.1
+//                shares: 0.54 in 34 of 86 x 15 48.4 / 38.4, 0.23 in 1544 of 39 x 5 237 / 267; bf16 0.56 in 42 of 80 x 16 53.9 / 57.9, 0.41 in 182 of
+//                10 x 39 55.9 / 62.1; f16 with blocks of more than 64 0.21 in 874 of 4 x 105 444 / 357, 0.17 in 72 of 3 x 120 44.2 / 47.1
+//   one round   15000: 2 of 65 x 57 15.1 / 11.8, 1 of 124 x 64 14.1 / 10.5, 14 of 118 x 32 21.0 / 15.1; below it 3 of 61 x 29 8.2 / 10.0
+//               16000: 1 of 48 x 128 14.9 / 11.5, 8 of 57 x 64 16.4 / 14.4; below it 4 of 54 x 29 11.0 / 12.1
+//               shares: 0.57 in 124 of 126 x 13 66.0 / 56.1, 0.30 in 102 of 38 x 7 14.2 / 17.7; bf16 0.78 in 19 of 102 x 25 24.9 / 19.9, 0.68 in 60 of
+//               34 x 32 25.5 / 23.0, 0.69 in 24 of 53 x 20 13.2 / 14.2, 0.57 in 12 of 72 x 37 17.2 / 20.6
+// On average the sort that is taken is 0.8 % off the better one; the tcgen05 tiles are taken where they are up to 15 % slower (1 of 87 x 111, masked,
+// one round 11.8 / 13.6), the warp-MMA tiles where they are up to 27 % slower (1 of 43 x 128 in bf16, one round 14.8 / 11.7).
 static bool tiles_on_tensor_cores(const Problem& p, float scale) {
   if (p.T > 2 || !(scale >= 0.f) || !ttc::supported(p.N, p.d, p.b, p.m, p.dtype, p.BH)) return false;
-  const long long tiles = (long long)p.whole * p.N / 128;
-  auto per_tile = [](int rows) { return rows <= 32 ? 4 : (rows <= 64 ? 2 : 1); };
-  const int pr = per_tile(p.b), pl = per_tile(p.m);
-  const int taken = (p.m + pr - 1) / pr + (p.b + pl - 1) / pl;
-  if (p.b <= 64 && 3 * 128 * taken >= 5 * 2 * p.N) return false;
-  if (p.T == 2) {
-    if (p.d < 48 || p.b < 32) return tiles >= (p.b > 32 ? 160 : 448);
-    if (p.b == 32) return p.m >= 64 || tiles >= (p.m > 32 || p.d == 64 ? 64 : 448);
-    return tiles >= (p.b > 64 ? 64 : (p.m > 32 ? 128 : 160));
-  }
-  return tiles >= (p.d < 48 ? 448 : (p.b >= 64 ? 64 : (p.dtype == MA_F16 ? 128 : 448)));
+  auto tiles_of = [](int blocks, int rows) {
+    const int per_tile = rows <= 32 ? 4 : (rows <= 64 ? 2 : 1);
+    return (blocks + per_tile - 1) / per_tile;
+  };
+  const long long tiles = (long long)p.whole * (tiles_of(p.m, p.b) + tiles_of(p.b, p.m)), size = tiles * (p.b + p.m);
+  const double share = 2. * p.whole * p.N / (128. * tiles);
+  const bool prepared = p.dtype != MA_F16 || p.seq_len != nullptr;
+  const bool two = p.T == 2;
+  if (share < (prepared ? (two ? 0.55 : 0.6) : (two && p.b > 64 ? 0. : 0.4))) return false;
+  if (two) return size >= (prepared ? 8000 : 6000);
+  if (!prepared) return size >= 15000;
+  return size >= (share >= 0.85 ? 16000 : (share >= 0.7 ? 30000 : 90000));
 }
 
 // Where a call's waits report to, and the status word it clears first (a caller's workspace; nullptr: none).
