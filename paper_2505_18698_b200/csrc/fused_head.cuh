@@ -637,21 +637,24 @@ inline bool get_maps(Params* P, const Args& a, const Plan& p, int dev) {
 }
 template <typename TIn, int NB, int NM, int ROUNDS, int WARPS = max_warps(NB, NM, ROUNDS), int RT = (NB + 1) / 2>
 inline int launch_k(const Params& P, const Plan& p, int num_sms, cudaStream_t st) {
-  auto kern = monarch_fused_head<TIn, NB, NM, ROUNDS, WARPS, RT>;
-  static warpmma::SmemOptIn opt_in;
-  if (!opt_in.done((const void*)kern, (int)kMaxSmem)) return 7;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  const int slots = p.ctas * num_sms, parts = p.parts * P.BH;
-  cfg.gridDim = dim3(parts < slots ? parts : slots);
-  cfg.blockDim = dim3(32 * p.warps);
-  cfg.dynamicSmemBytes = p.smem;
-  cfg.stream = st;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, P) == cudaSuccess ? 0 : 7;
+  if constexpr (!any_fits(NB, NM)) return 4;
+  else {
+    auto kern = monarch_fused_head<TIn, NB, NM, ROUNDS, WARPS, RT>;
+    static warpmma::SmemOptIn opt_in;
+    if (!opt_in.done((const void*)kern, (int)kMaxSmem)) return 7;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    const int slots = p.ctas * num_sms, parts = p.parts * P.BH;
+    cfg.gridDim = dim3(parts < slots ? parts : slots);
+    cfg.blockDim = dim3(32 * p.warps);
+    cfg.dynamicSmemBytes = p.smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, P) == cudaSuccess ? 0 : 7;
+  }
 }
 template <typename TIn, int ROUNDS>
 inline int launch_n(const Params& P, const Plan& p, int num_sms, cudaStream_t st) {

@@ -36,6 +36,9 @@ inline size_t smem_bytes(int tile, int bufs, int rounds, int b, int nm) {
   return (size_t)tile * (rounds == kMoreVLast ? 3 : 3 * bufs + (rounds == kMore ? 1 : 0)) + 128 + (size_t)b * nm * 8 * 4 + sizeof(Bars) + 1024;
 }
 
+// Whether any head of nb and nm 8-column tiles has a plan: Q, K and V of the smallest, 8 nb - 7 rows and 8 nm - 7 blocks, fit a CTA.  (25 x 25 does not.)
+constexpr bool any_fits(int nb, int nm) { return (size_t)3 * (8 * nb - 7) * (8 * nm - 7) * 128 <= kMaxSmem; }
+
 struct Plan {
   int bp, tile, bufs, warps, ctas, rounds, bound;      // ctas: per SM; bound: warps an SM that the kernel is compiled for
   int parts;      // CTAs a head goes to
