@@ -5,9 +5,8 @@
 // kernel is how many chains an SM has in flight and what the states cost on their way through L2.  So, against the one chain with
 // a stage per warpgroup of tensor_decoupled.cuh:
 //   * two CTAs per SM with two compute groups of four warps each; a group (thread = score row) takes a tile from its scores
-//     to its staged rows, and its first warp issues the tile's MMAs itself.  That warp alone looks at mbarriers, which means trying again
-//     and again; the others and the store warp wait in hardware barriers (64 heads of 4096, T = 2: 77.8 us with every warp
-//     at the mbarriers, 76.7 with one; trying in a tighter loop, a quarter more branches in all, cost 4 %).  Issuing a tile's eight score MMAs took
+//     to its staged rows, and its first warp issues the tile's MMAs itself (hand-overs: tile_group.cuh; trying at mbarriers in a tighter loop, a
+//     quarter more branches in all, cost 4 %).  Issuing a tile's eight score MMAs took
 //     a thread about 1000 cycles and a release 500 (clock stamps) while the warp's number came from threadIdx and the release's word
 //     went through shared memory: 74.0 us, 70.7 with uniform descriptors and a vote in the barrier;
 //   * three 16 KB slots a group.  Which of them a tile's operands take follows from the order in which the tile before gives
@@ -28,12 +27,13 @@
 #include <type_traits>
 
 #include "tensor_persistent.cuh"
+#include "tile_group.cuh"
 #include "tile_tc.cuh"
 
 namespace ma {
 namespace tp3 {
 
-using namespace ma::tensor;
+using namespace ma::group;
 using ma::tp::Params;
 using ma::tp::Tile;
 using ma::tp::bulk_load_1d;
@@ -67,92 +67,7 @@ struct __align__(16) Shared {
 static_assert(sizeof(Shared) <= 512, "barrier block");
 enum Rows { kAlphaL = 0, kY = 1, kAlphaR = 2, kOut = 3 };
 
-// A group's slots as the operands of its current tile; next(): in the order in which the tile gives them up.
-//   R:            first  alpha_R (Q), free after the score MMA; second K, alpha_L staged over it; third, last round, V and y over it
-//   L, not last:  first  Q(.,j), alpha_R staged over it; second alpha_L, then weights, free after the apply MMA (128 columns: and third)
-//   L, last:      first  Q(.,j), second alpha_L, both free after the score MMA; third y, Y staged over it
-template <int B>
-struct Slots {
-  int x0, x1, x2;
-  __device__ __forceinline__ explicit Slots(int w) : x0(3 * w), x1(3 * w + 1), x2(3 * w + 2) {}
-  __device__ __forceinline__ static bool uses_third(const Tile& t) { return t.isR ? t.withV : t.final_; }
-  __device__ __forceinline__ void next(const Tile& t) {
-    const int a = x0, b = x1, c = x2;
-    if (uses_third(t)) return;
-    if (B == 128 && !t.isR) {
-      x0 = b;
-      x1 = c;
-      x2 = a;
-      return;
-    }
-    x0 = c;
-    x1 = t.isR ? a : b;
-    x2 = t.isR ? b : a;
-  }
-};
-
-// Bounded wait: after a timeout (status word and abort flag set) every wait of the CTA returns at once (HEED: but for those that
-// come to an end by themselves).
-template <bool HEED = true>
-__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Shared* sh, const Params& P, int where) {
-  const uint32_t addr = smem_u32(bar);
-  long long t0 = 0;
-  for (int n = 0;; ++n) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(addr), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (HEED && sh->abort_flag) return false;
-    if (n == 0) {
-      t0 = clock64();
-    } else if (clock64() - t0 > P.wait_cycles) {
-      report_timeout(P.report, where);
-      sh->abort_flag = 1;
-      return false;
-    }
-  }
-}
-
-// Barriers in hardware, by group: the first warp lets the others go on, it waits for them, the store warp waits for staged
-// rows.
-__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-__device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-// The same with a vote: whether it is true for all of them.
-__device__ __forceinline__ bool bar_all(int id, int n, bool on) {
-  uint32_t all;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %3, 0;\n\tbarrier.cta.red.and.pred q, %1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
-      : "=r"(all)
-      : "r"(id), "r"(n), "r"((uint32_t)on)
-      : "memory");
-  return all != 0;
-}
-enum BarId { kRelease = 1, kCollect = 3, kStaged = 5 };
-// Tiles that a group is through with: its first warp says so once all warps have come by, the producer waits for it (bounded).
-__device__ __forceinline__ void say_through(Shared* sh, int w, uint32_t tiles) {
-  __threadfence_block();
-  *(volatile int*)&sh->through[w] = (int)tiles;
-}
-__device__ __forceinline__ bool wait_through(Shared* sh, int w, uint32_t tiles, const Params& P) {
-  const long long t0 = clock64();
-  while (*(volatile int*)&sh->through[w] < (int)tiles) {
-    if (sh->abort_flag) return false;
-    if (clock64() - t0 > P.wait_cycles) {
-      report_timeout(P.report, 12);
-      sh->abort_flag = 1;
-      return false;
-    }
-    __nanosleep(100);
-  }
-  __threadfence_block();
-  return true;
-}
-
+__device__ __forceinline__ bool uses_third(const Tile& t) { return t.isR ? t.withV : t.final_; }      // a half-step of the last round
 // Tile p, h, idx0 as its roles see it.
 __device__ __forceinline__ Tile tile_of(const Params& P, int p, int h, int idx0) {
   Tile t;
@@ -194,8 +109,7 @@ struct Chain {
     for (uint32_t q = 0;; ++q) {
       const int g = P.g_begin + claim;
       uint64_t *bar = &sh->full[w][q & 1], *bar3 = &sh->third[w][q & 1];
-      // The end: once all threads are through all tiles, the word and the barrier are free.  (A count: by the parity of a barrier a
-      // producer that comes late cannot tell the last tile from the one before the last but one.)
+      // The end: once all threads are through all tiles, the word and the barrier are free.
       if (g >= P.g_end) {
         if (!wait_through(sh, w, q, P)) return;
         sh->tile[w][q & 1] = make_int4(-1, 0, 0, 0);
@@ -263,7 +177,7 @@ struct Chain {
           mbar_arrive(bar3);
         }
       }
-      x.next(t);
+      x.next(t.isR, uses_third(t));
     }
   }
 
@@ -338,55 +252,18 @@ struct Chain {
     const int m = P.m;
     constexpr int NC = B / 16;
     Slots<B> x(w);
-    uint32_t par_o = 1, par_1 = 0;
+    uint32_t par_1 = 0;
     uint32_t par_3 = 0;                        // bit i: parity of third[w][i]
-    bool ok = true;                            // (the first warp's decides) no wait has run out
-    // The first warp alone looks at mbarriers and lets the others go on once it has seen one: four warps that try and try again take
-    // issue slots from those at work.  A wait that ran out reaches the others with the same release.
-    auto await = [&](uint64_t* bar, uint32_t parity, int where) { ok = __all_sync(0xffffffffu, wait_bar(bar, parity, sh, P, where)) && ok; };
-    auto release = [&](bool on) {              // of the group; false: no more tiles
-      tc_fence_before();
-      const bool go = bar_all(kRelease + w, 128, on);
-      tc_fence_after();
-      return go;
-    };
-    auto collect = [&]() {                     // all warps have come by: the first one waits
-      tc_fence_before();
-      if (warp == 0) {
-        bar_sync(kCollect + w, 128);
-        tc_fence_after();
-      } else {
-        bar_arrive(kCollect + w, 128);
-      }
-    };
-    // An accumulator is done, and the store warp has taken the word of the rows before: nobody comes by at kStaged a second time
-    // before the store warp has.
-    auto await_rows = [&](uint64_t* bar, uint32_t parity, int where) {
-      if (warp == 0) {
-        await(bar, parity, where);
-        if (ok) await(&sh->out_free[w], par_o, 38);
-        if (ok) par_o ^= 1;
-      }
-      return release(ok);
-    };
-    auto hand_over = [&](int h, int idx0, int what, int p) {
-      if (t_row == 0) sh->out[w] = make_int4(h, idx0, what, p);
-      __syncwarp();
-      bar_arrive(kStaged + w, 160);
-    };
+    Group<Shared, Params> group(sh, P, w, warp, t_row);
     for (uint32_t q = 0;; ++q) {
       const uint32_t par = q & 1;
       const uint32_t a0 = sm + x.x0 * kSlot, a1 = sm + x.x1 * kSlot, a2 = sm + x.x2 * kSlot;
       bool more = true;
       if (warp == 0) {
-        if (q > 0) {                           // every row of the tile before has left tensor memory
-          bar_sync(kCollect + w, 128);
-          tc_fence_after();
-          if (t_row == 0) say_through(sh, w, q);
-        }
-        await(&sh->full[w][q & 1], (q >> 1) & 1, 30);
+        group.begin(q);
+        group.await(&sh->full[w][q & 1], (q >> 1) & 1, 30);
         const int4 it = sh->tile[w][q & 1];
-        more = ok && it.x >= 0;
+        more = group.ok && it.x >= 0;
         if (more) {
           const Tile t = tile_of(P, it.x, it.y, it.z);
           if (elect_one()) {
@@ -396,11 +273,11 @@ struct Chain {
             if (t.final_) umma_commit(&sh->empty[x.x1]);
           }
           __syncwarp();
-          await(&sh->mma1[w], par, 31);
-          more = ok;
+          group.await(&sh->mma1[w], par, 31);
+          more = group.ok;
         }
       }
-      if (!release(more)) break;
+      if (!group.release(more)) break;
       const int4 it = sh->tile[w][q & 1];
       const Tile t = tile_of(P, it.x, it.y, it.z);
       // the state rows the score MMA consumed are read exactly once: drop them from L2
@@ -521,7 +398,7 @@ struct Chain {
           // the contraction runs over the rows of the weights: normalised in fp32, rounded once, to shared memory
           const float2 n2 = both(mul * kWeightScale);
           // (128 columns: the slot of the second half is free; every warp looks for itself)
-          if (B == 128) await(&sh->third[w][q & 1], (par_3 >> (q & 1)) & 1, 36);
+          if (B == 128) group.await(&sh->third[w][q & 1], (par_3 >> (q & 1)) & 1, 36);
           uint8_t* lower = smem + (B == 128 ? min(x.x1, x.x2) : x.x1) * kSlot + srow * 128;
           uint8_t* upper = smem + max(x.x1, x.x2) * kSlot + srow * 128;
           tmem_ld16(tS, c[0]);
@@ -544,11 +421,11 @@ struct Chain {
           fence_proxy_async();
         }
       }
-      collect();
-      const bool third = Slots<B>::uses_third(t) || (B == 128 && !t.isR);
+      group.collect();
+      const bool third = uses_third(t) || (B == 128 && !t.isR);
       if (warp == 0) {
-        if (t.final_) await(&sh->third[w][q & 1], (par_3 >> (q & 1)) & 1, 36);
-        if (ok && elect_one()) {
+        if (t.final_) group.await(&sh->third[w][q & 1], (par_3 >> (q & 1)) & 1, 36);
+        if (group.ok && elect_one()) {
           if (t.isR) {
             apply(d, a1);
             umma_commit(t.withV ? &sh->first[w] : &sh->mma2[w]);
@@ -569,15 +446,15 @@ struct Chain {
       // ============================================================== rows
       float o[64];
       if (t.isR && t.withV) {                  // alpha_L, over K; then y = R V through the same columns, over V
-        if (!await_rows(&sh->first[w], par_1, 32)) break;
+        if (!group.await_rows(&sh->first[w], par_1, 32)) break;
         par_1 ^= 1;
         tmem_ld32(tS + 64, o);
         tmem_ld32(tS + 96, o + 32);
         tmem_ld_wait();
-        collect();
+        group.collect();
         if (warp == 0) {
-          await(&sh->third[w][q & 1], (par_3 >> (q & 1)) & 1, 36);
-          if (ok && elect_one()) {
+          group.await(&sh->third[w][q & 1], (par_3 >> (q & 1)) & 1, 36);
+          if (group.ok && elect_one()) {
             apply(d, a2);
             umma_commit(&sh->mma2[w]);
           }
@@ -586,9 +463,9 @@ struct Chain {
         store_row32<T>(smem + x.x1 * kSlot, srow, 0, o, mul);
         store_row32<T>(smem + x.x1 * kSlot, srow, 32, o + 32, mul);
         fence_proxy_async();
-        hand_over(t.h, t.idx0, x.x1 | kAlphaL << 4, t.p);
+        group.hand_over(t.h, t.idx0, x.x1 | kAlphaL << 4, t.p);
       }
-      if (!await_rows(&sh->mma2[w], par, 33)) break;
+      if (!group.await_rows(&sh->mma2[w], par, 33)) break;
       if (t.final_) discard_line(P.y + ((size_t)(t.h * B + t.idx0) * m + t_row) * 128);
       const bool turned = !t.isR && !t.final_;
       float cr = 1.f;
@@ -597,21 +474,17 @@ struct Chain {
       tmem_ld32(tO, o);
       tmem_ld32(tO + 32, o + 32);
       tmem_ld_wait();
-      tc_fence_before();
-      if (warp != 0) bar_arrive(kCollect + w, 128);        // (the first warp waits for it before the next tile's scores)
+      group.leave();
       if (turned) mul = cr > 1e-30f ? 1.f / cr : 0.f;
       const int slot = t.isR ? (t.withV ? x.x2 : x.x1) : (t.final_ ? x.x2 : x.x0);
       store_row32<T>(smem + slot * kSlot, srow, 0, o, mul);
       store_row32<T>(smem + slot * kSlot, srow, 32, o + 32, mul);
       fence_proxy_async();
-      hand_over(t.h, t.idx0, slot | (t.isR ? (t.withV ? kY : kAlphaL) : (t.final_ ? kOut : kAlphaR)) << 4 | 1 << 8, t.p);
+      group.hand_over(t.h, t.idx0, slot | (t.isR ? (t.withV ? kY : kAlphaL) : (t.final_ ? kOut : kAlphaR)) << 4 | 1 << 8, t.p);
       if (third) par_3 ^= 1u << (q & 1);
-      x.next(t);
+      x.next(t.isR, uses_third(t));
     }
-    // (aborted or not: rows handed over before are on their way, and the store warp comes back for this word)
-    if (warp == 0) __all_sync(0xffffffffu, wait_bar<false>(&sh->out_free[w], par_o, sh, P, 38));
-    release(false);
-    hand_over(-1, 0, 0, 0);
+    group.finish();
   }
 };
 

@@ -34,12 +34,12 @@
 #include <type_traits>
 
 #include "status_word.cuh"
-#include "tensor_path.cuh"
+#include "tile_group.cuh"
 
 namespace ma {
 namespace ttc {
 
-using namespace ma::tensor;
+using namespace ma::group;
 
 constexpr int kThreads = 384;                // two compute groups of four warps, four service warps
 constexpr int kCtasPerSm = 2;
@@ -62,7 +62,7 @@ struct Params {
   uint8_t *aL, *aR, *y;    // state arrays, for L2 discards once a tile has been consumed (d = 64)
   float* lse;              // optional [BH][N]
   const int* seq_len;      // optional [BH / heads]
-  int* status;             // set by a wait that ran out
+  int* report;             // status word, set by a wait that ran out
   int* clear;              // status word to clear first, or nullptr
   int N, b, m, mp, BH, H, heads, n_valid;
   int first, last;         // this launch's half-step: of the first round, of the last round
@@ -84,64 +84,6 @@ struct __align__(16) Shared {
   volatile int abort_flag;
 };
 static_assert(sizeof(Shared) <= 384, "barrier block");
-
-// A group's slots as the operands of its current tile; next(): in the order in which the tile gives them up.
-//   R:            first  alpha_R (Q), free after the score MMA; second K, alpha_L staged over it; third, last round, V and y over it
-//   L, not last:  first  Q(.,j), alpha_R staged over it; second alpha_L, then weights, free after the apply MMA (128 columns: and third)
-//   L, last:      first  Q(.,j), second alpha_L, both free after the score MMA; third y, Y staged over it
-template <int B, bool R>
-struct Slots {
-  int x0, x1, x2;
-  __device__ __forceinline__ explicit Slots(int w) : x0(3 * w), x1(3 * w + 1), x2(3 * w + 2) {}
-  __device__ __forceinline__ void next(bool last) {
-    const int a = x0, b = x1, c = x2;
-    if (last) return;
-    if (B == 128 && !R) {
-      x0 = b;
-      x1 = c;
-      x2 = a;
-      return;
-    }
-    x0 = c;
-    x1 = R ? a : b;
-    x2 = R ? b : a;
-  }
-};
-
-// Barriers in hardware, by group: the first warp lets the others go on, it waits for them, the store warp waits for staged
-// rows.
-__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-__device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-// The same with a vote: whether it is true for all of them.
-__device__ __forceinline__ bool bar_all(int id, int n, bool on) {
-  uint32_t all;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %3, 0;\n\tbarrier.cta.red.and.pred q, %1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
-      : "=r"(all)
-      : "r"(id), "r"(n), "r"((uint32_t)on)
-      : "memory");
-  return all != 0;
-}
-enum BarId { kRelease = 1, kCollect = 3, kStaged = 5 };
-// Tiles that a group is through with: its first warp says so once all warps have come by, the producer waits for it (bounded).
-__device__ __forceinline__ void say_through(Shared* sh, int w, uint32_t tiles) {
-  __threadfence_block();
-  *(volatile int*)&sh->through[w] = (int)tiles;
-}
-__device__ __forceinline__ bool wait_through(Shared* sh, int w, uint32_t tiles, const Params& P) {
-  const long long t0 = clock64();
-  while (*(volatile int*)&sh->through[w] < (int)tiles) {
-    if (sh->abort_flag) return false;
-    if (clock64() - t0 > P.wait_cycles) {
-      report_timeout(P.status, 12);
-      sh->abort_flag = 1;
-      return false;
-    }
-    __nanosleep(100);
-  }
-  __threadfence_block();
-  return true;
-}
 
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -221,33 +163,6 @@ __device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64
       : "memory");
 }
 
-// Bounded wait: after a timeout (status word and abort flag set) every wait of the CTA returns at once (HEED: but for those that
-// come to an end by themselves), and its groups stop.
-template <bool HEED = true>
-__device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, Shared* sh, const Params& P, int where) {
-  const uint32_t addr = smem_u32(bar);
-  uint32_t done = 0;
-  long long t0 = 0;
-  for (int n = 0;; ++n) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(addr), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if (HEED && sh->abort_flag) return false;
-    if (n == 0) {
-      t0 = clock64();
-    } else if (clock64() - t0 > P.wait_cycles) {
-      report_timeout(P.status, where);
-      sh->abort_flag = 1;
-      return false;
-    }
-  }
-}
-
 __device__ __forceinline__ void arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
@@ -274,7 +189,7 @@ struct Kernel {
       grid_wait();
       grid_launch_dependents();
     }
-    Slots<B, R> x(w);
+    Slots<B> x(w);
     uint32_t busy = 0, par = 0;               // by slot: a use is to be waited for; parity of that wait
     auto take = [&](int s) {
       const uint32_t bit = 1u << s;
@@ -294,8 +209,7 @@ struct Kernel {
         idx0 = end ? 0 : (g - h * P.per_head) * kBlocks;
         if (!FULL && !end && P.seq_len != nullptr) n_valid = min(max(P.seq_len[h / P.heads], 1), P.N);
       } while (!FULL && R && !end && P.seq_len != nullptr && idx0 * P.b >= n_valid);      // key blocks that a shorter sequence does not have
-      // The end: once all threads are through all tiles, the word and the barrier are free.  (A count: by the parity of a barrier a
-      // producer that comes late cannot tell the last tile from the one before the last but one.)
+      // The end: once all threads are through all tiles, the word and the barrier are free.
       if (end) {
         if (!wait_through(sh, w, q, P)) return;
         sh->tile[w][q & 1] = make_int4(-1, 0, 0, 0);
@@ -341,7 +255,7 @@ struct Kernel {
         }
       }
       waited = true;
-      x.next(last);
+      x.next(R, last);
     }
   }
 
@@ -633,42 +547,8 @@ struct Kernel {
     const int row = threadIdx.x & 127, warp = warp_of_cta & 3, w = warp_of_cta >> 2, lane = threadIdx.x & 31;
     const uint32_t d = tmem + 128 * w, t_row = d + ((uint32_t)(warp * 32) << 16);     // the group's columns, this warp's lanes
     const bool prep = prepares(P), last = P.last != 0;
-    Slots<B, R> x(w);
-    uint32_t par_o = 1;
-    bool ok = true;                            // (the first warp's decides) no wait has run out
-    // The first warp alone looks at mbarriers and lets the others go on once it has seen one: four warps that try and try again take
-    // issue slots from those at work.  A wait that ran out reaches the others with the same release.
-    auto await = [&](uint64_t* bar, uint32_t parity, int where) { ok = __all_sync(0xffffffffu, wait_bar(bar, parity, sh, P, where)) && ok; };
-    auto release = [&](bool on) {              // of the group; false: no more tiles
-      tc_fence_before();
-      const bool go = bar_all(kRelease + w, 128, on);
-      tc_fence_after();
-      return go;
-    };
-    auto collect = [&]() {                     // all warps have come by: the first one waits
-      tc_fence_before();
-      if (warp == 0) {
-        bar_sync(kCollect + w, 128);
-        tc_fence_after();
-      } else {
-        bar_arrive(kCollect + w, 128);
-      }
-    };
-    // An accumulator is done, and the store warp has taken the word of the rows before: nobody comes by at kStaged a second time
-    // before the store warp has.
-    auto await_rows = [&](uint64_t* bar, uint32_t parity, int where) {
-      if (warp == 0) {
-        await(bar, parity, where);
-        if (ok) await(&sh->out_free[w], par_o, 38);
-        if (ok) par_o ^= 1;
-      }
-      return release(ok);
-    };
-    auto hand_over = [&](int h, int idx0, int slot, int is_y) {
-      if (row == 0) sh->out[w] = make_int4(h, idx0, slot, is_y);
-      __syncwarp();
-      bar_arrive(kStaged + w, 160);
-    };
+    Slots<B> x(w);
+    Group<Shared, Params> group(sh, P, w, warp, row);
     for (uint32_t q = 0;; ++q) {
       const uint32_t par = q & 1, par2 = (q >> 1) & 1;
       uint8_t *s0 = smem + x.x0 * kSlot, *s1 = smem + x.x1 * kSlot, *s2 = smem + x.x2 * kSlot;
@@ -681,33 +561,29 @@ struct Kernel {
           if (!R && last) umma_commit(&sh->empty[x.x1]);
         }
         __syncwarp();
-        await(&sh->mma1[w], par, 31);
-        if (prep && last) await(&sh->third[w][par], par2, 36);
+        group.await(&sh->mma1[w], par, 31);
+        if (prep && last) group.await(&sh->third[w][par], par2, 36);
       };
       bool more = true;
       if (warp == 0) {
-        if (q > 0) {                           // every row of the tile before has left tensor memory
-          bar_sync(kCollect + w, 128);
-          tc_fence_after();
-          if (row == 0) say_through(sh, w, q);
-        }
-        await(&sh->full[w][par], par2, 30);
-        more = ok && sh->tile[w][par].x >= 0;
+        group.begin(q);
+        group.await(&sh->full[w][par], par2, 30);
+        more = group.ok && sh->tile[w][par].x >= 0;
         if (more && !prep) {
           score();
-          more = ok;
+          more = group.ok;
         }
       }
-      if (!release(more)) break;
+      if (!group.release(more)) break;
       const int4 t = sh->tile[w][par];         // head, first block or position, keys that count
       const int h = t.x, idx0 = t.y;
       const int mv = FULL ? P.m : (t.z + P.b - 1) / P.b;                            // blocks that are present
       if (prep) {
         prepare(P, s0, !R || P.first, idx0, mv, row);      // Q, but not alpha_R
         prepare(P, s1, R, idx0, mv, row);                   // K, but not alpha_L
-        collect();
+        group.collect();
         if (warp == 0) score();
-        if (!release(ok)) break;
+        if (!group.release(group.ok)) break;
       }
       const float* sC = reinterpret_cast<const float*>(smem + kOffVec) + (2 * w + par) * 128;
       if (FULL && P.discard) {     // the state rows the score MMA consumed are read exactly once: drop them from L2
@@ -790,7 +666,7 @@ struct Kernel {
           }
           ld_frag32(tS, v);
           // (128 columns: the slot of the second half is free; every warp looks for itself)
-          if (B == 128) await(&sh->third[w][par], par2, 36);
+          if (B == 128) group.await(&sh->third[w][par], par2, 36);
           bar_sync(kRelease + w, 128);
           // (the set of the tile before: all warps are done with it, and none begins the next tile before all have come by)
           reinterpret_cast<unsigned*>(smem + kOffCol)[128 * (2 * w + (par ^ 1)) + row] = 0u;
@@ -812,10 +688,10 @@ struct Kernel {
         }
       }
       if (last && prep) prepare(P, s2, R, idx0, mv, row);   // V, but not y
-      collect();
+      group.collect();
       if (warp == 0) {
-        if (!R && last && !prep) await(&sh->third[w][par], par2, 36);
-        if (ok && elect_one()) {
+        if (!R && last && !prep) group.await(&sh->third[w][par], par2, 36);
+        if (group.ok && elect_one()) {
           if (R) {
             apply(d, s1);
             umma_commit(last ? &sh->first[w] : &sh->mma2[w]);
@@ -836,16 +712,16 @@ struct Kernel {
       // ============================================================== epilogue
       float o[32];
       if (R && last) {                           // alpha_L, over K; then y, over V
-        if (!await_rows(&sh->first[w], par, 32)) break;
+        if (!group.await_rows(&sh->first[w], par, 32)) break;
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
           tmem_ld32(t_row + 64 + 32 * hf, o);
           tmem_ld_wait();
           if (hf == 1) {
-            collect();
+            group.collect();
             if (warp == 0) {
-              if (!prep) await(&sh->third[w][par], par2, 36);
-              if (ok && elect_one()) {
+              if (!prep) group.await(&sh->third[w][par], par2, 36);
+              if (group.ok && elect_one()) {
                 apply(d, s2);
                 umma_commit(&sh->mma2[w]);
               }
@@ -855,9 +731,9 @@ struct Kernel {
           store_row32<TA>(s1, row, 32 * hf, o, mul);
         }
         fence_proxy_async();
-        hand_over(h, idx0, x.x1, 0);
+        group.hand_over(h, idx0, x.x1, 0);
       }
-      if (!await_rows(&sh->mma2[w], par, 33)) break;
+      if (!group.await_rows(&sh->mma2[w], par, 33)) break;
       int out_row = row;
       if (!R && !last) {
         if constexpr (!R && B < 128) out_row = ((lane >> 4) << 6) + 16 * warp + (lane & 15);
@@ -873,10 +749,7 @@ struct Kernel {
       for (int hf = 0; hf < 2; ++hf) {
         tmem_ld32(t_row + 64 + 32 * hf, o);
         tmem_ld_wait();
-        if (hf == 1) {                           // the next tile's scores may come (the first warp waits for it before them)
-          tc_fence_before();
-          if (warp != 0) bar_arrive(kCollect + w, 128);
-        }
+        if (hf == 1) group.leave();              // the next tile's scores may come
         if (R && last && !(mul == mul)) {      // NaN weights, and c_L is: the final L tiles hold several positions
           zero_row(dst, row);
         } else if (!R && last) {
@@ -890,13 +763,10 @@ struct Kernel {
         }
       }
       fence_proxy_async();
-      hand_over(h, idx0, slot, R && last);
-      x.next(last);
+      group.hand_over(h, idx0, slot, R && last);
+      x.next(R, last);
     }
-    // (aborted or not: rows handed over before are on their way, and the store warp comes back for this word)
-    if (warp == 0) __all_sync(0xffffffffu, wait_bar<false>(&sh->out_free[w], par_o, sh, P, 38));
-    release(false);
-    hand_over(-1, 0, 0, 0);
+    group.finish();
   }
 };
 
@@ -1114,7 +984,7 @@ inline int launch_t(const Args& a, const States& s, cudaStream_t st) {
   if (!current_device(&dev) || !cached_maps(&P, a, s, dev.dev)) return 7;
   P.cL = s.cL;
   P.aL = (uint8_t*)s.aL; P.aR = (uint8_t*)s.aR; P.y = (uint8_t*)s.y;
-  P.lse = a.lse; P.seq_len = a.seq_len; P.status = s.status; P.clear = s.clear;
+  P.lse = a.lse; P.seq_len = a.seq_len; P.report = s.status; P.clear = s.clear;
   P.N = a.N; P.b = a.b; P.m = a.m; P.mp = pad4(a.m); P.BH = a.BH; P.H = a.H; P.heads = a.heads; P.n_valid = a.n_valid;
   P.discard = a.d == 64;       // (a row is then a line)
   P.wait_cycles = a.waits.cycles;
