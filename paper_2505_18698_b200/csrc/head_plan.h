@@ -89,11 +89,15 @@ inline bool plan(int b, int m, int T, int BH, int num_sms, Plan* p) {
     if (nb == 3 && nm == 2 && rounds == kMore && p->ctas == 2) most = 24;
     // More than 16 positions and SMs enough for two CTAs a head: half of the positions each, so that a block is one 16-row tile instead of two
     // and a position has a warp to itself (us, one CTA / two: 12 heads of 16 x 24, one round 6.9 / 4.8, two 11.7 / 7.6, 36 of 19 x 22 9.0 / 6.3, 48 of 12 x 20, two
-    // rounds 10.0 / 6.8, 72 of 23 x 17 9.6 / 7.3, 24 of 14 x 30 7.6 / 5.1).
+    // rounds 10.0 / 6.8, 72 of 23 x 17 9.6 / 7.3, 24 of 14 x 30 7.6 / 5.1).  It takes more of the GPU in all: two such calls at once on two streams gain up to about a quarter
+    // of the SMs each and lose above (us for both: 12 heads of 16 x 24 6.9 / 4.8, 36 7.1 / 5.2, 60 of 10 x 18, two rounds 10.1 / 10.0, 72 of 16 x 24 7.8 / 9.6, of 20 x 20 10.0 / 12.5).
     p->parts = nb > 2 && 2 * BH <= num_sms ? 2 : 1;
     if (p->parts == 2) most = 16;
-    // A CTA an SM: so much shared memory that the next call's CTAs do not come to an SM at work (us in loops, without / with: 144 heads of 11 x 12
-    // 6.8 / 5.0, of 10 x 10 6.0 / 4.7, 108 of 10 x 10, two rounds 8.1 / 6.5, 72 of 10 x 17 5.6 / 4.6; never slower by more than 2 %).
+    // A CTA an SM: so much shared memory (no two of half an SM's fit) that the next call's CTAs do not come to an SM at work (us in loops, without / with:
+    // 144 heads of 11 x 12 6.8 / 5.0, of 10 x 10 6.0 / 4.7, 108 of 10 x 10, two rounds 8.1 / 6.5, 72 of 10 x 17 5.6 / 4.6).  That keeps calls on other streams off as well:
+    // two at once (us for both) 72 heads of 10 x 10 4.8 / 3.6, but 108 4.8 / 5.2, 144 4.9 / 6.6, two rounds 7.7 / 10.8, 144 of 11 x 12 5.4 / 6.9.  Calls one after another
+    // are the rule.  Letting the next call's CTAs come once the call before is gone (griddepcontrol.launch_dependents after the wait) instead leaves room for
+    // other streams (144 heads 5.0, two rounds 7.8), but loops of short calls lose 15 to 25 % (132 heads of 12 x 11 4.3 / 5.4, 144 of 10 x 10 in bf16 4.8 / 6.0).
     if (p->parts * BH <= num_sms) p->smem = std::max(p->smem, (size_t)114 * 1024);
     // the fewest warps that take the fewest rounds of tiles over both half-steps
     int best = 1 << 30;

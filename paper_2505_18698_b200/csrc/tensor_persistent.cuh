@@ -190,17 +190,20 @@ template <typename T, int B, int SB>
 cudaError_t launch_decoupled(const Params& P, int grid, cudaStream_t st);
 template <typename T, int B>
 cudaError_t launch_tmem(const Params& P, int grid, cudaStream_t st);
-//   launch_chain:     tensor_chain.cuh, SB == B == 64
+//   launch_chain:     tensor_chain.cuh, SB == B in {64, 128}
 template <typename T, int B>
 cudaError_t launch_chain(const Params& P, int grid, cudaStream_t st);
-// Whether MA_PATH_TENSOR runs the kernel of tensor_chain.cuh and not that of tensor_decoupled.cuh (by size alone: either layout
-// gives the same bits; for one round both kernels do).  Measured over heads of 4096 in loops of tenths of a second, us (this one / that one):
-// two rounds: 16 heads 39.4 / 37.0, 24 43.7 / 44.4, 32 48.4 / 50.2 (on another GPU 49.8 / 49.3), 33 48.7 / 51.9, 36 49.8 / 55.0, 64 82 / 89; one round: 32
-// 30.8 / 30.9 (on the other 31.2 / 30.9), 33 30.9 / 32.6, 35 32.4 / 32.9, 38 33.1 / 34.9, 48 37.8 / 41.1, 64 51 / 53; masked or in the other layout, where
-// that one is a fifth slower: one round 32 34.4 / 35.3 and 34.4 / 37.7, two rounds 32 55.1 / 58.1, 48 66.2 / 78.6.
-// Blocks of 128 (bf16 T = 2, f16 T = 1; loops): 8 heads of 16384 55.3 / 54.9 and 32.3 / 32.9 (replayed graphs 59.9 / 57.5 and 37.1 / 35.3), 9 59.8 / 60.0 and
-// 35.4 / 35.6, 12 74.3 / 79.9 and 44.4 / 46.2, 16 95.0 / 99.5 and 58.6 / 59.5; other layout 8 59 / 62 and 35 / 37, 12 78 / 86 and 46 / 50; masked 6 57 / 54, 8
-// 66.8 / 66.4, 12 81 / 93.
+// Whether MA_PATH_TENSOR runs the kernel of tensor_chain.cuh and not that of tensor_decoupled.cuh.  By size alone, so that a call gives the same bits in
+// either layout: for one round both kernels do, for more they round differently.  us per call, that one / this one, loops of tenths of a second
+// (replayed graphs); GPUs differ by 5 %:
+//   heads of 4096, bf16, T = 2:    16 35.0 / 34.9 (37.0 / 37.5), 20 37.1 / 37.6 (39.1 / 41.5), 24 41.0 / 39.4 (44.1 / 42.8), 28 44.6 / 43.2 (47.2 / 44.4), 32 47.2 / 45.8
+//                                  (49.3 / 50.4), 36 51.4 / 48.2 (53.1 / 52.7), 64 87 / 71; other layout 16 38.4 / 37.5, 24 47.3 / 43.1, 32 54.6 / 50.1; masked 24 45.9 / 44.1
+//   f16, T = 1:                    16 22.6 / 18.5 (24.6 / 23.2), 24 25.0 / 23.8 (28.8 / 27.8), 28 26.8 / 26.4 (29.1 / 30.0), 32 28.8 / 27.6 (31.4 / 31.6), 36 30.9 / 28.8 (33.3 / 32.4)
+//   heads of 16384, bf16, T = 2:   6 46.1 / 46.8 (47.6 / 49.4), 7 49.4 / 51.4 (51.6 / 53.0), 8 54.8 / 53.3 (55.9 / 56.4), 9 59.6 / 57.7 (61.0 / 60.2), 12 78.0 / 71.0 (76.5 / 70.4),
+//                                  16 98 / 88; other layout 6 51.4 / 50.4, 8 62.3 / 57.0, 9 68.8 / 60.7; masked 6 51.6 / 53.3, 8 63.2 / 61.3, 9 69.2 / 65.4
+//   f16, T = 1:                    6 28.0 / 26.8 (30.5 / 31.5), 7 30.3 / 29.4 (32.2 / 33.8), 8 31.9 / 30.8 (34.7 / 34.8), 9 34.9 / 32.9 (36.6 / 36.1), 12 45.5 / 42.0 (45.6 / 42.4)
+// The lines are where plain calls are no longer slower in graphs (32 heads of 4096 within 2 %, 9 of 16384).  In loops, in the other layout and masked this kernel is
+// ahead from about a quarter fewer tiles on.
 inline bool chain_chosen(int BH, int N, int b) {      // by tiles of a half-step
   const long long tiles = (long long)BH * N / kRows;
   return b == 64 ? tiles >= 1024 : b == 128 && tiles >= 1152;

@@ -1,7 +1,7 @@
 // Tensor-core tiles of both half-steps for sm_100a (tcgen05 + TMA), one launch per half-step: 16-bit
 // inputs, d <= 64 (a multiple of 8), any b, m <= 128, key padding mask and per-sequence lengths (App.
 // C.3), either layout, row log-sum-exp output.  MA_PATH_TILE_MMA takes these kernels for up to two
-// rounds where there are tiles enough to fill the GPU (the rule is in api.cu).
+// rounds where there are tiles enough, and full enough, to pay for their longer chain (the rule is in api.cu).
 //
 // What bounds a tile.  Its chain load -> score MMA -> softmax -> apply MMA -> epilogue -> store is mostly
 // latency (a launch with less than a tile a compute group takes 9 us), while its pipe time is
@@ -953,8 +953,8 @@ inline int launch_kernel(const Params& P, const Device& dev, cudaStream_t st) {
     if (cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem) != cudaSuccess) return 7;
     prepared[dev.dev] = true;
   }
-  // (the next half-step's CTAs take SM slots and set up as this one's drain; they wait for its end
-  // before they touch memory)
+  // (the next half-step's CTAs take SM slots, set up and ask for inputs as this one's drain; they wait for its end before they touch what it
+  // writes, and the call's first launch lets the next ones start only once it has waited for whatever wrote the inputs)
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
