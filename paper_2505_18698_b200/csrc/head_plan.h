@@ -95,7 +95,7 @@ inline bool plan(int b, int m, int T, int BH, int num_sms, Plan* p) {
     if (p->parts == 2) most = 16;
     // A CTA an SM: so much shared memory (no two of half an SM's fit) that the next call's CTAs do not come to an SM at work (us in loops, without / with:
     // 144 heads of 11 x 12 6.8 / 5.0, of 10 x 10 6.0 / 4.7, 108 of 10 x 10, two rounds 8.1 / 6.5, 72 of 10 x 17 5.6 / 4.6).  That keeps calls on other streams off as well:
-    // two at once (us for both) 72 heads of 10 x 10 4.8 / 3.6, but 108 4.8 / 5.2, 144 4.9 / 6.6, two rounds 7.7 / 10.8, 144 of 11 x 12 5.4 / 6.9.  Calls one after another
+    // two at once (us for both) 72 heads of 10 x 10 4.8 / 3.6, but 108 4.8 / 5.2, 144 4.9 / 6.6, two rounds 7.7 / 10.8, 144 of 12 x 11 5.4 / 6.9.  Calls one after another
     // are the rule.  Letting the next call's CTAs come once the call before is gone (griddepcontrol.launch_dependents after the wait) instead leaves room for
     // other streams (144 heads 5.0, two rounds 7.8), but loops of short calls lose 15 to 25 % (132 heads of 12 x 11 4.3 / 5.4, 144 of 10 x 10 in bf16 4.8 / 6.0).
     if (p->parts * BH <= num_sms) p->smem = std::max(p->smem, (size_t)114 * 1024);
