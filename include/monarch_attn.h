@@ -123,7 +123,8 @@ int monarch_attn_fwd_ex(const void* Q, const void* K, const void* V, void* Y,
  * than a few megabytes is cut into two or three chunks of units: a chunk's kernels and the copy of its
  * result run on two streams owned by the library while the next chunk's inputs come in on `stream`
  * (fork and join by events, so work queued on `stream` after the call still sees Y_host complete).
- * Where the kernels write each row of Y once (short sequences) and Y_host is pinned from its first byte to its
+ * A chunk runs on the kernels of the device call of all units, so that Y_host has its bits whatever the cut (fp32: to the last
+ * bits).  Where the kernels write each row of Y once (short sequences) and Y_host is pinned from its first byte to its
  * last, they write it directly instead of a copy back.  Grows the staging buffers on demand.  If a copy or a
  * launch fails, the status is returned, Y_host is undefined and `stream` is still ordered after what was queued. */
 int monarch_attn_fwd_host(const void* Q_host, const void* K_host, const void* V_host, void* Y_host,
